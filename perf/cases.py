@@ -1,0 +1,504 @@
+"""The workloads whose speed and accuracy are tracked on the GPU.
+
+Each case is one call (or one short sequence of calls) that a program using
+this library makes: BVP solves of different sizes, precisions and execution
+forms, solves through the resident pool, evaluations of the feedback
+interpolant in its three arithmetics, closed-loop simulations, and the whole
+off-line phase with the evaluation that follows it.  `exact` restates the
+discrete problem in plain 64-bit torch (no code of the library): the
+collocation root by damped Newton with a backward Riccati sweep over the
+condensed block rows, and the sparse-grid interpolant from the product form of
+its basis.
+"""
+from __future__ import annotations
+
+import math
+from types import SimpleNamespace
+
+import numpy as np
+import torch
+
+from paper_1507_04769_gb300 import sg
+
+DEV = "cuda"
+HALF = math.pi / 4.0                       # the box is [-pi/4, pi/4]^6
+PRECISION = {"fp64": sg.PREC_FP64, "mixed": sg.PREC_MIXED, "pair": sg.PREC_MIXED_PAIR}
+MODE = {"fp64": sg.EVAL_FP64, "df32": sg.EVAL_DF32, "tf32x3": sg.EVAL_TF32X3}
+GRID_NODES = {2: 85, 3: 389, 4: 1457, 5: 4865}   # d = 6
+NEWTON = {"attitude": 5, "lq": 1}          # typical Newton iterations per solve
+
+
+# ------------------------------------------------------------------ the cases
+def listed():
+    return [
+        # one state solved on its own, as an on-line controller or validation does
+        {"name": "solve_one_mixed", "what": "solve", "problem": "attitude", "precision": "mixed", "n": 1,
+         "mesh": "single", "graph": 1, "kept": True},
+        # the plain method: the level-2 node count, FP64, the default call with nothing preallocated
+        {"name": "solve_plain_85_fp64", "what": "solve", "problem": "attitude", "precision": "fp64", "n": 85,
+         "mesh": "single", "graph": 0, "kept": False},
+        # the linear-quadratic check at the level-3 node count, T = 10
+        {"name": "solve_lq_389_fp64", "what": "solve", "problem": "lq", "precision": "fp64", "n": 389,
+         "mesh": "short", "graph": 1, "kept": True},
+        # the batching form at the level-4 node count in FP64: horizons {10, 20, 40}, a graph per mesh size
+        {"name": "solve_batch_1457_fp64", "what": "solve", "problem": "attitude", "precision": "fp64", "n": 1457,
+         "mesh": "three", "graph": 2, "kept": True},
+        # a batch of arbitrary horizons: a different mesh size for nearly every node
+        {"name": "solve_ragged_777_pair", "what": "solve", "problem": "attitude", "precision": "pair", "n": 777,
+         "mesh": "ragged", "graph": 1, "kept": True},
+        # serving: two batches of states through the resident pool, the second joining the first
+        {"name": "pool_401_mixed", "what": "pool", "problem": "attitude", "precision": "mixed", "n": 401,
+         "mesh": "three"},
+        # the evaluation of the plain method: 1e4 queries of the level-2 interpolant in FP64
+        {"name": "eval_fp64_L2_10k", "what": "eval", "level": 2, "mode": "fp64", "queries": 10_000},
+        # the FP64 arm of the precision form: 1e6 queries of the level-4 interpolant
+        {"name": "eval_fp64_L4_1m", "what": "eval", "level": 4, "mode": "fp64", "queries": 1_000_000},
+        # the largest serving evaluation: 1e5 queries (a ragged count) of the level-5 interpolant, pairs of floats
+        {"name": "eval_df32_L5_100k", "what": "eval", "level": 5, "mode": "df32", "queries": 99_991},
+        # the precision form on the tensor cores: 1e6 queries of the level-4 interpolant
+        {"name": "eval_tf32x3_L4_1m", "what": "eval", "level": 4, "mode": "tf32x3", "queries": 1_000_000},
+        # serving: closed loops of 2000 steps from the level-4 feedback
+        {"name": "closed_loop_256_L4", "what": "loop", "level": 4, "mode": "df32", "n": 256, "steps": 2000},
+        # the whole path as the benchmark steps it: grid, level-4 mixed solves, surpluses, 1e6 evaluations
+        {"name": "offline_L4_mixed", "what": "offline", "level": 4, "precision": "mixed", "mode": "tf32x3",
+         "queries": 1_000_000},
+    ]
+
+
+def _log_int(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    """A case of the same ranges as the listed ones."""
+    what = rng.choice(["solve", "solve", "solve", "pool", "eval", "eval", "eval", "loop", "offline"])
+    if what == "solve":
+        precision = rng.choice(["fp64", "mixed", "pair"])
+        mesh = rng.choice(["single", "short", "three", "ragged"])
+        graph = rng.choice([0, 1, 2]) if mesh == "three" else rng.choice([0, 1])
+        return {"what": "solve", "problem": rng.choice(["attitude", "attitude", "lq"]), "precision": precision,
+                "n": _log_int(rng, 1, 1457 if precision == "fp64" else 4096), "mesh": mesh, "graph": graph,
+                "kept": rng.random() < 0.75}
+    if what == "pool":
+        return {"what": "pool", "problem": "attitude", "precision": rng.choice(["mixed", "pair"]),
+                "n": _log_int(rng, 2, 1024), "mesh": "three"}
+    if what == "eval":
+        level = rng.choice([2, 3, 4, 5])
+        mode = rng.choice(["fp64", "df32", "tf32x3"])
+        most = 1_000_000 if level < 5 else 100_000
+        return {"what": "eval", "level": level, "mode": mode, "queries": _log_int(rng, 1, most)}
+    if what == "loop":
+        level = rng.choice([2, 3, 4])
+        steps = rng.randint(200, 2000)
+        most = max(1, min(1024, 256 * 2000 * 1457 // (steps * GRID_NODES[level])))
+        return {"what": "loop", "level": level, "mode": rng.choice(["df32", "df32", "fp64"]),
+                "n": _log_int(rng, 1, most), "steps": steps}
+    return {"what": "offline", "level": rng.choice([2, 3, 4]), "precision": rng.choice(["mixed", "pair"]),
+            "mode": rng.choice(["df32", "tf32x3"]), "queries": _log_int(rng, 1_000, 1_000_000)}
+
+
+# ------------------------------------------------------------------ inputs
+def _params(problem, seed):
+    """Attitude: J = diag(2, 3, 4), a momentum vector of length one, B near the
+    identity.  LQ: a matrix shifted to spectral abscissa -0.1."""
+    rng = np.random.default_rng([11, seed])
+    if problem == "attitude":
+        h = rng.standard_normal(3)
+        B = np.eye(3) + rng.uniform(-0.1, 0.1, (3, 3)) * (1.0 - np.eye(3))
+        return SimpleNamespace(kind=sg.PROBLEM_ATTITUDE, J=np.array([2.0, 3.0, 4.0]), hmom=h / np.linalg.norm(h),
+                               B=B, wv=1.0, ww=1.0, r=0.1, tv=1.0, tw=1.0)
+    A = rng.standard_normal((6, 6))
+    A -= (np.linalg.eigvals(A).real.max() + 0.1) * np.eye(6)
+    return SimpleNamespace(kind=sg.PROBLEM_LQ, A=A, B=rng.standard_normal((6, 3)), Q=np.eye(6), R=0.1 * np.eye(3),
+                           QT=np.eye(6))
+
+
+def _horizons(mesh, n, seed):
+    """Horizons and mesh sizes of n nodes; one mesh width, 5/32, throughout."""
+    rng = np.random.default_rng([12, seed])
+    if mesh == "single":
+        T = np.full(n, 20.0)
+    elif mesh == "short":
+        T = np.full(n, 10.0)
+    elif mesh == "three":
+        T = rng.choice(np.array([10.0, 20.0, 40.0]), n)
+    else:
+        T = rng.uniform(5.0, 40.0, n)
+    return T, np.maximum(1, np.rint(6.4 * T)).astype(np.int32)
+
+
+def _states(n, seed):
+    return np.random.default_rng([13, seed]).uniform(-HALF, HALF, (n, 6))
+
+
+def _queries(n, seed):
+    """Half uniform on the box, half N(0, 0.2^2) clipped to it."""
+    rng = np.random.default_rng([14, seed])
+    x = rng.uniform(-HALF, HALF, (n, 6))
+    near = rng.random(n) < 0.5
+    x[near] = np.clip(0.2 * rng.standard_normal((int(near.sum()), 6)), -HALF, HALF)
+    return x
+
+
+def _feedback_values(x, seed):
+    """A smooth stabilising feedback (three controls) at states x (n, 6)."""
+    rng = np.random.default_rng([15, seed])
+    kv = torch.as_tensor(2.5 * np.eye(3) + 0.3 * rng.standard_normal((3, 3)), device=x.device)
+    kw = torch.as_tensor(4.0 * np.eye(3) + 0.3 * rng.standard_normal((3, 3)), device=x.device)
+    a = torch.as_tensor(0.4 * rng.standard_normal((6, 3)), device=x.device)
+    return -(torch.sin(x[:, :3]) @ kv + x[:, 3:] @ kw) * (1.0 + 0.1 * torch.cos(x @ a))
+
+
+def _t(a, dtype=torch.float64):
+    return torch.as_tensor(a, dtype=dtype, device=DEV)
+
+
+def _outputs(n):
+    f = dict(dtype=torch.float64, device=DEV)
+    i = dict(dtype=torch.int32, device=DEV)
+    return {"lambda0": torch.empty((n, 6), **f), "u0": torch.empty((n, 3), **f), "V": torch.empty((n,), **f),
+            "status": torch.empty((n,), **i), "iters": torch.empty((n,), **i)}
+
+
+def _workspace(n, n_max, precision):
+    return torch.empty(sg.workspace_bytes(n, n_max, precision), dtype=torch.uint8, device=DEV)
+
+
+def prepare(case, seed):
+    what = case["what"]
+    box = (np.full(6, -HALF), np.full(6, HALF))
+    if what in ("solve", "pool"):
+        n, precision = case["n"], PRECISION[case["precision"]]
+        T, N = _horizons(case["mesh"], n, seed)
+        st = {"case": case, "problem": sg.problem_from(_params(case["problem"], seed)), "x0": _t(_states(n, seed)),
+              "T": _t(T), "N": _t(N, torch.int32), "precision": precision}
+        if what == "pool":
+            st["pool"] = sg.SolverPool(st["problem"], max(64, n), 256, precision=precision)
+        elif case["kept"]:
+            # a program that solves again and again keeps its workspace and outputs
+            st["keep"] = {"n_max": int(N.max()), "workspace": _workspace(n, int(N.max()), precision),
+                          "out": _outputs(n)}
+        else:
+            st["keep"] = {}
+        return st
+    if what in ("eval", "loop"):
+        grid = sg.Grid(6, case["level"], *box)
+        st = {"case": case, "grid": grid, "surplus": sg.Surplus(grid, _feedback_values(grid.coords, seed))}
+        if what == "eval":
+            st["xq"] = _t(_queries(case["queries"], seed))
+        else:
+            st["problem"] = sg.problem_from(_params("attitude", seed))
+            st["x0"] = _t(_states(case["n"], seed))
+        return st
+    M, precision = GRID_NODES[case["level"]], PRECISION[case["precision"]]
+    T, N = _horizons("three", M, seed)
+    return {"case": case, "box": box, "problem": sg.problem_from(_params("attitude", seed)), "T": _t(T),
+            "N": _t(N, torch.int32), "precision": precision, "x0": _t(np.zeros((M, 6))), "out": _outputs(M),
+            "workspace": _workspace(M, int(N.max()), precision), "n_max": int(N.max()),
+            "xq": _t(_queries(case["queries"], seed))}
+
+
+# ------------------------------------------------------------------ one pass
+def run(state):
+    case = state["case"]
+    what = case["what"]
+    if what == "solve":
+        return sg.solve_bvps(state["problem"], state["x0"], state["T"], state["N"], precision=state["precision"],
+                             graph=case["graph"], **state["keep"])
+    if what == "pool":
+        pool, n = state["pool"], case["n"]
+        first = (n + 1) // 2
+        slots = [pool.admit(state["x0"][:first], state["T"][:first], state["N"][:first])]
+        pool.iterate()
+        pool.iterate()
+        slots.append(pool.admit(state["x0"][first:], state["T"][first:], state["N"][first:]))
+        while pool.iterate():
+            pass
+        return pool.collect(np.concatenate(slots))
+    if what == "eval":
+        return sg.eval_feedback(state["surplus"], state["xq"], mode=MODE[case["mode"]])
+    if what == "loop":
+        return sg.simulate_closed_loop(state["problem"], state["surplus"], state["x0"], case["steps"], 0.01,
+                                       mode=MODE[case["mode"]])
+    grid = sg.Grid(6, case["level"], *state["box"])
+    state["x0"].copy_(grid.coords)
+    out = sg.solve_bvps(state["problem"], state["x0"], state["T"], state["N"], precision=state["precision"], graph=2,
+                        n_max=state["n_max"], workspace=state["workspace"], out=state["out"])
+    surplus = sg.Surplus(grid, out["u0"])
+    u = sg.eval_feedback(surplus, state["xq"], mode=MODE[case["mode"]])
+    return {**out, "W": surplus.W.clone(), "u": u}
+
+
+# ------------------------------------------------------------------ work of one pass
+def _solve_work(problem, intervals, n):
+    """Per interval and Newton iteration: three points' right-hand side and
+    Jacobian (about 250 + 700 flops each), and the elimination of the two
+    interior stages, the block rows and the recovery (about 20,000)."""
+    return {"bytes": n * (6 + 1 + 6 + 3 + 1) * 8 + n * 12, "flops": NEWTON[problem] * intervals * (3 * 950 + 20_000)}
+
+
+def _eval_flops(M, k=3):
+    """The sum over the nodes nested by dimension: k multiply-adds per node."""
+    return M * 2 * k
+
+
+def work(case):
+    what = case["what"]
+    mean = {"single": 128.0, "short": 64.0, "three": 6.4 * 70.0 / 3.0, "ragged": 6.4 * 22.5}
+    if what in ("solve", "pool"):
+        return _solve_work(case["problem"], case["n"] * mean[case["mesh"]], case["n"])
+    M = GRID_NODES[case["level"]]
+    if what == "eval":
+        q = case["queries"]
+        return {"bytes": q * 9 * 8 + M * 3 * 8, "flops": q * _eval_flops(M)}
+    if what == "loop":
+        n = case["n"]
+        return {"bytes": n * 13 * 8 + M * 3 * 8, "flops": n * case["steps"] * (_eval_flops(M) + 4 * 120)}
+    s = _solve_work("attitude", M * mean["three"], M)
+    q = case["queries"]
+    return {"bytes": s["bytes"] + q * 9 * 8 + 2 * M * 3 * 8, "flops": s["flops"] + q * _eval_flops(M)}
+
+
+# ------------------------------------------------------------------ exact values (plain 64-bit torch)
+def _f0(p, x):
+    """Uncontrolled dynamics of the two problem families."""
+    if p.kind == sg.PROBLEM_LQ:
+        return x @ _t(p.A).T
+    (sp, st, ss), (cp, ct, cs) = torch.sin(x[..., :3]).unbind(-1), torch.cos(x[..., :3]).unbind(-1)
+    w1, w2, w3 = x[..., 3], x[..., 4], x[..., 5]
+    a = sp * w2 + cp * w3
+    h0, h1, h2 = (float(v) for v in p.hmom)
+    z0, z1 = cs * h0 + ss * h1, cs * h1 - ss * h0
+    y0, y2 = ct * z0 - st * h2, st * z0 + ct * h2
+    g0, g1, g2 = y0, cp * z1 + sp * y2, cp * y2 - sp * z1
+    return torch.stack([w1 + st / ct * a, cp * w2 - sp * w3, a / ct, (g1 * w3 - g2 * w2) / p.J[0],
+                        (g2 * w1 - g0 * w3) / p.J[1], (g0 * w2 - g1 * w1) / p.J[2]], -1)
+
+
+def _matrices(p):
+    """Plant input matrix (6 x 3), control weight, state weight, terminal weight."""
+    if p.kind == sg.PROBLEM_LQ:
+        return _t(p.B), _t(p.R), _t(p.Q), _t(p.QT)
+    Bu = np.zeros((6, 3))
+    Bu[3:] = p.B / p.J[:, None]
+    return _t(Bu), p.r * torch.eye(3, dtype=torch.float64, device=DEV), _t(np.diag([p.wv] * 3 + [p.ww] * 3)), \
+        _t(np.diag([p.tv] * 3 + [p.tw] * 3))
+
+
+def _characteristics(p, Y, jac):
+    """F = (H_lambda, -H_x) at Y (..., 12), and its Jacobian if asked."""
+    Bu, R, Q, _ = _matrices(p)
+    K = Bu @ torch.linalg.solve(R, Bu.T)
+    with torch.enable_grad():
+        y = Y.detach().clone().requires_grad_(True)
+        x, lam = y[..., :6], y[..., 6:]
+        H = 0.5 * ((x @ Q) * x).sum(-1) + (lam * _f0(p, x)).sum(-1) - 0.5 * ((lam @ K) * lam).sum(-1)
+        g, = torch.autograd.grad(H.sum(), y, create_graph=jac)
+        F = torch.cat([g[..., 6:], -g[..., :6]], -1)
+        if not jac:
+            return F.detach(), None
+        rows = [torch.autograd.grad(F[..., i].sum(), y, retain_graph=i < 11)[0] for i in range(12)]
+    return F.detach(), torch.stack(rows, -2)
+
+
+_S5 = math.sqrt(5.0)
+_LOBATTO = np.array([[(11 + _S5) / 120, (25 - _S5) / 120, (25 - 13 * _S5) / 120, (-1 + _S5) / 120],
+                     [(11 - _S5) / 120, (25 + 13 * _S5) / 120, (25 + _S5) / 120, (-1 - _S5) / 120],
+                     [1 / 12, 5 / 12, 5 / 12, 1 / 12]])
+
+
+def _stage(Y):
+    """Points (n, 3N + 1, c) as intervals (n, N, 4, c)."""
+    return torch.cat([Y[:, :-1].unflatten(1, (-1, 3)), Y[:, 3::3].unsqueeze(2)], 2)
+
+
+def _bvp_root(p, x0, T, N):
+    """The discrete Lobatto IIIA root at every node (intervals past a node's N
+    have width 0, so that all nodes share one layout)."""
+    n, Nm = len(N), int(N.max())
+    x0, A = _t(x0), _t(_LOBATTO)
+    Bu, R, Q, QT = _matrices(p)
+    h = _t(T / N)[:, None] * (torch.arange(Nm, device=DEV)[None, :] < _t(N, torch.int64)[:, None])
+    eye = torch.eye(12, dtype=torch.float64, device=DEV)
+
+    def residual(Y, F):
+        S = _stage(Y)
+        r = S[:, :, 1:] - S[:, :, :1] - h[..., None, None] * torch.einsum("kj,nijc->nikc", A, _stage(F))
+        ends = torch.cat([Y[:, 0, :6] - x0, Y[:, -1, 6:] - Y[:, -1, :6] @ QT], -1)
+        return r, ends
+
+    def norms(r, ends):
+        return (r * r).sum((1, 2, 3)) + (ends * ends).sum(-1), \
+            torch.maximum(r.abs().amax((1, 2, 3)), ends.abs().amax(-1))
+
+    Y = torch.cat([x0, torch.zeros_like(x0)], -1)[:, None, :].repeat(1, 3 * Nm + 1, 1)
+    for _ in range(40):
+        F, J = _characteristics(p, Y, True)
+        r, ends = residual(Y, F)
+        f2, fmax = norms(r, ends)
+        active = fmax > 1e-13
+        if not bool(active.any()):
+            break
+        Js = _stage(J.flatten(2)).unflatten(-1, (12, 12))
+        # rows: stages 2, 3, 4; columns: points 1 (y_i), 2, 3 (interior), 4 (y_{i+1})
+        blocks = -h[..., None, None, None, None] * torch.einsum("kj,nijab->nikajb", A, Js)
+        for k in range(3):
+            blocks[:, :, k, :, k + 1, :] += eye
+            blocks[:, :, k, :, 0, :] -= eye
+        inner = blocks[:, :, :2, :, 1:3, :].reshape(n, Nm, 24, 24)
+        outer = torch.cat([blocks[:, :, :2, :, 0, :].reshape(n, Nm, 24, 12),
+                           blocks[:, :, :2, :, 3, :].reshape(n, Nm, 24, 12), -r[:, :, :2].reshape(n, Nm, 24, 1)], -1)
+        X = torch.linalg.solve(inner, outer)
+        last = torch.cat([blocks[:, :, 2, :, 0, :], blocks[:, :, 2, :, 3, :], -r[:, :, 2].unsqueeze(-1)], -1) - \
+            blocks[:, :, 2, :, 1:3, :].reshape(n, Nm, 12, 24) @ X
+        # backward sweep: dlambda_i = P dx_i + q
+        P, q = QT.expand(n, 6, 6), -ends[:, 6:]
+        steps = [None] * Nm
+        for i in range(Nm - 1, -1, -1):
+            S, Tn, rr = last[:, i, :, :12], last[:, i, :, 12:24], last[:, i, :, 24]
+            M = torch.cat([S[..., 6:], Tn[..., :6] + Tn[..., 6:] @ P], -1)
+            rhs = torch.cat([-S[..., :6], (rr - (Tn[..., 6:] @ q[..., None])[..., 0])[..., None]], -1)
+            sol = torch.linalg.solve(M, rhs)
+            steps[i] = (P, q, sol)
+            P, q = sol[:, :6, :6], sol[:, :6, 6]
+        dx = -ends[:, :6]
+        dy = [torch.cat([dx, (P @ dx[..., None])[..., 0] + q], -1)]
+        for i in range(Nm):
+            Pn, qn, sol = steps[i]
+            dx = (sol[:, 6:, :6] @ dx[..., None])[..., 0] + sol[:, 6:, 6]
+            dy.append(torch.cat([dx, (Pn @ dx[..., None])[..., 0] + qn], -1))
+        dy = torch.stack(dy, 1)
+        z = torch.cat([dy[:, :-1], dy[:, 1:], torch.ones((n, Nm, 1), dtype=torch.float64, device=DEV)], -1)
+        z[..., :24] *= -1.0
+        inner_d = (X @ z[..., None])[..., 0].unflatten(-1, (2, 12))
+        D = torch.cat([torch.cat([dy[:, :-1, None], inner_d], 2).flatten(1, 2), dy[:, -1:]], 1)
+        # Armijo steps 1, 1/2, ..., 2^-10; a node whose residual is at rounding level takes the full step
+        alpha = torch.ones(n, dtype=torch.float64, device=DEV)
+        for trial in range(11):
+            Yt = Y + alpha[:, None, None] * D
+            t2, _ = norms(*residual(Yt, _characteristics(p, Yt, False)[0]))
+            ok = (t2 <= (1 - 2e-4 * alpha) * f2) | (fmax < 1e-9) | ~active
+            if bool(ok.all()) or trial == 10:
+                break
+            alpha = torch.where(ok, alpha, 0.5 * alpha)
+        step = D * (alpha * active)[:, None, None]
+        Y = Y + step
+        if float(step.abs().max()) < 1e-14:
+            break
+    lam = Y[..., 6:]
+    u = -torch.linalg.solve(R, Bu.T) @ lam[..., None]
+    u = u[..., 0]
+    L = 0.5 * (((Y[..., :6] @ Q) * Y[..., :6]).sum(-1) + ((u @ R) * u).sum(-1))
+    z = torch.einsum("j,nij,ni->n", A[2], _stage(L[..., None])[..., 0], h)
+    xT = Y[:, -1, :6]
+    return {"lambda0": lam[:, 0].clone(), "u0": u[:, 0].clone(), "V": z + 0.5 * ((xT @ QT) * xT).sum(-1),
+            "status": None, "iters": None}
+
+
+def _sparse_grid(level, d=6):
+    """Nodes by |i|, then i, then j: unit coordinates (M, d) and 1-D function ids (M, d)."""
+    fine = [[0.5], [0.0, 1.0]]                      # increment sets of the CGL points
+    for l in range(3, level + 2):
+        fine.append([math.sin(k * math.pi / 2 ** l) ** 2 for k in range(1, 2 ** (l - 1), 2)])
+    first = np.cumsum([0] + [len(s) for s in fine])
+
+    def multi(dim, total):
+        if dim == 1:
+            yield (total,)
+            return
+        for v in range(1, total - dim + 2):
+            for rest in multi(dim - 1, total - v):
+                yield (v,) + rest
+
+    ids = []
+    for total in range(d, d + level + 1):
+        for mi in multi(d, total):
+            axes = [np.arange(first[l - 1], first[l]) for l in mi]
+            ids.append(np.stack(np.meshgrid(*axes, indexing="ij"), -1).reshape(-1, d))
+    ids = np.concatenate(ids)
+    pts = np.concatenate([np.array(s) for s in fine])
+    level_of = np.repeat(np.arange(1, level + 2), [len(s) for s in fine])
+    return pts[ids], ids, pts, level_of
+
+
+def _basis(u, pts, level_of):
+    """Every 1-D basis function at u (...): the Lagrange polynomial of its
+    level's set that is 1 at its own point, in product form."""
+    out = []
+    for f in range(len(pts)):
+        v = torch.ones_like(u)
+        if level_of[f] > 1:
+            members = [x for g, x in enumerate(pts) if level_of[g] <= level_of[f] and g != f]
+            for x in members:
+                v = v * ((u - x) / (pts[f] - x))
+        out.append(v)
+    return torch.stack(out, -1)
+
+
+class _Interpolant:
+    def __init__(self, level):
+        self.unit, ids, self.pts, self.level_of = _sparse_grid(level)
+        self.ids = _t(ids, torch.int64)
+        self.total = _t(self.level_of, torch.int64)[self.ids].sum(-1)
+        self.coords = -HALF + (2.0 * HALF) * _t(self.unit)
+
+    def build(self, values):
+        phi = self.products(_t(self.unit))
+        W = torch.zeros_like(values)
+        for s in self.total.unique():
+            now, before = self.total == s, self.total < s
+            W[now] = values[now] - phi[now][:, before] @ W[before]
+        self.W = W
+        return self
+
+    def products(self, unit):
+        tab = _basis(unit, self.pts, self.level_of)
+        phi = tab[:, 0, :][:, self.ids[:, 0]]
+        for k in range(1, 6):
+            phi = phi * tab[:, k, :][:, self.ids[:, k]]
+        return phi
+
+    def __call__(self, x):
+        rows = max(1, 100_000_000 // len(self.ids))
+        return torch.cat([self.products((c + HALF) / (2.0 * HALF)) @ self.W for c in x.split(rows)])
+
+
+def _closed_loop(p, interp, x, steps, dt):
+    Bu, R, Q, _ = _matrices(p)
+    z = torch.zeros(len(x), dtype=torch.float64, device=DEV)
+
+    def f(x, u):
+        return _f0(p, x) + u @ Bu.T
+
+    def cost(x, u):
+        return 0.5 * (((x @ Q) * x).sum(-1) + ((u @ R) * u).sum(-1))
+
+    for _ in range(steps):
+        u = interp(x)
+        k1 = f(x, u)
+        x2 = x + 0.5 * dt * k1
+        k2 = f(x2, u)
+        x3 = x + 0.5 * dt * k2
+        k3 = f(x3, u)
+        x4 = x + dt * k3
+        k4 = f(x4, u)
+        z = z + dt / 6.0 * (cost(x, u) + 2.0 * cost(x2, u) + 2.0 * cost(x3, u) + cost(x4, u))
+        x = x + dt / 6.0 * (k1 + 2.0 * k2 + 2.0 * k3 + k4)
+    return {"xT": x, "cost": z}
+
+
+def exact(case, seed):
+    what = case["what"]
+    if what in ("solve", "pool"):
+        T, N = _horizons(case["mesh"], case["n"], seed)
+        return _bvp_root(_params(case["problem"], seed), _states(case["n"], seed), T, N)
+    interp = _Interpolant(case["level"])
+    if what in ("eval", "loop"):
+        interp.build(_feedback_values(interp.coords, seed))
+        if what == "eval":
+            return interp(_t(_queries(case["queries"], seed)))
+        return _closed_loop(_params("attitude", seed), interp, _t(_states(case["n"], seed)), case["steps"], 0.01)
+    T, N = _horizons("three", len(interp.ids), seed)
+    out = _bvp_root(_params("attitude", seed), interp.coords.cpu().numpy(), T, N)
+    interp.build(out["u0"])
+    return {**out, "W": interp.W, "u": interp(_t(_queries(case["queries"], seed)))}
