@@ -43,14 +43,15 @@ def listed():
         # the batching form at the level-4 node count in FP64: horizons {10, 20, 40}, a graph per mesh size
         {"name": "solve_batch_1457_fp64", "what": "solve", "problem": "attitude", "precision": "fp64", "n": 1457,
          "mesh": "three", "graph": 2, "kept": True},
+        # the same in the precision the benchmark solves in
+        {"name": "solve_batch_1457_mixed", "what": "solve", "problem": "attitude", "precision": "mixed", "n": 1457,
+         "mesh": "three", "graph": 2, "kept": True},
         # a batch of arbitrary horizons: a different mesh size for nearly every node
-        {"name": "solve_ragged_777_pair", "what": "solve", "problem": "attitude", "precision": "pair", "n": 777,
+        {"name": "solve_ragged_301_pair", "what": "solve", "problem": "attitude", "precision": "pair", "n": 301,
          "mesh": "ragged", "graph": 1, "kept": True},
         # serving: two batches of states through the resident pool, the second joining the first
         {"name": "pool_401_mixed", "what": "pool", "problem": "attitude", "precision": "mixed", "n": 401,
          "mesh": "three"},
-        # the evaluation of the plain method: 1e4 queries of the level-2 interpolant in FP64
-        {"name": "eval_fp64_L2_10k", "what": "eval", "level": 2, "mode": "fp64", "queries": 10_000},
         # the FP64 arm of the precision form: 1e6 queries of the level-4 interpolant
         {"name": "eval_fp64_L4_1m", "what": "eval", "level": 4, "mode": "fp64", "queries": 1_000_000},
         # the largest serving evaluation: 1e5 queries (a ragged count) of the level-5 interpolant, pairs of floats
@@ -59,9 +60,9 @@ def listed():
         {"name": "eval_tf32x3_L4_1m", "what": "eval", "level": 4, "mode": "tf32x3", "queries": 1_000_000},
         # serving: closed loops of 2000 steps from the level-4 feedback
         {"name": "closed_loop_256_L4", "what": "loop", "level": 4, "mode": "df32", "n": 256, "steps": 2000},
-        # the whole path as the benchmark steps it: grid, level-4 mixed solves, surpluses, 1e6 evaluations
-        {"name": "offline_L4_mixed", "what": "offline", "level": 4, "precision": "mixed", "mode": "tf32x3",
-         "queries": 1_000_000},
+        # the whole path as a model is rebuilt: grid, level-3 mixed solves, surpluses, 1e4 evaluations in FP64
+        {"name": "offline_L3_mixed", "what": "offline", "level": 3, "precision": "mixed", "mode": "fp64",
+         "queries": 10_000},
     ]
 
 
@@ -94,7 +95,7 @@ def draw(rng):
         return {"what": "loop", "level": level, "mode": rng.choice(["df32", "df32", "fp64"]),
                 "n": _log_int(rng, 1, most), "steps": steps}
     return {"what": "offline", "level": rng.choice([2, 3, 4]), "precision": rng.choice(["mixed", "pair"]),
-            "mode": rng.choice(["df32", "tf32x3"]), "queries": _log_int(rng, 1_000, 1_000_000)}
+            "mode": rng.choice(["df32", "fp64"]), "queries": _log_int(rng, 1_000, 1_000_000)}
 
 
 # ------------------------------------------------------------------ inputs
@@ -225,8 +226,7 @@ def run(state):
     out = sg.solve_bvps(state["problem"], state["x0"], state["T"], state["N"], precision=state["precision"], graph=2,
                         n_max=state["n_max"], workspace=state["workspace"], out=state["out"])
     surplus = sg.Surplus(grid, out["u0"])
-    u = sg.eval_feedback(surplus, state["xq"], mode=MODE[case["mode"]])
-    return {**out, "W": surplus.W.clone(), "u": u}
+    return {**out, "u": sg.eval_feedback(surplus, state["xq"], mode=MODE[case["mode"]])}
 
 
 # ------------------------------------------------------------------ work of one pass
@@ -256,7 +256,7 @@ def work(case):
         return {"bytes": n * 13 * 8 + M * 3 * 8, "flops": n * case["steps"] * (_eval_flops(M) + 4 * 120)}
     s = _solve_work("attitude", M * mean["three"], M)
     q = case["queries"]
-    return {"bytes": s["bytes"] + q * 9 * 8 + 2 * M * 3 * 8, "flops": s["flops"] + q * _eval_flops(M)}
+    return {"bytes": s["bytes"] + q * 9 * 8, "flops": s["flops"] + q * _eval_flops(M)}
 
 
 # ------------------------------------------------------------------ exact values (plain 64-bit torch)
@@ -501,4 +501,4 @@ def exact(case, seed):
     T, N = _horizons("three", len(interp.ids), seed)
     out = _bvp_root(_params("attitude", seed), interp.coords.cpu().numpy(), T, N)
     interp.build(out["u0"])
-    return {**out, "W": interp.W, "u": interp(_t(_queries(case["queries"], seed)))}
+    return {**out, "u": interp(_t(_queries(case["queries"], seed)))}
