@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "bvp_direction.cuh"
 #include "bvp_kernels.cuh"
 #include "bvp_persistent.cuh"
 #include "common.cuh"
@@ -177,21 +178,12 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
                      double* V, int32_t* status, int32_t* iters, double* Yout) {
   const int64_t P = npts(a.Nmax);
   const int64_t npoint = a.n * P;
-  const int64_t nint = a.n * a.Nmax;
   const unsigned gp = static_cast<unsigned>(ceil_div(npoint, 128));
   const unsigned gupd = static_cast<unsigned>(ceil_div(npoint * kUpdPer, 128));
   const unsigned ginit = static_cast<unsigned>(ceil_div(npoint * kInitPer, 128));
   const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
   const unsigned gnode_thr = static_cast<unsigned>(ceil_div(a.n, 128));
   const unsigned gnode_warp = static_cast<unsigned>(ceil_div(a.n * 32, 128));
-  const unsigned gwarp_int = static_cast<unsigned>(ceil_div(nint, 4));
-  const unsigned gwarp_node = static_cast<unsigned>(ceil_div(a.n, 4));
-  const unsigned gwarp_seg = static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), 4));
-  const unsigned gseg_blk = static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), seg_warps<T>()));
-  const size_t cond_smem = sizeof(double) * kCondWarps * 36 * kCols;
-  if constexpr (sizeof(T) == sizeof(double)) {
-    SG_CUDA_TRY(ensure_dynamic_smem(k_condense_smem, static_cast<int>(cond_smem)));
-  }
   if (a.persistent) {
     // one warp per node, nodes from a device queue, no host round trip
     const int smem = 4 * persist_smem_per_warp<T>();
@@ -213,6 +205,9 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
     if (a.sync_at_end) SG_CUDA_TRY(cudaStreamSynchronize(st));
     return SG_OK;
   }
+  SG_CUDA_TRY(direction_setup<T>(a));
+  DirLaunch dir[kDirLaunches<T>];
+  direction_launches<T>(a, dir);
   int h_cnt[2] = {0, 0};
   auto read_counters = [&]() -> int {
     cudaError_t e = cudaMemcpyAsync(h_cnt, w.counters, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -230,24 +225,17 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
   if ((rc = read_counters()) != SG_OK) return rc;
   int active = h_cnt[1];
   for (int it = 0; it < a.max_iter && active > 0; ++it) {
-    SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 2 * sizeof(int), st));
+    SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, kCounters * sizeof(int), st));
     if (!a.jac_in_trial) SG_TIMED(kname<T>("k_point"), st, (k_point<T><<<gp, 128, 0, st>>>(a, w)));   // else stored by the last trial
-    if constexpr (sizeof(T) == sizeof(float)) {
-      const int cw = condense_reg_warps(a.cond_warps);
-      SG_TIMED("k_condense_reg_fp32", st,
-               (condense_reg_kernel(cw)<<<static_cast<unsigned>(ceil_div(nint, cw)), 32 * cw, 0, st>>>(a, w)));
-    } else {
-      SG_TIMED("k_condense_smem_fp64", st,
-               (k_condense_smem<<<static_cast<unsigned>(ceil_div(nint, kCondWarps)), 32 * kCondWarps, cond_smem,
-                                  st>>>(a, w)));
-    }
-    SG_TIMED(kname<T>("k_abd_seg"), st, (k_abd_seg<T><<<gseg_blk, 32 * seg_warps<T>(), 0, st>>>(a, w)));
-    SG_TIMED(kname<T>("k_abd_red"), st, (k_abd_red<T><<<gwarp_node, 128, 0, st>>>(a, w)));
-    SG_TIMED(kname<T>("k_abd_segback"), st, (k_abd_segback<T><<<gwarp_seg, 128, 0, st>>>(a, w)));
-    SG_TIMED(kname<T>("k_recover"), st, (k_recover<T><<<gwarp_int, 128, 0, st>>>(a, w)));
+    for (const DirLaunch& d : dir)
+      SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
     SG_TIMED("k_ls_begin", st, (k_ls_begin<<<gnode_thr, 128, 0, st>>>(a, w)));
     SG_LAUNCH_CHECK("newton kernels");
-    for (int trial = 0; trial < 12; ++trial) {
+    for (int trial = 0; trial < 13; ++trial) {   // alpha = 1, 1/2, ..., 2^-10 (and one at 0 in the FP64 form)
+      if constexpr (sizeof(T) == sizeof(double)) {
+        const DirLaunch d = elim_launch(a);
+        SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
+      }
       SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, sizeof(int), st));
       SG_TIMED("k_trial", st, (trial_kernel<T>(a)<<<gi, 128, 0, st>>>(a, w)));
       SG_TIMED("k_ls_reduce", st, (k_ls_reduce<<<gnode_warp, 128, 0, st>>>(a, w, 1)));
@@ -339,15 +327,10 @@ static cudaError_t build_solve_graph(const SolveArgs& a, const Workspace& w, dou
                                      double* V, int32_t* status, int32_t* iters, double* Yout,
                                      cudaGraph_t* out) {
   const int64_t P = npts(a.Nmax);
-  const int64_t nint = a.n * a.Nmax;
   const unsigned gp = static_cast<unsigned>(ceil_div(a.n * P, 128));
   const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
   const unsigned gnt = static_cast<unsigned>(ceil_div(a.n, 128));
   const unsigned gnw = static_cast<unsigned>(ceil_div(a.n * 32, 128));
-  const unsigned gwi = static_cast<unsigned>(ceil_div(nint, 4));
-  const unsigned gwn = static_cast<unsigned>(ceil_div(a.n, 4));
-  const unsigned gws = static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), 4));
-  const size_t cond_smem = sizeof(double) * kCondWarps * 36 * kCols;
   cudaGraph_t root;
   cudaError_t e = cudaGraphCreate(&root, 0);
   if (e != cudaSuccess) return e;
@@ -367,19 +350,12 @@ static cudaError_t build_solve_graph(const SolveArgs& a, const Workspace& w, dou
   if (rb.err != cudaSuccess) return rb.err;
 
   GraphBuilder nb{newton_body, {}};
-  nb.memset0(w.counters, 2 * sizeof(int));
+  nb.memset0(w.counters, kCounters * sizeof(int));
   if (!a.jac_in_trial) nb.kernel(k_point<T>, gp, 128, 0, a, w);   // else stored by the last trial
-  if constexpr (sizeof(T) == sizeof(float)) {
-    const int cw = condense_reg_warps(a.cond_warps);
-    nb.kernel(condense_reg_kernel(cw), static_cast<unsigned>(ceil_div(nint, cw)), 32 * cw, 0, a, w);
-  } else {
-    nb.kernel(k_condense_smem, static_cast<unsigned>(ceil_div(nint, kCondWarps)), 32 * kCondWarps, cond_smem, a, w);
-  }
-  nb.kernel(k_abd_seg<T>, static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), seg_warps<T>())),
-            32 * seg_warps<T>(), 0, a, w);
-  nb.kernel(k_abd_red<T>, gwn, 128, 0, a, w);
-  nb.kernel(k_abd_segback<T>, gws, 128, 0, a, w);
-  nb.kernel(k_recover<T>, gwi, 128, 0, a, w);
+  if (nb.err == cudaSuccess) nb.err = direction_setup<T>(a);
+  DirLaunch dir[kDirLaunches<T>];
+  direction_launches<T>(a, dir);
+  for (const DirLaunch& d : dir) nb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
   nb.kernel(k_ls_begin, gnt, 128, 0, a, w);
   nb.kernel(k_set_cond_one, 1, 1, 0, hl);
   cudaGraph_t ls_body;
@@ -392,6 +368,10 @@ static cudaError_t build_solve_graph(const SolveArgs& a, const Workspace& w, dou
   if (nb.err != cudaSuccess) return nb.err;
 
   GraphBuilder lb{ls_body, {}};
+  if constexpr (sizeof(T) == sizeof(double)) {
+    const DirLaunch d = elim_launch(a);
+    lb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+  }
   lb.memset0(w.counters, sizeof(int));
   lb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);
   lb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 1);
@@ -475,8 +455,6 @@ static int launch_solve_graph(const SolveArgs& a, Workspace w, cudaStream_t st, 
     if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
     const int64_t want = ceil_div(a.n, 4);
     grid = static_cast<unsigned>(want < int64_t(sms) * per_sm ? want : int64_t(sms) * per_sm);
-  } else if constexpr (sizeof(T) == sizeof(double)) {
-    SG_CUDA_TRY(ensure_dynamic_smem(k_condense_smem, static_cast<int>(sizeof(double) * kCondWarps * 36 * kCols)));
   }
   // key: every byte that is baked into the graph's kernel parameters
   GraphKey key;
@@ -731,6 +709,7 @@ extern "C" int sg_solve_bvps(const sg_problem* prob, const double* d_x0, int64_t
   // the FP32 Jacobian from the FP64 residual kernel (its FP32 pipe is idle
   // beside the FP64 work) in the launch-per-phase and graph forms
   a.jac_in_trial = fp32_direction(o.precision) && !a.res_pair && !o.persistent ? 1 : 0;
+  a.tree = o.precision == SG_PREC_FP64 && !o.persistent ? 1 : 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (o.graph == 2 && !d_Y) {
     bool ran = false;
@@ -833,6 +812,7 @@ extern "C" int sg_solve_bvps_static(const sg_problem* prob, const double* d_x0, 
   a.sync_at_end = 1;
   a.Yin = o.warm_start ? d_Y : nullptr;
   a.res_pair = o.precision == SG_PREC_MIXED_PAIR ? 1 : 0;
+  a.tree = o.precision == SG_PREC_FP64 && !o.persistent ? 1 : 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // Every region the solver reads is written first in this call (k_init sets the
   // iterate, the corrections and the per-node state; the counters are zeroed
@@ -955,15 +935,10 @@ __global__ void k_pool_release(Workspace w, const int64_t* list, int64_t count) 
 template <typename T>
 static cudaError_t build_pool_graph(const SolveArgs& a, const Workspace& w, uint8_t* flags, cudaGraph_t* out) {
   const int64_t P = npts(a.Nmax);
-  const int64_t nint = a.n * a.Nmax;
   const unsigned gp = static_cast<unsigned>(ceil_div(a.n * P, 128));
   const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
   const unsigned gnt = static_cast<unsigned>(ceil_div(a.n, 128));
   const unsigned gnw = static_cast<unsigned>(ceil_div(a.n * 32, 128));
-  const unsigned gwi = static_cast<unsigned>(ceil_div(nint, 4));
-  const unsigned gwn = static_cast<unsigned>(ceil_div(a.n, 4));
-  const unsigned gws = static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), 4));
-  const size_t cond_smem = sizeof(double) * kCondWarps * 36 * kCols;
   cudaGraph_t root;
   cudaError_t e = cudaGraphCreate(&root, 0);
   if (e != cudaSuccess) return e;
@@ -973,19 +948,12 @@ static cudaError_t build_pool_graph(const SolveArgs& a, const Workspace& w, uint
   rb.memset0(w.counters, 4 * sizeof(int));
   rb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);     // new slots only (searching at alpha = 0)
   rb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 0);
-  rb.memset0(w.counters, 2 * sizeof(int));
+  rb.memset0(w.counters, kCounters * sizeof(int));
   rb.kernel(k_point<T>, gp, 128, 0, a, w);
-  if constexpr (sizeof(T) == sizeof(float)) {
-    const int cw = condense_reg_warps(a.cond_warps);
-    rb.kernel(condense_reg_kernel(cw), static_cast<unsigned>(ceil_div(nint, cw)), 32 * cw, 0, a, w);
-  } else {
-    rb.kernel(k_condense_smem, static_cast<unsigned>(ceil_div(nint, kCondWarps)), 32 * kCondWarps, cond_smem, a, w);
-  }
-  rb.kernel(k_abd_seg<T>, static_cast<unsigned>(ceil_div(a.n * seg_count(a.Nmax), seg_warps<T>())),
-            32 * seg_warps<T>(), 0, a, w);
-  rb.kernel(k_abd_red<T>, gwn, 128, 0, a, w);
-  rb.kernel(k_abd_segback<T>, gws, 128, 0, a, w);
-  rb.kernel(k_recover<T>, gwi, 128, 0, a, w);
+  if (rb.err == cudaSuccess) rb.err = direction_setup<T>(a);
+  DirLaunch dir[kDirLaunches<T>];
+  direction_launches<T>(a, dir);
+  for (const DirLaunch& d : dir) rb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
   rb.kernel(k_ls_begin, gnt, 128, 0, a, w);
   rb.kernel(k_set_cond_one, 1, 1, 0, hl);
   cudaGraph_t ls_body;
@@ -996,6 +964,10 @@ static cudaError_t build_pool_graph(const SolveArgs& a, const Workspace& w, uint
   rb.kernel(k_pool_flags, gnt, 128, 0, a, w, flags);
   if (rb.err != cudaSuccess) return rb.err;
   GraphBuilder lb{ls_body, {}};
+  if constexpr (sizeof(T) == sizeof(double)) {
+    const DirLaunch d = elim_launch(a);
+    lb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+  }
   lb.memset0(w.counters, sizeof(int));
   lb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);
   lb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 1);
@@ -1064,6 +1036,7 @@ extern "C" int sg_pool_create(const sg_problem* prob, int64_t slots, int n_max_i
   p->a.sync_at_end = 1;
   p->a.res_pair = o.precision == SG_PREC_MIXED_PAIR ? 1 : 0;
   p->fp32 = fp32_direction(o.precision);
+  p->a.tree = p->fp32 ? 0 : 1;
   p->w = carve(base + L.ws, slots, n_max_intervals, p->fp32 ? sizeof(float) : sizeof(double));
   p->d_list = reinterpret_cast<int64_t*>(base + L.list);
   p->d_flags = reinterpret_cast<uint8_t*>(base + L.flags);
@@ -1090,10 +1063,6 @@ extern "C" int sg_pool_create(const sg_problem* prob, int64_t slots, int n_max_i
     return bail(e, "sg_pool_create: clearing the node states");
   if ((e = cudaMemsetAsync(base + L.x0, 0, L.ws - L.x0, st)) != cudaSuccess)
     return bail(e, "sg_pool_create: clearing the inputs");
-  if (!p->fp32) {
-    if ((e = ensure_dynamic_smem(k_condense_smem, static_cast<int>(sizeof(double) * kCondWarps * 36 * kCols))) != cudaSuccess)
-      return bail(e, "sg_pool_create: condensation shared memory");
-  }
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(e, "sg_pool_create");
   *out = new sg_pool{p};
   return SG_OK;

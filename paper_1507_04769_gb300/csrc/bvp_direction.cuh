@@ -1,0 +1,814 @@
+// The FP64 Newton direction of the launch-per-phase and graph forms: stage
+// condensation, elimination over the intervals and stage recovery.  All three
+// are bound by the FP64 pipe (a warp's FP64 instruction holds it for 20
+// cycles, whatever its active lanes), so the formulation is the one with the
+// fewest FP64 operations, and rows are packed onto all 32 lanes.
+//
+// Condensation.  With the 2 x 2 inverse B of the interior block of the
+// Lobatto IIIA matrix, B [[a22, a23], [a32, a33]] = I, the two interior stage
+// rows of an interval become
+//   (hJ2 - B11 I) dY2 - B12 dY3 = g1,    -B21 dY2 + (hJ3 - B22 I) dY3 = g2,
+//   g_i = -s_i dy_i - alpha_i hJ1 dy_i - gamma_i hJ4 dy_{i+1} + rho_i
+// (points 1..4 of the interval; s, alpha, gamma: scalars; rho: combinations
+// of the residual rows): the blocks off the diagonal are multiples of the
+// identity, so one 12 x 12 system is left of the 24 x 24 one,
+//   C dY3 = G = (hJ2 - B11 I) g2 + B21 g1,  C = (hJ2 - B11 I)(hJ3 - B22 I) - B12 B21 I,
+//   dY2 = ((hJ3 - B22 I) dY3 - g2) / B21,
+// and the last stage row, in which hJ2 dY2 and hJ3 dY3 are replaced by the
+// same combinations, needs only L G with L = E C^-1, E = c (hJ3 - B22 I) + d I.
+// That is 12,200 multiply-adds per interval (12 x 12 products and one 12 x 12
+// inversion with partial pivoting) instead of the 23,000 of the elimination
+// of the 24 interior columns, and what the recovery needs is C^-1 (144
+// numbers) instead of 24 pivot rows (1,248).  The FP32 forms keep the
+// elimination: a direction rounded otherwise moves their residuals near the
+// tolerance by about a thousandth, and with them the iteration counts of one
+// node in 5,000.
+//
+// Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
+// iterations): condensation 74.8 -> 31.5 ms, elimination and back substitution
+// over the intervals 23.9 -> 9.6 ms, recovery 4.3 -> 2.5 ms; the solve (a graph
+// per mesh size) 112.0 -> 48.7 ms; one node at 128 intervals 1.80 -> 1.01 ms.
+//
+// Elimination over the intervals.  An interval's condensed row
+// S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
+// (dx_i, dlambda_{i+1}): the scattering form of the two-point relation, whose
+// composition (Redheffer's star product) does not grow along the mesh as
+// products of transition matrices do.  Composing [a, m] and [m, b] solves one
+// 6 x 6 system I - B_1 C_2 for (dx_m, dlambda_m) in terms of (dx_a,
+// dlambda_b); a binary tree of compositions over the N intervals (depth
+// log2 N) leaves the relation over [0, T], the boundary rows close it, and
+// the tree is walked down for the mesh-point corrections.
+//
+// A node with a pivot too small for the arithmetic, and a node whose full step
+// is rejected by the line search, take the direction of the elimination with
+// full partial pivoting instead (k_elim_fp64, the FP32 forms' algorithm in
+// FP64).  The first has no scattering form; the second is far from its root,
+// where the path of damped Newton depends on the last bits of the direction
+// and whether it arrives is found out by following it.
+#pragma once
+
+#include "bvp_kernels.cuh"
+#include "bvp_persistent.cuh"
+
+namespace sg {
+
+// Scalars of the combined stage rows, from a = A of Lobatto IIIA (closed
+// forms in sqrt 5).
+namespace lob {
+constexpr double s5 = SG_S5;
+constexpr double B11 = (25.0 + s5) / 7.0, B21 = -(25.0 + 13.0 * s5) / 7.0, B22 = (25.0 - s5) / 7.0;
+constexpr double P12 = -220.0 / 49.0;                                              // B12 B21
+constexpr double S1 = 2.0 * s5;                                                    // s_1; s_2 = -s_1
+constexpr double A1 = (17.0 * s5 - 5.0) / 70.0, A2 = -(17.0 * s5 + 5.0) / 70.0;    // alpha
+constexpr double G1 = (3.0 * s5 - 5.0) / 70.0, G2 = -(3.0 * s5 + 5.0) / 70.0;      // gamma
+constexpr double B12 = (13.0 * s5 - 25.0) / 7.0;
+constexpr double CE = 5.0 * s5 / (25.0 + 13.0 * s5);                               // E = CE (hJ3 - B22 I) + C2 I
+constexpr double C2 = 5.0 * s5 / 7.0;
+constexpr double W1 = 5.0 / 12.0, W2 = 5.0 / 12.0 - CE;                            // factors of g1, g2 in the last row
+constexpr double KD = -1.0 + W1 * S1 - W2 * S1;                                    // dy_i, hJ1 dy_i and hJ4 dy_{i+1}
+constexpr double K0 = -1.0 / 12.0 + W1 * A1 + W2 * A2;
+constexpr double K3 = -1.0 / 12.0 + W1 * G1 + W2 * G2;
+}  // namespace lob
+
+constexpr int kOp = 13 * 12;   // a scattering relation: columns (dx_a 6 | dlambda_b 6 | 1), rows (dx_b 6 | dlambda_a 6)
+constexpr int kCi = 144;       // C^-1 of an interval, row-major
+
+// n x Nmax x kCi inverses and n x Nmax x kOp relations share the region that
+// holds the segments' pivot rows in the FP32 forms.
+__host__ __device__ __forceinline__ double* dir_ci(const Workspace& w) { return static_cast<double*>(w.Seg); }
+__host__ __device__ __forceinline__ double* dir_op(const SolveArgs& a, const Workspace& w) {
+  return static_cast<double*>(w.Seg) + a.n * a.Nmax * int64_t(kCi);
+}
+static_assert(kCi + kOp <= kSegBlk, "the direction's arrays fit the region");
+
+// 1/p for the pivots of the direction: Newton's iteration (one cubic step)
+// from the approximate reciprocal instruction, which is good to about 20
+// bits.  `good` is false for a pivot too small for the arithmetic (the rows
+// are of order one) or not finite; the result is then 0.
+__device__ __forceinline__ double dir_recip(double p, bool& good) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+  const double e = fma(-p, r, 1.0);
+  r = fma(r, fma(e, e, e), r);
+  const unsigned hi = static_cast<unsigned>(__double_as_longlong(p) >> 32) & 0x7FFFFFFFu;
+  good = hi >= 0x3E300000u && hi < 0x7E300000u;   // 2^-28 .. 2^996
+  return good ? r : 0.0;
+}
+
+__device__ __forceinline__ void mark_elim(const Workspace& w, int64_t node) {
+  if (!(atomicOr(&w.ns[node].singular, kElimNode) & kElimNode)) atomicAdd(&w.counters[kElimCount], 1);
+}
+
+// n contiguous entries (16-byte vectors) from or to shared or global memory
+template <int n>
+__device__ __forceinline__ void ld_vec(const double* src, double (&r)[n]) {
+  static_assert(n % 2 == 0, "whole vectors");
+#pragma unroll
+  for (int q = 0; q < n / 2; ++q) {
+    const double2 v = reinterpret_cast<const double2*>(src)[q];
+    r[2 * q] = v.x; r[2 * q + 1] = v.y;
+  }
+}
+// vectors q0 .. of n entries
+template <int n>
+__device__ __forceinline__ void st_vec(double* dst, const double (&r)[n], int q0 = 0) {
+  static_assert(n % 2 == 0, "whole vectors");
+#pragma unroll
+  for (int q = 0; q < n / 2; ++q)
+    if (q >= q0) reinterpret_cast<double2*>(dst)[q] = make_double2(r[2 * q], r[2 * q + 1]);
+}
+
+// ---------------------------------------------------------------- condensation
+// Eight intervals per block of 96 threads, a thread per row of an interval's
+// 12-row matrices (every lane of the three warps a row; two intervals per
+// warp would leave a quarter of the FP64 pipe's lanes idle); the other operand
+// of every product is broadcast from shared memory.  Block barriers hide
+// behind the FP64 pipe.
+constexpr int kCondIv = 8;                       // intervals per block
+constexpr int kCondThreads = 12 * kCondIv;
+constexpr int kCondU = 28;                       // a published pivot row
+// J (4 x 144), C^-1 (144), U (2), rho_2 (12), last column of G (12), pivot keys and pivot rows (24 words)
+constexpr int kCondElems = 576 + 144 + 2 * kCondU + 24 + 12;
+constexpr int kCondSmem = kCondIv * kCondElems * 8;
+__host__ __device__ __forceinline__ int cond_chunks(int Nmax) { return (Nmax + kCondIv - 1) / kCondIv; }
+
+// Whether this thread's row holds the pivot: the largest |v| among the
+// interval's candidate rows, ties to the lower row (the low four bits of the
+// magnitude key are replaced by a row tag).  A block barrier.
+__device__ __forceinline__ bool row_pivot(double v, bool cand, int row, unsigned* keys) {
+  const unsigned key = cand ? ((mag_key(v) & ~15u) | unsigned(15 - row)) : 0u;
+  keys[row] = key;
+  __syncthreads();
+  unsigned best = 0u;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const uint4 k = reinterpret_cast<const uint4*>(keys)[q];
+    best = max(best, max(max(k.x, k.y), max(k.z, k.w)));
+  }
+  return cand && key == best;
+}
+
+__global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, Workspace w) {
+  extern __shared__ __align__(16) unsigned char cond_smem[];
+  const int chunks = cond_chunks(a.Nmax);
+  const int64_t node = blockIdx.x / chunks;
+  int i = static_cast<int>(blockIdx.x % chunks) * kCondIv;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  if (i >= N) return;
+  const int slot = threadIdx.x / 12, r = threadIdx.x % 12;
+  // intervals past the mesh repeat the last one and store nothing
+  const bool valid = i + slot < N;
+  i = valid ? i + slot : N - 1;
+
+  double* sm = reinterpret_cast<double*>(cond_smem) + slot * kCondElems;
+  double* J_s = sm;                 // hJ of the four points; points 2 and 3 are overwritten by G [12][24]
+  double* G_s = sm + 144;
+  double* Ci_s = sm + 576;
+  double* U_s = Ci_s + 144;         // [2][28]
+  double* rho_s = U_s + 2 * kCondU;
+  double* gr_s = rho_s + 12;        // last column of G
+  unsigned* keys = reinterpret_cast<unsigned*>(gr_s + 12);
+  int* perm_s = reinterpret_cast<int*>(keys + 12);
+
+  const int64_t wid = node * a.Nmax + i;
+  const double h = a.T[node] / N;
+  {
+    const double* J = static_cast<const double*>(w.Jm) + (node * npts(a.Nmax) + 3 * int64_t(i)) * 144;
+#pragma unroll
+    for (int e = 0; e < 576 / 2 / 12; ++e) {
+      double v[2];
+      ld_vec<2>(J + (r + e * 12) * 2, v);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) v[t] *= h;
+      st_vec<2>(J_s + (r + e * 12) * 2, v);
+    }
+  }
+  double rho1, rho2, res3;
+  {
+    const double* res = static_cast<const double*>(w.Res) + wid * kResRows;
+    const double r1 = res[r], r2 = res[12 + r];
+    res3 = res[24 + r];
+    rho1 = lob::B11 * r1 + lob::B12 * r2;
+    rho2 = lob::B21 * r1 + lob::B22 * r2;
+    rho_s[r] = rho2;
+  }
+  __syncthreads();
+
+  bool bad = false;
+  // ---- C and its inverse (Gauss-Jordan in place, partial pivoting, rows
+  // stay where they are)
+  {
+    double c[12];
+    {
+      double e1[12];
+      ld_vec<12>(J_s + 144 + r * 12, e1);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) {
+        if (j == r) e1[j] -= lob::B11;
+        c[j] = -lob::B22 * e1[j];
+        if (j == r) c[j] -= lob::P12;
+      }
+#pragma unroll
+      for (int m = 0; m < 12; ++m) {
+        double u[12];
+        ld_vec<12>(J_s + 288 + m * 12, u);
+#pragma unroll
+        for (int j = 0; j < 12; ++j) c[j] = fma(e1[m], u[j], c[j]);
+      }
+    }
+    bool cand = true;
+    int my = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      double* U = U_s + (k & 1) * kCondU;
+      const bool is_p = row_pivot(c[k], cand, r, keys);
+      if (is_p) {
+        st_vec<12>(U, c);
+        perm_s[k] = r;
+        my = k;
+        cand = false;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) c[j] = 0.0;
+      }
+      __syncthreads();
+      bool good;
+      double u[12];
+      ld_vec<12>(U, u);
+      const double inv = dir_recip(u[k], good);
+      bad = bad || !good;
+      // row r: c -= (c_k / p) u, c_k = -c_k / p; the pivot row: u / p, 1 / p
+      const double l = is_p ? -inv : c[k] * inv;
+#pragma unroll
+      for (int j = 0; j < 12; ++j)
+        if (j != k) c[j] = fma(-l, u[j], c[j]);
+      c[k] = -l;
+    }
+    // register j of the row of step k is entry (k, pivot row of step j) of the inverse
+#pragma unroll
+    for (int j = 0; j < 12; ++j) Ci_s[my * 12 + perm_s[j]] = c[j];
+  }
+  __syncthreads();
+  if (valid) {
+    double* dst = dir_ci(w) + wid * kCi;
+    for (int e = r; e < kCi / 2; e += 12) {
+      double v[2];
+      ld_vec<2>(Ci_s + e * 2, v);
+      st_vec<2>(dst + e * 2, v);
+    }
+  }
+
+  // ---- L = E C^-1
+  double L[12];
+  {
+    double e[12];
+    ld_vec<12>(J_s + 288 + r * 12, e);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) {
+      e[j] *= lob::CE;
+      if (j == r) e[j] += (lob::C2 - lob::CE * lob::B22);
+      L[j] = 0.0;
+    }
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      double u[12];
+      ld_vec<12>(Ci_s + m * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) L[j] = fma(e[m], u[j], L[j]);
+    }
+  }
+
+  // ---- G = (hJ2 - B11 I) g2 + B21 g1
+  {
+    double e1[12], g[24], gr = lob::B21 * rho1;
+    ld_vec<12>(J_s + 144 + r * 12, e1);
+#pragma unroll
+    for (int j = 0; j < 12; ++j)
+      if (j == r) e1[j] -= lob::B11;
+#pragma unroll
+    for (int j = 0; j < 24; ++j) g[j] = 0.0;
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      double u[12];
+      ld_vec<12>(J_s + m * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) g[j] = fma(e1[m], u[j], g[j]);
+      ld_vec<12>(J_s + 432 + m * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) g[12 + j] = fma(e1[m], u[j], g[12 + j]);
+    }
+    {
+      double u[12];
+      ld_vec<12>(rho_s, u);
+#pragma unroll
+      for (int m = 0; m < 12; ++m) gr = fma(e1[m], u[m], gr);
+      ld_vec<12>(J_s + r * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) {
+        g[j] = fma(-lob::A2, g[j], lob::S1 * e1[j]);
+        g[j] = fma(-lob::B21 * lob::A1, u[j], g[j]);
+        if (j == r) g[j] -= lob::B21 * lob::S1;
+      }
+      ld_vec<12>(J_s + 432 + r * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j)
+        g[12 + j] = fma(-lob::G2, g[12 + j], -lob::B21 * lob::G1 * u[j]);
+    }
+    __syncthreads();   // points 2 and 3 have been read by every row
+    st_vec<24>(G_s + r * 24, g);
+    gr_s[r] = gr;
+  }
+  __syncthreads();
+
+  // ---- the condensed row [S | T | r] as [T_x | S_lambda | -S_x | -T_lambda | r]
+  double v[28];
+  {
+    double g[24], gr = 0.0;
+#pragma unroll
+    for (int j = 0; j < 24; ++j) g[j] = 0.0;
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      double u[24];
+      ld_vec<24>(G_s + m * 24, u);
+#pragma unroll
+      for (int j = 0; j < 24; ++j) g[j] = fma(L[m], u[j], g[j]);
+    }
+    double u[12];
+    ld_vec<12>(gr_s, u);
+#pragma unroll
+    for (int m = 0; m < 12; ++m) gr = fma(L[m], u[m], gr);
+    ld_vec<12>(J_s + r * 12, u);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) {
+      double s = fma(lob::K0, u[j], -g[j]);
+      if (j == r) s += lob::KD;
+      if (j < 6) v[12 + j] = -s;
+      else v[j] = s;
+    }
+    ld_vec<12>(J_s + 432 + r * 12, u);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) {
+      double t = fma(lob::K3, u[j], -g[12 + j]);
+      if (j == r) t += 1.0;
+      if (j < 6) v[j] = t;
+      else v[12 + j] = -t;
+    }
+    v[24] = gr + lob::W1 * rho1 + lob::W2 * rho2 - res3;
+    v[25] = v[26] = v[27] = 0.0;
+  }
+
+  // ---- (dx_{i+1}, dlambda_i) from (dx_i, dlambda_{i+1}): Gauss-Jordan with
+  // partial pivoting on the first 12 columns
+  {
+    bool cand = true;
+    int my = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      double* U = U_s + (k & 1) * kCondU;
+      const bool is_p = row_pivot(v[k], cand, r, keys);
+      if (is_p) {
+        st_vec<28>(U, v, k / 2);
+        my = k;
+        cand = false;
+#pragma unroll
+        for (int j = k; j < 25; ++j) v[j] = 0.0;
+      }
+      __syncthreads();
+      bool good;
+      const double inv = dir_recip(U[k], good);
+      bad = bad || !good;
+      const double l = is_p ? -inv : v[k] * inv;
+#pragma unroll
+      for (int q = k / 2; q < (25 + 2 - 1) / 2; ++q) {
+        double u[2];
+        ld_vec<2>(U + q * 2, u);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const int j = q * 2 + t;
+          if (j > k && j < 25) v[j] = fma(-l, u[t], v[j]);
+        }
+      }
+    }
+    // column-major relation through shared memory (J is no longer read)
+#pragma unroll
+    for (int j = 0; j < 13; ++j) J_s[j * 12 + my] = v[12 + j];
+    __syncthreads();
+    if (valid) {
+      double* dst = dir_op(a, w) + wid * kOp;
+      for (int e = r; e < kOp / 2; e += 12) {
+        double x[2];
+        ld_vec<2>(J_s + e * 2, x);
+        st_vec<2>(dst + e * 2, x);
+      }
+    }
+  }
+  if (bad && valid && r == 0) mark_elim(w, node);
+}
+
+// ---------------------------------------------------------------- tree
+// Composition of o1 over [a, m] with o2 over [m, b] by 16 lanes, lane c < 13 a
+// column (dx_a | dlambda_b | 1): km = (dx_m, dlambda_m), nw = the relation over
+// [a, b].  The 6 x 6 matrix I - B_1 C_2 has its columns on lanes 0..5;
+// Gauss-Jordan with partial pivoting, the pivot column passed through `pub`.
+// All 32 lanes of the warp call it.
+__device__ __forceinline__ void compose(const double* o1, const double* o2, double* pub, int c, double (&km)[12],
+                                        double (&nw)[12], bool& bad) {
+  double c2[12], c1[12], q[6], b[6];
+  ld_vec<12>(o2 + c * 12, c2);   // A2 | B2 | f2 above C2 | D2 | e2
+  ld_vec<12>(o1 + c * 12, c1);
+#pragma unroll
+  for (int t = 0; t < 6; ++t) q[t] = 0.0;
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {     // B1 times (C2 | D2 | e2)
+    const double* col = o1 + (6 + m) * 12;
+#pragma unroll
+    for (int t = 0; t < 6; ++t) q[t] = fma(col[t], c2[6 + m], q[t]);
+  }
+  const bool left = c < 6, one = c == 12;
+#pragma unroll
+  for (int t = 0; t < 6; ++t) {
+    b[t] = left ? c1[t] : (one ? c1[t] + q[t] : q[t]);
+    q[t] = -q[t];
+    if (t == c) q[t] += 1.0;
+  }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    double* p_s = pub + (k & 1) * 8;
+    int p = k;
+    unsigned best = mag_key(q[k]);
+#pragma unroll
+    for (int t = k + 1; t < 6; ++t) {
+      const unsigned x = mag_key(q[t]);
+      if (x > best) {
+        best = x;
+        p = t;
+      }
+    }
+    if (c == k) {
+#pragma unroll
+      for (int t = 0; t < 6; ++t) p_s[t] = q[t];
+      *reinterpret_cast<int*>(p_s + 6) = p;
+    }
+    __syncwarp();
+    double l[6];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) l[t] = p_s[t];
+    p = *reinterpret_cast<const int*>(p_s + 6);
+    double piv = l[k];
+#pragma unroll
+    for (int t = k + 1; t < 6; ++t) {
+      if (p == t) {
+        piv = l[t];
+        l[t] = l[k];
+        const double x = q[k], y = b[k];
+        q[k] = q[t];
+        q[t] = x;
+        b[k] = b[t];
+        b[t] = y;
+      }
+    }
+    bool good;
+    const double inv = dir_recip(piv, good);
+    bad = bad || !good;
+    q[k] *= inv;
+    b[k] *= inv;
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      if (t != k) {
+        q[t] = fma(-l[t], q[k], q[t]);
+        b[t] = fma(-l[t], b[k], b[t]);
+      }
+    }
+  }
+  double y[12];
+#pragma unroll
+  for (int t = 0; t < 12; ++t) y[t] = left ? 0.0 : c2[t];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {     // (A2 | C2) dx_m
+    double u[12];
+    ld_vec<12>(o2 + m * 12, u);
+#pragma unroll
+    for (int t = 0; t < 12; ++t) y[t] = fma(u[t], b[m], y[t]);
+  }
+#pragma unroll
+  for (int t = 0; t < 6; ++t) {
+    km[t] = b[t];
+    km[6 + t] = y[6 + t];
+    nw[t] = y[t];
+    nw[6 + t] = (left || one) ? c1[6 + t] : 0.0;
+  }
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {     // D1 dlambda_m
+    const double* col = o1 + (6 + m) * 12 + 6;
+#pragma unroll
+    for (int t = 0; t < 6; ++t) nw[6 + t] = fma(col[t], km[6 + m], nw[6 + t]);
+  }
+}
+
+constexpr int kTreeMaxThreads = 512;
+constexpr int kTreeGroupElems = 4 * kOp + 16;   // two pairs of relations in flight, pivot columns
+constexpr int tree_smem(int threads) { return threads / 16 * kTreeGroupElems * 8; }
+// Threads per block: many nodes fill the chip with small blocks; few nodes
+// take the levels of their trees in fewer rounds.
+inline int tree_threads(int64_t n, int Nmax) {
+  int t = n >= 4 * kNumSMs ? 128 : (n >= kNumSMs ? 256 : kTreeMaxThreads);
+  while (t > 32 && t / 16 >= Nmax) t /= 2;
+  return t;
+}
+
+// Block per node.  Relations are composed in place: the result over [a, b)
+// replaces the left operand, and the interior solution (dx_m, dlambda_m) of
+// the composition takes the right operand's place, to be used on the way
+// down.  The boundary rows x(0), lambda(T) close the tree as one more
+// composition, with the relation (dlambda_N = H dx_N + eta).
+__global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, Workspace w) {
+  extern __shared__ __align__(16) unsigned char tree_smem_raw[];
+  const int64_t node = blockIdx.x;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  const int tid = threadIdx.x, lane16 = tid & 15, g = tid >> 4, ng = blockDim.x >> 4;
+  const int c = lane16 < 13 ? lane16 : 12;
+  double* buf = reinterpret_cast<double*>(tree_smem_raw) + g * kTreeGroupElems;   // [2][o1 | o2]
+  double* pub = buf + 4 * kOp;
+  double* ops = dir_op(a, w) + node * a.Nmax * int64_t(kOp);
+  bool bad = false;
+
+  auto fetch = [&](int i, int st, int b) {   // relations i and i + st to buffer b
+    double* dst = buf + b * 2 * kOp;
+    for (int e = lane16; e < 2 * kOp / 2; e += 16) {
+      const double* src = ops + (e < kOp / 2 ? int64_t(i) * kOp + e * 2 : int64_t(i + st) * kOp + (e - kOp / 2) * 2);
+      cp_async16(dst + e * 2, src);
+    }
+    cp_async_commit();
+  };
+
+  for (int st = 1; st < N; st *= 2) {
+    const int pairs = (N - st + 2 * st - 1) / (2 * st);   // left ends 2 st j with 2 st j + st < N
+    int b = 0;
+    if (g < pairs) fetch(2 * st * g, st, 0);
+    for (int j0 = 0; j0 < pairs; j0 += ng, b ^= 1) {
+      const int j = j0 + g;
+      cp_async_wait_all();
+      __syncwarp();
+      if (j + ng < pairs) fetch(2 * st * (j + ng), st, b ^ 1);
+      if (j0 + (g & ~1) >= pairs) continue;   // the whole warp
+      double km[12], nw[12];
+      bool bd = false;
+      compose(buf + b * 2 * kOp, buf + b * 2 * kOp + kOp, pub, c, km, nw, bd);
+      if (j < pairs) {
+        bad = bad || bd;
+        if (lane16 < 13) {
+          st_vec<12>(ops + int64_t(2 * st * j) * kOp + c * 12, nw);
+          st_vec<12>(ops + int64_t(2 * st * j + st) * kOp + c * 12, km);
+        }
+      }
+      __syncwarp();   // buffer b is fetched again in the next round
+    }
+    __syncthreads();
+  }
+
+  // boundary rows
+  const int64_t pb = node * npts(a.Nmax);
+  double* D = w.D + pb * 12;
+  if (tid < 32) {
+    const double* Y = (w.ns[node].ybuf ? w.Y2 : w.Y) + pb * 12;
+    const double* yN = Y + 3 * int64_t(N) * 12;
+    double* o1 = reinterpret_cast<double*>(tree_smem_raw);
+    double* o2 = o1 + kOp;
+    for (int e = tid; e < kOp; e += 32) {
+      o1[e] = ops[e];
+      const int cc = e / 12, rr = e % 12 - 6;
+      double x = 0.0;
+      if (rr >= 0 && cc < 6) x = terminal_hess(a.P, rr, cc);
+      if (rr >= 0 && cc == 12) x = -(yN[6 + rr] - terminal_grad(a.P, yN, rr));
+      o2[e] = x;
+    }
+    __syncwarp();
+    double km[12], nw[12];
+    compose(o1, o2, o1 + 4 * kOp, c, km, nw, bad);
+    __syncwarp();
+    if (tid < 13) {
+      st_vec<12>(o1 + c * 12, km);
+      st_vec<12>(o2 + c * 12, nw);
+    }
+    __syncwarp();
+    if (tid < 12) {
+      const double* x0 = a.x0 + node * 6;
+      double xi[6];
+#pragma unroll
+      for (int m = 0; m < 6; ++m) xi[m] = -(Y[m] - x0[m]);
+      double yn = o1[144 + tid], y0 = o2[144 + tid];
+#pragma unroll
+      for (int m = 0; m < 6; ++m) {
+        yn = fma(o1[m * 12 + tid], xi[m], yn);
+        y0 = fma(o2[m * 12 + tid], xi[m], y0);
+      }
+#pragma unroll
+      for (int m = 0; m < 6; ++m)
+        if (m == tid) y0 = xi[m];
+      D[3 * int64_t(N) * 12 + tid] = yn;
+      D[tid] = y0;
+    }
+  }
+  if (__syncthreads_or(bad)) {
+    if (tid == 0) mark_elim(w, node);
+    return;   // k_elim_fp64 solves it
+  }
+
+  // down the tree: the corrections at the middle of [i, e) from those at its ends
+  int top = 1;
+  while (2 * top < N) top *= 2;
+  if (N < 2) return;
+  for (int st = top; st >= 1; st /= 2) {
+    for (int j = g; 2 * st * j + st < N; j += ng) {
+      const int i = 2 * st * j, m = i + st, e = i + 2 * st < N ? i + 2 * st : N;
+      const double* K = ops + int64_t(m) * kOp;
+      const int r = lane16 < 12 ? lane16 : 11;
+      double k[13];
+#pragma unroll
+      for (int cc = 0; cc < 13; ++cc) k[cc] = K[cc * 12 + r];
+      const double* ya = D + 3 * int64_t(i) * 12;
+      const double* yb = D + 3 * int64_t(e) * 12;
+      double y = k[12];
+#pragma unroll
+      for (int cc = 0; cc < 12; ++cc) y = fma(k[cc], cc < 6 ? ya[cc] : yb[cc], y);
+      if (lane16 < 12) D[3 * int64_t(m) * 12 + r] = y;
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------- marked nodes
+// Block per marked node: condensation by elimination of the 24 interior
+// columns, segmented staircase, back substitution and recovery, each phase
+// over the block's warps.  A small grid, with nothing to do unless a node was
+// marked.  (The relations and inverses in the segments' region are no longer
+// read when it runs.)
+constexpr int kElimBlocks = 2 * kNumSMs, kElimWarps = 4;
+constexpr int kElimWarpSmem = 36 * kCols * 8;   // the condensation's system; the segments' tables are smaller
+static_assert(seg_smem_elems<double>() * 8 <= kElimWarpSmem && 2 * 12 * kSegLd * 8 <= kElimWarpSmem, "tables fit");
+__global__ void __launch_bounds__(32 * kElimWarps) k_elim_fp64(SolveArgs a, Workspace w) {
+  if (w.counters[kElimCount] == 0) return;
+  extern __shared__ __align__(16) unsigned char elim_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* sm = reinterpret_cast<double*>(elim_smem + warp * kElimWarpSmem);
+  for (int64_t node = blockIdx.x; node < a.n; node += gridDim.x) {
+    const bool marked = w.ns[node].active && (w.ns[node].singular & kElimNode);
+    __syncthreads();   // every warp has read the mark before one of them changes the state
+    if (!marked) continue;
+    const int N = a.N[node], nseg = seg_count(N);
+    for (int i = warp; i < N; i += kElimWarps) condense_interval_smem(a, w, node, i, N, lane, sm);
+    __syncthreads();
+    for (int s = warp; s < nseg; s += kElimWarps) {
+      abd_segment<double>(a, w, node, s, N, lane, sm);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (warp == 0) abd_reduced<double>(a, w, node, N, lane);
+    __syncthreads();
+    for (int s = warp; s < nseg; s += kElimWarps) {
+      abd_segment_back<double>(a, w, node, s, N, lane, reinterpret_cast<double(*)[12 * kSegLd]>(sm));
+      __syncwarp();
+    }
+    __syncthreads();
+    for (int i = warp; i < N; i += kElimWarps) recover_interval<double>(a, w, node, i, lane);
+    if (threadIdx.x == 0) {
+      NodeState& s = w.ns[node];
+      if (s.singular & 1) {
+        s.status = SG_SINGULAR;
+        s.active = 0;
+        s.searching = 0;
+      }
+      s.singular = kElimDone;
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------- recovery
+// Interior-stage corrections from the mesh-point corrections: two intervals
+// per warp, 16 lanes each, a lane per row; the Jacobians and C^-1 are staged
+// in shared memory by asynchronous copies, the vectors pass through it.
+constexpr int kRecWarps = 4;
+constexpr int kRecElems = 576 + kCi + 5 * 12;   // per interval: J, C^-1, five vectors
+constexpr int kRecSmem = 2 * kRecWarps * kRecElems * 8;
+
+__device__ __forceinline__ double dot12(const double* row, const double* vec) {
+  double x[12], y[12];
+  ld_vec<12>(row, x);
+  ld_vec<12>(vec, y);
+  double s = x[0] * y[0], t = x[1] * y[1];
+#pragma unroll
+  for (int m = 2; m < 12; m += 2) {
+    s = fma(x[m], y[m], s);
+    t = fma(x[m + 1], y[m + 1], t);
+  }
+  return s + t;
+}
+
+__global__ void __launch_bounds__(32 * kRecWarps) k_recover_fp64(SolveArgs a, Workspace w) {
+  extern __shared__ __align__(16) unsigned char rec_smem[];
+  const int chunks = (a.Nmax + 1) / 2;
+  const int64_t c = blockIdx.x * int64_t(kRecWarps) + (threadIdx.x >> 5);
+  const int64_t node = c / chunks;
+  if (node >= a.n) return;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  int i = static_cast<int>(c % chunks) * 2;
+  if (i >= N) return;
+  const int lane16 = threadIdx.x & 15;
+  i += (threadIdx.x >> 4) & 1;
+  const bool valid = i < N;
+  if (!valid) i = N - 1;
+  const bool on = lane16 < 12;
+  const int r = on ? lane16 : 11;
+  double* sm = reinterpret_cast<double*>(rec_smem) + (threadIdx.x >> 4) * kRecElems;
+  double* Ci_s = sm + 576;
+  double* v0 = Ci_s + kCi;          // dy_i, dy_{i+1}, then g2, G, dY3
+  const int64_t wid = node * a.Nmax + i;
+  const double* J = static_cast<const double*>(w.Jm) + (node * npts(a.Nmax) + 3 * int64_t(i)) * 144;
+  const double* Ci = dir_ci(w) + wid * kCi;
+  for (int e = lane16; e < (576 + kCi) / 2; e += 16)
+    cp_async16(sm + e * 2, e < 576 / 2 ? J + e * 2 : Ci + (e - 576 / 2) * 2);
+  cp_async_commit();
+  double* D = w.D + (node * npts(a.Nmax) + 3 * int64_t(i)) * 12;
+  const double d0 = D[r], d3 = D[36 + r];
+  const double* res = static_cast<const double*>(w.Res) + wid * kResRows;
+  const double r1 = res[r], r2 = res[12 + r];
+  const double h = a.T[node] / N;
+  if (on) {
+    v0[r] = d0;
+    v0[12 + r] = d3;
+  }
+  cp_async_wait_all();
+  __syncwarp();
+  const double u0 = h * dot12(sm + r * 12, v0), u3 = h * dot12(sm + 432 + r * 12, v0 + 12);
+  const double g1 = lob::B11 * r1 + lob::B12 * r2 - lob::S1 * d0 - lob::A1 * u0 - lob::G1 * u3;
+  const double g2 = lob::B21 * r1 + lob::B22 * r2 + lob::S1 * d0 - lob::A2 * u0 - lob::G2 * u3;
+  if (on) v0[24 + r] = g2;
+  __syncwarp();
+  const double G = h * dot12(sm + 144 + r * 12, v0 + 24) - lob::B11 * g2 + lob::B21 * g1;
+  if (on) v0[36 + r] = G;
+  __syncwarp();
+  const double x = dot12(Ci_s + r * 12, v0 + 36);   // dY3
+  if (on) v0[48 + r] = x;
+  __syncwarp();
+  const double y = (h * dot12(sm + 288 + r * 12, v0 + 48) - lob::B22 * x - g2) * (1.0 / lob::B21);
+  if (valid && on) {
+    D[12 + r] = y;
+    D[24 + r] = x;
+  }
+}
+
+// The launches of a Newton direction (after the Jacobians): kernel, grid,
+// block and shared memory of each, in order, for the host loop and the graphs.
+struct DirLaunch {
+  const char* name;
+  void (*fn)(SolveArgs, Workspace);
+  int64_t grid;
+  int block, smem;
+};
+template <typename T>
+constexpr int kDirLaunches = sizeof(T) == sizeof(float) ? 5 : 3;
+
+template <typename T>
+inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches<T>]) {
+  const int64_t nint = a.n * a.Nmax;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    const int64_t nseg = a.n * seg_count(a.Nmax);
+    const int cw = condense_reg_warps(a.cond_warps);
+    out[0] = {"k_condense_reg_fp32", condense_reg_kernel(cw), ceil_div(nint, cw), 32 * cw, 0};
+    out[1] = {"k_abd_seg_fp32", k_abd_seg, ceil_div(nseg, seg_warps<float>()), 32 * seg_warps<float>(), 0};
+    out[2] = {"k_abd_red_fp32", k_abd_red, ceil_div(a.n, 4), 128, 0};
+    out[3] = {"k_abd_segback_fp32", k_abd_segback, ceil_div(nseg, 4), 128, 0};
+    out[4] = {"k_recover_fp32", k_recover_fp32, ceil_div(nint, 4), 128, 0};
+  } else {
+    const int tt = tree_threads(a.n, a.Nmax);
+    out[0] = {"k_condense_fp64", k_condense_fp64, a.n * cond_chunks(a.Nmax), kCondThreads, kCondSmem};
+    out[1] = {"k_tree_fp64", k_tree_fp64, a.n, tt, tree_smem(tt)};
+    out[2] = {"k_recover_fp64", k_recover_fp64, ceil_div(a.n * ((a.Nmax + 1) / 2), kRecWarps), 32 * kRecWarps,
+              kRecSmem};
+  }
+}
+
+// The elimination of marked nodes, launched in front of every trial of the line
+// search of the FP64 form.
+inline DirLaunch elim_launch(const SolveArgs& a) {
+  return {"k_elim_fp64", k_elim_fp64, a.n < kElimBlocks ? a.n : kElimBlocks, 32 * kElimWarps,
+          kElimWarps * kElimWarpSmem};
+}
+
+// Raises the dynamic shared-memory caps of a direction's kernels.
+template <typename T>
+inline cudaError_t direction_setup(const SolveArgs& a) {
+  DirLaunch d[kDirLaunches<T>];
+  direction_launches<T>(a, d);
+  for (auto& x : d) {
+    const cudaError_t e = ensure_dynamic_smem(x.fn, x.smem);
+    if (e != cudaSuccess) return e;
+  }
+  if constexpr (sizeof(T) == sizeof(double)) return ensure_dynamic_smem(k_elim_fp64, elim_launch(a).smem);
+  return cudaSuccess;
+}
+
+}  // namespace sg

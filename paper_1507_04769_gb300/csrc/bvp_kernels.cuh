@@ -21,7 +21,10 @@
 //               in a fixed reduction order
 // T = double gives the FP64 form, T = float the mixed forms (FP32 Jacobian,
 // elimination and direction; FP64 line search and update; the residual in
-// FP64, or in pairs of floats in the mixed-pair form).
+// FP64, or in pairs of floats in the mixed-pair form).  The condensation, the
+// elimination and the recovery described here are the FP32 forms'; the FP64
+// form takes them only for a node whose full step is rejected, and has its own
+// for the others (bvp_direction.cuh).
 #pragma once
 
 #include <cmath>
@@ -53,11 +56,17 @@ struct NodeState {
   double alpha;    // current step length
   int active;      // still iterating
   int searching;   // in the line search
-  int singular;    // a zero pivot was met this iteration
+  int singular;    // bit 0: a zero pivot was met this iteration; kElimNode, kElimDone
   int iters;
   int status;
   int ybuf;        // 1: the current iterate is in Y2 (see Workspace)
 };
+
+// NodeState::singular, FP64 form: the node waits for the direction of the
+// elimination with full partial pivoting (k_elim_fp64) / has it
+constexpr int kElimNode = 2, kElimDone = 4;
+constexpr int kCounters = 5;     // ints of Workspace::counters zeroed per Newton iteration
+constexpr int kElimCount = 4;    // index in Workspace::counters: nodes marked kElimNode
 
 constexpr int kCols = 49;        // 24 interior + 12 (y_i) + 12 (y_{i+1}) + rhs
 constexpr int kRecLd = 52;       // row stride of a stored interior pivot row (16-byte multiple)
@@ -87,7 +96,8 @@ struct Workspace {
   void* Cond;      // n x Nmax x kBlk (T), condensed block rows
   void* Rec;       // n x Nmax x kRec (T), interior pivot rows (FP32: chunk-major, rec_at)
   void* Abd;       // n x Nmax x kBlk (T), staircase pivot rows
-  void* Seg;       // n x Nmax x kSegBlk (T), pivot rows of the segment eliminations
+  void* Seg;       // n x Nmax x kSegBlk (T), pivot rows of the segment eliminations; FP64 form:
+                   // also the direction's arrays (dir_ci, dir_op), which end before it is used
   void* Red;       // n x seg_count(Nmax) x kBlk (T), reduced block rows of the segments
   double* part;    // n x Nmax x 2, partial |F|^2 and |F|_inf
   NodeState* ns;   // n
@@ -111,6 +121,7 @@ struct SolveArgs {
   int sync_at_end;
   const double* Yin;   // initial iterate (n x P x 12), or null for the zero-control guess
   int res_pair;        // FP32-direction form: 1 = residual in pairs of floats, 0 = in FP64
+  int tree;            // FP64 form, launch per phase or graph: direction from bvp_direction.cuh
   int jac_in_trial;    // FP32-direction form with the FP64 residual: the residual kernel also stores the Jacobian
 };
 
@@ -243,7 +254,12 @@ __global__ void __launch_bounds__(128, 5) k_trial(SolveArgs a, Workspace w) {
 #pragma unroll
   for (int c = 0; c < 12; ++c) yf[c] = 0.0f;
   const double* Ycur = s.ybuf ? w.Y2 : w.Y;
-  auto ypoint = [&](int64_t pt, int c) { return __fma_rn(alpha, w.D[pt * 12 + c], Ycur[pt * 12 + c]); };
+  auto ypoint = [&](int64_t pt, int c) {
+    if constexpr (sizeof(T) == sizeof(double)) {   // at the iterate whatever the direction holds
+      if (alpha == 0.0) return Ycur[pt * 12 + c];
+    }
+    return __fma_rn(alpha, w.D[pt * 12 + c], Ycur[pt * 12 + c]);
+  };
   // the stage coefficients h a_kj once per block (the last 12 threads)
   if (tid >= 128 - 12) {
     const int e = tid - (128 - 12), k = e / 4 + 1, jj = e % 4;
@@ -453,6 +469,16 @@ __global__ void k_ls_reduce(SolveArgs a, Workspace w, int mode) {
       atomicAdd(&w.counters[1], 1);
     }
   } else {
+    if (s.alpha == 0.0) {
+      // the residual rows at the iterate are back: the direction of the
+      // elimination next, and the search goes on at 1/2
+      s.alpha = 0.5;
+      s.singular |= kElimNode;
+      w.ns[node] = s;
+      atomicAdd(&w.counters[0], 1);
+      atomicAdd(&w.counters[kElimCount], 1);
+      return;
+    }
     const bool finite = ss < INFINITY;
     const bool accept = !a.damping || (finite && ss <= (1.0 - 2e-4 * s.alpha) * s.fnorm2) ||
                         s.alpha <= 0x1p-10;
@@ -462,7 +488,10 @@ __global__ void k_ls_reduce(SolveArgs a, Workspace w, int mode) {
       s.searching = 0;
       if (a.jac_in_trial) s.ybuf ^= 1;   // the trial point is the iterate
     } else {
-      s.alpha *= 0.5;
+      // FP64 form: a node far from its root follows the elimination's direction
+      // (its path depends on the last bits of it); alpha = 0 evaluates the
+      // rows at the iterate again, which that direction needs
+      s.alpha = a.tree && !(s.singular & kElimDone) ? 0.0 : 0.5 * s.alpha;
       atomicAdd(&w.counters[0], 1);
     }
   }
@@ -954,10 +983,9 @@ inline void (*condense_reg_kernel(int cond_warps))(SolveArgs, Workspace) {
 }
 inline int condense_reg_warps(int cond_warps) { return cond_warps == 2 || cond_warps == 8 ? cond_warps : 4; }
 
-// Shared-memory FP64 form (used by the FP64 solve): the 36 x 49 system of one
+// Shared-memory FP64 form (persistent form, k_elim_fp64): the 36 x 49 system of one
 // interval in shared memory, one warp per interval, elimination of the first
 // 24 columns with partial pivoting over all 36 rows (warp_eliminate).
-constexpr int kCondWarps = 4;
 __device__ __forceinline__ void condense_interval_smem(const SolveArgs& a, const Workspace& w, int64_t node,
                                                        int i, int N, int lane, double* M) {
   const int64_t wid = node * a.Nmax + i;
@@ -1008,19 +1036,6 @@ __device__ __forceinline__ void condense_interval_smem(const SolveArgs& a, const
     cond[r * kBlkLd + c] = M[(24 + r) * kCols + 24 + c];
   }
   __syncwarp();
-}
-
-__global__ void __launch_bounds__(32 * kCondWarps) k_condense_smem(SolveArgs a, Workspace w) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t wid = blockIdx.x * int64_t(kCondWarps) + warp;
-  if (wid >= a.n * a.Nmax) return;
-  const int64_t node = wid / a.Nmax;
-  const int i = static_cast<int>(wid % a.Nmax);
-  if (!w.ns[node].active) return;
-  const int N = a.N[node];
-  if (i >= N) return;
-  condense_interval_smem(a, w, node, i, N, lane, reinterpret_cast<double*>(smem_raw) + warp * (36 * kCols));
 }
 
 // ---------------------------------------------------------------- staircase
@@ -1269,23 +1284,15 @@ __device__ __forceinline__ void store_row12_from(T* __restrict__ dst, const T (&
   }
 }
 
+// (the warp's tables at P_s: seg_smem_elems<T>() elements)
 template <typename T>
-__global__ void __launch_bounds__(32 * seg_warps<T>()) k_abd_seg(SolveArgs a, Workspace w) {
-  constexpr int W = seg_warps<T>();
+__device__ __forceinline__ void abd_segment(const SolveArgs& a, const Workspace& w, int64_t node, int s, int N,
+                                            int lane, T* P_s) {
   constexpr int V = 16 / int(sizeof(T));   // entries per 16-byte vector
-  __shared__ __align__(16) T sm[W][seg_smem_elems<T>()];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int smax = seg_count(a.Nmax);
-  const int64_t wid = blockIdx.x * int64_t(W) + warp;
-  const int64_t node = wid / smax;
-  const int s = static_cast<int>(wid % smax);
-  if (node >= a.n) return;
-  if (!w.ns[node].active) return;
-  const int N = a.N[node];
-  if (s >= seg_count(N)) return;
   const int i0 = s * kSegLen;
   const int i1 = i0 + kSegLen < N ? i0 + kSegLen : N;
-  T* P_s = sm[warp];                  // [24][kSegP] passive parts [F | Z | rhs] of the panel rows
+  // P_s: [24][kSegP] passive parts [F | Z | rhs] of the panel rows
   T* Y_s = P_s + 24 * kSegP;          // [24][12] y_i parts
   T* L_s = Y_s + 24 * 12;             // [24][12] multipliers l(r, k)
   T* U_s = L_s + 24 * 12;             // [12][12] pivot rows (y_i part), 1/pivot on the diagonal
@@ -1460,37 +1467,25 @@ __global__ void __launch_bounds__(32 * seg_warps<T>()) k_abd_seg(SolveArgs a, Wo
     }
     __syncwarp();   // tables written before the next panel reads them
   }
-  if (__any_sync(0xffffffffu, bad) && lane == 0) w.ns[node].singular = 1;
+  if (__any_sync(0xffffffffu, bad) && lane == 0) w.ns[node].singular |= 1;
 }
 
+// the reduced staircase of one node by one warp
 template <typename T>
-__global__ void __launch_bounds__(128) k_abd_red(SolveArgs a, Workspace w) {
-  const int lane = threadIdx.x & 31;
-  const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
-  if (node >= a.n) return;
-  if (!w.ns[node].active) return;
-  const int N = a.N[node];
+__device__ __forceinline__ void abd_reduced(const SolveArgs& a, const Workspace& w, int64_t node, int N, int lane) {
   const int smax = seg_count(a.Nmax);
   const T* red = static_cast<const T*>(w.Red) + node * smax * int64_t(kBlk);
   T* abd = static_cast<T*>(w.Abd) + node * a.Nmax * int64_t(kBlk);
   const bool ok = abd_staircase<T>(a, w, node, N, red, seg_count(N), 3 * kSegLen, abd, lane);
-  if (!ok && lane == 0) w.ns[node].singular = 1;
+  if (!ok && lane == 0) w.ns[node].singular |= 1;
 }
 
+// the back substitution of one segment by one warp: the pivot rows of panel
+// i - 1 are copied to shared memory (asynchronously) while panel i is
+// substituted
 template <typename T>
-__global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
-  // the pivot rows of panel i - 1 are copied to shared memory (asynchronously)
-  // while panel i is substituted
-  __shared__ __align__(16) T buf_s[4][2][12 * kSegLd];
-  const int lane = threadIdx.x & 31;
-  const int smax = seg_count(a.Nmax);
-  const int64_t wid = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
-  const int64_t node = wid / smax;
-  const int s = static_cast<int>(wid % smax);
-  if (node >= a.n) return;
-  if (!w.ns[node].active) return;
-  const int N = a.N[node];
-  if (s >= seg_count(N)) return;
+__device__ __forceinline__ void abd_segment_back(const SolveArgs& a, const Workspace& w, int64_t node, int s, int N,
+                                                 int lane, T (*buf)[12 * kSegLd]) {
   const int i0 = s * kSegLen;
   const int i1 = i0 + kSegLen < N ? i0 + kSegLen : N;
   if (i1 - i0 < 2) return;
@@ -1502,7 +1497,6 @@ __global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
     dya[c] = T(D[3 * int64_t(i0) * 12 + c]);
     dyn[c] = T(D[3 * int64_t(i1) * 12 + c]);
   }
-  T (*buf)[12 * kSegLd] = buf_s[threadIdx.x >> 5];
   auto fetch = [&](int i, int b) {   // panel i's 12 pivot rows to buf[b]
     const char* src = reinterpret_cast<const char*>(seg + int64_t(i) * 12 * kSegLd);
     for (int e = lane; e < 12 * kSegLd * int(sizeof(T)) / 16; e += 32)
@@ -1544,6 +1538,41 @@ __global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
       D[3 * int64_t(i) * 12 + lane] = double(mine);
     }
   }
+}
+
+__global__ void __launch_bounds__(32 * seg_warps<float>()) k_abd_seg(SolveArgs a, Workspace w) {
+  constexpr int W = seg_warps<float>();
+  __shared__ __align__(16) float sm[W][seg_smem_elems<float>()];
+  const int warp = threadIdx.x >> 5;
+  const int smax = seg_count(a.Nmax);
+  const int64_t wid = blockIdx.x * int64_t(W) + warp;
+  const int64_t node = wid / smax;
+  const int s = static_cast<int>(wid % smax);
+  if (node >= a.n) return;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  if (s >= seg_count(N)) return;
+  abd_segment<float>(a, w, node, s, N, threadIdx.x & 31, sm[warp]);
+}
+
+__global__ void __launch_bounds__(128) k_abd_red(SolveArgs a, Workspace w) {
+  const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
+  if (node >= a.n) return;
+  if (!w.ns[node].active) return;
+  abd_reduced<float>(a, w, node, a.N[node], threadIdx.x & 31);
+}
+
+__global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
+  __shared__ __align__(16) float buf_s[4][2][12 * kSegLd];
+  const int smax = seg_count(a.Nmax);
+  const int64_t wid = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
+  const int64_t node = wid / smax;
+  const int s = static_cast<int>(wid % smax);
+  if (node >= a.n) return;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  if (s >= seg_count(N)) return;
+  abd_segment_back<float>(a, w, node, s, N, threadIdx.x & 31, buf_s[threadIdx.x >> 5]);
 }
 
 // Interior-stage corrections from the stored condensation pivot rows: lane
@@ -1600,8 +1629,7 @@ __device__ __forceinline__ void recover_interval(const SolveArgs& a, const Works
   if (lane < 24) D[12 + lane] = double(x);   // points 3i+1 and 3i+2 are contiguous
 }
 
-template <typename T>
-__global__ void k_recover(SolveArgs a, Workspace w) {
+__global__ void k_recover_fp32(SolveArgs a, Workspace w) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t wid = blockIdx.x * int64_t(4) + warp;
   if (wid >= a.n * a.Nmax) return;
@@ -1609,7 +1637,7 @@ __global__ void k_recover(SolveArgs a, Workspace w) {
   const int i = static_cast<int>(wid % a.Nmax);
   if (!w.ns[node].active) return;
   if (i >= a.N[node]) return;
-  recover_interval<T>(a, w, node, i, lane);
+  recover_interval<float>(a, w, node, i, lane);
 }
 
 // ---------------------------------------------------------------- update
@@ -1618,10 +1646,11 @@ __global__ void k_ls_begin(SolveArgs a, Workspace w) {
   if (node >= a.n) return;
   NodeState s = w.ns[node];
   if (!s.active) return;
-  if (s.singular) {
+  if (s.singular & 1) {
     s.status = SG_SINGULAR;
     s.active = 0;
   } else {
+    s.singular &= kElimNode;
     s.searching = 1;
     s.alpha = 1.0;
   }

@@ -137,6 +137,28 @@ __device__ __forceinline__ void residual_node(const SolveArgs& a, const Workspac
   residual_node_t<T, false>(a, w, node, N, alpha, lane, ss_out, mx_out);
 }
 
+// Newton direction of one node by one warp, from its Jacobians and residual
+// rows: condensation of every interval with partial pivoting over the
+// interior rows, staircase elimination, stage recovery.  False if a pivot of
+// the staircase was zero (the condensation reports its own in the node state).
+template <typename T>
+__device__ __forceinline__ bool direction_node(const SolveArgs& a, const Workspace& w, int64_t node, int N, int lane,
+                                               unsigned char* scratch) {
+  for (int i = 0; i < N; ++i) {
+    if constexpr (sizeof(T) == sizeof(float)) {
+      condense_interval_reg(a, w, node, i, N, lane, reinterpret_cast<float*>(scratch));
+    } else {
+      condense_interval_smem(a, w, node, i, N, lane, reinterpret_cast<double*>(scratch));
+    }
+  }
+  __syncwarp();
+  const bool ok = abd_node_reg<T>(a, w, node, N, lane);
+  __syncwarp();
+  for (int i = 0; i < N; ++i) recover_interval<T>(a, w, node, i, lane);
+  __syncwarp();
+  return ok;
+}
+
 template <typename T>
 __device__ void solve_node_persistent(const SolveArgs& a, const Workspace& w, int64_t node, int lane,
                                       unsigned char* scratch) {
@@ -162,20 +184,7 @@ __device__ void solve_node_persistent(const SolveArgs& a, const Workspace& w, in
         char_jacobian<T>(a.P, y, static_cast<T*>(w.Jm) + (pb + p) * 144, nullptr);
       }
       __syncwarp();
-      // condensation of every interval
-      bool ok = true;
-      for (int i = 0; i < N; ++i) {
-        if constexpr (sizeof(T) == sizeof(float)) {
-          condense_interval_reg(a, w, node, i, N, lane, reinterpret_cast<float*>(scratch));
-        } else {
-          condense_interval_smem(a, w, node, i, N, lane, reinterpret_cast<double*>(scratch));
-        }
-      }
-      __syncwarp();
-      ok = abd_node_reg<T>(a, w, node, N, lane) && ok;
-      __syncwarp();
-      for (int i = 0; i < N; ++i) recover_interval<T>(a, w, node, i, lane);
-      __syncwarp();
+      const bool ok = direction_node<T>(a, w, node, N, lane, scratch);
       // the condensation reports zero pivots through the node state
       const bool sing = !__all_sync(0xffffffffu, ok) || w.ns[node].singular;
       if (sing) {
