@@ -60,6 +60,84 @@ __device__ inline void basis_row(double u, int level, const double* __restrict__
 }
 
 
+// 1/x by Newton's iteration (one cubic step) from the approximate reciprocal
+// instruction, which is good to about 20 bits: three FP64 operations and
+// within one unit in the last place, where the correctly rounded reciprocal
+// takes about seven.
+__device__ __forceinline__ double recip_newton(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// The FP64 basis for a level fixed at compile time (every loop unrolls, the
+// reciprocals stay in registers).  The denominators of the nested sets follow
+// from one another: the points of X^l are the even points of X^{l+1}, so with P
+// the sum of |w_m| / (u - x_m) over X^l and N the sum over the new points, the
+// denominator of X^{l+1} is P - N and its own P is P + N.  Written out(id, v).
+template <int L, typename Out>
+__device__ __forceinline__ void basis_row_t(double u, const double* __restrict__ xf, Out out) {
+  constexpr int fine_n = 1 << L;
+  out(0, 1.0);
+  double rinv[fine_n + 1];
+  int hit = -1;
+#pragma unroll
+  for (int p = 0; p <= fine_n; ++p) {
+    const double diff = u - xf[p];
+    const bool zero = (static_cast<unsigned long long>(__double_as_longlong(diff)) << 1) == 0ull;
+    if (zero) hit = p;
+    const double r = recip_newton(diff);
+    rinv[p] = zero ? 0.0 : r;
+  }
+  double P = 0.0;
+  int id = 1;
+#pragma unroll
+  for (int l = 2; l <= L + 1; ++l) {
+    const int n = 1 << (l - 1);
+    const int sf = fine_n / n;
+    const bool exact = hit >= 0 && (hit % sf) == 0;
+    double nw, ends = 0.0;
+    if (l == 2) {
+      ends = 0.5 * (rinv[0] + rinv[fine_n]);
+      nw = rinv[sf];
+      P = ends;
+    } else {
+      nw = rinv[sf];
+#pragma unroll
+      for (int m = 3; m < n; m += 2) nw += rinv[m * sf];
+    }
+    const double inv = recip_newton(P - nw);
+    P += nw;
+    const int cnt = l == 2 ? 2 : (n >> 1);
+    // increment points: l = 2 the two ends (weight +1/2), l >= 3 the odd points (weight -1)
+    const double wi = l == 2 ? 0.5 * inv : -inv;
+#pragma unroll
+    for (int j = 0; j < cnt; ++j) {
+      const int m = l == 2 ? j * n : 2 * j + 1;
+      const double v = wi * rinv[m * sf];
+      out(id + j, exact ? ((m * sf == hit) ? 1.0 : 0.0) : v);
+    }
+    id += cnt;
+  }
+}
+
+// All 1-D basis values at u to tab[id * stride]: levels 1..5 unrolled, the
+// others by the general form.
+__device__ __forceinline__ void basis_row_fast(double u, int level, const double* __restrict__ xf, double* tab,
+                                               int stride) {
+  auto out = [&](int id, double v) { tab[id * stride] = v; };
+  switch (level) {
+    case 1: return basis_row_t<1>(u, xf, out);
+    case 2: return basis_row_t<2>(u, xf, out);
+    case 3: return basis_row_t<3>(u, xf, out);
+    case 4: return basis_row_t<4>(u, xf, out);
+    case 5: return basis_row_t<5>(u, xf, out);
+    default: return basis_row(u, level, xf, tab, stride);
+  }
+}
+
+
 struct df {
   float hi, lo;
 };

@@ -117,138 +117,314 @@ __global__ void __launch_bounds__(32 * kSurpWarps)
   }
 }
 
-// Gather rows of W into the evaluation order.
-__global__ void k_gather_rows(int64_t M, int k, const int32_t* __restrict__ order,
-                              const double* __restrict__ W, double* __restrict__ Ws) {
+// Gathers rows of W into the evaluation order and into the nested order.
+__global__ void k_gather_rows(int64_t M, int k, const int32_t* __restrict__ order, const int32_t* __restrict__ nested,
+                              const double* __restrict__ W, double* __restrict__ Ws, double* __restrict__ Wt) {
   const int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (e >= M * k) return;
   const int64_t r = e / k, c = e % k;
   Ws[e] = W[int64_t(order[r]) * k + c];
+  Wt[e] = W[int64_t(nested[r]) * k + c];
 }
 
-// FP64 evaluation: thread per query.  The d x nf basis table of each query
-// lives in shared memory (query index fastest, so a warp's accesses are
-// consecutive).  The node loop is uniform across the block.  Each node
-// carries the table offsets of its active dimensions only (level >= 2; the
-// level-1 factor is the constant 1), so its basis product costs
-// (active - 1) multiplications, taken by a warp-uniform branch, and the
-// contraction costs K fused multiply-adds.
+// ---------------------------------------------------------------- FP64 evaluation
+// Both kernels are bound by the FP64 pipe, which a warp's instruction holds for
+// 20 cycles whatever its active lanes.
+//
+// Nested form (many queries).  In lexicographic order of the function ids the
+// nodes are the preorder of a tree: a node's parent is the node with its last
+// active dimension set to level 1 (in the grid, which is downward closed), and
+//   u = value(root),  value(n) = W_n + sum over the children c of phi_c value(c)
+// with phi_c the one 1-D basis value of c's last active dimension.  That is K
+// multiply-adds per node and no products (the sum over nodes of products of
+// their active factors takes A - 1 products more per node: 7.7 FP64 operations
+// per node against 4.4 on the level-4 6-D grid).  A lane per query, 32 queries
+// per block; the block's warps take equal ranges of the preorder (a range
+// starts by entering its first node's ancestors with value 0), so that every
+// warp's control flow is uniform, and their sums are added in order.
+// Measured (K = 3, d = 6) against the per-node form at 128 threads, one query
+// each: 1e6 queries 20.2 -> 8.7 ms on the level-4 grid (the FP64 pipe's time
+// for the multiply-adds and the tables) and 114 -> 26.5 ms on the level-5 grid.
+constexpr int kNestQ = 32;
+
+// prog[m] of a node: table offset of its last active dimension (12 bits), its
+// depth (active dimensions, 4 bits), and for a node without children the
+// number of entries from it on that are such nodes at its depth (16 bits):
+// three quarters of the nodes are taken in runs, by a short loop.
+__host__ __device__ constexpr uint32_t nested_entry(uint32_t off, uint32_t depth, uint32_t run) {
+  return off | depth << 12 | run << 16;
+}
+
 template <int K>
-__device__ __forceinline__ void eval_accumulate(const EvalArgs& e, const double* __restrict__ tab,
-                                                int tid, double* acc) {
-  for (int64_t m = 0; m < e.M; ++m) {
-    const int na = e.nact[m];
-    const uint16_t* o = e.ops + m * kMaxDim;
-    double phi;
-    switch (na) {
-      case 0: phi = 1.0; break;
-      case 1: phi = tab[o[0] * kEvalThreads + tid]; break;
-      case 2: phi = tab[o[0] * kEvalThreads + tid] * tab[o[1] * kEvalThreads + tid]; break;
-      case 3:
-        phi = tab[o[0] * kEvalThreads + tid] * tab[o[1] * kEvalThreads + tid] * tab[o[2] * kEvalThreads + tid];
-        break;
-      default: {
-        phi = tab[o[0] * kEvalThreads + tid] * tab[o[1] * kEvalThreads + tid] *
-              tab[o[2] * kEvalThreads + tid] * tab[o[3] * kEvalThreads + tid];
-        for (int j = 4; j < na; ++j) phi *= tab[o[j] * kEvalThreads + tid];
-      }
-    }
-    const double* w = e.W + m * K;
+struct Nested {
+  const uint32_t* prog;
+  const double* W;         // K columns of the surpluses in nested order, row stride k
+  const double* tab;       // this query's table column
+  int k, kc, m1;           // kc: columns that exist (<= K); m1: end of the range
+  // entries base .. base + 31 of the range, staged in shared memory (an
+  // entry steers the walk, so a load from L2 would stand in its path); lp, lw:
+  // the 32 after them, one per lane, on their way
+  uint32_t* sp;            // [32]
+  double* sw;              // [32][K]
+  int lane, base, pos;
+  uint32_t lp;
+  double lw[K];
+  __device__ __forceinline__ void load(int m0) {
+    const int i = m0 + lane;
+    lp = i < m1 ? prog[i] : 0u;   // depth 0 ends every loop
 #pragma unroll
-    for (int c = 0; c < K; ++c) acc[c] = fma(phi, w[c], acc[c]);
+    for (int c = 0; c < K; ++c) lw[c] = i < m1 && c < kc ? W[int64_t(i) * k + c] : 0.0;
+  }
+  __device__ __forceinline__ void refill() {
+    __syncwarp();
+    sp[lane] = lp;
+#pragma unroll
+    for (int c = 0; c < K; ++c) sw[lane * K + c] = lw[c];
+    __syncwarp();
+    base += 32;
+    pos = 0;
+    load(base + 32);
+  }
+};
+constexpr int nested_stage_bytes(int K) { return 32 * (8 * K + 4); }   // per warp
+
+// Adds the children (and theirs) at depth D from the current entry on to acc;
+// the first `resume` depths are ancestors of the range's first node (path:
+// their table offsets), entered with value 0.
+template <int K, int D>
+__device__ __forceinline__ void nested_children(Nested<K>& t, int resume, const uint16_t* path, double (&acc)[K]) {
+  if constexpr (D <= kMaxDim) {
+    while (true) {
+      double v[K];
+      uint32_t off;
+      const bool again = resume >= D;
+      if (again) {
+        off = path[D - 1];
+#pragma unroll
+        for (int c = 0; c < K; ++c) v[c] = 0.0;
+      } else {
+        if (t.pos == 32) t.refill();
+        const uint32_t p = t.sp[t.pos];
+        if (((p >> 12) & 15u) != uint32_t(D)) break;
+        int run = static_cast<int>(p >> 16);
+        if (run != 0) {
+          run = min(run, min(32 - t.pos, t.m1 - t.base - t.pos));
+          const uint32_t* sp = t.sp + t.pos;
+          const double* sw = t.sw + t.pos * K;
+          t.pos += run;
+#pragma unroll 2
+          for (; run > 0; --run, ++sp, sw += K) {
+            const double phi = t.tab[(*sp & 0xFFFu) * kNestQ];
+#pragma unroll
+            for (int c = 0; c < K; ++c) acc[c] = fma(phi, sw[c], acc[c]);
+          }
+          continue;
+        }
+        off = p & 0xFFFu;
+#pragma unroll
+        for (int c = 0; c < K; ++c) v[c] = t.sw[t.pos * K + c];
+        ++t.pos;
+      }
+      const double phi = t.tab[off * kNestQ];
+      nested_children<K, D + 1>(t, again ? resume : 0, path, v);
+      resume = 0;
+#pragma unroll
+      for (int c = 0; c < K; ++c) acc[c] = fma(phi, v[c], acc[c]);
+    }
   }
 }
 
-template <int D, int K>
-__global__ void __launch_bounds__(kEvalThreads) k_eval_fp64(EvalArgs e) {
-  extern __shared__ double tabs_s[];
-  const int tid = threadIdx.x;
-  const int64_t q = blockIdx.x * int64_t(kEvalThreads) + tid;
+template <int K>
+__global__ void __launch_bounds__(512, 1) k_eval_fp64_nested(EvalArgs e, int d, int c0, size_t stage0) {
+  extern __shared__ double tabs_s[];   // [d * nf][kNestQ] (then the warps' sums), the warps' stages
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int64_t q = blockIdx.x * int64_t(kNestQ) + lane;
   const bool live = q < e.Q;
-  const int nf = e.nf;
-  // tab[(dim * nf + id) * kEvalThreads + tid]
-  for (int dim = 0; dim < D; ++dim) {
-    const double u = live ? (e.xq[q * D + dim] - e.lo[dim]) / e.width[dim] : 0.5;
-    basis_row(u, e.level, e.xf, tabs_s + (dim * nf) * kEvalThreads + tid, kEvalThreads);
+  for (int dim = warp; dim < d; dim += nw) {
+    const double u = live ? (e.xq[q * d + dim] - e.lo[dim]) / e.width[dim] : 0.5;
+    basis_row_fast(u, e.level, e.xf, tabs_s + (dim * e.nf) * kNestQ + lane, kNestQ);
   }
   __syncthreads();
+  Nested<K> t;
+  t.prog = e.prog;
+  t.W = e.Wt + c0;
+  t.tab = tabs_s + lane;
+  t.k = e.k;
+  t.kc = e.k - c0 < K ? e.k - c0 : K;
+  const int m0 = static_cast<int>(e.M * warp / nw);
+  t.m1 = static_cast<int>(e.M * (warp + 1) / nw);
+  t.lane = lane;
+  t.sw = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(tabs_s) + stage0 + warp * nested_stage_bytes(K));
+  t.sp = reinterpret_cast<uint32_t*>(t.sw + 32 * K);
   double acc[K];
 #pragma unroll
   for (int c = 0; c < K; ++c) acc[c] = 0.0;
-  eval_accumulate<K>(e, tabs_s, tid, acc);
-  if (live) {
+  if (m0 < t.m1) {
+    t.base = m0 - 32;
+    t.load(m0);
+    t.refill();
+    int resume = 0;
+    if (m0 == 0) {   // the root
 #pragma unroll
-    for (int c = 0; c < K; ++c) e.out[q * K + c] = acc[c];
+      for (int c = 0; c < K; ++c) acc[c] = t.sw[c];
+      t.pos = 1;
+    } else {
+      resume = static_cast<int>((t.sp[0] >> 12) & 15u) - 1;
+    }
+    nested_children<K, 1>(t, resume, e.path + int64_t(m0) * kMaxDim, acc);
+  }
+  __syncthreads();   // the tables are read; their space takes the sums
+  double* sum = tabs_s;
+#pragma unroll
+  for (int c = 0; c < K; ++c) sum[(warp * K + c) * 32 + lane] = acc[c];
+  __syncthreads();
+  if (warp == 0 && live) {
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+      double v = sum[c * 32 + lane];
+      for (int s = 1; s < nw; ++s) v += sum[(s * K + c) * 32 + lane];
+      if (c < t.kc) e.out[q * e.k + c0 + c] = v;
+    }
   }
 }
 
-// Any output count: the same loop with a runtime count (rarely used shapes).
-template <int D>
-__global__ void __launch_bounds__(kEvalThreads) k_eval_fp64_anyk(EvalArgs e) {
-  extern __shared__ double tabs_s[];
-  const int tid = threadIdx.x;
-  const int64_t q = blockIdx.x * int64_t(kEvalThreads) + tid;
-  const bool live = q < e.Q;
-  const int nf = e.nf;
-  for (int dim = 0; dim < D; ++dim) {
-    const double u = live ? (e.xq[q * D + dim] - e.lo[dim]) / e.width[dim] : 0.5;
-    basis_row(u, e.level, e.xf, tabs_s + (dim * nf) * kEvalThreads + tid, kEvalThreads);
+// Per-node form (few queries): the lanes of a block are QB queries x node
+// streams, so that a handful of queries fills the FP64 pipe of its SM and a
+// few hundred all SMs.  A node's basis product is that of its active factors
+// (level 1 is the constant 1); nodes come in groups of equal active count.
+constexpr int kNodesThreads = 256;
+
+template <int K, int A, int QB>
+__device__ __forceinline__ void nodes_group(const EvalArgs& e, int64_t n0, int64_t n1, int stream,
+                                            const double* __restrict__ tab, int c0, int kc, double (&acc)[K]) {
+  constexpr int NS = kNodesThreads / QB;
+  for (int64_t m = n0 + stream; m < n1; m += NS) {
+    double phi = 1.0;
+    if constexpr (A > 0) {
+      const uint4 ov = *reinterpret_cast<const uint4*>(e.ops + m * kMaxDim);
+      const uint32_t o[4] = {ov.x, ov.y, ov.z, ov.w};
+      phi = tab[(o[0] & 0xFFFFu) * QB];
+#pragma unroll
+      for (int a = 1; a < A; ++a) phi *= tab[((a & 1) ? (o[a >> 1] >> 16) : (o[a >> 1] & 0xFFFFu)) * QB];
+    }
+    const double* w = e.W + m * e.k + c0;
+#pragma unroll
+    for (int c = 0; c < K; ++c)
+      if (c < kc) acc[c] = fma(phi, w[c], acc[c]);
+  }
+}
+
+template <int K, int QB>
+__global__ void __launch_bounds__(kNodesThreads) k_eval_fp64_nodes(EvalArgs e, int d, int c0) {
+  extern __shared__ double tabs_s[];   // [d * nf][QB], then the partial sums
+  const int tid = threadIdx.x, ql = tid % QB, stream = tid / QB;
+  const int64_t q0 = blockIdx.x * int64_t(QB);
+  for (int task = tid; task < QB * d; task += kNodesThreads) {
+    const int tq = task % QB, dim = task / QB;
+    const int64_t q = q0 + tq;
+    const double u = q < e.Q ? (e.xq[q * d + dim] - e.lo[dim]) / e.width[dim] : 0.5;
+    basis_row_fast(u, e.level, e.xf, tabs_s + (dim * e.nf) * QB + tq, QB);
   }
   __syncthreads();
-  const int k = e.k;
-  for (int c0 = 0; c0 < k; c0 += 4) {
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t m = 0; m < e.M; ++m) {
-      const int na = e.nact[m];
-      const uint16_t* o = e.ops + m * kMaxDim;
-      double phi = 1.0;
-      for (int j = 0; j < na; ++j) phi *= tabs_s[o[j] * kEvalThreads + tid];
-      const double* w = e.W + m * k;
+  const int kc = e.k - c0 < K ? e.k - c0 : K;
+  double acc[K];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c0 + c < k) acc[c] = fma(phi, w[c0 + c], acc[c]);
+  for (int c = 0; c < K; ++c) acc[c] = 0.0;
+  for (int a = 0; a <= kMaxDim; ++a) {
+    const int64_t n0 = e.grp[a], n1 = e.grp[a + 1];
+    if (n0 >= n1) continue;
+    switch (a) {
+      case 0: nodes_group<K, 0, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 1: nodes_group<K, 1, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 2: nodes_group<K, 2, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 3: nodes_group<K, 3, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 4: nodes_group<K, 4, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 5: nodes_group<K, 5, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 6: nodes_group<K, 6, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      case 7: nodes_group<K, 7, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+      default: nodes_group<K, 8, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
     }
-    if (live)
-      for (int c = 0; c < 4 && c0 + c < k; ++c) e.out[q * k + c0 + c] = acc[c];
+  }
+  // streams of a warp by shuffles, then the warps in order
+#pragma unroll
+  for (int c = 0; c < K; ++c)
+#pragma unroll
+    for (int o = 16; o >= QB; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+  __syncthreads();
+  const int lane = tid & 31, warp = tid >> 5;
+  if (lane < QB) {
+#pragma unroll
+    for (int c = 0; c < K; ++c) tabs_s[(warp * QB + lane) * K + c] = acc[c];
+  }
+  __syncthreads();
+  if (tid < QB && q0 + tid < e.Q) {
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+      double v = tabs_s[tid * K + c];
+      for (int s = 1; s < kNodesThreads / 32; ++s) v += tabs_s[(s * QB + tid) * K + c];
+      if (c < kc) e.out[(q0 + tid) * e.k + c0 + c] = v;
+    }
   }
 }
 
-template <int D>
-static int launch_eval_fp64(const EvalArgs& e, cudaStream_t st) {
-  const size_t smem = sizeof(double) * D * e.nf * kEvalThreads;
-  if (smem > 200 * 1024) return fail(SG_EUNSUPPORTED, "sg_eval_feedback: grid level too high for the FP64 kernel");
-  const unsigned blocks = static_cast<unsigned>(ceil_div(e.Q, kEvalThreads));
-#define SG_EVAL_K(KK)                                                                              \
-  case KK:                                                                                         \
-    SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64<D, KK>, smem));                                  \
-    SG_TIMED("k_eval_fp64", st, (k_eval_fp64<D, KK><<<blocks, kEvalThreads, smem, st>>>(e)));      \
-    break;
-  switch (e.k) {
-    SG_EVAL_K(1)
-    SG_EVAL_K(2)
-    SG_EVAL_K(3)
-    SG_EVAL_K(4)
-    SG_EVAL_K(6)
-    default:
-      SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64_anyk<D>, static_cast<int>(smem)));
-      SG_TIMED("k_eval_fp64", st, (k_eval_fp64_anyk<D><<<blocks, kEvalThreads, smem, st>>>(e)));
-  }
-#undef SG_EVAL_K
-  SG_LAUNCH_CHECK("k_eval_fp64");
+template <int K>
+static int launch_eval_fp64_nested(const EvalArgs& e, int d, int c0, cudaStream_t st) {
+  const int64_t blocks = ceil_div(e.Q, kNestQ);
+  // four warps per block fill the SMs (the FP64 pipe needs about four warps in
+  // flight per scheduler); with fewer blocks than that, more warps per block
+  int nw = 4;
+  while (nw < 16 && blocks * nw < int64_t(kNumSMs) * 16) nw *= 2;
+  const size_t tab = sizeof(double) * d * e.nf * kNestQ, sum = sizeof(double) * nw * K * 32;
+  const size_t stage0 = tab > sum ? tab : sum, smem = stage0 + nw * nested_stage_bytes(K);
+  SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64_nested<K>, smem));
+  SG_TIMED("k_eval_fp64_nested", st,
+           (k_eval_fp64_nested<K><<<static_cast<unsigned>(blocks), 32 * nw, smem, st>>>(e, d, c0, stage0)));
+  SG_LAUNCH_CHECK("k_eval_fp64_nested");
   return SG_OK;
 }
 
+template <int K, int QB>
+static int launch_eval_fp64_nodes(const EvalArgs& e, int d, int c0, cudaStream_t st) {
+  const size_t tab = sizeof(double) * d * e.nf * QB, sum = sizeof(double) * kNodesThreads / 32 * QB * K;
+  const size_t smem = tab > sum ? tab : sum;
+  SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64_nodes<K, QB>, smem));
+  SG_TIMED("k_eval_fp64_nodes", st,
+           (k_eval_fp64_nodes<K, QB><<<static_cast<unsigned>(ceil_div(e.Q, QB)), kNodesThreads, smem, st>>>(e, d, c0)));
+  SG_LAUNCH_CHECK("k_eval_fp64_nodes");
+  return SG_OK;
+}
+
+// K columns from c0 on.  The nested form needs 0.6 of the per-node form's
+// FP64 operations but comes in blocks of 32 queries, one SM's work at least: it
+// is taken when the queries fill two thirds of the waves of blocks they need
+// (level 4: 5,000 queries 0.124 ms per node; 8,000 queries 0.117 ms nested,
+// which the per-node form would take 0.19 ms for).  Below, the smallest number
+// of queries per block that leaves at most four blocks per SM.
+template <int K>
+static int launch_eval_fp64(const EvalArgs& e, int d, int c0, cudaStream_t st) {
+  const int64_t waves = ceil_div(ceil_div(e.Q, kNestQ), kNumSMs);
+  if (3 * e.Q >= 2 * waves * kNumSMs * kNestQ) return launch_eval_fp64_nested<K>(e, d, c0, st);
+  if (e.Q <= 4 * kNumSMs) return launch_eval_fp64_nodes<K, 1>(e, d, c0, st);
+  if (e.Q <= 16 * kNumSMs) return launch_eval_fp64_nodes<K, 4>(e, d, c0, st);
+  return launch_eval_fp64_nodes<K, 16>(e, d, c0, st);
+}
+
 int eval_fp64(const EvalArgs& e, int d, cudaStream_t st) {
-  switch (d) {
-    case 1: return launch_eval_fp64<1>(e, st);
-    case 2: return launch_eval_fp64<2>(e, st);
-    case 3: return launch_eval_fp64<3>(e, st);
-    case 4: return launch_eval_fp64<4>(e, st);
-    case 5: return launch_eval_fp64<5>(e, st);
-    case 6: return launch_eval_fp64<6>(e, st);
-    case 7: return launch_eval_fp64<7>(e, st);
-    case 8: return launch_eval_fp64<8>(e, st);
-    default: return fail(SG_EUNSUPPORTED, "sg_eval_feedback: d must be 1..8");
+  if (d < 1 || d > kMaxDim) return fail(SG_EUNSUPPORTED, "sg_eval_feedback: d must be 1..8");
+  if (sizeof(double) * d * e.nf * kEvalThreads > 200 * 1024)
+    return fail(SG_EUNSUPPORTED, "sg_eval_feedback: grid level too high for the FP64 kernel");
+  switch (e.k) {
+    case 1: return launch_eval_fp64<1>(e, d, 0, st);
+    case 2: return launch_eval_fp64<2>(e, d, 0, st);
+    case 3: return launch_eval_fp64<3>(e, d, 0, st);
+    case 4: return launch_eval_fp64<4>(e, d, 0, st);
+    case 6: return launch_eval_fp64<6>(e, d, 0, st);
+    default:   // any output count, four columns at a time (rarely used shapes)
+      for (int c0 = 0; c0 < e.k; c0 += 4) {
+        const int rc = launch_eval_fp64<4>(e, d, c0, st);
+        if (rc != SG_OK) return rc;
+      }
+      return SG_OK;
   }
 }
 
@@ -277,6 +453,7 @@ struct SurplusHost {
   SfPlan sf;                    // scalar fields (its tables are in the staged bytes)
   size_t npack = 0, off = 0, ohost = 0;
   size_t oW = 0, oWs = 0, oWdf = 0, oxf = 0, oxfdf = 0, otab1 = 0, obp = 0, oerr = 0, osfb = 0;
+  size_t oWt = 0, oprog = 0, opath = 0, onested = 0;   // nested order (FP64 evaluation)
   size_t obox = 0, onact = 0, oops = 0, otcoff = 0, ofid = 0, ofpt = 0, oorder = 0, ometa = 0, obmap = 0;
   std::vector<unsigned char> staging;   // bytes [ohost, off) of the allocation, box zero
   // The same bytes in page-locked memory when it could be had (then
@@ -356,6 +533,34 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   // grp[a] = first node with at least a active dimensions (non-decreasing)
   for (int a = kMaxDim; a >= 0; --a) h->grp[a] = h->grp[a] < h->grp[a + 1] ? h->grp[a] : h->grp[a + 1];
 
+  // the nested order (preorder of the tree of active dimensions): function
+  // ids lexicographically; per node its depth and last table offset, and the
+  // offsets of its whole path
+  std::vector<int32_t> nested(M);
+  std::iota(nested.begin(), nested.end(), 0);
+  std::stable_sort(nested.begin(), nested.end(), [&](int32_t a, int32_t b) {
+    return std::lexicographical_compare(&fid[int64_t(a) * d], &fid[int64_t(a) * d] + d, &fid[int64_t(b) * d],
+                                        &fid[int64_t(b) * d] + d);
+  });
+  std::vector<uint32_t> prog(M, 0), depth(M, 0);
+  std::vector<uint16_t> path(M * kMaxDim, 0);
+  for (int64_t r = 0; r < M; ++r) {
+    int na = 0;
+    for (int dim = 0; dim < d; ++dim) {
+      const int id = fid[int64_t(nested[r]) * d + dim];
+      if (id != 0) path[r * kMaxDim + na++] = static_cast<uint16_t>(dim * h->nf + id);
+    }
+    depth[r] = na;
+  }
+  // a node's first child, if any, is the entry after it
+  uint32_t run = 0;
+  for (int64_t r = M - 1; r >= 0; --r) {
+    const bool leaf = r + 1 == M || depth[r + 1] <= depth[r];
+    const bool joins = r + 1 < M && run != 0 && depth[r + 1] == depth[r] && run < 0xFFFFu;
+    run = leaf ? (joins ? run + 1 : 1) : 0;
+    prog[r] = nested_entry(depth[r] ? path[r * kMaxDim + depth[r] - 1] : 0u, depth[r], run);
+  }
+
   // one device allocation: the surplus's arrays and the build's tables; the
   // device-computed ones first, then the host-made ones (one copy)
   size_t off = 0;
@@ -366,6 +571,7 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   };
   h->oW = take(M * k * sizeof(double));
   h->oWs = take(M * k * sizeof(double));
+  h->oWt = take(M * k * sizeof(double));
   h->oWdf = take(M * k * sizeof(float2));
   h->oxf = take((fine_n + 1) * sizeof(double));
   h->oxfdf = take((fine_n + 1) * sizeof(float2));
@@ -388,6 +594,9 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   h->ofid = take(M * d * sizeof(uint16_t));
   h->ofpt = take(M * d * sizeof(int16_t));
   h->oorder = take(M * sizeof(int32_t));
+  h->onested = take(M * sizeof(int32_t));
+  h->oprog = take(M * sizeof(uint32_t));
+  h->opath = take(M * kMaxDim * sizeof(uint16_t));
   h->ometa = take(h->sf_ok ? h->sf.meta.size() : 0);
   h->obmap = take(h->sf_ok ? h->sf.bmap.size() * sizeof(int32_t) : 0);
   h->off = off;
@@ -404,6 +613,9 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   std::memcpy(st.data() + (h->ofid - oh), fid.data(), M * d * sizeof(uint16_t));
   std::memcpy(st.data() + (h->ofpt - oh), fpt.data(), M * d * sizeof(int16_t));
   std::memcpy(st.data() + (h->oorder - oh), order.data(), M * sizeof(int32_t));
+  std::memcpy(st.data() + (h->onested - oh), nested.data(), M * sizeof(int32_t));
+  std::memcpy(st.data() + (h->oprog - oh), prog.data(), M * sizeof(uint32_t));
+  std::memcpy(st.data() + (h->opath - oh), path.data(), M * kMaxDim * sizeof(uint16_t));
   if (h->sf_ok) {
     std::memcpy(st.data() + (h->ometa - oh), h->sf.meta.data(), h->sf.meta.size());
     std::memcpy(st.data() + (h->obmap - oh), h->sf.bmap.data(), h->sf.bmap.size() * sizeof(int32_t));
@@ -478,6 +690,9 @@ extern "C" int sg_build_surpluses(const sg_grid* g, const double* d_values, int 
   char* base = static_cast<char*>(s->block);
   s->W = reinterpret_cast<double*>(base + h.oW);
   s->Ws = reinterpret_cast<double*>(base + h.oWs);
+  s->Wt = reinterpret_cast<double*>(base + h.oWt);
+  s->prog = reinterpret_cast<uint32_t*>(base + h.oprog);
+  s->path = reinterpret_cast<uint16_t*>(base + h.opath);
   s->Wdf = reinterpret_cast<float2*>(base + h.oWdf);
   s->xf = reinterpret_cast<double*>(base + h.oxf);
   s->xfdf = reinterpret_cast<float2*>(base + h.oxfdf);
@@ -491,6 +706,7 @@ extern "C" int sg_build_surpluses(const sg_grid* g, const double* d_values, int 
   auto* d_fpt = reinterpret_cast<int16_t*>(base + h.ofpt);
   auto* d_tab1 = reinterpret_cast<double*>(base + h.otab1);
   auto* d_order = reinterpret_cast<int32_t*>(base + h.oorder);
+  auto* d_nested = reinterpret_cast<int32_t*>(base + h.onested);
   if (h.sf_ok) {
     const SfPlan& sf = h.sf;
     s->sf_ok = 1;
@@ -542,7 +758,7 @@ extern "C" int sg_build_surpluses(const sg_grid* g, const double* d_values, int 
                  n0, n1, d, k, fine_n, d_fid, d_fpt, d_tab1, d_values, s->W)));
     SG_TRY_CLEAN(cudaGetLastError());
   }
-  SG_TIMED("k_gather_rows", st, (k_gather_rows<<<static_cast<unsigned>(ceil_div(M * k, 256)), 256, 0, st>>>(M, k, d_order, s->W, s->Ws)));
+  SG_TIMED("k_gather_rows", st, (k_gather_rows<<<static_cast<unsigned>(ceil_div(M * k, 256)), 256, 0, st>>>(M, k, d_order, d_nested, s->W, s->Ws, s->Wt)));
   SG_TRY_CLEAN(cudaGetLastError());
   if (split_df(fine_n + 1, s->xf, s->xfdf, st) != SG_OK || split_df(M * k, s->Ws, s->Wdf, st) != SG_OK)
     return cleanup(cudaGetLastError(), "split_df");
@@ -588,6 +804,9 @@ extern "C" int sg_eval_feedback(const sg_surplus* s, const double* d_xq, int64_t
   e.nact = s->nact;
   e.ops = s->ops;
   e.W = s->Ws;
+  e.Wt = s->Wt;
+  e.prog = s->prog;
+  e.path = s->path;
   e.lo = s->box;
   e.width = s->box + s->d;
   e.xf = s->xf;

@@ -22,6 +22,9 @@ struct EvalArgs {
   const uint8_t* nact;    // M: number of active (level >= 2) dimensions
   const uint16_t* ops;    // M x kMaxDim: table offsets dim * nf + id of the active dimensions
   const double* W;        // M x k, evaluation order
+  const double* Wt;       // M x k, nested order
+  const uint32_t* prog;   // M, nested order: nested_entry of each node
+  const uint16_t* path;   // M x kMaxDim, nested order: table offsets of the active dimensions
   const double* lo;       // d
   const double* width;    // d: hi - lo (divided, so that nodes map exactly)
   const double* xf;       // 2^L + 1 points of the finest 1-D set
@@ -65,6 +68,9 @@ struct sg_surplus {
   int64_t M = 0;
   double* W = nullptr;            // M x k, grid order
   double* Ws = nullptr;           // M x k, evaluation order
+  double* Wt = nullptr;           // M x k, nested order (function ids lexicographically)
+  uint32_t* prog = nullptr;       // M, nested order: nested_entry of each node
+  uint16_t* path = nullptr;       // M x kMaxDim, nested order
   uint8_t* nact = nullptr;        // M, evaluation order (sorted by this count)
   int64_t grp[sg::kMaxDim + 2] = {};  // first node with >= a active dimensions
   uint16_t* ops = nullptr;        // M x kMaxDim
