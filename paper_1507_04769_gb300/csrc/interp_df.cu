@@ -28,20 +28,6 @@ constexpr int kDfChunk = 256;      // nodes staged in shared memory at a time
 template <int K>
 constexpr int df_kp() { return (K + 1) & ~1; }
 
-// Product of a pair with a pair, left unnormalised: the result (p, e) has
-// p = fl(a.hi b.hi) and e = the exact rounding error of p plus the cross
-// terms, so p + e carries the product to about 2^-46 relative.  Skipping the
-// renormalisation is safe because |e| stays below about 2^-22 |p| and every
-// consumer (the next product, the compensated dot) treats hi and lo only
-// through products and exact sums.
-__device__ __forceinline__ df df_mul_raw(df a, df b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  float e = __fmaf_rn(a.hi, b.hi, -p);
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  return {p, e};
-}
-
 struct DfAcc {
   double total;
   float ah, al;
