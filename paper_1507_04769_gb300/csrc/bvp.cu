@@ -182,7 +182,6 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
   const unsigned gupd = static_cast<unsigned>(ceil_div(npoint * kUpdPer, 128));
   const unsigned ginit = static_cast<unsigned>(ceil_div(npoint * kInitPer, 128));
   const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
-  const unsigned gnode_thr = static_cast<unsigned>(ceil_div(a.n, 128));
   const unsigned gnode_warp = static_cast<unsigned>(ceil_div(a.n * 32, 128));
   if (a.persistent) {
     // one warp per node, nodes from a device queue, no host round trip
@@ -199,7 +198,7 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
     SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 4 * sizeof(int), st));
     SG_TIMED("k_init", st, (k_init<<<ginit, 128, 0, st>>>(a, w)));
     SG_TIMED(kname<T>("k_newton_persistent"), st, (k_newton_persistent<T><<<grid, 128, smem, st>>>(a, w)));
-    SG_TIMED("k_outputs", st, (k_outputs<<<gnode_warp, 128, 0, st>>>(a, w, lambda0, u0, V, status, iters)));
+    SG_TIMED("k_outputs", st, (k_outputs<<<static_cast<unsigned>(a.n), kOutThreads, 0, st>>>(a, w, lambda0, u0, V, status, iters)));
     if (Yout) SG_TIMED("k_copy_Y", st, (k_copy_Y<<<gp, 128, 0, st>>>(a, w, Yout)));
     SG_LAUNCH_CHECK("persistent solve");
     if (a.sync_at_end) SG_CUDA_TRY(cudaStreamSynchronize(st));
@@ -208,49 +207,44 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
   SG_CUDA_TRY(direction_setup<T>(a));
   DirLaunch dir[kDirLaunches<T>];
   direction_launches<T>(a, dir);
-  int h_cnt[2] = {0, 0};
+  int h_cnt[2] = {0, 0};   // nodes still in the line search, nodes left to iterate
   auto read_counters = [&]() -> int {
-    cudaError_t e = cudaMemcpyAsync(h_cnt, w.counters, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(h_cnt, w.counters + kSearchOut, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, "counter copy");
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "solver kernels");
     return SG_OK;
   };
+  static_assert(kActiveOut == kSearchOut + 1, "read together");
   int rc;
-  SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 2 * sizeof(int), st));
+  SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, kCounters * sizeof(int), st));
   SG_TIMED("k_init", st, (k_init<<<ginit, 128, 0, st>>>(a, w)));
   SG_TIMED("k_trial", st, (trial_kernel<T>(a)<<<gi, 128, 0, st>>>(a, w)));
   SG_TIMED("k_ls_reduce", st, (k_ls_reduce<<<gnode_warp, 128, 0, st>>>(a, w, 0)));
   SG_LAUNCH_CHECK("init kernels");
   if ((rc = read_counters()) != SG_OK) return rc;
-  int active = h_cnt[1];
-  for (int it = 0; it < a.max_iter && active > 0; ++it) {
-    SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, kCounters * sizeof(int), st));
-    if (!a.jac_in_trial) SG_TIMED(kname<T>("k_point"), st, (k_point<T><<<gp, 128, 0, st>>>(a, w)));   // else stored by the last trial
+  for (int it = 0; it < a.max_iter && h_cnt[1] > 0; ++it) {
+    if constexpr (sizeof(T) == sizeof(double)) SG_TIMED("k_point_fp64", st, (k_point_fp64<<<gp, 128, 0, st>>>(a, w)));
     for (const DirLaunch& d : dir)
       SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
-    SG_TIMED("k_ls_begin", st, (k_ls_begin<<<gnode_thr, 128, 0, st>>>(a, w)));
     SG_LAUNCH_CHECK("newton kernels");
     for (int trial = 0; trial < 13; ++trial) {   // alpha = 1, 1/2, ..., 2^-10 (and one at 0 in the FP64 form)
       if constexpr (sizeof(T) == sizeof(double)) {
         const DirLaunch d = elim_launch(a);
         SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
       }
-      SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, sizeof(int), st));
       SG_TIMED("k_trial", st, (trial_kernel<T>(a)<<<gi, 128, 0, st>>>(a, w)));
       SG_TIMED("k_ls_reduce", st, (k_ls_reduce<<<gnode_warp, 128, 0, st>>>(a, w, 1)));
       SG_LAUNCH_CHECK("line search kernels");
       if ((rc = read_counters()) != SG_OK) return rc;
       if (h_cnt[0] == 0) break;
     }
-    SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 2 * sizeof(int), st));
-    if (!a.jac_in_trial) SG_TIMED("k_update", st, (k_update<<<gupd, 128, 0, st>>>(a, w)));   // else the accepted trial point
-    SG_TIMED("k_after_update", st, (k_after_update<<<gnode_thr, 128, 0, st>>>(a, w)));
-    SG_LAUNCH_CHECK("update kernels");
-    if ((rc = read_counters()) != SG_OK) return rc;
-    active = h_cnt[1];
+    if constexpr (sizeof(T) == sizeof(double)) {
+      SG_TIMED("k_update", st, (k_update<<<gupd, 128, 0, st>>>(a, w)));
+      SG_LAUNCH_CHECK("k_update");
+    }
   }
-  SG_TIMED("k_outputs", st, (k_outputs<<<gnode_warp, 128, 0, st>>>(a, w, lambda0, u0, V, status, iters)));
+  SG_TIMED("k_outputs", st, (k_outputs<<<static_cast<unsigned>(a.n), kOutThreads, 0, st>>>(a, w, lambda0, u0, V, status, iters)));
   if (Yout) SG_TIMED("k_copy_Y", st, (k_copy_Y<<<gp, 128, 0, st>>>(a, w, Yout)));
   SG_LAUNCH_CHECK("output kernels");
   SG_CUDA_TRY(cudaStreamSynchronize(st));
@@ -263,18 +257,6 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
 // device from the active / searching counters, so the data-dependent loop
 // trip counts never reach the host.  Executable graphs are cached per
 // (sizes, precision, buffers, problem): one per mesh size for a given batch.
-__global__ void k_set_cond(cudaGraphConditionalHandle h, const int* cnt) {
-  cudaGraphSetConditional(h, cnt[0] > 0 ? 1u : 0u);
-}
-__global__ void k_set_cond_one(cudaGraphConditionalHandle h) { cudaGraphSetConditional(h, 1u); }
-
-// Counts the nodes that start a line search (replaces the host read).
-__global__ void k_count_searching(SolveArgs a, Workspace w) {
-  const int64_t node = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (node >= a.n) return;
-  if (w.ns[node].searching) atomicAdd(&w.counters[0], 1);
-}
-
 struct GraphBuilder {
   cudaGraph_t g;
   std::vector<cudaGraphNode_t> last;   // dependencies for the next node
@@ -322,61 +304,65 @@ struct GraphBuilder {
   }
 };
 
+// One trial of the line search: the elimination of marked nodes (FP64 form), the
+// residual at the trial point, the decision.
 template <typename T>
-static cudaError_t build_solve_graph(const SolveArgs& a, const Workspace& w, double* lambda0, double* u0,
+static void add_trial(GraphBuilder& b, const SolveArgs& a, const Workspace& w) {
+  if constexpr (sizeof(T) == sizeof(double)) {
+    const DirLaunch d = elim_launch(a);
+    b.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+  }
+  b.kernel(trial_kernel<T>(a), static_cast<unsigned>(a.n * trial_chunks(a.Nmax)), 128, 0, a, w);
+  b.kernel(k_ls_reduce, static_cast<unsigned>(ceil_div(a.n, 4)), 128, 0, a, w, 1);
+}
+
+// One Newton iteration; the first trial is in line (it is the only one for
+// nearly every node), further ones are a WHILE loop on a.h_search.
+template <typename T>
+static void add_iteration(GraphBuilder& b, const SolveArgs& a, const Workspace& w) {
+  const int64_t np = a.n * npts(a.Nmax);
+  if (b.err == cudaSuccess) b.err = direction_setup<T>(a);
+  if constexpr (sizeof(T) == sizeof(double))
+    b.kernel(k_point_fp64, static_cast<unsigned>(ceil_div(np, 128)), 128, 0, a, w);
+  DirLaunch dir[kDirLaunches<T>];
+  direction_launches<T>(a, dir);
+  for (const DirLaunch& d : dir) b.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+  add_trial<T>(b, a, w);
+  cudaGraph_t body = nullptr;
+  b.loop(a.h_search, &body);
+  if (b.err == cudaSuccess) {
+    GraphBuilder lb{body, {}};
+    add_trial<T>(lb, a, w);
+    b.err = lb.err;
+  }
+  if constexpr (sizeof(T) == sizeof(double))   // FP32: the accepted trial point is the iterate
+    b.kernel(k_update, static_cast<unsigned>(ceil_div(np * kUpdPer, 128)), 128, 0, a, w);
+}
+
+template <typename T>
+static cudaError_t build_solve_graph(SolveArgs a, const Workspace& w, double* lambda0, double* u0,
                                      double* V, int32_t* status, int32_t* iters, double* Yout,
                                      cudaGraph_t* out) {
-  const int64_t P = npts(a.Nmax);
-  const unsigned gp = static_cast<unsigned>(ceil_div(a.n * P, 128));
-  const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
-  const unsigned gnt = static_cast<unsigned>(ceil_div(a.n, 128));
-  const unsigned gnw = static_cast<unsigned>(ceil_div(a.n * 32, 128));
+  const int64_t np = a.n * npts(a.Nmax);
   cudaGraph_t root;
   cudaError_t e = cudaGraphCreate(&root, 0);
   if (e != cudaSuccess) return e;
-  cudaGraphConditionalHandle hn, hl;
-  if ((e = cudaGraphConditionalHandleCreate(&hn, root, 0, 0)) != cudaSuccess) return e;
-  if ((e = cudaGraphConditionalHandleCreate(&hl, root, 0, 0)) != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&a.h_newton, root, 0, 0)) != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&a.h_search, root, 0, 0)) != cudaSuccess) return e;
+  a.conds = 3;
   GraphBuilder rb{root, {}};
-  rb.memset0(w.counters, 4 * sizeof(int));
-  rb.kernel(k_init, static_cast<unsigned>(ceil_div(a.n * P * kInitPer, 128)), 128, 0, a, w);
-  rb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);
-  rb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 0);
-  rb.kernel(k_set_cond, 1, 1, 0, hn, static_cast<const int*>(w.counters + 1));
-  cudaGraph_t newton_body;
-  rb.loop(hn, &newton_body);
-  rb.kernel(k_outputs, gnw, 128, 0, a, w, lambda0, u0, V, status, iters);
-  if (Yout) rb.kernel(k_copy_Y, gp, 128, 0, a, w, Yout);
+  rb.memset0(w.counters, kCounters * sizeof(int));
+  rb.kernel(k_init, static_cast<unsigned>(ceil_div(np * kInitPer, 128)), 128, 0, a, w);
+  rb.kernel(trial_kernel<T>(a), static_cast<unsigned>(a.n * trial_chunks(a.Nmax)), 128, 0, a, w);
+  rb.kernel(k_ls_reduce, static_cast<unsigned>(ceil_div(a.n, 4)), 128, 0, a, w, 0);
+  cudaGraph_t newton_body = nullptr;
+  rb.loop(a.h_newton, &newton_body);
+  rb.kernel(k_outputs, static_cast<unsigned>(a.n), kOutThreads, 0, a, w, lambda0, u0, V, status, iters);
+  if (Yout) rb.kernel(k_copy_Y, static_cast<unsigned>(ceil_div(np, 128)), 128, 0, a, w, Yout);
   if (rb.err != cudaSuccess) return rb.err;
-
   GraphBuilder nb{newton_body, {}};
-  nb.memset0(w.counters, kCounters * sizeof(int));
-  if (!a.jac_in_trial) nb.kernel(k_point<T>, gp, 128, 0, a, w);   // else stored by the last trial
-  if (nb.err == cudaSuccess) nb.err = direction_setup<T>(a);
-  DirLaunch dir[kDirLaunches<T>];
-  direction_launches<T>(a, dir);
-  for (const DirLaunch& d : dir) nb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
-  nb.kernel(k_ls_begin, gnt, 128, 0, a, w);
-  nb.kernel(k_set_cond_one, 1, 1, 0, hl);
-  cudaGraph_t ls_body;
-  nb.loop(hl, &ls_body);
-  nb.memset0(w.counters, 2 * sizeof(int));
-  if (!a.jac_in_trial)   // else the accepted trial point is the iterate
-    nb.kernel(k_update, static_cast<unsigned>(ceil_div(a.n * npts(a.Nmax) * kUpdPer, 128)), 128, 0, a, w);
-  nb.kernel(k_after_update, gnt, 128, 0, a, w);
-  nb.kernel(k_set_cond, 1, 1, 0, hn, static_cast<const int*>(w.counters + 1));
+  add_iteration<T>(nb, a, w);
   if (nb.err != cudaSuccess) return nb.err;
-
-  GraphBuilder lb{ls_body, {}};
-  if constexpr (sizeof(T) == sizeof(double)) {
-    const DirLaunch d = elim_launch(a);
-    lb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
-  }
-  lb.memset0(w.counters, sizeof(int));
-  lb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);
-  lb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 1);
-  lb.kernel(k_set_cond, 1, 1, 0, hl, static_cast<const int*>(w.counters));
-  if (lb.err != cudaSuccess) return lb.err;
   *out = root;
   return cudaSuccess;
 }
@@ -394,7 +380,7 @@ static cudaError_t build_persistent_graph(const SolveArgs& a, const Workspace& w
   rb.memset0(w.counters, 4 * sizeof(int));
   rb.kernel(k_init, static_cast<unsigned>(ceil_div(a.n * P * kInitPer, 128)), 128, 0, a, w);
   rb.kernel(k_newton_persistent<T>, grid, 128, static_cast<size_t>(smem), a, w);
-  rb.kernel(k_outputs, static_cast<unsigned>(ceil_div(a.n * 32, 128)), 128, 0, a, w, lambda0, u0, V, status, iters);
+  rb.kernel(k_outputs, static_cast<unsigned>(a.n), kOutThreads, 0, a, w, lambda0, u0, V, status, iters);
   if (Yout) rb.kernel(k_copy_Y, static_cast<unsigned>(ceil_div(a.n * P, 128)), 128, 0, a, w, Yout);
   if (rb.err != cudaSuccess) return rb.err;
   *out = root;
@@ -706,9 +692,6 @@ extern "C" int sg_solve_bvps(const sg_problem* prob, const double* d_x0, int64_t
   a.sync_at_end = 1;
   a.Yin = o.warm_start ? d_Y : nullptr;
   a.res_pair = o.precision == SG_PREC_MIXED_PAIR ? 1 : 0;
-  // the FP32 Jacobian from the FP64 residual kernel (its FP32 pipe is idle
-  // beside the FP64 work) in the launch-per-phase and graph forms
-  a.jac_in_trial = fp32_direction(o.precision) && !a.res_pair && !o.persistent ? 1 : 0;
   a.tree = o.precision == SG_PREC_FP64 && !o.persistent ? 1 : 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (o.graph == 2 && !d_Y) {
@@ -912,12 +895,10 @@ __global__ void k_pool_flags(SolveArgs a, Workspace w, uint8_t* flags) {
   flags[node] = w.ns[node].active ? 1 : 0;
 }
 
-__global__ void k_pool_outputs(SolveArgs a, Workspace w, const int64_t* list, int64_t count, double* lambda0,
-                               double* u0, double* V, int32_t* status, int32_t* iters) {
-  const int lane = threadIdx.x & 31;
-  const int64_t j = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-  if (j >= count) return;
-  node_outputs(a, w, list[j], j, lane, lambda0, u0, V, status, iters);
+__global__ void __launch_bounds__(kOutThreads)
+    k_pool_outputs(SolveArgs a, Workspace w, const int64_t* list, double* lambda0, double* u0, double* V,
+                   int32_t* status, int32_t* iters) {
+  node_outputs(a, w, list[blockIdx.x], blockIdx.x, lambda0, u0, V, status, iters);
 }
 
 // Marks the slots of `list` free for the solver kernels (inactive, not searching).
@@ -930,49 +911,22 @@ __global__ void k_pool_release(Workspace w, const int64_t* list, int64_t count) 
 }
 
 // One pool iteration as a graph: the initial residual of new slots, then one
-// Newton step of every active slot (the body of the Newton loop of
-// build_solve_graph, run once).
+// Newton iteration of every active slot (that of build_solve_graph, run once).
 template <typename T>
-static cudaError_t build_pool_graph(const SolveArgs& a, const Workspace& w, uint8_t* flags, cudaGraph_t* out) {
-  const int64_t P = npts(a.Nmax);
-  const unsigned gp = static_cast<unsigned>(ceil_div(a.n * P, 128));
-  const unsigned gi = static_cast<unsigned>(a.n * trial_chunks(a.Nmax));
-  const unsigned gnt = static_cast<unsigned>(ceil_div(a.n, 128));
-  const unsigned gnw = static_cast<unsigned>(ceil_div(a.n * 32, 128));
+static cudaError_t build_pool_graph(SolveArgs a, const Workspace& w, uint8_t* flags, cudaGraph_t* out) {
   cudaGraph_t root;
   cudaError_t e = cudaGraphCreate(&root, 0);
   if (e != cudaSuccess) return e;
-  cudaGraphConditionalHandle hl;
-  if ((e = cudaGraphConditionalHandleCreate(&hl, root, 0, 0)) != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&a.h_search, root, 0, 0)) != cudaSuccess) return e;
+  a.conds = 2;
   GraphBuilder rb{root, {}};
-  rb.memset0(w.counters, 4 * sizeof(int));
-  rb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);     // new slots only (searching at alpha = 0)
-  rb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 0);
-  rb.memset0(w.counters, kCounters * sizeof(int));
-  rb.kernel(k_point<T>, gp, 128, 0, a, w);
-  if (rb.err == cudaSuccess) rb.err = direction_setup<T>(a);
-  DirLaunch dir[kDirLaunches<T>];
-  direction_launches<T>(a, dir);
-  for (const DirLaunch& d : dir) rb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
-  rb.kernel(k_ls_begin, gnt, 128, 0, a, w);
-  rb.kernel(k_set_cond_one, 1, 1, 0, hl);
-  cudaGraph_t ls_body;
-  rb.loop(hl, &ls_body);
-  rb.memset0(w.counters, 2 * sizeof(int));
-  rb.kernel(k_update, static_cast<unsigned>(ceil_div(a.n * P * kUpdPer, 128)), 128, 0, a, w);
-  rb.kernel(k_after_update, gnt, 128, 0, a, w);
-  rb.kernel(k_pool_flags, gnt, 128, 0, a, w, flags);
+  rb.memset0(w.counters, kEpoch * sizeof(int));
+  // new slots only (searching at alpha = 0)
+  rb.kernel(trial_kernel<T>(a), static_cast<unsigned>(a.n * trial_chunks(a.Nmax)), 128, 0, a, w);
+  rb.kernel(k_ls_reduce, static_cast<unsigned>(ceil_div(a.n, 4)), 128, 0, a, w, 0);
+  add_iteration<T>(rb, a, w);
+  rb.kernel(k_pool_flags, static_cast<unsigned>(ceil_div(a.n, 128)), 128, 0, a, w, flags);
   if (rb.err != cudaSuccess) return rb.err;
-  GraphBuilder lb{ls_body, {}};
-  if constexpr (sizeof(T) == sizeof(double)) {
-    const DirLaunch d = elim_launch(a);
-    lb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
-  }
-  lb.memset0(w.counters, sizeof(int));
-  lb.kernel(trial_kernel<T>(a), gi, 128, 0, a, w);
-  lb.kernel(k_ls_reduce, gnw, 128, 0, a, w, 1);
-  lb.kernel(k_set_cond, 1, 1, 0, hl, static_cast<const int*>(w.counters));
-  if (lb.err != cudaSuccess) return lb.err;
   *out = root;
   return cudaSuccess;
 }
@@ -1061,6 +1015,8 @@ extern "C" int sg_pool_create(const sg_problem* prob, int64_t slots, int n_max_i
   // of a valid empty node so that no kernel reads garbage
   if ((e = cudaMemsetAsync(p->w.ns, 0, slots * sizeof(NodeState), st)) != cudaSuccess)
     return bail(e, "sg_pool_create: clearing the node states");
+  if ((e = cudaMemsetAsync(p->w.counters, 0, kCounters * sizeof(int), st)) != cudaSuccess)
+    return bail(e, "sg_pool_create: clearing the counters");
   if ((e = cudaMemsetAsync(base + L.x0, 0, L.ws - L.x0, st)) != cudaSuccess)
     return bail(e, "sg_pool_create: clearing the inputs");
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(e, "sg_pool_create");
@@ -1196,8 +1152,8 @@ extern "C" int sg_pool_collect(sg_pool* pool, const int64_t* slots, int64_t coun
   for (int64_t j = 0; j < count; ++j) p->h_list[j] = slots[j];
   SG_CUDA_TRY(cudaMemcpyAsync(p->d_list, p->h_list, count * sizeof(int64_t), cudaMemcpyHostToDevice, st));
   SG_TIMED("k_pool_outputs", st,
-           (k_pool_outputs<<<static_cast<unsigned>(ceil_div(count * 32, 128)), 128, 0, st>>>(
-               p->a, p->w, p->d_list, count, d_lambda0, d_u0, d_V, d_status, d_iters)));
+           (k_pool_outputs<<<static_cast<unsigned>(count), kOutThreads, 0, st>>>(
+               p->a, p->w, p->d_list, d_lambda0, d_u0, d_V, d_status, d_iters)));
   SG_TIMED("k_pool_release", st,
            (k_pool_release<<<static_cast<unsigned>(ceil_div(count, 128)), 128, 0, st>>>(p->w, p->d_list, count)));
   SG_LAUNCH_CHECK("sg_pool_collect");

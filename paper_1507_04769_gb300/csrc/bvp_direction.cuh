@@ -610,10 +610,12 @@ __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, W
       D[tid] = y0;
     }
   }
-  if (__syncthreads_or(bad)) {
-    if (tid == 0) mark_elim(w, node);
-    return;   // k_elim_fp64 solves it
+  bad = __syncthreads_or(bad);
+  if (tid == 0) {
+    if (bad) mark_elim(w, node);
+    ls_start(w, node);
   }
+  if (bad) return;   // k_elim_fp64 solves it
 
   // down the tree: the corrections at the middle of [i, e) from those at its ends
   int top = 1;

@@ -2,10 +2,9 @@
 // four-stage Lobatto IIIA collocation on N equal intervals, damped Newton.
 //
 // One Newton iteration:
-//   k_point     Jacobian dF/dy (precision T) at every collocation point (in
-//               the mixed form with the FP64 residual, k_trial stores it
-//               instead: the last trial of a line search is the next
-//               iterate)
+//   k_point     FP64 form: Jacobian dF/dy at every collocation point (in the
+//               FP32 forms k_trial stores it: the last trial of a line search
+//               is the next iterate)
 //   k_condense  the 36 linearised stage equations of one interval; Gaussian
 //               elimination of the two interior stages (24 columns, partial
 //               pivoting over the 24 interior rows) leaves the 12 x 25 block
@@ -48,14 +47,13 @@ namespace sg {
    {1.0 / 12.0, 5.0 / 12.0, 5.0 / 12.0, 1.0 / 12.0}}
 __constant__ double kLobA[4][4] = SG_LOB_A;
 __constant__ float kLobAf[4][4] = SG_LOB_A;
-__constant__ double kLobB[4] = {1.0 / 12.0, 5.0 / 12.0, 5.0 / 12.0, 1.0 / 12.0};
 
 struct NodeState {
   double fnorm2;   // |F|_2^2 at the current iterate
   double fmax;     // |F|_inf at the current iterate
   double alpha;    // current step length
   int active;      // still iterating
-  int searching;   // in the line search
+  int searching;   // 1: in the line search; -e: step accepted in iteration e (FP64 form, for k_update)
   int singular;    // bit 0: a zero pivot was met this iteration; kElimNode, kElimDone
   int iters;
   int status;
@@ -65,8 +63,12 @@ struct NodeState {
 // NodeState::singular, FP64 form: the node waits for the direction of the
 // elimination with full partial pivoting (k_elim_fp64) / has it
 constexpr int kElimNode = 2, kElimDone = 4;
-constexpr int kCounters = 5;     // ints of Workspace::counters zeroed per Newton iteration
-constexpr int kElimCount = 4;    // index in Workspace::counters: nodes marked kElimNode
+// Workspace::counters (zeroed before a solve): nodes still in the line search
+// and nodes left to iterate so far in this iteration; nodes marked kElimNode;
+// the same two as the last block of k_ls_reduce found them (read by the host
+// loop); that kernel's finished blocks; Newton iterations so far
+constexpr int kSearchCount = 0, kActiveCount = 1, kElimCount = 4, kSearchOut = 5, kActiveOut = 6, kTicket = 7, kEpoch = 8,
+              kCounters = 16;
 
 constexpr int kCols = 49;        // 24 interior + 12 (y_i) + 12 (y_{i+1}) + rhs
 constexpr int kRecLd = 52;       // row stride of a stored interior pivot row (16-byte multiple)
@@ -122,7 +124,9 @@ struct SolveArgs {
   const double* Yin;   // initial iterate (n x P x 12), or null for the zero-control guess
   int res_pair;        // FP32-direction form: 1 = residual in pairs of floats, 0 = in FP64
   int tree;            // FP64 form, launch per phase or graph: direction from bvp_direction.cuh
-  int jac_in_trial;    // FP32-direction form with the FP64 residual: the residual kernel also stores the Jacobian
+  // graph form: the loops' conditions, set by k_ls_reduce
+  int conds;           // bit 0: h_newton exists, bit 1: h_search
+  cudaGraphConditionalHandle h_newton, h_search;
 };
 
 __host__ __device__ __forceinline__ int64_t npts(int Nmax) { return 3 * int64_t(Nmax) + 1; }
@@ -224,15 +228,17 @@ constexpr int kTrialJLd = 40;   // staged rows of one point in the fused Jacobia
 
 // (kJac: five blocks per SM, 96 registers with a few spilled dual values,
 // against 126 registers and four blocks; 2 % faster)
-template <typename T, bool kPair, bool kJac>
+template <typename T, bool kPair>
 __global__ void __launch_bounds__(128, 5) k_trial(SolveArgs a, Workspace w) {
+  constexpr bool kJac = sizeof(T) == sizeof(float);
   // kPair = false: points and rows in FP64 (the FP64 and mixed forms).
   // kPair = true (the mixed-pair form): the right-hand side and the stage rows
   // in pair-of-floats arithmetic (about 48 bits, on the FP32 pipe); the
   // boundary rows and the iterate Y + alpha D stay FP64.
-  // kJac (mixed form): the FP32 Jacobian at the trial point as well, on the
-  // FP32 pipe beside the FP64 residual; the last trial of a line search is
-  // the accepted iterate, so its Jacobian is the next iteration's.
+  // kJac (FP32 forms): the FP32 Jacobian at the trial point as well (in the
+  // mixed form on the FP32 pipe beside the FP64 residual); the last trial of a
+  // line search is the accepted iterate, so its Jacobian is the next
+  // iteration's.
   __shared__ __align__(16) double yfs[2][kTrialPts][12];   // points and F (dfnum in the mixed-pair form)
   auto& ys = yfs[0];
   auto& fs = yfs[1];
@@ -244,7 +250,7 @@ __global__ void __launch_bounds__(128, 5) k_trial(SolveArgs a, Workspace w) {
   const int i0 = static_cast<int>(blockIdx.x % nchunk) * kTrialIv;
   if (node >= a.n) return;
   const NodeState& s = w.ns[node];
-  if (!s.searching) return;
+  if (s.searching != 1) return;
   const int N = a.N[node];
   if (i0 >= N) return;
   const int niv = N - i0 < kTrialIv ? N - i0 : kTrialIv;
@@ -273,8 +279,16 @@ __global__ void __launch_bounds__(128, 5) k_trial(SolveArgs a, Workspace w) {
   if (tid <= 3 * niv) {
     if constexpr (kPair) {
       dfnum y[12], F[12];
+      double2* alt = reinterpret_cast<double2*>((s.ybuf ? w.Y : w.Y2) + (base + tid) * 12);
 #pragma unroll
-      for (int c = 0; c < 12; ++c) y[c] = dfnum(ypoint(base + tid, c));
+      for (int c = 0; c < 12; c += 2) {
+        const double y0 = ypoint(base + tid, c), y1 = ypoint(base + tid, c + 1);
+        y[c] = dfnum(y0);
+        y[c + 1] = dfnum(y1);
+        yf[c] = y[c].hi;
+        yf[c + 1] = y[c + 1].hi;
+        alt[c / 2] = make_double2(y0, y1);   // as below
+      }
       char_rhs_t<dfnum>(a.P, y, F, node_target(a.P, node));
       dfnum* yp = reinterpret_cast<dfnum*>(ys[tid]);
       dfnum* fp = reinterpret_cast<dfnum*>(fs[tid]);
@@ -430,22 +444,34 @@ __global__ void __launch_bounds__(128, 5) k_trial(SolveArgs a, Workspace w) {
 template <typename T>
 inline void (*trial_kernel(const SolveArgs& a))(SolveArgs, Workspace) {
   if constexpr (sizeof(T) == sizeof(float)) {
-    if (a.res_pair) return k_trial<float, true, false>;
-    return a.jac_in_trial ? k_trial<float, false, true> : k_trial<float, false, false>;
+    return a.res_pair ? k_trial<float, true> : k_trial<float, false>;
   } else {
-    return k_trial<double, false, false>;
+    return k_trial<double, false>;
   }
 }
 
-// Warp per node: reduce the partial norms in a fixed order and decide.
-// mode 0: initial residual (convergence test at iteration 0);
-// mode 1: Armijo test for the current alpha.
-__global__ void k_ls_reduce(SolveArgs a, Workspace w, int mode) {
-  const int lane = threadIdx.x & 31;
-  const int64_t node = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-  if (node >= a.n) return;
+// A node's line search starts (after its direction's elimination).
+__device__ __forceinline__ void ls_start(const Workspace& w, int64_t node) {
   NodeState s = w.ns[node];
-  if (!s.searching) return;
+  if (!s.active) return;
+  if (s.singular & 1) {
+    s.status = SG_SINGULAR;
+    s.active = 0;
+  } else {
+    s.singular &= kElimNode;
+    s.searching = 1;
+    s.alpha = 1.0;
+  }
+  w.ns[node] = s;
+}
+
+// One warp reduces a node's partial norms in a fixed order and decides.
+// mode 0: initial residual (convergence test at iteration 0);
+// mode 1: Armijo test for the current alpha, and when the step is taken the
+// iteration's end: convergence, iteration cap.
+__device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, int64_t node, int lane, int mode) {
+  NodeState s = w.ns[node];
+  if (s.searching != 1) return;
   const int N = a.N[node];
   double ss = 0.0, mx = 0.0;
   for (int i = lane; i < N; i += 32) {
@@ -455,98 +481,86 @@ __global__ void k_ls_reduce(SolveArgs a, Workspace w, int mode) {
   ss = warp_sum(ss);
   mx = warp_max(mx);
   if (lane != 0) return;
-  if (mode == 0) {
-    s.fnorm2 = ss;
-    s.fmax = mx;
-    s.searching = 0;
-    if (!(mx < INFINITY)) {
-      s.status = SG_NONFINITE;
-      s.active = 0;
-    } else if (mx <= a.tol) {
-      s.status = SG_CONVERGED;
-      s.active = 0;
-    } else {
-      atomicAdd(&w.counters[1], 1);
-    }
+  if (mode == 1 && s.alpha == 0.0) {
+    // the residual rows at the iterate are back: the direction of the
+    // elimination next, and the search goes on at 1/2
+    s.alpha = 0.5;
+    s.singular |= kElimNode;
+    w.ns[node] = s;
+    atomicAdd(&w.counters[kSearchCount], 1);
+    atomicAdd(&w.counters[kElimCount], 1);
+    return;
+  }
+  const bool accept = mode == 0 || !a.damping || (ss < INFINITY && ss <= (1.0 - 2e-4 * s.alpha) * s.fnorm2) ||
+                      s.alpha <= 0x1p-10;
+  if (!accept) {
+    // FP64 form: a node far from its root follows the elimination's direction
+    // (its path depends on the last bits of it); alpha = 0 evaluates the
+    // rows at the iterate again, which that direction needs
+    s.alpha = a.tree && !(s.singular & kElimDone) ? 0.0 : 0.5 * s.alpha;
+    w.ns[node] = s;
+    atomicAdd(&w.counters[kSearchCount], 1);
+    return;
+  }
+  s.fnorm2 = ss;
+  s.fmax = mx;
+  s.searching = 0;
+  if (mode == 1) {
+    s.iters += 1;
+    if (a.tree) s.searching = -(w.counters[kEpoch] + 1);   // k_update takes the step
+    else s.ybuf ^= 1;                                      // the trial point is the iterate
+  }
+  if (!(mx < INFINITY)) {
+    s.status = SG_NONFINITE;
+    s.active = 0;
+  } else if (mx <= a.tol) {
+    s.status = SG_CONVERGED;
+    s.active = 0;
+  } else if (mode == 1 && s.iters >= a.max_iter) {
+    s.status = SG_MAXITER;
+    s.active = 0;
   } else {
-    if (s.alpha == 0.0) {
-      // the residual rows at the iterate are back: the direction of the
-      // elimination next, and the search goes on at 1/2
-      s.alpha = 0.5;
-      s.singular |= kElimNode;
-      w.ns[node] = s;
-      atomicAdd(&w.counters[0], 1);
-      atomicAdd(&w.counters[kElimCount], 1);
-      return;
-    }
-    const bool finite = ss < INFINITY;
-    const bool accept = !a.damping || (finite && ss <= (1.0 - 2e-4 * s.alpha) * s.fnorm2) ||
-                        s.alpha <= 0x1p-10;
-    if (accept) {
-      s.fnorm2 = ss;
-      s.fmax = mx;
-      s.searching = 0;
-      if (a.jac_in_trial) s.ybuf ^= 1;   // the trial point is the iterate
-    } else {
-      // FP64 form: a node far from its root follows the elimination's direction
-      // (its path depends on the last bits of it); alpha = 0 evaluates the
-      // rows at the iterate again, which that direction needs
-      s.alpha = a.tree && !(s.singular & kElimDone) ? 0.0 : 0.5 * s.alpha;
-      atomicAdd(&w.counters[0], 1);
-    }
+    atomicAdd(&w.counters[kActiveCount], 1);
   }
   w.ns[node] = s;
 }
 
-// ---------------------------------------------------------------- Jacobian
-constexpr int kPtWarps = 4;    // warps per block of k_point
-constexpr int kPtLd = 76;      // staged row stride of a point: six rows (72) + 4, 16-byte aligned
+// A warp per node; the block that finishes last publishes the counts, sets the
+// graph's loop conditions and clears the counters: no other launch and no
+// memset per trial or iteration.
+__global__ void __launch_bounds__(128) k_ls_reduce(SolveArgs a, Workspace w, int mode) {
+  const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
+  if (node < a.n) ls_node(a, w, node, threadIdx.x & 31, mode);
+  __threadfence();   // this warp's counts before the block's ticket
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (atomicAdd(&w.counters[kTicket], 1) != static_cast<int>(gridDim.x) - 1) return;
+  __threadfence();
+  const int searching = atomicExch(&w.counters[kSearchCount], 0);
+  w.counters[kTicket] = 0;
+  w.counters[kSearchOut] = searching;
+  if (searching == 0) {   // the iteration's end
+    const int active = atomicExch(&w.counters[kActiveCount], 0);
+    w.counters[kActiveOut] = active;
+    w.counters[kElimCount] = 0;
+    if (mode == 1) w.counters[kEpoch] += 1;
+    if (a.conds & 1) cudaGraphSetConditional(a.h_newton, active > 0 ? 1u : 0u);
+  }
+  if ((a.conds & 2) && mode == 1) cudaGraphSetConditional(a.h_search, searching > 0 ? 1u : 0u);
+}
 
-template <typename T>
-__global__ void __launch_bounds__(32 * kPtWarps) k_point(SolveArgs a, Workspace w) {
+// ---------------------------------------------------------------- Jacobian
+// FP64 form (in the FP32 forms the residual kernel stores the Jacobian).
+__global__ void __launch_bounds__(128) k_point_fp64(SolveArgs a, Workspace w) {
   const int64_t P = npts(a.Nmax);
   const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  bool valid = t < a.n * P;
-  if (valid) {
-    const int64_t node = t / P, p = t % P;
-    valid = w.ns[node].active && p <= 3 * int64_t(a.N[node]);
-  }
+  if (t >= a.n * P) return;
+  const int64_t node = t / P, p = t % P;
+  if (!w.ns[node].active || p > 3 * int64_t(a.N[node])) return;
   double y[12];
 #pragma unroll
-  for (int c = 0; c < 12; ++c) y[c] = valid ? w.Y[t * 12 + c] : 0.0;
-  if constexpr (sizeof(T) == 8) {
-    if (valid) char_jacobian<T>(a.P, y, static_cast<T*>(w.Jm) + t * 144, nullptr);
-  } else {
-    // The 32 points of a warp are consecutive in Jm.  Rows are staged in
-    // shared memory six at a time and the warp writes them as contiguous
-    // 288-byte runs (one per point) instead of 48-byte rows 576 bytes apart.
-    __shared__ __align__(16) float stage[kPtWarps][32 * kPtLd];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-    if (vmask == 0u) return;   // the whole warp
-    float* mine = stage[warp] + lane * kPtLd;
-    float* Jw = static_cast<float*>(w.Jm) + (t - lane) * 144;   // the warp's first point
-    char_jacobian_rows<float>(
-        a.P, y,
-        [&](int r, const float (&row)[12]) {
-          float4* dst = reinterpret_cast<float4*>(mine + 12 * (r % 6));
-#pragma unroll
-          for (int q4 = 0; q4 < 3; ++q4)
-            dst[q4] = make_float4(row[4 * q4], row[4 * q4 + 1], row[4 * q4 + 2], row[4 * q4 + 3]);
-          if (r % 6 == 5) {
-            __syncwarp();
-            const int h = r / 6;
-            for (int e = lane; e < 32 * 18; e += 32) {
-              const int pt = e / 18, q = e % 18;
-              if ((vmask >> pt) & 1u)
-                reinterpret_cast<float4*>(Jw + pt * 144 + 72 * h)[q] =
-                    reinterpret_cast<const float4*>(stage[warp] + pt * kPtLd)[q];
-            }
-            __syncwarp();
-          }
-        },
-        nullptr);
-  }
+  for (int c = 0; c < 12; ++c) y[c] = w.Y[t * 12 + c];
+  char_jacobian<double>(a.P, y, static_cast<double*>(w.Jm) + t * 144, nullptr);
 }
 
 // ---------------------------------------------------------------- helpers
@@ -1560,6 +1574,8 @@ __global__ void __launch_bounds__(128) k_abd_red(SolveArgs a, Workspace w) {
   if (node >= a.n) return;
   if (!w.ns[node].active) return;
   abd_reduced<float>(a, w, node, a.N[node], threadIdx.x & 31);
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) ls_start(w, node);   // (the rest of the direction skips a singular node)
 }
 
 __global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
@@ -1641,23 +1657,8 @@ __global__ void k_recover_fp32(SolveArgs a, Workspace w) {
 }
 
 // ---------------------------------------------------------------- update
-__global__ void k_ls_begin(SolveArgs a, Workspace w) {
-  const int64_t node = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (node >= a.n) return;
-  NodeState s = w.ns[node];
-  if (!s.active) return;
-  if (s.singular & 1) {
-    s.status = SG_SINGULAR;
-    s.active = 0;
-  } else {
-    s.singular &= kElimNode;
-    s.searching = 1;
-    s.alpha = 1.0;
-  }
-  w.ns[node] = s;
-}
-
-// Y += alpha D, a thread per pair of components (consecutive threads touch
+// Y += alpha D at the nodes whose step was accepted in this iteration (FP64
+// form), a thread per pair of components (consecutive threads touch
 // consecutive 16-byte words).
 constexpr int kUpdPer = 6;   // threads per collocation point
 __global__ void k_update(SolveArgs a, Workspace w) {
@@ -1666,7 +1667,7 @@ __global__ void k_update(SolveArgs a, Workspace w) {
   if (u >= a.n * P * kUpdPer) return;
   const int64_t t = u / kUpdPer;
   const int64_t node = t / P;
-  if (!w.ns[node].active) return;
+  if (w.ns[node].searching != -w.counters[kEpoch]) return;
   if (t % P > 3 * int64_t(a.N[node])) return;
   const double alpha = w.ns[node].alpha;
   double2* y2 = reinterpret_cast<double2*>(w.Y) + u;
@@ -1675,37 +1676,22 @@ __global__ void k_update(SolveArgs a, Workspace w) {
   *y2 = make_double2(__fma_rn(alpha, d.x, y.x), __fma_rn(alpha, d.y, y.y));
 }
 
-__global__ void k_after_update(SolveArgs a, Workspace w) {
-  const int64_t node = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (node >= a.n) return;
-  NodeState s = w.ns[node];
-  if (!s.active) return;
-  s.iters += 1;
-  if (!(s.fmax < INFINITY)) {
-    s.status = SG_NONFINITE;
-    s.active = 0;
-  } else if (s.fmax <= a.tol) {
-    s.status = SG_CONVERGED;
-    s.active = 0;
-  } else if (s.iters >= a.max_iter) {
-    s.status = SG_MAXITER;
-    s.active = 0;
-  } else {
-    atomicAdd(&w.counters[1], 1);
-  }
-  w.ns[node] = s;
-}
-
 // Outputs (Eq. optuv): lambda(0), u*(x0, lambda(0)), V = z(T) + h(x(T)) with
-// z(T) = h sum_i sum_j b_j L(Y_ij) (the Lobatto IIIA step of z' = L).  One
-// warp per node; the results go to output row `row`.
+// z(T) = h sum_i sum_j b_j L(Y_ij) (the Lobatto IIIA step of z' = L; a shared mesh
+// point counts once with both intervals' weights).  A block of 128 threads
+// per node, a thread per point and pass; the results go to output row `row`.
+// (A warp per node, four evaluations per interval: 28 us for one node of 128
+// intervals, FP64-issue-bound on one quarter of an SM.)
+constexpr int kOutThreads = 128;
 __device__ __forceinline__ void node_outputs(const SolveArgs& a, const Workspace& w, int64_t node, int64_t row,
-                                             int lane, double* lambda0, double* u0, double* V, int32_t* status,
+                                             double* lambda0, double* u0, double* V, int32_t* status,
                                              int32_t* iters) {
+  __shared__ double z_s[kOutThreads / 32];
+  const int tid = threadIdx.x;
   const NodeState s = w.ns[node];
   const double* Y = (s.ybuf ? w.Y2 : w.Y) + node * npts(a.Nmax) * 12;
   if (s.status == SG_BADINPUT) {
-    if (lane == 0) {
+    if (tid == 0) {
       for (int c = 0; c < 6; ++c) lambda0[row * 6 + c] = NAN;
       for (int c = 0; c < 3; ++c) u0[row * 3 + c] = NAN;
       V[row] = NAN;
@@ -1714,19 +1700,20 @@ __device__ __forceinline__ void node_outputs(const SolveArgs& a, const Workspace
     }
     return;
   }
-  const int N = a.N[node];
-  const double h = a.T[node] / N;
+  const int N = a.N[node], last = 3 * N;
+  const double* ve = node_target(a.P, node);
   double z = 0.0;
-  for (int i = lane; i < N; i += 32) {
-    const double* yi = Y + 3 * int64_t(i) * 12;
-    const double* ve = node_target(a.P, node);
-    z += h * (kLobB[0] * running_cost(a.P, yi, ve) + kLobB[1] * running_cost(a.P, yi + 12, ve) +
-              kLobB[2] * running_cost(a.P, yi + 24, ve) + kLobB[3] * running_cost(a.P, yi + 36, ve));
+  for (int p = tid; p <= last; p += kOutThreads) {
+    const double wt = p % 3 ? 5.0 : (p == 0 || p == last ? 1.0 : 2.0);
+    z = fma(wt, running_cost(a.P, Y + 12 * int64_t(p), ve), z);
   }
   z = warp_sum(z);
-  if (lane == 0) {
-    const double* yN = Y + 3 * int64_t(N) * 12;
-    V[row] = z + terminal_cost(a.P, yN);
+  if ((tid & 31) == 0) z_s[tid >> 5] = z;
+  __syncthreads();
+  if (tid == 0) {
+    z = (z_s[0] + z_s[1]) + (z_s[2] + z_s[3]);
+    const double* yN = Y + 12 * int64_t(last);
+    V[row] = fma(a.T[node] / N / 12.0, z, terminal_cost(a.P, yN));
     double u[3];
     optimal_control(a.P, Y, Y + 6, u);
     for (int c = 0; c < 6; ++c) lambda0[row * 6 + c] = Y[6 + c];
@@ -1736,12 +1723,9 @@ __device__ __forceinline__ void node_outputs(const SolveArgs& a, const Workspace
   }
 }
 
-__global__ void k_outputs(SolveArgs a, Workspace w, double* lambda0, double* u0, double* V,
-                          int32_t* status, int32_t* iters) {
-  const int lane = threadIdx.x & 31;
-  const int64_t node = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-  if (node >= a.n) return;
-  node_outputs(a, w, node, node, lane, lambda0, u0, V, status, iters);
+__global__ void __launch_bounds__(kOutThreads) k_outputs(SolveArgs a, Workspace w, double* lambda0, double* u0,
+                                                         double* V, int32_t* status, int32_t* iters) {
+  node_outputs(a, w, blockIdx.x, blockIdx.x, lambda0, u0, V, status, iters);
 }
 
 __global__ void k_copy_Y(SolveArgs a, Workspace w, double* out) {
