@@ -16,18 +16,21 @@
 //   dY2 = ((hJ3 - B22 I) dY3 - g2) / B21,
 // and the last stage row, in which hJ2 dY2 and hJ3 dY3 are replaced by the
 // same combinations, needs only L G with L = E C^-1, E = c (hJ3 - B22 I) + d I.
-// That is 12,200 multiply-adds per interval (12 x 12 products and one 12 x 12
-// inversion with partial pivoting) instead of the 23,000 of the elimination
-// of the 24 interior columns, and what the recovery needs is C^-1 (144
-// numbers) instead of 24 pivot rows (1,248).  The FP32 forms keep the
+// G is not formed: L G is the product of hJ1 and of hJ4 with a combination of
+// L and L hJ2 each, two 12 x 12 products less.  That is 9,700 multiply-adds
+// per interval (five 12 x 12 products and one 12 x 12 inversion with partial
+// pivoting) instead of the 23,000 of the elimination of the 24 interior
+// columns, and what the recovery needs is C^-1 (144 numbers) instead of 24
+// pivot rows (1,248).  The FP32 forms keep the
 // elimination: a direction rounded otherwise moves their residuals near the
 // tolerance by about a thousandth, and with them the iteration counts of one
 // node in 5,000.
 //
 // Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
-// iterations): condensation 74.8 -> 31.5 ms, elimination and back substitution
-// over the intervals 23.9 -> 9.6 ms, recovery 4.3 -> 2.5 ms; the solve (a graph
-// per mesh size) 112.0 -> 48.7 ms; one node at 128 intervals 1.80 -> 1.01 ms.
+// iterations): condensation 74.8 -> 25.5 ms (FP64 pipe 95 % busy), elimination
+// and back substitution over the intervals 23.9 -> 9.4 ms, recovery 4.3 -> 2.5
+// ms; the solve (a graph per mesh size) 112.0 -> 42.4 ms; one node at 128
+// intervals 1.80 -> 0.95 ms.
 //
 // Elimination over the intervals.  An interval's condensed row
 // S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
@@ -58,6 +61,7 @@ namespace lob {
 constexpr double s5 = SG_S5;
 constexpr double B11 = (25.0 + s5) / 7.0, B21 = -(25.0 + 13.0 * s5) / 7.0, B22 = (25.0 - s5) / 7.0;
 constexpr double P12 = -220.0 / 49.0;                                              // B12 B21
+constexpr double R2 = -120.0 / 7.0;                                                // B12 B21 - B11 B22
 constexpr double S1 = 2.0 * s5;                                                    // s_1; s_2 = -s_1
 constexpr double A1 = (17.0 * s5 - 5.0) / 70.0, A2 = -(17.0 * s5 + 5.0) / 70.0;    // alpha
 constexpr double G1 = (3.0 * s5 - 5.0) / 70.0, G2 = -(3.0 * s5 + 5.0) / 70.0;      // gamma
@@ -127,7 +131,7 @@ __device__ __forceinline__ void st_vec(double* dst, const double (&r)[n], int q0
 constexpr int kCondIv = 8;                       // intervals per block
 constexpr int kCondThreads = 12 * kCondIv;
 constexpr int kCondU = 28;                       // a published pivot row
-// J (4 x 144), C^-1 (144), U (2), rho_2 (12), last column of G (12), pivot keys and pivot rows (24 words)
+// J (4 x 144), C^-1 (144), U (2), the residuals' two vectors (24), pivot keys and pivot rows (24 words)
 constexpr int kCondElems = 576 + 144 + 2 * kCondU + 24 + 12;
 constexpr int kCondSmem = kCondIv * kCondElems * 8;
 __host__ __device__ __forceinline__ int cond_chunks(int Nmax) { return (Nmax + kCondIv - 1) / kCondIv; }
@@ -162,13 +166,11 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
   i = valid ? i + slot : N - 1;
 
   double* sm = reinterpret_cast<double*>(cond_smem) + slot * kCondElems;
-  double* J_s = sm;                 // hJ of the four points; points 2 and 3 are overwritten by G [12][24]
-  double* G_s = sm + 144;
+  double* J_s = sm;                 // J of the four points
   double* Ci_s = sm + 576;
   double* U_s = Ci_s + 144;         // [2][28]
   double* rho_s = U_s + 2 * kCondU;
-  double* gr_s = rho_s + 12;        // last column of G
-  unsigned* keys = reinterpret_cast<unsigned*>(gr_s + 12);
+  unsigned* keys = reinterpret_cast<unsigned*>(rho_s + 24);
   int* perm_s = reinterpret_cast<int*>(keys + 12);
 
   const int64_t wid = node * a.Nmax + i;
@@ -176,23 +178,19 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
   {
     const double* J = static_cast<const double*>(w.Jm) + (node * npts(a.Nmax) + 3 * int64_t(i)) * 144;
 #pragma unroll
-    for (int e = 0; e < 576 / 2 / 12; ++e) {
-      double v[2];
-      ld_vec<2>(J + (r + e * 12) * 2, v);
-#pragma unroll
-      for (int t = 0; t < 2; ++t) v[t] *= h;
-      st_vec<2>(J_s + (r + e * 12) * 2, v);
-    }
+    for (int e = 0; e < 576 / 2 / 12; ++e) cp_async16(J_s + (r + e * 12) * 2, J + (r + e * 12) * 2);
+    cp_async_commit();
   }
-  double rho1, rho2, res3;
+  double res_c;   // the stage residuals' part that needs no product
   {
     const double* res = static_cast<const double*>(w.Res) + wid * kResRows;
-    const double r1 = res[r], r2 = res[12 + r];
-    res3 = res[24 + r];
-    rho1 = lob::B11 * r1 + lob::B12 * r2;
-    rho2 = lob::B21 * r1 + lob::B22 * r2;
-    rho_s[r] = rho2;
+    const double r1 = res[r], r2 = res[12 + r], r3 = res[24 + r];
+    const double rho1 = lob::B11 * r1 + lob::B12 * r2, rho2 = lob::B21 * r1 + lob::B22 * r2;
+    res_c = lob::W1 * rho1 + lob::W2 * rho2 - r3;
+    rho_s[r] = h * rho2;
+    rho_s[12 + r] = lob::R2 * r2;   // B21 rho_1 - B11 rho_2
   }
+  cp_async_wait_all();
   __syncthreads();
 
   bool bad = false;
@@ -205,9 +203,9 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
       ld_vec<12>(J_s + 144 + r * 12, e1);
 #pragma unroll
       for (int j = 0; j < 12; ++j) {
-        if (j == r) e1[j] -= lob::B11;
-        c[j] = -lob::B22 * e1[j];
-        if (j == r) c[j] -= lob::P12;
+        e1[j] = fma(h, e1[j], j == r ? -lob::B11 : 0.0);
+        c[j] = fma(-lob::B22, e1[j], j == r ? -lob::P12 : 0.0);
+        e1[j] *= h;
       }
 #pragma unroll
       for (int m = 0; m < 12; ++m) {
@@ -258,16 +256,16 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
     }
   }
 
-  // ---- L = E C^-1
-  double L[12];
+  // ---- L = E C^-1 and L J2
+  double L[12], M[12];
   {
     double e[12];
     ld_vec<12>(J_s + 288 + r * 12, e);
+    const double ce = lob::CE * h;
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
-      e[j] *= lob::CE;
-      if (j == r) e[j] += (lob::C2 - lob::CE * lob::B22);
-      L[j] = 0.0;
+      e[j] = fma(ce, e[j], j == r ? lob::C2 - lob::CE * lob::B22 : 0.0);
+      L[j] = M[j] = 0.0;
     }
 #pragma unroll
     for (int m = 0; m < 12; ++m) {
@@ -276,84 +274,58 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
 #pragma unroll
       for (int j = 0; j < 12; ++j) L[j] = fma(e[m], u[j], L[j]);
     }
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      double u[12];
+      ld_vec<12>(J_s + 144 + m * 12, u);
+#pragma unroll
+      for (int j = 0; j < 12; ++j) M[j] = fma(L[m], u[j], M[j]);
+    }
   }
 
-  // ---- G = (hJ2 - B11 I) g2 + B21 g1
+  // ---- the condensed row [S | T | r] as [T_x | S_lambda | -S_x | -T_lambda | r]:
+  // with M = L (hJ2 - B11 I),
+  //   S = (K0 I + alpha_2 M + B21 alpha_1 L) hJ1 + KD I - s_1 M + B21 s_1 L,
+  //   T = (K3 I + gamma_2 M + B21 gamma_1 L) hJ4 + I
+  double v[28];
   {
-    double e1[12], g[24], gr = lob::B21 * rho1;
-    ld_vec<12>(J_s + 144 + r * 12, e1);
+    const double cm = -lob::S1 * h, hK0 = lob::K0 * h, hK3 = lob::K3 * h, h2 = h * h;
+    const double am = lob::A2 * h2, al = (lob::B21 * lob::A1 - lob::A2 * lob::B11) * h;
+    const double gm = lob::G2 * h2, gl = (lob::B21 * lob::G1 - lob::G2 * lob::B11) * h;
+    double t[12];
 #pragma unroll
     for (int j = 0; j < 12; ++j)
-      if (j == r) e1[j] -= lob::B11;
-#pragma unroll
-    for (int j = 0; j < 24; ++j) g[j] = 0.0;
+      t[j] = fma(cm, M[j], fma(lob::S1 * (lob::B11 + lob::B21), L[j], j == r ? lob::KD : 0.0));
 #pragma unroll
     for (int m = 0; m < 12; ++m) {
       double u[12];
       ld_vec<12>(J_s + m * 12, u);
+      const double x = fma(am, M[m], fma(al, L[m], m == r ? hK0 : 0.0));
 #pragma unroll
-      for (int j = 0; j < 12; ++j) g[j] = fma(e1[m], u[j], g[j]);
-      ld_vec<12>(J_s + 432 + m * 12, u);
-#pragma unroll
-      for (int j = 0; j < 12; ++j) g[12 + j] = fma(e1[m], u[j], g[12 + j]);
+      for (int j = 0; j < 12; ++j) t[j] = fma(x, u[j], t[j]);
     }
-    {
-      double u[12];
-      ld_vec<12>(rho_s, u);
 #pragma unroll
-      for (int m = 0; m < 12; ++m) gr = fma(e1[m], u[m], gr);
-      ld_vec<12>(J_s + r * 12, u);
-#pragma unroll
-      for (int j = 0; j < 12; ++j) {
-        g[j] = fma(-lob::A2, g[j], lob::S1 * e1[j]);
-        g[j] = fma(-lob::B21 * lob::A1, u[j], g[j]);
-        if (j == r) g[j] -= lob::B21 * lob::S1;
-      }
-      ld_vec<12>(J_s + 432 + r * 12, u);
-#pragma unroll
-      for (int j = 0; j < 12; ++j)
-        g[12 + j] = fma(-lob::G2, g[12 + j], -lob::B21 * lob::G1 * u[j]);
+    for (int j = 0; j < 12; ++j) {
+      if (j < 6) v[12 + j] = -t[j];
+      else v[j] = t[j];
+      t[j] = j == r ? 1.0 : 0.0;
     }
-    __syncthreads();   // points 2 and 3 have been read by every row
-    st_vec<24>(G_s + r * 24, g);
-    gr_s[r] = gr;
-  }
-  __syncthreads();
-
-  // ---- the condensed row [S | T | r] as [T_x | S_lambda | -S_x | -T_lambda | r]
-  double v[28];
-  {
-    double g[24], gr = 0.0;
-#pragma unroll
-    for (int j = 0; j < 24; ++j) g[j] = 0.0;
+    double rr = res_c;
 #pragma unroll
     for (int m = 0; m < 12; ++m) {
-      double u[24];
-      ld_vec<24>(G_s + m * 24, u);
+      double u[12];
+      ld_vec<12>(J_s + 432 + m * 12, u);
+      const double x = fma(gm, M[m], fma(gl, L[m], m == r ? hK3 : 0.0));
 #pragma unroll
-      for (int j = 0; j < 24; ++j) g[j] = fma(L[m], u[j], g[j]);
+      for (int j = 0; j < 12; ++j) t[j] = fma(x, u[j], t[j]);
+      rr = fma(M[m], rho_s[m], fma(L[m], rho_s[12 + m], rr));
     }
-    double u[12];
-    ld_vec<12>(gr_s, u);
-#pragma unroll
-    for (int m = 0; m < 12; ++m) gr = fma(L[m], u[m], gr);
-    ld_vec<12>(J_s + r * 12, u);
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
-      double s = fma(lob::K0, u[j], -g[j]);
-      if (j == r) s += lob::KD;
-      if (j < 6) v[12 + j] = -s;
-      else v[j] = s;
+      if (j < 6) v[j] = t[j];
+      else v[12 + j] = -t[j];
     }
-    ld_vec<12>(J_s + 432 + r * 12, u);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) {
-      double t = fma(lob::K3, u[j], -g[12 + j]);
-      if (j == r) t += 1.0;
-      if (j < 6) v[j] = t;
-      else v[12 + j] = -t;
-    }
-    v[24] = gr + lob::W1 * rho1 + lob::W2 * rho2 - res3;
+    v[24] = rr;
     v[25] = v[26] = v[27] = 0.0;
   }
 
