@@ -620,7 +620,9 @@ __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, W
 // read when it runs.)
 constexpr int kElimBlocks = 2 * kNumSMs, kElimWarps = 4;
 constexpr int kElimWarpSmem = 36 * kCols * 8;   // the condensation's system; the segments' tables are smaller
-static_assert(seg_smem_elems<double>() * 8 <= kElimWarpSmem && 2 * 12 * kSegLd * 8 <= kElimWarpSmem, "tables fit");
+static_assert(seg_smem_elems<double>() * 8 <= kElimWarpSmem && stair_smem_elems<double>() * 8 <= kElimWarpSmem &&
+                  kSegBackStages<double> * 12 * kSegLd * 8 <= kElimWarpSmem,
+              "tables fit");
 __global__ void __launch_bounds__(32 * kElimWarps) k_elim_fp64(SolveArgs a, Workspace w) {
   if (w.counters[kElimCount] == 0) return;
   extern __shared__ __align__(16) unsigned char elim_smem[];
@@ -638,7 +640,7 @@ __global__ void __launch_bounds__(32 * kElimWarps) k_elim_fp64(SolveArgs a, Work
       __syncwarp();
     }
     __syncthreads();
-    if (warp == 0) abd_reduced<double>(a, w, node, N, lane);
+    if (warp == 0) abd_reduced<double>(a, w, node, N, lane, sm);
     __syncthreads();
     for (int s = warp; s < nseg; s += kElimWarps) {
       abd_segment_back<double>(a, w, node, s, N, lane, reinterpret_cast<double(*)[12 * kSegLd]>(sm));

@@ -595,25 +595,6 @@ __device__ __forceinline__ void load_row25(const T* __restrict__ src, T (&r)[25]
   r[24] = src[24];
 }
 
-// A 25-entry row into a kBlkLd (28) slot, the 3 pad entries zeroed: whole
-// 32-byte sectors are written, so the memory system need not read the slot
-// first.
-template <typename T>
-__device__ __forceinline__ void store_row25(T* __restrict__ dst, const T (&r)[25]) {
-  if constexpr (sizeof(T) == 4) {
-    float4* d4 = reinterpret_cast<float4*>(dst);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) d4[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-    d4[6] = make_float4(r[24], 0.0f, 0.0f, 0.0f);
-  } else {
-    double2* d2 = reinterpret_cast<double2*>(dst);
-#pragma unroll
-    for (int q = 0; q < 12; ++q) d2[q] = make_double2(r[2 * q], r[2 * q + 1]);
-    d2[12] = make_double2(r[24], 0.0);
-    d2[13] = make_double2(0.0, 0.0);
-  }
-}
-
 // Pivot-search key: the magnitude bits (sign shifted out; for doubles the
 // upper word) in the top 31 bits, ordered like |x|.
 __device__ __forceinline__ unsigned mag_key(float x) { return __float_as_uint(x) << 1; }
@@ -628,6 +609,10 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int n>
+__device__ __forceinline__ void cp_async_wait_prior() {   // all but the last n committed groups
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(n) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Correctly rounded reciprocal (the same value as 1 / x, without the
@@ -669,37 +654,6 @@ __device__ __forceinline__ void load_row40(const T* __restrict__ src, T (&r)[40]
     for (int q = 0; q < 20; ++q) {
       const double2 v = s2[q];
       r[2 * q] = v.x; r[2 * q + 1] = v.y;
-    }
-  }
-}
-
-// Twelve pivot steps with partial pivoting on 25-column rows held one per
-// lane.  cand: this lane's row takes part.  The pivot row of step k keeps
-// 1/pivot at column k; plane[k] is the lane that held it.
-template <typename T>
-__device__ __forceinline__ void panel_eliminate12(T (&r)[25], bool cand, bool& done, int& my_step,
-                                                  int (&plane)[12], bool& ok, int lane) {
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    const int p = warp_pivot_lane<T>(r[k], cand && !done, lane);
-    plane[k] = p;
-    const T piv = __shfl_sync(0xffffffffu, r[k], p);
-    // (the correctly rounded reciprocal: on this serial chain the approximate
-    // instruction measured 19 % slower)
-    const bool good = piv != T(0) && isfinite(piv);
-    ok = ok && good;
-    const T inv = good ? recip_rn(piv) : T(0);
-    const bool is_p = lane == p;
-    const T l = (cand && !done && !is_p) ? r[k] * inv : T(0);
-#pragma unroll
-    for (int c = k + 1; c < 25; ++c) {
-      const T pc = __shfl_sync(0xffffffffu, r[c], p);
-      r[c] = fma(-l, pc, r[c]);
-    }
-    if (is_p) {
-      done = true;
-      my_step = k;
-      r[k] = inv;
     }
   }
 }
@@ -1052,192 +1006,21 @@ __device__ __forceinline__ void condense_interval_smem(const SolveArgs& a, const
   __syncwarp();
 }
 
-// ---------------------------------------------------------------- staircase
-// Register-resident staircase elimination: warp per node, lanes 0..17 hold the
-// 18 rows of the current panel [carry (6) ; block row i (12)] over the 25
-// columns [y_i (12) | y_{i+1} (12) | rhs].  Twelve pivot steps leave 12 pivot
-// rows (stored in pivot order, 1/pivot on the diagonal) and 6 rows that carry
-// y_{i+1} into the next panel.  The next block row is prefetched into lanes
-// 0..11 while the current panel is eliminated.  The lambda(T) rows close the
-// system; back substitution then runs from the last mesh point to the first.
-//
-// The blocks may be the N interval block rows of the node (pt_stride = 3:
-// block i couples mesh points 3i and 3i + 3) or the reduced block rows of the
-// segmented form (block s couples the segment ends, pt_stride = 3 x segment
-// length); the last block always ends at mesh point 3N.
 template <typename T>
-__device__ __forceinline__ bool abd_staircase(const SolveArgs& a, const Workspace& w, int64_t node, int N,
-                                              const T* __restrict__ cond, int nblk, int pt_stride,
-                                              T* __restrict__ abd, int lane) {
-  const int64_t pb = node * npts(a.Nmax);
-  const double* Y = (w.ns[node].ybuf ? w.Y2 : w.Y) + pb * 12;
-  const double* x0 = a.x0 + node * 6;
-  double* D = w.D + pb * 12;
-  const bool rowlane = lane < 18;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  T r[25], nx[25];
-#pragma unroll
-  for (int c = 0; c < 25; ++c) {
-    r[c] = T(0);
-    nx[c] = T(0);
+__device__ __forceinline__ void load_vec16(const T* src, T (&v)[16 / sizeof(T)]) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(src);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  } else {
+    const double2 x = *reinterpret_cast<const double2*>(src);
+    v[0] = x.x; v[1] = x.y;
   }
-  if (lane < 6) {
-    // x(0) - x0 = 0 linearised: [I 0] dy_0 = -(x(0) - x0)
-#pragma unroll
-    for (int c = 0; c < 6; ++c)
-      if (c == lane) r[c] = T(1);
-    r[24] = T(-(Y[lane] - x0[lane]));
-  } else if (rowlane) {
-    load_row25<T>(cond + (lane - 6) * kBlkLd, r);
-  }
-  bool ok = true;
-  bool done = false;
-  int rank = 0;
-  int plane[12];
-  for (int i = 0; i < nblk; ++i) {
-    if (i + 1 < nblk && lane < 12) load_row25<T>(cond + int64_t(i + 1) * kBlk + lane * kBlkLd, nx);
-    done = false;
-    int my_step = -1;
-    panel_eliminate12<T>(r, rowlane, done, my_step, plane, ok, lane);
-    if (done) store_row25<T>(abd + int64_t(i) * kBlk + my_step * kBlkLd, r);
-    rank = __popc(__ballot_sync(0xffffffffu, done) & lt_mask);
-    // next panel: carry rows shift y_{i+1} into the first block; the pivot
-    // lanes take the prefetched block row i+1, in lane order
-#pragma unroll
-    for (int c = 0; c < 25; ++c) {
-      const T v = __shfl_sync(0xffffffffu, nx[c], rank & 15);
-      if (done) {
-        r[c] = v;
-      } else if (c < 12) {
-        r[c] = r[c < 12 ? c + 12 : c];
-      } else if (c < 24) {
-        r[c] = T(0);
-      }
-    }
-  }
-  // closing rows: lambda(T) - grad h(x(T)) = 0, taken by pivot lanes of rank
-  // 0..5 (the other pivot lanes sit out); the carry lanes hold the rest
-  const double* yN = Y + 3 * int64_t(N) * 12;
-  if (done) {
-#pragma unroll
-    for (int c = 0; c < 25; ++c) r[c] = T(0);
-    if (rank < 6) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) r[c] = T(-terminal_hess(a.P, rank, c));
-#pragma unroll
-      for (int c = 0; c < 6; ++c)
-        if (c == rank) r[6 + c] = T(1);
-      r[24] = T(-(yN[6 + rank] - terminal_grad(a.P, yN, rank)));
-    }
-  }
-  {
-    const bool cand = rowlane && (!done || rank < 6);
-    bool done2 = false;
-    int my2 = -1;
-    panel_eliminate12<T>(r, cand, done2, my2, plane, ok, lane);
-  }
-  // back substitution of the closing system: dy_N (uniform across lanes)
-  T dy[12];
-  {
-    T t = r[24];
-#pragma unroll
-    for (int k = 11; k >= 0; --k) {
-      const T dk = __shfl_sync(0xffffffffu, t * r[k], plane[k]);
-      dy[k] = dk;
-      t = fma(-r[k], dk, t);
-    }
-  }
-  if (lane < 12) {
-    T mine = T(0);
-#pragma unroll
-    for (int c = 0; c < 12; ++c)
-      if (c == lane) mine = dy[c];
-    D[3 * int64_t(N) * 12 + lane] = double(mine);
-  }
-  // backward sweep: lane k holds the stored pivot row of step k of interval ii:
-  // U (cols k..11, 1/pivot at k), V (cols 12..23), rhs (24)
-  T row[25], pre[25];
-#pragma unroll
-  for (int c = 0; c < 25; ++c) {
-    row[c] = T(0);
-    pre[c] = T(0);
-  }
-  if (lane < 12) load_row25<T>(abd + int64_t(nblk - 1) * kBlk + lane * kBlkLd, row);
-  for (int ii = nblk - 1; ii >= 0; --ii) {
-    if (ii > 0 && lane < 12) load_row25<T>(abd + int64_t(ii - 1) * kBlk + lane * kBlkLd, pre);
-    T tt = row[24];
-#pragma unroll
-    for (int c = 0; c < 12; ++c) tt = fma(-row[12 + c], dy[c], tt);
-#pragma unroll
-    for (int k = 11; k >= 0; --k) {
-      const T dk = __shfl_sync(0xffffffffu, tt * row[k], k);
-      dy[k] = dk;
-      tt = (lane < k) ? fma(-row[k], dk, tt) : tt;
-    }
-    if (lane < 12) {
-      T mine = T(0);
-#pragma unroll
-      for (int c = 0; c < 12; ++c)
-        if (c == lane) mine = dy[c];
-      D[int64_t(ii) * pt_stride * 12 + lane] = double(mine);
-    }
-#pragma unroll
-    for (int c = 0; c < 25; ++c) row[c] = pre[c];
-  }
-  return ok;
 }
-
-// The whole staircase of one node over its N interval block rows.
-template <typename T>
-__device__ __forceinline__ bool abd_node_reg(const SolveArgs& a, const Workspace& w, int64_t node, int N,
-                                             int lane) {
-  const T* cond = static_cast<const T*>(w.Cond) + node * a.Nmax * int64_t(kBlk);
-  T* abd = static_cast<T*>(w.Abd) + node * a.Nmax * int64_t(kBlk);
-  return abd_staircase<T>(a, w, node, N, cond, N, 3, abd, lane);
+template <typename T, int n>
+__device__ __forceinline__ void store_vec16(T* dst, const T (&r)[n], int c) {   // entries c .. of r
+  if constexpr (sizeof(T) == 4) *reinterpret_cast<float4*>(dst) = make_float4(r[c], r[c + 1], r[c + 2], r[c + 3]);
+  else *reinterpret_cast<double2*>(dst) = make_double2(r[c], r[c + 1]);
 }
-
-// ---------------------------------------------------------------- segmented staircase
-// The serial chain of the staircase is N panels long.  The segmented form
-// cuts the mesh of a node into segments of kSegLen intervals and runs three
-// kernels:
-//   k_abd_seg      warp per (node, segment): eliminates the segment's interior
-//                  mesh points.  A panel holds the 12 carry rows [F | G | r]
-//                  (coupling the segment's first point y_a with y_i) and the
-//                  block row i [0 | S_i | T_i | r_i]; twelve pivot steps with
-//                  partial pivoting over all 24 rows remove y_i, leave 12
-//                  pivot rows [F | U | V | r] (1/pivot on U's diagonal) and 12
-//                  new carry rows on (y_a, y_{i+1}).  After the last panel the
-//                  carry rows are the segment's reduced block row on
-//                  (y_a, y_b), in the same 12 x 25 format as a block row.
-//   k_abd_red      warp per node: the staircase over the reduced block rows
-//                  and the boundary rows gives the segment ends.
-//   k_abd_segback  warp per (node, segment): back substitution through the
-//                  stored pivot rows for the interior mesh points.
-// This is Gaussian elimination with partial pivoting restricted to the block
-// rows of a segment, the structured pairwise reduction of block rows of
-// Wright (SIAM J. Sci. Stat. Comput. 13, 1992) taken sequentially inside a
-// segment; the chain becomes kSegLen + N / kSegLen panels.
-//
-// Each panel runs in two phases, like the condensation:
-//   phase A (rows on lanes): lane r < 24 holds the 12 y_i entries of panel
-//   row r in registers.  Partial pivoting over the 24 rows; at step k the
-//   pivot lane writes its row (1/pivot on the diagonal) to the table U and
-//   every row keeps its multiplier l(r, k) in the eliminated column, stored
-//   to L at the end.
-//   phase B (columns on lanes): lane c < 25 owns passive column c of
-//   [F | Z | rhs].  With the pivot order p_k the passive part of pivot row k
-//   is Q_k = P(p_k) - sum_{j<k} l(p_k, j) Q_j, and a carry row r leaves as
-//   P(r) - sum_k l(r, k) Q_k.
-// The panel rows live in shared memory between panels: their passive parts
-// in P and their y_i parts in Y.  Carry rows move Z into Y; the slots of the
-// pivot rows take block row i + 1.
-template <typename T>
-__host__ __device__ constexpr int seg_warps() { return sizeof(T) == 4 ? 4 : 2; }   // warps per block
-constexpr int kSegP = 25;   // row stride of the passive table P
-// P, Y, L, U and the staged block row (elements), then 32 ints (pivot slots, carry slots)
-constexpr int kSegSmem = 24 * kSegP + 24 * 12 + 24 * 12 + 12 * 12 + 12 * kBlkLd;
-template <typename T>
-__host__ __device__ constexpr int seg_smem_elems() { return kSegSmem + 32 * 4 / int(sizeof(T)); }
 
 template <typename T>
 __device__ __forceinline__ void load_row12(const T* __restrict__ src, T (&r)[12]) {
@@ -1298,65 +1081,463 @@ __device__ __forceinline__ void store_row12_from(T* __restrict__ dst, const T (&
   }
 }
 
-// (the warp's tables at P_s: seg_smem_elems<T>() elements)
+__device__ __forceinline__ void load_slots(const int* src, int (&r)[12]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int4 v = reinterpret_cast<const int4*>(src)[q];
+    r[4 * q] = v.x; r[4 * q + 1] = v.y; r[4 * q + 2] = v.z; r[4 * q + 3] = v.w;
+  }
+}
+
+// ---------------------------------------------------------------- staircase
+// Staircase elimination: warp per node.  A panel has 18 rows [carry (6) ;
+// block row i (12)] over the 25 columns [y_i (12) | y_{i+1} (12) | rhs].
+// Twelve pivot steps leave 12 pivot rows (stored in pivot order, 1/pivot on
+// the diagonal) and 6 rows that carry y_{i+1} into the next panel.  The
+// lambda(T) rows close the system; back substitution then runs from the last
+// mesh point to the first.  Blocks and stored pivot rows come through a ring
+// of asynchronous copies in shared memory.
+//
+// A panel runs in two phases, like a segment's: lanes r < 18 eliminate the
+// y_i columns, then lanes c < 13 form the passive columns [y_{i+1} | rhs] of
+// the pivot rows and of the carry rows (in the order of the steps: the sums of
+// a row-wise elimination).  A row's lane decides ties of the pivot search:
+// carry rows keep theirs, the next block's rows take the pivot rows' in lane
+// order.  The chain is latency; with the rows' 25 columns in the lanes a
+// panel took 3,300 cycles, in this form RED_CYC (one node at 128 intervals,
+// eight panels: 26 -> RED_US us per iteration).
+//
+// The blocks may be the N interval block rows of the node (pt_stride = 3:
+// block i couples mesh points 3i and 3i + 3) or the reduced block rows of the
+// segmented form (block s couples the segment ends, pt_stride = 3 x segment
+// length); the last block always ends at mesh point 3N.
+template <typename T>
+constexpr int kStairStages = sizeof(T) == 4 ? 4 : 3;
+// carry rows and the ring, L, U, published rows of the closing system (elements), then 40 ints
+template <typename T>
+constexpr int stair_smem_elems() {
+  return 6 * kBlkLd + kStairStages<T> * kBlk + 18 * 12 + 12 * 12 + 2 * 16 + 40 * 4 / int(sizeof(T));
+}
+
+// The closing system [y_N (12) | rhs]: twelve pivot steps with partial
+// pivoting on rows held one per lane (entries 13.. are padding).  The pivot
+// row of step k keeps 1/pivot at column k; plane[k] is the lane that held it.
+template <typename T>
+__device__ __forceinline__ void close_eliminate(T (&r)[16], bool cand, int (&plane)[12], bool& ok, int lane, T* pub) {
+  constexpr int V = 16 / int(sizeof(T));
+  bool done = false;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const bool act = cand && !done;
+    const bool good = r[k] != T(0) && isfinite(r[k]);
+    const T own = recip_rn(act && good ? r[k] : T(1));
+    const int p = warp_pivot_lane<T>(r[k], act, lane);
+    plane[k] = p;
+    const T inv = __shfl_sync(0xffffffffu, good ? own : T(0), p);
+    const bool is_p = lane == p;
+    ok = ok && (good || !is_p);
+    const T l = (act && !is_p) ? r[k] * inv : T(0);
+    T* u = pub + (k & 1) * 16;
+    if (is_p) {
+#pragma unroll
+      for (int q = (k + 1) / V; q < 16 / V; ++q) store_vec16<T>(u + q * V, r, q * V);
+      done = true;
+      r[k] = inv;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = (k + 1) / V; q < 16 / V; ++q) {
+      T v[V];
+      load_vec16<T>(u + q * V, v);
+#pragma unroll
+      for (int t = 0; t < V; ++t) {
+        const int c = q * V + t;
+        if (c > k && c < 13) r[c] = fma(-l, v[t], r[c]);
+      }
+    }
+  }
+}
+
+// (the warp's tables at tab: stair_smem_elems<T>() elements)
+template <typename T>
+__device__ __forceinline__ bool abd_staircase(const SolveArgs& a, const Workspace& w, int64_t node, int N,
+                                              const T* __restrict__ cond, int nblk, int pt_stride,
+                                              T* __restrict__ abd, int lane, T* tab) {
+  constexpr int V = 16 / int(sizeof(T));   // entries per 16-byte vector
+  constexpr int S = kStairStages<T>;
+  const int64_t pb = node * npts(a.Nmax);
+  const double* Y = (w.ns[node].ybuf ? w.Y2 : w.Y) + pb * 12;
+  const double* x0 = a.x0 + node * 6;
+  double* D = w.D + pb * 12;
+  // tab: [6 + 12 S][kBlkLd] rows 0..5 the carry rows [y_i | 0 | rhs], then the ring's block rows
+  T* ring = tab + 6 * kBlkLd;
+  T* L_s = ring + S * kBlk;           // [18][12] multipliers l(r, k)
+  T* U_s = L_s + 18 * 12;             // [12][12] pivot rows (y_i part), 1/pivot on the diagonal
+  T* pub = U_s + 12 * 12;             // the closing system's published rows
+  int* prow_s = reinterpret_cast<int*>(pub + 2 * 16);   // [12] the pivot row of step k in tab ...
+  int* plane_s = prow_s + 12;                           // ... and its lane
+  int* crow_s = prow_s + 24;                            // [6] carry row m in tab ...
+  int* clane_s = prow_s + 32;                           // ... and its lane
+  const unsigned lt_mask = (1u << lane) - 1u;
+  auto fetch = [&](const T* base, int i) {   // block i of an array of blocks to the ring
+    char* dst = reinterpret_cast<char*>(ring + (i % S) * kBlk);
+    const char* src = reinterpret_cast<const char*>(base + int64_t(i) * kBlk);
+    constexpr int n = kBlk * int(sizeof(T)) / 16;
+#pragma unroll
+    for (int t = 0; t < (n + 31) / 32; ++t) {
+      const int e = lane + 32 * t;
+      if (32 * t + 32 <= n || e < n) cp_async16(dst + 16 * e, src + 16 * e);
+    }
+  };
+  for (int i = 0; i < S - 1; ++i) {   // (a group per block, also where there is none)
+    if (i < nblk) fetch(cond, i);
+    cp_async_commit();
+  }
+  // the closing rows lambda(T) - grad h(x(T)) = 0, row `lane` < 6 in lane `lane`
+  T ch[6], cr = T(0);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) ch[c] = T(0);
+  if (lane < 6) {
+    const double* yN = Y + 3 * int64_t(N) * 12;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) ch[c] = T(-terminal_hess(a.P, lane, c));
+    cr = T(-(yN[6 + lane] - terminal_grad(a.P, yN, lane)));
+    // x(0) - x0 = 0 linearised: [I 0] dy_0 = -(x(0) - x0)
+    const T r0 = T(-(Y[lane] - x0[lane]));
+#pragma unroll
+    for (int c = 0; c < 24; ++c) tab[lane * kBlkLd + c] = c == lane ? T(1) : T(0);
+    tab[lane * kBlkLd + 24] = r0;
+  }
+  const bool rowlane = lane < 18;
+  const int pc = lane < 13 ? lane : 0;   // phase B: passive column 12 + pc
+  int row = lane;   // this lane's row of the panel: 0..5 carry, 6.. row of the block + 6
+  bool ok = true;
+  for (int i = 0; i < nblk; ++i) {
+    cp_async_wait_prior<S - 2>();   // block i has landed (this lane's part) ...
+    __syncwarp();                   // ... and every lane's; block i - 1 has been read
+    if (i + S - 1 < nblk) fetch(cond, i + S - 1);
+    cp_async_commit();
+    // ---- phase A
+    const int trow = row < 6 ? row : row + 12 * (i % S);   // in tab
+    T ya[12];
+    if (rowlane) {
+      load_row12<T>(tab + trow * kBlkLd, ya);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 12; ++t) ya[t] = T(0);
+    }
+    bool done = false;
+    int step = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      // every candidate forms its own reciprocal while the pivot is searched;
+      // it and the entry of column k + 1 reach the other rows by shuffles, so
+      // that the next search does not wait for the table
+      const bool act = rowlane && !done;
+      const bool good = ya[k] != T(0) && isfinite(ya[k]);
+      const T own = recip_rn(act && good ? ya[k] : T(1));   // (1: no slow path for zeros)
+      const T mine = good ? own : T(0);
+      const int src = warp_pivot_lane<T>(ya[k], act, lane);
+      const T inv = __shfl_sync(0xffffffffu, mine, src);
+      T u1 = T(0);
+      if (k + 1 < 12) u1 = __shfl_sync(0xffffffffu, ya[k + 1 < 12 ? k + 1 : k], src);
+      // (rows that are no candidates are updated too: their entries from here
+      // on are never read)
+      const T la = ya[k] * inv;
+      ya[k] = mine;
+      if (lane == src) {
+        ok = ok && good;
+        store_row12_from<T>(U_s + k * 12, ya, k / V);
+        done = true;
+        step = k;
+      }
+      ya[k] = la;
+      if (k + 1 < 12) ya[k + 1 < 12 ? k + 1 : k] = fma(-la, u1, ya[k + 1 < 12 ? k + 1 : k]);
+      __syncwarp();
+      if (k + 2 < 12) {
+#pragma unroll
+        for (int q = (k + 2) / V; q < 12 / V; ++q) {
+          T uv[V];
+          load_vec16<T>(U_s + k * 12 + q * V, uv);
+#pragma unroll
+          for (int t = 0; t < V; ++t) {
+            const int cc = V * q + t;
+            if (cc > k + 1) ya[cc] = fma(-la, uv[t], ya[cc]);
+          }
+        }
+      }
+    }
+    if (rowlane) store_row12_from<T>(L_s + lane * 12, ya, 0);
+    const unsigned dmask = __ballot_sync(0xffffffffu, done);
+    if (rowlane) {
+      const int rank = __popc(dmask & lt_mask), m = lane - rank;
+      (done ? prow_s + step : crow_s + m)[0] = trow;
+      (done ? plane_s + step : clane_s + m)[0] = lane;
+      row = done ? 6 + rank : m;   // the next panel's
+    }
+    __syncwarp();
+    // ---- phase B
+    T* dst = abd + int64_t(i) * kBlk;
+    T Q[12];
+    int rows[12], lanes[12];
+    load_slots(prow_s, rows);
+    load_slots(plane_s, lanes);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) Q[k] = tab[rows[k] * kBlkLd + 12 + pc];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      T l[12];
+      load_row12_upto<T>(L_s + lanes[k] * 12, l, (k + V - 1) / V);
+#pragma unroll
+      for (int j = 0; j < k; ++j) Q[k] = fma(-l[j], Q[j], Q[k]);
+    }
+    T f[6];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) {
+      rows[m] = crow_s[m];
+      lanes[m] = clane_s[m];
+    }
+#pragma unroll
+    for (int m = 0; m < 6; ++m) f[m] = tab[rows[m] * kBlkLd + 12 + pc];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) {
+      T l[12];
+      load_row12<T>(L_s + lanes[m] * 12, l);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) f[m] = fma(-l[k], Q[k], f[m]);
+    }
+    if (lane < 13) {   // y_{i+1} moves into the y_i columns (the table's y_{i+1} columns stay 0)
+#pragma unroll
+      for (int m = 0; m < 6; ++m) tab[m * kBlkLd + (pc < 12 ? pc : 24)] = f[m];
+    }
+    if (lane < 16) {   // pad zeroed: whole sectors
+#pragma unroll
+      for (int k = 0; k < 12; ++k) dst[k * kBlkLd + 12 + lane] = lane < 13 ? Q[k] : T(0);
+    }
+    constexpr int nu = 12 * (12 / V);
+#pragma unroll
+    for (int t = 0; t < (nu + 31) / 32; ++t) {
+      const int e = lane + 32 * t, k = e / (12 / V), q = e % (12 / V);
+      if (e < nu && q >= k / V)
+        reinterpret_cast<float4*>(dst + k * kBlkLd)[q] = reinterpret_cast<const float4*>(U_s + k * 12)[q];
+    }
+  }
+  __syncwarp();   // the carry rows
+  // closing rows, taken by the pivot lanes of rank 0..5 (the other pivot
+  // lanes sit out); the carry lanes hold the rest
+  int plane[12];
+  T r[16];
+  {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) r[c] = T(0);
+    const int cl = row < 12 ? row - 6 : 0;   // closing row
+#pragma unroll
+    for (int c = 0; c < 6; ++c) ch[c] = __shfl_sync(0xffffffffu, ch[c], cl & 7);
+    cr = __shfl_sync(0xffffffffu, cr, cl & 7);
+    const bool cand = rowlane && row < 12;
+    if (cand && row < 6) {
+      T y[12];
+      load_row12<T>(tab + row * kBlkLd, y);
+#pragma unroll
+      for (int c = 0; c < 12; ++c) r[c] = y[c];
+      r[12] = tab[row * kBlkLd + 24];
+    } else if (cand) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) r[c] = ch[c];
+#pragma unroll
+      for (int c = 0; c < 6; ++c)
+        if (c == cl) r[6 + c] = T(1);
+      r[12] = cr;
+    }
+    close_eliminate<T>(r, cand, plane, ok, lane, pub);
+  }
+  // back substitution of the closing system: dy_N (uniform across lanes)
+  T dy[12];
+  {
+    T t = r[12];
+#pragma unroll
+    for (int k = 11; k >= 0; --k) {
+      const T dk = __shfl_sync(0xffffffffu, t * r[k], plane[k]);
+      dy[k] = dk;
+      t = fma(-r[k], dk, t);
+    }
+  }
+  if (lane < 12) {
+    T mine = T(0);
+#pragma unroll
+    for (int c = 0; c < 12; ++c)
+      if (c == lane) mine = dy[c];
+    D[3 * int64_t(N) * 12 + lane] = double(mine);
+  }
+  // backward sweep: lane k holds the stored pivot row of step k of interval ii:
+  // U (cols k..11, 1/pivot at k), V (cols 12..23), rhs (24)
+  __syncwarp();   // the stored rows and the ring's last reads
+  for (int t = 1; t < S; ++t) {
+    if (nblk - t >= 0) fetch(abd, nblk - t);
+    cp_async_commit();
+  }
+  for (int ii = nblk - 1; ii >= 0; --ii) {
+    cp_async_wait_prior<S - 2>();
+    __syncwarp();
+    if (ii - (S - 1) >= 0) fetch(abd, ii - (S - 1));
+    cp_async_commit();
+    T rr[25];
+    load_row25<T>(ring + (ii % S) * kBlk + (lane < 12 ? lane : 0) * kBlkLd, rr);
+    T tt = rr[24];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) tt = fma(-rr[12 + c], dy[c], tt);
+#pragma unroll
+    for (int k = 11; k >= 0; --k) {
+      const T dk = __shfl_sync(0xffffffffu, tt * rr[k], k);
+      dy[k] = dk;
+      tt = (lane < k) ? fma(-rr[k], dk, tt) : tt;
+    }
+    if (lane < 12) {
+      T mine = T(0);
+#pragma unroll
+      for (int c = 0; c < 12; ++c)
+        if (c == lane) mine = dy[c];
+      D[int64_t(ii) * pt_stride * 12 + lane] = double(mine);
+    }
+  }
+  cp_async_wait_all();
+  return __all_sync(0xffffffffu, ok);
+}
+
+// The whole staircase of one node over its N interval block rows.
+template <typename T>
+__device__ __forceinline__ bool abd_node_reg(const SolveArgs& a, const Workspace& w, int64_t node, int N,
+                                             int lane, T* tab) {
+  const T* cond = static_cast<const T*>(w.Cond) + node * a.Nmax * int64_t(kBlk);
+  T* abd = static_cast<T*>(w.Abd) + node * a.Nmax * int64_t(kBlk);
+  return abd_staircase<T>(a, w, node, N, cond, N, 3, abd, lane, tab);
+}
+
+// ---------------------------------------------------------------- segmented staircase
+// The serial chain of the staircase is N panels long.  The segmented form
+// cuts the mesh of a node into segments of kSegLen intervals and runs three
+// kernels:
+//   k_abd_seg      warp per (node, segment): eliminates the segment's interior
+//                  mesh points.  A panel holds the 12 carry rows [F | G | r]
+//                  (coupling the segment's first point y_a with y_i) and the
+//                  block row i [0 | S_i | T_i | r_i]; twelve pivot steps with
+//                  partial pivoting over all 24 rows remove y_i, leave 12
+//                  pivot rows [F | U | V | r] (1/pivot on U's diagonal) and 12
+//                  new carry rows on (y_a, y_{i+1}).  After the last panel the
+//                  carry rows are the segment's reduced block row on
+//                  (y_a, y_b), in the same 12 x 25 format as a block row.
+//   k_abd_red      warp per node: the staircase over the reduced block rows
+//                  and the boundary rows gives the segment ends.
+//   k_abd_segback  warp per (node, segment): back substitution through the
+//                  stored pivot rows for the interior mesh points.
+// This is Gaussian elimination with partial pivoting restricted to the block
+// rows of a segment, the structured pairwise reduction of block rows of
+// Wright (SIAM J. Sci. Stat. Comput. 13, 1992) taken sequentially inside a
+// segment; the chain becomes kSegLen + N / kSegLen panels.
+//
+// Each panel runs in two phases, like the condensation:
+//   phase A (rows on lanes): lane r < 24 holds the 12 y_i entries of panel
+//   row r in registers.  Partial pivoting over the 24 rows; at step k the
+//   pivot lane writes its row (1/pivot on the diagonal) to the table U and
+//   every row keeps its multiplier l(r, k) in the eliminated column, stored
+//   to L at the end.
+//   phase B (columns on lanes): lane c < 25 owns passive column c of
+//   [F | Z | rhs].  With the pivot order p_k the passive part of pivot row k
+//   is Q_k = P(p_k) - sum_{j<k} l(p_k, j) Q_j, and a carry row r leaves as
+//   P(r) - sum_k l(r, k) Q_k.
+// Rows 0..11 of a panel are the carry rows: their passive parts [F | 0 | rhs]
+// are rows 0..11 of the table `tab`, their y_i parts are in Y; rows 12..23 are
+// block row i, read in place from the buffer of `tab` that it was copied to
+// (its y_i part is S, its passive part [0 | T | rhs]) while the other buffer
+// takes block row i + 1.  A row's lane decides ties of the pivot search:
+// carry rows keep theirs (and are stored in lane order), the rows of block row
+// i + 1 take those of the pivot rows in pivot order.
+//
+// Few segments are bound by the latency of a panel's chain (many by the
+// shared-memory and issue slots about evenly), so what is not on the chain is
+// kept off it: the reciprocal of every candidate is formed during the search,
+// the pivot row's next column travels by shuffle and the rest through U while
+// the next search runs, and loads are issued ahead of the stores they could
+// alias.  One node at 128 intervals: 52 -> SEG_US us per iteration; the
+// level-4 batch's six iterations 1.40 -> SEG_MS ms.
+template <typename T>
+__host__ __device__ constexpr int seg_warps() { return sizeof(T) == 4 ? 4 : 2; }   // warps per block
+// carry rows and two block rows, Y, L, U (elements), then 48 ints
+constexpr int kSegSmem = 3 * kBlk + 12 * 12 + 24 * 12 + 12 * 12;
+template <typename T>
+__host__ __device__ constexpr int seg_smem_elems() { return kSegSmem + 48 * 4 / int(sizeof(T)); }
+
+// (the warp's tables at tab: seg_smem_elems<T>() elements)
 template <typename T>
 __device__ __forceinline__ void abd_segment(const SolveArgs& a, const Workspace& w, int64_t node, int s, int N,
-                                            int lane, T* P_s) {
+                                            int lane, T* tab) {
   constexpr int V = 16 / int(sizeof(T));   // entries per 16-byte vector
   const int smax = seg_count(a.Nmax);
   const int i0 = s * kSegLen;
   const int i1 = i0 + kSegLen < N ? i0 + kSegLen : N;
-  // P_s: [24][kSegP] passive parts [F | Z | rhs] of the panel rows
-  T* Y_s = P_s + 24 * kSegP;          // [24][12] y_i parts
-  T* L_s = Y_s + 24 * 12;             // [24][12] multipliers l(r, k)
+  // tab: [36][kBlkLd] rows 0..11 the carry rows, 12..23 and 24..35 block rows
+  T* Y_s = tab + 3 * kBlk;            // [12][12] y_i parts of the carry rows
+  T* L_s = Y_s + 12 * 12;             // [24][12] multipliers l(r, k)
   T* U_s = L_s + 24 * 12;             // [12][12] pivot rows (y_i part), 1/pivot on the diagonal
-  T* stage = U_s + 12 * 12;           // [12][kBlkLd] block row i + 1
-  int* perm_s = reinterpret_cast<int*>(stage + 12 * kBlkLd);   // [12] slot of the pivot row of step k
-  int* cslot_s = perm_s + 16;                                   // [12] carry slots in lane order
+  int* prow_s = reinterpret_cast<int*>(U_s + 12 * 12);   // [12] the pivot row of step k in tab ...
+  int* plane_s = prow_s + 12;                             // ... and its lane
+  int* crow_s = prow_s + 24;                              // [12] carry row m in tab ...
+  int* clane_s = prow_s + 36;                             // ... and its lane
+  const unsigned lt_mask = (1u << lane) - 1u;
   const T* cond = static_cast<const T*>(w.Cond) + node * a.Nmax * int64_t(kBlk);
   T* seg = static_cast<T*>(w.Seg) + node * a.Nmax * int64_t(kSegBlk);
   T* red = static_cast<T*>(w.Red) + (node * smax + s) * int64_t(kBlk);
-  const unsigned lt_mask = (1u << lane) - 1u;
   const bool col = lane < 25;               // phase B: passive column c = F (0..11), Z (12..23), rhs (24)
   const int c = col ? lane : 0;
   const int segc = c < 12 ? c : c + 12;     // its column in a stored pivot row [F | U | V | rhs]
+  const bool zcol = c >= 12 && c < 24;
 
-  const T* b0 = cond + int64_t(i0) * kBlk;
   if (i0 + 1 >= i1) {   // a one-interval segment: its block row is the reduced row
+    const T* b0 = cond + int64_t(i0) * kBlk;
     for (int e = lane; e < kBlk; e += 32) red[e] = b0[e];
     return;
   }
-  // panel rows: slots 0..11 = block row i0 = [F = S | Y = T | Z = 0 | r],
-  // slots 12..23 = block row i0 + 1 = [F = 0 | Y = S | Z = T | r]
-  const T* b1 = b0 + kBlk;
-  if (col) {
-#pragma unroll 4
-    for (int r = 0; r < 12; ++r) {
-      P_s[r * kSegP + c] = c < 12 ? b0[r * kBlkLd + c] : (c < 24 ? T(0) : b0[r * kBlkLd + 24]);
-      P_s[(12 + r) * kSegP + c] = c < 12 ? T(0) : b1[r * kBlkLd + c];
+  auto fetch = [&](int i, int buf) {   // block row i to buffer buf (asynchronous copy)
+    char* dst = reinterpret_cast<char*>(tab + (1 + buf) * kBlk);
+    const char* src = reinterpret_cast<const char*>(cond + int64_t(i) * kBlk);
+    constexpr int n = kBlk * int(sizeof(T)) / 16;
+#pragma unroll
+    for (int t = 0; t < (n + 31) / 32; ++t) {
+      const int e = lane + 32 * t;
+      if (32 * t + 32 <= n || e < n) cp_async16(dst + 16 * e, src + 16 * e);
     }
-  }
-  if (lane < 24) {
-    T y[12];
-    load_row12<T>(lane < 12 ? b0 + lane * kBlkLd + 12 : b1 + (lane - 12) * kBlkLd, y);
-    store_row12_from<T>(Y_s + lane * 12, y, 0);
+  };
+  // the first panel: carry rows = block row i0 = [F = S | Y = T | Z = 0 | r]
+  fetch(i0, 1);
+  fetch(i0 + 1, 0);
+  cp_async_wait_all();
+  __syncwarp();
+  {
+    T v[12], y[12];
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      v[m] = tab[(24 + m) * kBlkLd + c];
+      if (lane < 12) y[m] = tab[(24 + m) * kBlkLd + 12 + lane];
+    }
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      if (col) tab[m * kBlkLd + c] = zcol ? T(0) : v[m];
+      if (lane < 12) Y_s[m * 12 + lane] = y[m];
+    }
   }
   __syncwarp();
 
-  const unsigned itag = 31u - unsigned(lane);
+  int row = lane;   // this lane's row of the panel: 0..11 carry, 12.. row of the block row + 12
+  int cur = 0;      // the buffer of block row i
   bool bad = false;
-  for (int i = i0 + 1; i < i1; ++i) {
+  for (int i = i0 + 1; i < i1; ++i, cur ^= 1) {
     const bool more = i + 1 < i1;
-    if (more) {   // block row i + 1 to the stage (asynchronous copy)
-      const char* src = reinterpret_cast<const char*>(cond + int64_t(i + 1) * kBlk);
-      for (int e = lane; e < 12 * kBlkLd * int(sizeof(T)) / 16; e += 32)
-        cp_async16(reinterpret_cast<char*>(stage) + 16 * e, src + 16 * e);
-      cp_async_commit();
-    }
+    if (more) fetch(i + 1, cur ^ 1);
     // ---- phase A
+    const int trow = row < 12 ? row : row + 12 * cur;   // in tab
     T ya[12];
     if (lane < 24) {
-      load_row12<T>(Y_s + lane * 12, ya);
+      load_row12<T>(row < 12 ? Y_s + row * 12 : tab + trow * kBlkLd, ya);
     } else {
 #pragma unroll
       for (int t = 0; t < 12; ++t) ya[t] = T(0);
@@ -1364,75 +1545,73 @@ __device__ __forceinline__ void abd_segment(const SolveArgs& a, const Workspace&
     // pivot key: magnitude with the low 5 bits replaced by a lane tag (ties
     // to the lower lane); rows that are no candidates have zero mask and tag
     unsigned kmask = lane < 24 ? ~31u : 0u;
-    unsigned ktag = lane < 24 ? itag : 0u;
+    unsigned ktag = lane < 24 ? 31u - unsigned(lane) : 0u;
+    int step = 0;   // a pivot row's
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      const int q0 = k / V;
+      bool good;
+      const T own = pivot_recip(ya[k], good);
       const unsigned key = (mag_key(ya[k]) & kmask) | ktag;
       const unsigned best = __reduce_max_sync(0xffffffffu, key);
-      if (key == best) {   // candidates' keys are nonzero and differ in the tag; the others are 0
-        if constexpr (sizeof(T) == sizeof(double)) {   // FP64: the pivot lane publishes 1/pivot
-          const T piv = ya[k];
-          const bool good = piv != T(0) && isfinite(piv);
-          bad = bad || !good;
-          ya[k] = good ? recip_rn(piv) : T(0);
-        }
-        store_row12_from<T>(U_s + k * 12, ya, q0);
-        perm_s[k] = lane;
-        kmask = 0u;
-        ktag = 0u;
-      }
-      __syncwarp();
-      const T* u = U_s + k * 12;
-      T inv = u[k];
-      if constexpr (sizeof(T) == sizeof(float)) {
-        // FP32: the row is published with its raw pivot and every lane forms
-        // the same 1/pivot (off the pivot lane's path)
-        bool good;
-        inv = pivot_recip(inv, good);
-        bad = bad || !good;
-      }
+      const int src = 31 - int(best & 31u);
+      const T inv = __shfl_sync(0xffffffffu, own, src);
+      T u1 = T(0);
+      if (k + 1 < 12) u1 = __shfl_sync(0xffffffffu, ya[k + 1 < 12 ? k + 1 : k], src);
       // (lanes that are no candidate update rows whose entries from here on
       // are never read)
       const T la = ya[k] * inv;
-#pragma unroll
-      for (int q = q0; q < 12 / V; ++q) {
-        T uv[V];
-        if constexpr (sizeof(T) == 4) {
-          const float4 v4 = reinterpret_cast<const float4*>(u)[q];
-          uv[0] = v4.x; uv[1] = v4.y; uv[2] = v4.z; uv[3] = v4.w;
-        } else {
-          const double2 v2 = reinterpret_cast<const double2*>(u)[q];
-          uv[0] = v2.x; uv[1] = v2.y;
-        }
-#pragma unroll
-        for (int t = 0; t < V; ++t) {
-          const int cc = V * q + t;
-          if (cc > k) ya[cc] = fma(-la, uv[t], ya[cc]);
-        }
+      ya[k] = own;
+      if (lane == src) {   // the pivot row, 1/pivot on the diagonal
+        bad = bad || !good;
+        store_row12_from<T>(U_s + k * 12, ya, k / V);
+        step = k;
+        kmask = 0u;
+        ktag = 0u;
       }
       ya[k] = la;   // column k is done: the row keeps its multiplier there
-    }
-    if (lane < 24) store_row12_from<T>(L_s + lane * 12, ya, 0);   // a pivot row's entries from its step on are never read
-    if constexpr (sizeof(T) == sizeof(float)) {
-      if (lane < 12) {   // 1/pivot on the diagonal of the stored rows (formed again: the same value)
-        bool gd;
-        U_s[lane * 12 + lane] = pivot_recip(U_s[lane * 12 + lane], gd);
+      if (k + 1 < 12) ya[k + 1 < 12 ? k + 1 : k] = fma(-la, u1, ya[k + 1 < 12 ? k + 1 : k]);
+      __syncwarp();
+      if (k + 2 < 12) {
+#pragma unroll
+        for (int q = (k + 2) / V; q < 12 / V; ++q) {
+          T uv[V];
+          load_vec16<T>(U_s + k * 12 + q * V, uv);
+#pragma unroll
+          for (int t = 0; t < V; ++t) {
+            const int cc = V * q + t;
+            if (cc > k + 1) ya[cc] = fma(-la, uv[t], ya[cc]);
+          }
+        }
       }
     }
-    const unsigned cmask = __ballot_sync(0xffffffffu, ktag != 0u);   // the 12 rows that were no pivot
-    if (ktag != 0u) cslot_s[__popc(cmask & lt_mask)] = lane;
-    __syncwarp();
+    if (lane < 24) store_row12_from<T>(L_s + lane * 12, ya, 0);   // a pivot row's entries from its step on are never read
+    const bool carry = ktag != 0u;   // one of the 12 rows that were no pivot
+    const unsigned cmask = __ballot_sync(0xffffffffu, carry);
+    if (lane < 24) {
+      const int m = __popc(cmask & lt_mask);
+      (carry ? crow_s + m : prow_s + step)[0] = trow;
+      (carry ? clane_s + m : plane_s + step)[0] = lane;
+      row = carry ? m : 12 + step;   // the next panel's
+    }
+    if (more) cp_async_wait_all();   // this lane's part of block row i + 1 has landed
+    __syncwarp();                    // ... and every lane's
 
-    // ---- phase B
+    // ---- phase B: all loads of a part before its stores, so that they overlap
     T* segp = seg + int64_t(i) * 12 * kSegLd;
+    int rows[12], lanes[12];
+    load_slots(prow_s, rows);
+    load_slots(plane_s, lanes);
     T Q[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      const int pk = perm_s[k];
-      T x = P_s[pk * kSegP + c], y = T(0);
+      Q[k] = tab[rows[k] * kBlkLd + c];
+      if (rows[k] >= 12 && c < 12) Q[k] = T(0);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      T x = Q[k], y = T(0);
       T l[12];
-      load_row12_upto<T>(L_s + pk * 12, l, (k + V - 1) / V);
+      load_row12_upto<T>(L_s + lanes[k] * 12, l, (k + V - 1) / V);
 #pragma unroll
       for (int j = 0; j < k; ++j) {
         if (j & 1) y = fma(-l[j], Q[j], y);
@@ -1440,44 +1619,50 @@ __device__ __forceinline__ void abd_segment(const SolveArgs& a, const Workspace&
       }
       x += y;
       Q[k] = x;
-      if (col) segp[k * kSegLd + segc] = x;
     }
-    // y_i part of the pivot rows (1/pivot on the diagonal; left of it unread)
-    for (int e = lane; e < 12 * (12 / V); e += 32) {
-      const int k = e / (12 / V), q = e % (12 / V);
-      if (q >= k / V)
-        reinterpret_cast<float4*>(segp + k * kSegLd + 12)[q] = reinterpret_cast<const float4*>(U_s + k * 12)[q];
-    }
-    const bool zcol = c >= 12 && c < 24;
+    load_slots(crow_s, rows);
+    load_slots(clane_s, lanes);
+    T f[12];
 #pragma unroll
     for (int m = 0; m < 12; ++m) {
-      const int r = cslot_s[m];
-      T f = P_s[r * kSegP + c], g = T(0);
+      f[m] = tab[rows[m] * kBlkLd + c];
+      if (rows[m] >= 12 && c < 12) f[m] = T(0);
+    }
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      T g = T(0);
       T l[12];
-      load_row12<T>(L_s + r * 12, l);
+      load_row12<T>(L_s + lanes[m] * 12, l);
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
         if (k & 1) g = fma(-l[k], Q[k], g);
-        else f = fma(-l[k], Q[k], f);
+        else f[m] = fma(-l[k], Q[k], f[m]);
       }
-      f += g;
-      if (more) {
-        // Z moves into the y_i slot
-        if (col) P_s[r * kSegP + c] = zcol ? T(0) : f;
-        if (zcol) Y_s[r * 12 + c - 12] = f;
-      } else if (col) {
-        red[m * kBlkLd + c] = f;   // last panel: the carry rows are the reduced row [F | Y | rhs]
-      }
+      f[m] += g;
     }
-    if (more) {   // the pivot slots take block row i + 1 = [0 | S | T | r]
-      cp_async_wait_all();   // this lane's part of the stage has landed
-      __syncwarp();          // ... and every lane's
+    if (more) {   // Z moves into the y_i slot (the table's Z columns stay 0)
+      T* dst = zcol ? Y_s + c - 12 : tab + c;
+      const int ld = zcol ? 12 : kBlkLd;
+      if (col) {
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const int slot = perm_s[k];
-        if (col) P_s[slot * kSegP + c] = c < 12 ? T(0) : stage[k * kBlkLd + c];
-        if (lane < 12) Y_s[slot * 12 + lane] = stage[k * kBlkLd + lane];
+        for (int m = 0; m < 12; ++m) dst[m * ld] = f[m];
       }
+    } else if (col) {   // last panel: the carry rows are the reduced row [F | Y | rhs]
+#pragma unroll
+      for (int m = 0; m < 12; ++m) red[m * kBlkLd + c] = f[m];
+    }
+    // the stored pivot rows: passive columns, then the y_i part (1/pivot on
+    // the diagonal; left of it unread)
+    if (col) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) segp[k * kSegLd + segc] = Q[k];
+    }
+    constexpr int nu = 12 * (12 / V);
+#pragma unroll
+    for (int t = 0; t < (nu + 31) / 32; ++t) {
+      const int e = lane + 32 * t, k = e / (12 / V), q = e % (12 / V);
+      if (e < nu && q >= k / V)
+        reinterpret_cast<float4*>(segp + k * kSegLd + 12)[q] = reinterpret_cast<const float4*>(U_s + k * 12)[q];
     }
     __syncwarp();   // tables written before the next panel reads them
   }
@@ -1486,20 +1671,25 @@ __device__ __forceinline__ void abd_segment(const SolveArgs& a, const Workspace&
 
 // the reduced staircase of one node by one warp
 template <typename T>
-__device__ __forceinline__ void abd_reduced(const SolveArgs& a, const Workspace& w, int64_t node, int N, int lane) {
+__device__ __forceinline__ void abd_reduced(const SolveArgs& a, const Workspace& w, int64_t node, int N, int lane,
+                                            T* tab) {
   const int smax = seg_count(a.Nmax);
   const T* red = static_cast<const T*>(w.Red) + node * smax * int64_t(kBlk);
   T* abd = static_cast<T*>(w.Abd) + node * a.Nmax * int64_t(kBlk);
-  const bool ok = abd_staircase<T>(a, w, node, N, red, seg_count(N), 3 * kSegLen, abd, lane);
+  const bool ok = abd_staircase<T>(a, w, node, N, red, seg_count(N), 3 * kSegLen, abd, lane, tab);
   if (!ok && lane == 0) w.ns[node].singular |= 1;
 }
 
-// the back substitution of one segment by one warp: the pivot rows of panel
-// i - 1 are copied to shared memory (asynchronously) while panel i is
-// substituted
+// the back substitution of one segment by one warp: the pivot rows of the
+// panels before panel i are copied to shared memory (asynchronously) while
+// panel i is substituted; a panel takes less time than a copy's latency, so
+// the FP32 form keeps three in flight
+template <typename T>
+constexpr int kSegBackStages = sizeof(T) == 4 ? 4 : 2;
 template <typename T>
 __device__ __forceinline__ void abd_segment_back(const SolveArgs& a, const Workspace& w, int64_t node, int s, int N,
                                                  int lane, T (*buf)[12 * kSegLd]) {
+  constexpr int S = kSegBackStages<T>;
   const int i0 = s * kSegLen;
   const int i1 = i0 + kSegLen < N ? i0 + kSegLen : N;
   if (i1 - i0 < 2) return;
@@ -1513,15 +1703,23 @@ __device__ __forceinline__ void abd_segment_back(const SolveArgs& a, const Works
   }
   auto fetch = [&](int i, int b) {   // panel i's 12 pivot rows to buf[b]
     const char* src = reinterpret_cast<const char*>(seg + int64_t(i) * 12 * kSegLd);
-    for (int e = lane; e < 12 * kSegLd * int(sizeof(T)) / 16; e += 32)
-      cp_async16(reinterpret_cast<char*>(buf[b]) + 16 * e, src + 16 * e);
-    cp_async_commit();
+    constexpr int n = 12 * kSegLd * int(sizeof(T)) / 16;
+#pragma unroll
+    for (int t = 0; t < (n + 31) / 32; ++t) {
+      const int e = lane + 32 * t;
+      if (32 * t + 32 <= n || e < n) cp_async16(reinterpret_cast<char*>(buf[b]) + 16 * e, src + 16 * e);
+    }
   };
-  fetch(i1 - 1, 0);
-  for (int i = i1 - 1, b = 0; i > i0; --i, b ^= 1) {
-    cp_async_wait_all();   // panel i has landed (this lane's part) ...
-    __syncwarp();          // ... and every lane's; buf[b ^ 1] was read in the last pass
-    if (i - 1 > i0) fetch(i - 1, b ^ 1);
+#pragma unroll
+  for (int t = 0; t < S - 1; ++t) {   // (a group per panel, also where there is none)
+    if (i1 - 1 - t > i0) fetch(i1 - 1 - t, t);
+    cp_async_commit();
+  }
+  for (int i = i1 - 1, b = 0; i > i0; --i, b = b + 1 < S ? b + 1 : 0) {
+    cp_async_wait_prior<S - 2>();   // panel i has landed (this lane's part) ...
+    __syncwarp();                   // ... and every lane's; the buffer before b was read in the last pass
+    if (i - (S - 1) > i0) fetch(i - (S - 1), b > 0 ? b - 1 : S - 1);
+    cp_async_commit();
     // lane k holds pivot row k of panel i: [F | U (1/pivot at k) | V | rhs]
     T r[37];
 #pragma unroll
@@ -1570,16 +1768,17 @@ __global__ void __launch_bounds__(32 * seg_warps<float>()) k_abd_seg(SolveArgs a
 }
 
 __global__ void __launch_bounds__(128) k_abd_red(SolveArgs a, Workspace w) {
+  __shared__ __align__(16) float stair_s[4][stair_smem_elems<float>()];
   const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
   if (node >= a.n) return;
   if (!w.ns[node].active) return;
-  abd_reduced<float>(a, w, node, a.N[node], threadIdx.x & 31);
+  abd_reduced<float>(a, w, node, a.N[node], threadIdx.x & 31, stair_s[threadIdx.x >> 5]);
   __syncwarp();
   if ((threadIdx.x & 31) == 0) ls_start(w, node);   // (the rest of the direction skips a singular node)
 }
 
 __global__ void __launch_bounds__(128) k_abd_segback(SolveArgs a, Workspace w) {
-  __shared__ __align__(16) float buf_s[4][2][12 * kSegLd];
+  __shared__ __align__(16) float buf_s[4][kSegBackStages<float>][12 * kSegLd];
   const int smax = seg_count(a.Nmax);
   const int64_t wid = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
   const int64_t node = wid / smax;

@@ -21,6 +21,10 @@ __host__ __device__ constexpr int persist_smem_per_warp() {
   return sizeof(T) == sizeof(double) ? 36 * kCols * 8 : kCondSmemFloats * 4;
 }
 
+static_assert(stair_smem_elems<float>() * 4 <= persist_smem_per_warp<float>() &&
+                  stair_smem_elems<double>() * 8 <= persist_smem_per_warp<double>(),
+              "the staircase's tables fit");
+
 // Residual at Y + alpha D for the whole node, by one warp.  The
 // right-hand side F at every point goes to `Fs` (the node's Jacobian slot,
 // free during the line search); each lane then forms the stage rows of the
@@ -152,7 +156,7 @@ __device__ __forceinline__ bool direction_node(const SolveArgs& a, const Workspa
     }
   }
   __syncwarp();
-  const bool ok = abd_node_reg<T>(a, w, node, N, lane);
+  const bool ok = abd_node_reg<T>(a, w, node, N, lane, reinterpret_cast<T*>(scratch));
   __syncwarp();
   for (int i = 0; i < N; ++i) recover_interval<T>(a, w, node, i, lane);
   __syncwarp();
