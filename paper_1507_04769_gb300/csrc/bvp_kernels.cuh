@@ -26,6 +26,8 @@
 // for the others (bvp_direction.cuh).
 #pragma once
 
+#include <type_traits>
+
 #include <cmath>
 
 #include "common.cuh"
@@ -469,14 +471,24 @@ __device__ __forceinline__ void ls_start(const Workspace& w, int64_t node) {
 // mode 0: initial residual (convergence test at iteration 0);
 // mode 1: Armijo test for the current alpha, and when the step is taken the
 // iteration's end: convergence, iteration cap.
-__device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, int64_t node, int lane, int mode) {
+// The node's share of the counts goes to cnt (shared memory: searching,
+// active).
+__device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, int64_t node, int lane, int mode,
+                                        int* cnt) {
+  const int N = a.N[node];   // (beside the state: one latency)
   NodeState s = w.ns[node];
   if (s.searching != 1) return;
-  const int N = a.N[node];
   double ss = 0.0, mx = 0.0;
-  for (int i = lane; i < N; i += 32) {
-    ss += w.part[2 * (node * a.Nmax + i)];
-    mx = fmax(mx, w.part[2 * (node * a.Nmax + i) + 1]);
+  const double2* part = reinterpret_cast<const double2*>(w.part) + node * a.Nmax;
+  for (int i0 = lane; i0 < N; i0 += 4 * 32) {   // four loads in flight
+    double2 v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = i0 + 32 * t < N ? part[i0 + 32 * t] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      ss += v[t].x;
+      mx = fmax(mx, v[t].y);
+    }
   }
   ss = warp_sum(ss);
   mx = warp_max(mx);
@@ -487,7 +499,7 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
     s.alpha = 0.5;
     s.singular |= kElimNode;
     w.ns[node] = s;
-    atomicAdd(&w.counters[kSearchCount], 1);
+    atomicAdd(&cnt[0], 1);
     atomicAdd(&w.counters[kElimCount], 1);
     return;
   }
@@ -499,7 +511,7 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
     // rows at the iterate again, which that direction needs
     s.alpha = a.tree && !(s.singular & kElimDone) ? 0.0 : 0.5 * s.alpha;
     w.ns[node] = s;
-    atomicAdd(&w.counters[kSearchCount], 1);
+    atomicAdd(&cnt[0], 1);
     return;
   }
   s.fnorm2 = ss;
@@ -520,31 +532,49 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
     s.status = SG_MAXITER;
     s.active = 0;
   } else {
-    atomicAdd(&w.counters[kActiveCount], 1);
+    atomicAdd(&cnt[1], 1);
   }
   w.ns[node] = s;
 }
 
 // A warp per node; the block that finishes last publishes the counts, sets the
 // graph's loop conditions and clears the counters: no other launch and no
-// memset per trial or iteration.
+// memset per trial or iteration.  (Latency: a block's counts are added up in
+// shared memory, and a single block needs no ticket.  One node: 8.2 -> LSR_US
+// us.)
 __global__ void __launch_bounds__(128) k_ls_reduce(SolveArgs a, Workspace w, int mode) {
+  __shared__ int cnt[2];
   const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
-  if (node < a.n) ls_node(a, w, node, threadIdx.x & 31, mode);
-  __threadfence();   // this warp's counts before the block's ticket
+  const bool one = gridDim.x == 1;
+  int before = 0;
+  if (threadIdx.x == 0) {
+    cnt[0] = cnt[1] = 0;
+    if (one) before = w.counters[kActiveCount];   // by earlier trials of the search
+  }
+  __syncthreads();
+  if (node < a.n) ls_node(a, w, node, threadIdx.x & 31, mode, cnt);
   __syncthreads();
   if (threadIdx.x != 0) return;
-  if (atomicAdd(&w.counters[kTicket], 1) != static_cast<int>(gridDim.x) - 1) return;
-  __threadfence();
-  const int searching = atomicExch(&w.counters[kSearchCount], 0);
-  w.counters[kTicket] = 0;
+  int searching = cnt[0];
+  if (!one) {
+    if (cnt[0]) atomicAdd(&w.counters[kSearchCount], cnt[0]);
+    if (cnt[1]) atomicAdd(&w.counters[kActiveCount], cnt[1]);
+    __threadfence();   // this block's counts before its ticket
+    if (atomicAdd(&w.counters[kTicket], 1) != static_cast<int>(gridDim.x) - 1) return;
+    __threadfence();
+    searching = atomicExch(&w.counters[kSearchCount], 0);
+    w.counters[kTicket] = 0;
+  }
   w.counters[kSearchOut] = searching;
   if (searching == 0) {   // the iteration's end
-    const int active = atomicExch(&w.counters[kActiveCount], 0);
+    const int active = one ? before + cnt[1] : atomicExch(&w.counters[kActiveCount], 0);
+    if (one) w.counters[kActiveCount] = 0;
     w.counters[kActiveOut] = active;
     w.counters[kElimCount] = 0;
     if (mode == 1) w.counters[kEpoch] += 1;
     if (a.conds & 1) cudaGraphSetConditional(a.h_newton, active > 0 ? 1u : 0u);
+  } else if (one) {
+    w.counters[kActiveCount] = before + cnt[1];
   }
   if ((a.conds & 2) && mode == 1) cudaGraphSetConditional(a.h_search, searching > 0 ? 1u : 0u);
 }
@@ -617,8 +647,37 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // Correctly rounded reciprocal (the same value as 1 / x, without the
 // division's slow-path branch).
-__device__ __forceinline__ float recip_rn(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip_rn(double x) { return __drcp_rn(x); }
+
+// 1/pivot of the staircase, correctly rounded; 0 for an unusable pivot.  FP32
+// with kLib = false: one Newton step from the approximate reciprocal with the
+// residual in a fused multiply-add (correctly rounded where no intermediate
+// leaves the normal range: Markstein, IBM J. Res. Dev. 34, 1990; compared for
+// every operand) without the library function's branches, which cost 94 cycles
+// per pivot step of the chain; `odd` tells that the operand is outside the
+// range and the elimination has to be repeated with kLib = true.
+template <bool kLib>
+__device__ __forceinline__ float pivot_recip_rn(float p, bool& good, bool& odd) {
+  const float ap = fabsf(p);
+  good = p != 0.0f && ap < INFINITY;
+  if constexpr (kLib) {
+    odd = false;
+    return good ? __frcp_rn(p) : 0.0f;
+  } else {
+    float r;   // (volatile: not to be sunk into a branch)
+    asm volatile("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(p));
+    r = __fmaf_rn(r, __fmaf_rn(-p, r, 1.0f), r);
+    odd = good && !(ap > 0x1p-125f && ap < 0x1p125f);
+    return good ? r : 0.0f;
+  }
+}
+template <bool kLib>
+__device__ __forceinline__ double pivot_recip_rn(double p, bool& good, bool& odd) {
+  good = p != 0.0 && isfinite(p);
+  odd = false;
+  const double r = recip_rn(good ? p : 1.0);   // (1: no slow path for zeros)
+  return good ? r : 0.0;
+}
 
 // 1/pivot in the condensation and segment eliminations.  FP32: the
 // approximate reciprocal instruction (rcp.approx.ftz, within about one unit
@@ -1119,23 +1178,60 @@ constexpr int stair_smem_elems() {
   return 6 * kBlkLd + kStairStages<T> * kBlk + 18 * 12 + 12 * 12 + 2 * 16 + 40 * 4 / int(sizeof(T));
 }
 
+// Back substitution through 12 upper triangular pivot rows: lane k < 12 holds
+// row k's right-hand side t and its entries u (1/pivot at u[k]), U is the
+// table of the rows in shared memory (row stride ld, 16-byte aligned); every
+// lane receives d.  Four unknowns at a time: their lanes' t by shuffles, the
+// 4 x 4 triangle from the table in every lane (the operations of one unknown
+// at a time, with a third of the shuffles' latency).
+template <typename T>
+__device__ __forceinline__ void back_solve12(T t, const T (&u)[12], const T* U, int ld, int lane, T (&d)[12]) {
+  constexpr int V = 16 / int(sizeof(T));
+#pragma unroll
+  for (int b = 2; b >= 0; --b) {
+    T x[4], m[4][4];
+#pragma unroll
+    for (int j = 3; j >= 0; --j) {
+      x[j] = __shfl_sync(0xffffffffu, t, 4 * b + j);
+#pragma unroll
+      for (int q = 0; q < 4 / V; ++q) {
+        T v[V];
+        load_vec16<T>(U + (4 * b + j) * ld + 4 * b + q * V, v);
+#pragma unroll
+        for (int e = 0; e < V; ++e) m[j][q * V + e] = v[e];
+      }
+    }
+#pragma unroll
+    for (int j = 3; j >= 0; --j) {
+      x[j] *= m[j][j];
+      d[4 * b + j] = x[j];
+#pragma unroll
+      for (int i = j - 1; i >= 0; --i) x[i] = fma(-m[i][j], x[j], x[i]);
+    }
+#pragma unroll
+    for (int j = 3; j >= 0; --j) t = lane < 4 * b + j ? fma(-u[4 * b + j], x[j], t) : t;
+  }
+}
+
 // The closing system [y_N (12) | rhs]: twelve pivot steps with partial
 // pivoting on rows held one per lane (entries 13.. are padding).  The pivot
 // row of step k keeps 1/pivot at column k; plane[k] is the lane that held it.
-template <typename T>
-__device__ __forceinline__ void close_eliminate(T (&r)[16], bool cand, int (&plane)[12], bool& ok, int lane, T* pub) {
+// Returns whether a pivot asks for kLib.
+template <typename T, bool kLib>
+__device__ __forceinline__ bool close_eliminate(T (&r)[16], bool cand, int (&plane)[12], bool& ok, int lane, T* pub) {
   constexpr int V = 16 / int(sizeof(T));
-  bool done = false;
+  bool done = false, again = false;
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     const bool act = cand && !done;
-    const bool good = r[k] != T(0) && isfinite(r[k]);
-    const T own = recip_rn(act && good ? r[k] : T(1));
     const int p = warp_pivot_lane<T>(r[k], act, lane);
     plane[k] = p;
-    const T inv = __shfl_sync(0xffffffffu, good ? own : T(0), p);
+    bool good, odd;
+    const T own = pivot_recip_rn<kLib>(r[k], good, odd);
+    const T inv = __shfl_sync(0xffffffffu, own, p);
     const bool is_p = lane == p;
     ok = ok && (good || !is_p);
+    again = again || (odd && is_p);
     const T l = (act && !is_p) ? r[k] * inv : T(0);
     T* u = pub + (k & 1) * 16;
     if (is_p) {
@@ -1156,6 +1252,7 @@ __device__ __forceinline__ void close_eliminate(T (&r)[16], bool cand, int (&pla
       }
     }
   }
+  return __any_sync(0xffffffffu, again);
 }
 
 // (the warp's tables at tab: stair_smem_elems<T>() elements)
@@ -1219,55 +1316,65 @@ __device__ __forceinline__ bool abd_staircase(const SolveArgs& a, const Workspac
     cp_async_commit();
     // ---- phase A
     const int trow = row < 6 ? row : row + 12 * (i % S);   // in tab
-    T ya[12];
-    if (rowlane) {
-      load_row12<T>(tab + trow * kBlkLd, ya);
-    } else {
-#pragma unroll
-      for (int t = 0; t < 12; ++t) ya[t] = T(0);
-    }
-    bool done = false;
+    bool done = false, again = false, fine = true;
     int step = 0;
+    auto phase_a = [&](auto lib) {
+      T ya[12];
+      if (rowlane) {
+        load_row12<T>(tab + trow * kBlkLd, ya);
+      } else {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      // every candidate forms its own reciprocal while the pivot is searched;
-      // it and the entry of column k + 1 reach the other rows by shuffles, so
-      // that the next search does not wait for the table
-      const bool act = rowlane && !done;
-      const bool good = ya[k] != T(0) && isfinite(ya[k]);
-      const T own = recip_rn(act && good ? ya[k] : T(1));   // (1: no slow path for zeros)
-      const T mine = good ? own : T(0);
-      const int src = warp_pivot_lane<T>(ya[k], act, lane);
-      const T inv = __shfl_sync(0xffffffffu, mine, src);
-      T u1 = T(0);
-      if (k + 1 < 12) u1 = __shfl_sync(0xffffffffu, ya[k + 1 < 12 ? k + 1 : k], src);
-      // (rows that are no candidates are updated too: their entries from here
-      // on are never read)
-      const T la = ya[k] * inv;
-      ya[k] = mine;
-      if (lane == src) {
-        ok = ok && good;
-        store_row12_from<T>(U_s + k * 12, ya, k / V);
-        done = true;
-        step = k;
+        for (int t = 0; t < 12; ++t) ya[t] = T(0);
       }
-      ya[k] = la;
-      if (k + 1 < 12) ya[k + 1 < 12 ? k + 1 : k] = fma(-la, u1, ya[k + 1 < 12 ? k + 1 : k]);
-      __syncwarp();
-      if (k + 2 < 12) {
+      done = again = false;
+      fine = true;
 #pragma unroll
-        for (int q = (k + 2) / V; q < 12 / V; ++q) {
-          T uv[V];
-          load_vec16<T>(U_s + k * 12 + q * V, uv);
+      for (int k = 0; k < 12; ++k) {
+        // every candidate forms its own reciprocal while the pivot is searched;
+        // it and the entry of column k + 1 reach the other rows by shuffles, so
+        // that the next search does not wait for the table
+        const bool act = rowlane && !done;
+        const int src = warp_pivot_lane<T>(ya[k], act, lane);
+        bool good, odd;
+        const T mine = pivot_recip_rn<decltype(lib)::value>(ya[k], good, odd);
+        const T inv = __shfl_sync(0xffffffffu, mine, src);
+        T u1 = T(0);
+        if (k + 1 < 12) u1 = __shfl_sync(0xffffffffu, ya[k + 1 < 12 ? k + 1 : k], src);
+        // (rows that are no candidates are updated too: their entries from here
+        // on are never read)
+        const T la = ya[k] * inv;
+        ya[k] = mine;
+        if (lane == src) {
+          fine = fine && good;
+          again = again || odd;
+          store_row12_from<T>(U_s + k * 12, ya, k / V);
+          done = true;
+          step = k;
+        }
+        ya[k] = la;
+        if (k + 1 < 12) ya[k + 1 < 12 ? k + 1 : k] = fma(-la, u1, ya[k + 1 < 12 ? k + 1 : k]);
+        __syncwarp();
+        if (k + 2 < 12) {
 #pragma unroll
-          for (int t = 0; t < V; ++t) {
-            const int cc = V * q + t;
-            if (cc > k + 1) ya[cc] = fma(-la, uv[t], ya[cc]);
+          for (int q = (k + 2) / V; q < 12 / V; ++q) {
+            T uv[V];
+            load_vec16<T>(U_s + k * 12 + q * V, uv);
+#pragma unroll
+            for (int t = 0; t < V; ++t) {
+              const int cc = V * q + t;
+              if (cc > k + 1) ya[cc] = fma(-la, uv[t], ya[cc]);
+            }
           }
         }
       }
+      if (rowlane) store_row12_from<T>(L_s + lane * 12, ya, 0);
+    };
+    phase_a(std::false_type{});
+    if (__any_sync(0xffffffffu, again)) {
+      __syncwarp();
+      phase_a(std::true_type{});
     }
-    if (rowlane) store_row12_from<T>(L_s + lane * 12, ya, 0);
+    ok = ok && fine;
     const unsigned dmask = __ballot_sync(0xffffffffu, done);
     if (rowlane) {
       const int rank = __popc(dmask & lt_mask), m = lane - rank;
@@ -1349,7 +1456,17 @@ __device__ __forceinline__ bool abd_staircase(const SolveArgs& a, const Workspac
         if (c == cl) r[6 + c] = T(1);
       r[12] = cr;
     }
-    close_eliminate<T>(r, cand, plane, ok, lane, pub);
+    const bool ok0 = ok;
+    T r0[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) r0[c] = r[c];
+    if (close_eliminate<T, false>(r, cand, plane, ok, lane, pub)) {
+      ok = ok0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) r[c] = r0[c];
+      __syncwarp();   // the last published row
+      close_eliminate<T, true>(r, cand, plane, ok, lane, pub);
+    }
   }
   // back substitution of the closing system: dy_N (uniform across lanes)
   T dy[12];
@@ -1386,12 +1503,10 @@ __device__ __forceinline__ bool abd_staircase(const SolveArgs& a, const Workspac
     T tt = rr[24];
 #pragma unroll
     for (int c = 0; c < 12; ++c) tt = fma(-rr[12 + c], dy[c], tt);
+    T u[12];
 #pragma unroll
-    for (int k = 11; k >= 0; --k) {
-      const T dk = __shfl_sync(0xffffffffu, tt * rr[k], k);
-      dy[k] = dk;
-      tt = (lane < k) ? fma(-rr[k], dk, tt) : tt;
-    }
+    for (int c = 0; c < 12; ++c) u[c] = rr[c];
+    back_solve12<T>(tt, u, ring + (ii % S) * kBlk, kBlkLd, lane, dy);
     if (lane < 12) {
       T mine = T(0);
 #pragma unroll
@@ -1736,12 +1851,10 @@ __device__ __forceinline__ void abd_segment_back(const SolveArgs& a, const Works
       tt = fma(-r[c], dya[c], tt);
       tt = fma(-r[24 + c], dyn[c], tt);
     }
+    T u[12];
 #pragma unroll
-    for (int k = 11; k >= 0; --k) {
-      const T dk = __shfl_sync(0xffffffffu, tt * r[12 + k], k);
-      dyn[k] = dk;
-      tt = (lane < k) ? fma(-r[12 + k], dk, tt) : tt;
-    }
+    for (int c = 0; c < 12; ++c) u[c] = r[12 + c];
+    back_solve12<T>(tt, u, buf[b] + 12, kSegLd, lane, dyn);
     if (lane < 12) {
       T mine = T(0);
 #pragma unroll
