@@ -540,8 +540,7 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
 // A warp per node; the block that finishes last publishes the counts, sets the
 // graph's loop conditions and clears the counters: no other launch and no
 // memset per trial or iteration.  (Latency: a block's counts are added up in
-// shared memory, and a single block needs no ticket.  One node: 8.2 -> LSR_US
-// us.)
+// shared memory, and a single block needs no ticket.)
 __global__ void __launch_bounds__(128) k_ls_reduce(SolveArgs a, Workspace w, int mode) {
   __shared__ int cnt[2];
   const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
@@ -1163,8 +1162,8 @@ __device__ __forceinline__ void load_slots(const int* src, int (&r)[12]) {
 // a row-wise elimination).  A row's lane decides ties of the pivot search:
 // carry rows keep theirs, the next block's rows take the pivot rows' in lane
 // order.  The chain is latency; with the rows' 25 columns in the lanes a
-// panel took 3,300 cycles, in this form RED_CYC (one node at 128 intervals,
-// eight panels: 26 -> RED_US us per iteration).
+// panel took 3,300 cycles, in this form 2,500 (one node at 128 intervals,
+// eight panels: 26 -> 22 us per iteration).
 //
 // The blocks may be the N interval block rows of the node (pt_stride = 3:
 // block i couples mesh points 3i and 3i + 3) or the reduced block rows of the
@@ -1573,8 +1572,8 @@ __device__ __forceinline__ bool abd_node_reg(const SolveArgs& a, const Workspace
 // kept off it: the reciprocal of every candidate is formed during the search,
 // the pivot row's next column travels by shuffle and the rest through U while
 // the next search runs, and loads are issued ahead of the stores they could
-// alias.  One node at 128 intervals: 52 -> SEG_US us per iteration; the
-// level-4 batch's six iterations 1.40 -> SEG_MS ms.
+// alias.  One node at 128 intervals: 52 -> 23 us per iteration; the
+// level-4 batch's six iterations 1.40 -> 1.12 ms.
 template <typename T>
 __host__ __device__ constexpr int seg_warps() { return sizeof(T) == 4 ? 4 : 2; }   // warps per block
 // carry rows and two block rows, Y, L, U (elements), then 48 ints
