@@ -226,7 +226,7 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
   for (int it = 0; it < a.max_iter && h_cnt[1] > 0; ++it) {
     if constexpr (sizeof(T) == sizeof(double)) SG_TIMED("k_point_fp64", st, (k_point_fp64<<<gp, 128, 0, st>>>(a, w)));
     for (const DirLaunch& d : dir)
-      SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
+      if (d.grid > 0) SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
     SG_LAUNCH_CHECK("newton kernels");
     for (int trial = 0; trial < 13; ++trial) {   // alpha = 1, 1/2, ..., 2^-10 (and one at 0 in the FP64 form)
       if constexpr (sizeof(T) == sizeof(double)) {
@@ -326,7 +326,8 @@ static void add_iteration(GraphBuilder& b, const SolveArgs& a, const Workspace& 
     b.kernel(k_point_fp64, static_cast<unsigned>(ceil_div(np, 128)), 128, 0, a, w);
   DirLaunch dir[kDirLaunches<T>];
   direction_launches<T>(a, dir);
-  for (const DirLaunch& d : dir) b.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+  for (const DirLaunch& d : dir)
+    if (d.grid > 0) b.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
   add_trial<T>(b, a, w);
   cudaGraph_t body = nullptr;
   b.loop(a.h_search, &body);

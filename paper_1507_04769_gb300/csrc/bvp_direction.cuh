@@ -29,8 +29,8 @@
 // Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
 // iterations): condensation 74.8 -> 25.5 ms (FP64 pipe 95 % busy), elimination
 // and back substitution over the intervals 23.9 -> 9.4 ms, recovery 4.3 -> 2.5
-// ms; the solve (a graph per mesh size) 112.0 -> 42.4 ms; one node at 128
-// intervals 1.80 -> 0.95 ms.
+// ms; the solve (a graph per mesh size) 112.0 -> 42.0 ms; 85 nodes at 128
+// intervals 8.09 -> 3.31 ms.
 //
 // Elimination over the intervals.  An interval's condensed row
 // S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
@@ -488,6 +488,72 @@ inline int tree_threads(int64_t n, int Nmax) {
   return t;
 }
 
+// The compositions of the relations [i0, i1) at strides st0, 2 st0, .. below
+// st1, by the block's groups of 16 lanes.  A block barrier per stride.
+__device__ __forceinline__ bool tree_up(double* ops, int i0, int i1, int st0, int st1, double* buf, double* pub, int c,
+                                        int lane16, int g, int ng) {
+  bool bad = false;
+  auto fetch = [&](int i, int st, int b) {   // relations i and i + st to buffer b
+    double* dst = buf + b * 2 * kOp;
+    for (int e = lane16; e < 2 * kOp / 2; e += 16) {
+      const double* src = ops + (e < kOp / 2 ? int64_t(i) * kOp + e * 2 : int64_t(i + st) * kOp + (e - kOp / 2) * 2);
+      cp_async16(dst + e * 2, src);
+    }
+    cp_async_commit();
+  };
+  const int n = i1 - i0;
+  for (int st = st0; st < n && st < st1; st *= 2) {
+    const int pairs = (n - st + 2 * st - 1) / (2 * st);   // left ends i0 + 2 st j with 2 st j + st < n
+    int b = 0;
+    if (g < pairs) fetch(i0 + 2 * st * g, st, 0);
+    for (int j0 = 0; j0 < pairs; j0 += ng, b ^= 1) {
+      const int j = j0 + g;
+      cp_async_wait_all();
+      __syncwarp();
+      if (j + ng < pairs) fetch(i0 + 2 * st * (j + ng), st, b ^ 1);
+      if (j0 + (g & ~1) >= pairs) continue;   // the whole warp
+      double km[12], nw[12];
+      bool bd = false;
+      compose(buf + b * 2 * kOp, buf + b * 2 * kOp + kOp, pub, c, km, nw, bd);
+      if (j < pairs) {
+        bad = bad || bd;
+        if (lane16 < 13) {
+          st_vec<12>(ops + int64_t(i0 + 2 * st * j) * kOp + c * 12, nw);
+          st_vec<12>(ops + int64_t(i0 + 2 * st * j + st) * kOp + c * 12, km);
+        }
+      }
+      __syncwarp();   // buffer b is fetched again in the next round
+    }
+    __syncthreads();
+  }
+  return bad;
+}
+
+// With fewer than two nodes per SM a block per node leaves SMs idle or unevenly
+// loaded through the tree's lowest levels, which hold most of its work: then a
+// block per kLeafIv intervals runs those first.  (85 nodes at 128 intervals: the
+// tree 0.92 -> 0.76 ms, the solve 3.52 -> 3.31 ms; at 389 nodes of 64 intervals
+// the solve would go from 1.29 to 1.31 ms, at 486 per graph from 41.9 to 43.3.)
+constexpr int kLeafIv = 16;
+__host__ __device__ __forceinline__ bool tree_leaves(int64_t n, int Nmax) {
+  return n < 2 * kNumSMs && Nmax >= 2 * kLeafIv;
+}
+constexpr int kLeafThreads = kLeafIv / 2 * 16;   // a group per pair of intervals
+__global__ void __launch_bounds__(kLeafThreads) k_tree_leaf_fp64(SolveArgs a, Workspace w) {
+  extern __shared__ __align__(16) unsigned char tree_smem_raw[];
+  const int chunks = (a.Nmax + kLeafIv - 1) / kLeafIv;
+  const int64_t node = blockIdx.x / chunks;
+  const int i0 = static_cast<int>(blockIdx.x % chunks) * kLeafIv;
+  if (!w.ns[node].active) return;
+  const int N = a.N[node];
+  if (i0 >= N) return;
+  const int tid = threadIdx.x, lane16 = tid & 15, g = tid >> 4;
+  double* buf = reinterpret_cast<double*>(tree_smem_raw) + g * kTreeGroupElems;
+  const bool bad = tree_up(dir_op(a, w) + node * a.Nmax * int64_t(kOp), i0, i0 + kLeafIv < N ? i0 + kLeafIv : N, 1,
+                           kLeafIv, buf, buf + 4 * kOp, lane16 < 13 ? lane16 : 12, lane16, g, kLeafThreads / 16);
+  if (__syncthreads_or(bad) && tid == 0) mark_elim(w, node);
+}
+
 // Block per node.  Relations are composed in place: the result over [a, b)
 // replaces the left operand, and the interior solution (dx_m, dlambda_m) of
 // the composition takes the right operand's place, to be used on the way
@@ -503,41 +569,7 @@ __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, W
   double* buf = reinterpret_cast<double*>(tree_smem_raw) + g * kTreeGroupElems;   // [2][o1 | o2]
   double* pub = buf + 4 * kOp;
   double* ops = dir_op(a, w) + node * a.Nmax * int64_t(kOp);
-  bool bad = false;
-
-  auto fetch = [&](int i, int st, int b) {   // relations i and i + st to buffer b
-    double* dst = buf + b * 2 * kOp;
-    for (int e = lane16; e < 2 * kOp / 2; e += 16) {
-      const double* src = ops + (e < kOp / 2 ? int64_t(i) * kOp + e * 2 : int64_t(i + st) * kOp + (e - kOp / 2) * 2);
-      cp_async16(dst + e * 2, src);
-    }
-    cp_async_commit();
-  };
-
-  for (int st = 1; st < N; st *= 2) {
-    const int pairs = (N - st + 2 * st - 1) / (2 * st);   // left ends 2 st j with 2 st j + st < N
-    int b = 0;
-    if (g < pairs) fetch(2 * st * g, st, 0);
-    for (int j0 = 0; j0 < pairs; j0 += ng, b ^= 1) {
-      const int j = j0 + g;
-      cp_async_wait_all();
-      __syncwarp();
-      if (j + ng < pairs) fetch(2 * st * (j + ng), st, b ^ 1);
-      if (j0 + (g & ~1) >= pairs) continue;   // the whole warp
-      double km[12], nw[12];
-      bool bd = false;
-      compose(buf + b * 2 * kOp, buf + b * 2 * kOp + kOp, pub, c, km, nw, bd);
-      if (j < pairs) {
-        bad = bad || bd;
-        if (lane16 < 13) {
-          st_vec<12>(ops + int64_t(2 * st * j) * kOp + c * 12, nw);
-          st_vec<12>(ops + int64_t(2 * st * j + st) * kOp + c * 12, km);
-        }
-      }
-      __syncwarp();   // buffer b is fetched again in the next round
-    }
-    __syncthreads();
-  }
+  bool bad = tree_up(ops, 0, N, tree_leaves(a.n, a.Nmax) ? kLeafIv : 1, N, buf, pub, c, lane16, g, ng);
 
   // boundary rows
   const int64_t pb = node * npts(a.Nmax);
@@ -737,7 +769,8 @@ __global__ void __launch_bounds__(32 * kRecWarps) k_recover_fp64(SolveArgs a, Wo
 }
 
 // The launches of a Newton direction (after the Jacobians): kernel, grid,
-// block and shared memory of each, in order, for the host loop and the graphs.
+// block and shared memory of each, in order, for the host loop and the graphs
+// (none where the grid is 0).
 struct DirLaunch {
   const char* name;
   void (*fn)(SolveArgs, Workspace);
@@ -745,7 +778,7 @@ struct DirLaunch {
   int block, smem;
 };
 template <typename T>
-constexpr int kDirLaunches = sizeof(T) == sizeof(float) ? 5 : 3;
+constexpr int kDirLaunches = sizeof(T) == sizeof(float) ? 5 : 4;
 
 template <typename T>
 inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches<T>]) {
@@ -761,8 +794,11 @@ inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches
   } else {
     const int tt = tree_threads(a.n, a.Nmax);
     out[0] = {"k_condense_fp64", k_condense_fp64, a.n * cond_chunks(a.Nmax), kCondThreads, kCondSmem};
-    out[1] = {"k_tree_fp64", k_tree_fp64, a.n, tt, tree_smem(tt)};
-    out[2] = {"k_recover_fp64", k_recover_fp64, ceil_div(a.n * ((a.Nmax + 1) / 2), kRecWarps), 32 * kRecWarps,
+    out[1] = {"k_tree_leaf_fp64", k_tree_leaf_fp64,
+              tree_leaves(a.n, a.Nmax) ? a.n * ((a.Nmax + kLeafIv - 1) / kLeafIv) : 0, kLeafThreads,
+              tree_smem(kLeafThreads)};
+    out[2] = {"k_tree_fp64", k_tree_fp64, a.n, tt, tree_smem(tt)};
+    out[3] = {"k_recover_fp64", k_recover_fp64, ceil_div(a.n * ((a.Nmax + 1) / 2), kRecWarps), 32 * kRecWarps,
               kRecSmem};
   }
 }

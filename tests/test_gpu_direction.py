@@ -84,3 +84,19 @@ def test_interval_without_scattering_form():
     for j in range(5):
         s = obvp.solve(pr, X0[j], N * lo, N)
         assert np.max(np.abs(res["lambda0"][j].cpu().numpy() - s.lambda0)) <= 1e-8 * np.max(np.abs(s.lambda0))
+
+
+def test_tree_leaves_by_blocks_give_the_same_bits():
+    """Fewer than 304 nodes run the tree's lowest levels in blocks of their own:
+    the same compositions, so the same results to the last bit as in a solve of
+    more nodes."""
+    params = synth.lq_params(1)
+    n, more = 303, 305
+    sizes = [1, 15, 16, 17, 32, 33, 47, 64, 100, 129]
+    N = np.array([sizes[k % len(sizes)] for k in range(more)])
+    T = 10.0 * N / N.max()
+    X0 = synth.uniform_queries(more, LO, HI, seed=79)
+    few = sg.solve_bvps(sg.problem_from(params), cuda(X0[:n]), cuda(T[:n]), cuda(N[:n], torch.int32))
+    many = sg.solve_bvps(sg.problem_from(params), cuda(X0), cuda(T), cuda(N, torch.int32))
+    for key in ("lambda0", "u0", "V", "status", "iters"):
+        assert torch.equal(few[key], many[key][:n]), key
