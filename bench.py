@@ -97,6 +97,26 @@ def flops_abd_segback_interval() -> float:
     return 2 * 2 * 144 + 144 + 12
 
 
+def flops_condense_fp64_interval() -> float:
+    """FP64 condensation of one interval: C = (hJ2 - B11)(hJ3 - B22) - B12 B21
+    and its inverse, E C^-1, L J2, two products with J1 and J4, Gauss-Jordan of
+    the 12 x 25 condensed row, and the combinations between them (11 per
+    entry of a 12 x 12 block)."""
+    return 2.0 * (5 * 12 ** 3 + 12 * 12 * 11 + 12 * sum(24 - k for k in range(12)) + 11 * 144)
+
+
+def flops_tree_interval() -> float:
+    """One composition of two scattering relations (13 columns: the product with
+    B1, the 6 x 6 Gauss-Jordan, the products with A2 | C2 and with D1), and the
+    12 x 13 product on the way down."""
+    return 2.0 * (13 * (36 + 60 + 72 + 36) + 12 * 13)
+
+
+def flops_recover_fp64_interval() -> float:
+    """Four 12 x 12 products with the Jacobians, one with C^-1, the combinations."""
+    return 2.0 * (5 * 144 + 12 * 14)
+
+
 def flops_recover_interval() -> float:
     """Per interval: 24 x 24 product and 24 x 24 triangular solve."""
     return 2 * 576 + 576 + 24
@@ -849,14 +869,19 @@ def roofline(kt, iters, N_h, M, prec, nq=N_QUERIES, peaks=None):
         "k_abd_seg" + suffix: ("alu", flops_abd_seg_interval() * seg_units, peak_lin, "TFLOP/s"),
         "k_abd_red" + suffix: ("alu", flops_abd_interval() * red_units, peak_lin, "TFLOP/s"),
         "k_abd_segback" + suffix: ("alu", flops_abd_segback_interval() * seg_units, peak_lin, "TFLOP/s"),
-        "k_recover" + suffix: ("alu", flops_recover_interval() * int_units, peak_lin, "TFLOP/s"),
+        "k_recover" + suffix: ("alu", (flops_recover_interval() if fp32 else flops_recover_fp64_interval()) * int_units,
+                               peak_lin, "TFLOP/s"),
         "k_newton_persistent" + suffix: ("alu", (flops_condense_interval() + flops_abd_interval()
                                                   + flops_recover_interval()) * int_units, peak_lin, "TFLOP/s"),
         "k_point" + suffix: ("hbm", bytes_point(tsize) * pt_units, None, "GB/s"),
+        "k_condense_fp64": ("alu", flops_condense_fp64_interval() * int_units, pk64, "TFLOP/s"),
+        "k_tree_fp64": ("alu", flops_tree_interval() * int_units, pk64, "TFLOP/s"),
         "k_condense_smem_fp64": ("alu", flops_condense_interval() * int_units, pk64, "TFLOP/s"),
         # the interpolant: the method's M (2k + 1) flops per query whatever the
         # arithmetic (pairs of floats and split TF32 do more operations)
-        "k_eval_fp64": ("alu", flops_eval_query(M, 3) * nq, pk64, "TFLOP/s"),
+        # (nested over the dimensions: no products)
+        "k_eval_fp64_nested": ("alu", 2.0 * 3 * M * nq, pk64, "TFLOP/s"),
+        "k_eval_fp64_nodes": ("alu", flops_eval_query(M, 3) * nq, pk64, "TFLOP/s"),
         "k_eval_df32": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),
         "k_eval_tf32x3": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),
         "k_eval_sf_tf32x3": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),

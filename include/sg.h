@@ -433,7 +433,7 @@ int sg_fma_probe(int precision, void* d_scratch, size_t scratch_bytes, int block
                  int iters, double* flops_per_launch, void* stream);
 
 /* Evaluates the library's FP64 sine and cosine (the ones inside the
- * characteristic right-hand side: Taylor polynomials on |x| <= pi/4, the CUDA
+ * characteristic right-hand side: minimax polynomials on |x| <= pi/4, the CUDA
  * library beyond) at n points.  d_x, d_s, d_c: n doubles each on the device
  * (caller-owned).  Used to test those functions against a reference and an
  * error bound.  Asynchronous on `stream`; SG_EINVAL for n < 0 or null
@@ -465,7 +465,7 @@ int sg_theorem1_bound(int d, int q, double* bound);
  *           ntraj x nsteps x 3 held controls
  * The running cost is that of the problem with no target attitude: an
  * attitude problem with d_target set is rejected (SG_EINVAL).
- * One warp per trajectory.  Asynchronous on `stream`.  Errors: SG_EINVAL, SG_ECUDA. */
+ * A block per one, two or four trajectories.  Asynchronous on `stream`.  Errors: SG_EINVAL, SG_ECUDA. */
 int sg_simulate_closed_loop(const sg_problem* prob, const sg_surplus* s, const double* d_x0,
                             int64_t ntraj, int nsteps, double dt, int mode, double* d_xT,
                             double* d_cost, double* d_traj, double* d_ctrl, void* stream);
