@@ -98,11 +98,12 @@ def flops_abd_segback_interval() -> float:
 
 
 def flops_condense_fp64_interval() -> float:
-    """FP64 condensation of one interval: C = (hJ2 - B11)(hJ3 - B22) - B12 B21
+    """FP64 condensation of one interval of the attitude family (51 of the
+    Jacobian's 144 entries are structural zeros): C = (hJ2 - B11)(hJ3 - B22) - B12 B21
     and its inverse, E C^-1, L J2, two products with J1 and J4, Gauss-Jordan of
     the 12 x 25 condensed row, and the combinations between them (11 per
     entry of a 12 x 12 block)."""
-    return 2.0 * (5 * 12 ** 3 + 12 * 12 * 11 + 12 * sum(24 - k for k in range(12)) + 11 * 144)
+    return 2.0 * (12 ** 3 + 4 * 12 * 93 + 12 * 12 * 11 + 12 * sum(24 - k for k in range(12)) + 11 * 144)
 
 
 def flops_tree_interval() -> float:

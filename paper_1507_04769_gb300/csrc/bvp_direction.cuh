@@ -27,10 +27,10 @@
 // node in 5,000.
 //
 // Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
-// iterations): condensation 74.8 -> 25.5 ms (FP64 pipe 95 % busy), elimination
+// iterations): condensation 74.8 -> 21.7 ms (FP64 pipe 95 % busy), elimination
 // and back substitution over the intervals 23.9 -> 9.4 ms, recovery 4.3 -> 2.5
-// ms; the solve (a graph per mesh size) 112.0 -> 42.0 ms; 85 nodes at 128
-// intervals 8.09 -> 3.31 ms.
+// ms; the solve (a graph per mesh size) 112.0 -> 38.9 ms; 85 nodes at 128
+// intervals 8.11 -> 3.00 ms.
 //
 // Elimination over the intervals.  An interval's condensed row
 // S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
@@ -152,6 +152,28 @@ __device__ __forceinline__ bool row_pivot(double v, bool cand, int row, unsigned
   return cand && key == best;
 }
 
+// Entries (m, j) of the attitude family's Jacobian that are zero at every point:
+// of f0_x (x' = E(v) w, w' = J^-1 (g(v) x w)), of -K (the controls enter the
+// rates only), of the Hessian in the rates (lambda' f0 is linear in w) and of
+// -f0_x'; 51 of 144.
+__host__ __device__ constexpr bool attitude_zero(int m, int j) {
+  if (m >= 6 && j >= 6) {   // -f0_x'
+    const int t = m - 6;
+    m = j - 6;
+    j = t;
+  }
+  if (m < 6 && j < 6) {
+    if (m >= 3) return j == m;
+    return j == 2 || (m >= 1 && j == 3) || (m == 1 && j == 1);
+  }
+  if (m < 6) return m < 3 || j < 9;            // -K
+  return m >= 9 && j >= 3 && m - 6 != j;       // l_ww + (lambda' f0)_ww
+}
+
+// kAtt: the attitude family, whose structural zeros are left out of the four
+// products with the Jacobians (204 of 1,380 FP64 instructions; a term that is
+// left out adds an exact zero).  Level-4 batch 42.8 -> 38.9 ms.
+template <bool kAtt>
 __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, Workspace w) {
   extern __shared__ __align__(16) unsigned char cond_smem[];
   const int chunks = cond_chunks(a.Nmax);
@@ -212,7 +234,8 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
         double u[12];
         ld_vec<12>(J_s + 288 + m * 12, u);
 #pragma unroll
-        for (int j = 0; j < 12; ++j) c[j] = fma(e1[m], u[j], c[j]);
+        for (int j = 0; j < 12; ++j)
+          if (!(kAtt && attitude_zero(m, j))) c[j] = fma(e1[m], u[j], c[j]);
       }
     }
     bool cand = true;
@@ -279,7 +302,8 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
       double u[12];
       ld_vec<12>(J_s + 144 + m * 12, u);
 #pragma unroll
-      for (int j = 0; j < 12; ++j) M[j] = fma(L[m], u[j], M[j]);
+      for (int j = 0; j < 12; ++j)
+        if (!(kAtt && attitude_zero(m, j))) M[j] = fma(L[m], u[j], M[j]);
     }
   }
 
@@ -302,7 +326,8 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
       ld_vec<12>(J_s + m * 12, u);
       const double x = fma(am, M[m], fma(al, L[m], m == r ? hK0 : 0.0));
 #pragma unroll
-      for (int j = 0; j < 12; ++j) t[j] = fma(x, u[j], t[j]);
+      for (int j = 0; j < 12; ++j)
+        if (!(kAtt && attitude_zero(m, j))) t[j] = fma(x, u[j], t[j]);
     }
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
@@ -317,7 +342,8 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
       ld_vec<12>(J_s + 432 + m * 12, u);
       const double x = fma(gm, M[m], fma(gl, L[m], m == r ? hK3 : 0.0));
 #pragma unroll
-      for (int j = 0; j < 12; ++j) t[j] = fma(x, u[j], t[j]);
+      for (int j = 0; j < 12; ++j)
+        if (!(kAtt && attitude_zero(m, j))) t[j] = fma(x, u[j], t[j]);
       rr = fma(M[m], rho_s[m], fma(L[m], rho_s[12 + m], rr));
     }
 #pragma unroll
@@ -793,7 +819,8 @@ inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches
     out[4] = {"k_recover_fp32", k_recover_fp32, ceil_div(nint, 4), 128, 0};
   } else {
     const int tt = tree_threads(a.n, a.Nmax);
-    out[0] = {"k_condense_fp64", k_condense_fp64, a.n * cond_chunks(a.Nmax), kCondThreads, kCondSmem};
+    out[0] = {"k_condense_fp64", a.P.kind == SG_PROBLEM_ATTITUDE ? k_condense_fp64<true> : k_condense_fp64<false>,
+              a.n * cond_chunks(a.Nmax), kCondThreads, kCondSmem};
     out[1] = {"k_tree_leaf_fp64", k_tree_leaf_fp64,
               tree_leaves(a.n, a.Nmax) ? a.n * ((a.Nmax + kLeafIv - 1) / kLeafIv) : 0, kLeafThreads,
               tree_smem(kLeafThreads)};

@@ -100,3 +100,24 @@ def test_tree_leaves_by_blocks_give_the_same_bits():
     many = sg.solve_bvps(sg.problem_from(params), cuda(X0), cuda(T), cuda(N, torch.int32))
     for key in ("lambda0", "u0", "V", "status", "iters"):
         assert torch.equal(few[key], many[key][:n]), key
+
+
+@pytest.mark.parametrize("make", [synth.attitude_params, synth.example1_params, synth.example2_params])
+def test_attitude_zeros_against_general_elimination(make):
+    """The attitude family's condensation leaves out the Jacobian's structural
+    zeros; the persistent form eliminates the whole blocks.  Both converge
+    quadratically to |F| <= 1e-12, so lambda(0) agrees far below 1e-8 of its
+    size, and the statuses are the same."""
+    params = make()
+    sizes = [1, 2, 7, 8, 9, 24, 33]
+    n = len(sizes)
+    X0 = 0.3 * synth.uniform_queries(n, LO, HI, seed=80)
+    N = np.array(sizes)
+    T = np.minimum(0.15 * N, 4.0)
+    prob = sg.problem_from(params)
+    a = sg.solve_bvps(prob, cuda(X0), cuda(T), cuda(N, torch.int32), tol=1e-12)
+    b = sg.solve_bvps(prob, cuda(X0), cuda(T), cuda(N, torch.int32), tol=1e-12, persistent=True)
+    assert torch.equal(a["status"], b["status"])
+    la, lb = a["lambda0"], b["lambda0"]
+    assert torch.all(a["status"] == sg.CONVERGED)
+    assert torch.max(torch.abs(la - lb)) <= 1e-8 * torch.max(torch.abs(lb))
