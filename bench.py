@@ -108,9 +108,9 @@ def flops_condense_fp64_interval() -> float:
 
 def flops_tree_interval() -> float:
     """One composition of two scattering relations (13 columns: the product with
-    B1, the 6 x 6 Gauss-Jordan, the products with A2 | C2 and with D1), and the
+    B1, the 6 x 6 elimination, the products with A2 | C2 and with D1), and the
     12 x 13 product on the way down."""
-    return 2.0 * (13 * (36 + 60 + 72 + 36) + 12 * 13)
+    return 2.0 * (13 * (36 + 45 + 72 + 36) + 12 * 13)
 
 
 def flops_recover_fp64_interval() -> float:

@@ -28,9 +28,9 @@
 //
 // Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
 // iterations): condensation 74.8 -> 21.7 ms (FP64 pipe 95 % busy), elimination
-// and back substitution over the intervals 23.9 -> 9.4 ms, recovery 4.3 -> 2.5
-// ms; the solve (a graph per mesh size) 112.0 -> 38.9 ms; 85 nodes at 128
-// intervals 8.11 -> 3.00 ms.
+// and back substitution over the intervals 23.9 -> 8.5 ms, recovery 4.3 -> 2.5
+// ms; the solve (a graph per mesh size) 112.0 -> 38.1 ms; 85 nodes at 128
+// intervals 8.08 -> 2.97 ms.
 //
 // Elimination over the intervals.  An interval's condensed row
 // S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
@@ -407,28 +407,31 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
 // Composition of o1 over [a, m] with o2 over [m, b] by 16 lanes, lane c < 13 a
 // column (dx_a | dlambda_b | 1): km = (dx_m, dlambda_m), nw = the relation over
 // [a, b].  The 6 x 6 matrix I - B_1 C_2 has its columns on lanes 0..5;
-// Gauss-Jordan with partial pivoting, the pivot column passed through `pub`.
-// All 32 lanes of the warp call it.
+// elimination with partial pivoting, the pivot column (above it a column of the
+// unit upper triangle, kept for the back substitution) passed through `pub`.
+// All 32 lanes of the warp call it.  (FP64 instructions are its time: 219, with
+// Gauss-Jordan and the identity and the right-hand side added apart 246.)
 __device__ __forceinline__ void compose(const double* o1, const double* o2, double* pub, int c, double (&km)[12],
                                         double (&nw)[12], bool& bad) {
   double c2[12], c1[12], q[6], b[6];
   ld_vec<12>(o2 + c * 12, c2);   // A2 | B2 | f2 above C2 | D2 | e2
   ld_vec<12>(o1 + c * 12, c1);
+  const bool left = c < 6, one = c == 12;
+  // -I + B1 C2, B1 D2, f1 + B1 e2
 #pragma unroll
-  for (int t = 0; t < 6; ++t) q[t] = 0.0;
+  for (int t = 0; t < 6; ++t) q[t] = one ? c1[t] : (t == c ? -1.0 : 0.0);
 #pragma unroll
   for (int m = 0; m < 6; ++m) {     // B1 times (C2 | D2 | e2)
     const double* col = o1 + (6 + m) * 12;
 #pragma unroll
     for (int t = 0; t < 6; ++t) q[t] = fma(col[t], c2[6 + m], q[t]);
   }
-  const bool left = c < 6, one = c == 12;
 #pragma unroll
   for (int t = 0; t < 6; ++t) {
-    b[t] = left ? c1[t] : (one ? c1[t] + q[t] : q[t]);
+    b[t] = left ? c1[t] : q[t];
     q[t] = -q[t];
-    if (t == c) q[t] += 1.0;
   }
+  double up[6][6];   // up[k][t], t < k: the unit upper triangle
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     double* p_s = pub + (k & 1) * 8;
@@ -472,12 +475,17 @@ __device__ __forceinline__ void compose(const double* o1, const double* o2, doub
     b[k] *= inv;
 #pragma unroll
     for (int t = 0; t < 6; ++t) {
-      if (t != k) {
+      if (t < k) up[k][t] = l[t];
+      if (t > k) {
         q[t] = fma(-l[t], q[k], q[t]);
         b[t] = fma(-l[t], b[k], b[t]);
       }
     }
   }
+#pragma unroll
+  for (int k = 5; k > 0; --k)
+#pragma unroll
+    for (int t = 0; t < k; ++t) b[t] = fma(-up[k][t], b[k], b[t]);
   double y[12];
 #pragma unroll
   for (int t = 0; t < 12; ++t) y[t] = left ? 0.0 : c2[t];
@@ -558,14 +566,15 @@ __device__ __forceinline__ bool tree_up(double* ops, int i0, int i1, int st0, in
 // With fewer than two nodes per SM a block per node leaves SMs idle or unevenly
 // loaded through the tree's lowest levels, which hold most of its work: then a
 // block per kLeafIv intervals runs those first.  (85 nodes at 128 intervals: the
-// tree 0.92 -> 0.76 ms, the solve 3.52 -> 3.31 ms; at 389 nodes of 64 intervals
+// tree 0.92 -> 0.72 ms, the solve 3.52 -> 3.31 ms; five blocks per SM, which
+// the shared memory allows, with a few spills: 0.45 ms against 0.52; at 389 nodes of 64 intervals
 // the solve would go from 1.29 to 1.31 ms, at 486 per graph from 41.9 to 43.3.)
 constexpr int kLeafIv = 16;
 __host__ __device__ __forceinline__ bool tree_leaves(int64_t n, int Nmax) {
   return n < 2 * kNumSMs && Nmax >= 2 * kLeafIv;
 }
 constexpr int kLeafThreads = kLeafIv / 2 * 16;   // a group per pair of intervals
-__global__ void __launch_bounds__(kLeafThreads) k_tree_leaf_fp64(SolveArgs a, Workspace w) {
+__global__ void __launch_bounds__(kLeafThreads, 5) k_tree_leaf_fp64(SolveArgs a, Workspace w) {
   extern __shared__ __align__(16) unsigned char tree_smem_raw[];
   const int chunks = (a.Nmax + kLeafIv - 1) / kLeafIv;
   const int64_t node = blockIdx.x / chunks;
