@@ -114,8 +114,9 @@ def flops_tree_interval() -> float:
 
 
 def flops_recover_fp64_interval() -> float:
-    """Four 12 x 12 products with the Jacobians, one with C^-1, the combinations."""
-    return 2.0 * (5 * 144 + 12 * 14)
+    """12 x 12 products with the Jacobians (one per mesh point, two per interval),
+    one with C^-1, the combinations."""
+    return 2.0 * (4 * 144 + 12 * 14)
 
 
 def flops_recover_interval() -> float:

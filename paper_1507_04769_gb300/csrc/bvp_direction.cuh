@@ -28,9 +28,9 @@
 //
 // Measured on the level-4 batch (1,457 nodes, horizons 10 / 20 / 40, six
 // iterations): condensation 74.8 -> 21.7 ms (FP64 pipe 95 % busy), elimination
-// and back substitution over the intervals 23.9 -> 8.5 ms, recovery 4.3 -> 2.5
-// ms; the solve (a graph per mesh size) 112.0 -> 38.1 ms; 85 nodes at 128
-// intervals 8.08 -> 2.97 ms.
+// and back substitution over the intervals 23.9 -> 8.5 ms, recovery 4.3 -> 1.8
+// ms; the solve (a graph per mesh size) 112.0 -> 37.0 ms; 85 nodes at 128
+// intervals 8.09 -> 2.92 ms.
 //
 // Elimination over the intervals.  An interval's condensed row
 // S dy_i + double dy_{i+1} = r is solved for (dx_{i+1}, dlambda_i) in terms of
@@ -729,12 +729,17 @@ __global__ void __launch_bounds__(32 * kElimWarps) k_elim_fp64(SolveArgs a, Work
 }
 
 // ---------------------------------------------------------------- recovery
-// Interior-stage corrections from the mesh-point corrections: two intervals
-// per warp, 16 lanes each, a lane per row; the Jacobians and C^-1 are staged
-// in shared memory by asynchronous copies, the vectors pass through it.
-constexpr int kRecWarps = 4;
-constexpr int kRecElems = 576 + kCi + 5 * 12;   // per interval: J, C^-1, five vectors
-constexpr int kRecSmem = 2 * kRecWarps * kRecElems * 8;
+// Interior-stage corrections from the mesh-point corrections: eight intervals
+// per block of 96 threads, a thread per row (every lane of the three warps, as
+// in the condensation: the FP64 pipe is its time); the Jacobians and C^-1 are
+// staged in shared memory by asynchronous copies, the vectors pass through it.
+// J dy at a mesh point serves the intervals on both sides.  (Two intervals per
+// warp, 16 lanes each, both products per interval: 2.6 ms of the level-4 batch
+// against 1.8.)
+constexpr int kRecIv = kCondIv;
+// J of the 3 kRecIv + 1 points, C^-1, dy and J dy at the kRecIv + 1 mesh points, three vectors per interval
+constexpr int kRecElems = (3 * kRecIv + 1) * 144 + kRecIv * kCi + 2 * (kRecIv + 1) * 12 + 3 * kRecIv * 12;
+constexpr int kRecSmem = kRecElems * 8;
 
 __device__ __forceinline__ double dot12(const double* row, const double* vec) {
   double x[12], y[12];
@@ -749,57 +754,59 @@ __device__ __forceinline__ double dot12(const double* row, const double* vec) {
   return s + t;
 }
 
-__global__ void __launch_bounds__(32 * kRecWarps) k_recover_fp64(SolveArgs a, Workspace w) {
+__global__ void __launch_bounds__(12 * kRecIv) k_recover_fp64(SolveArgs a, Workspace w) {
   extern __shared__ __align__(16) unsigned char rec_smem[];
-  const int chunks = (a.Nmax + 1) / 2;
-  const int64_t c = blockIdx.x * int64_t(kRecWarps) + (threadIdx.x >> 5);
-  const int64_t node = c / chunks;
-  if (node >= a.n) return;
+  const int chunks = cond_chunks(a.Nmax);
+  const int64_t node = blockIdx.x / chunks;
+  const int i0 = static_cast<int>(blockIdx.x % chunks) * kRecIv;
   if (!w.ns[node].active) return;
   const int N = a.N[node];
-  int i = static_cast<int>(c % chunks) * 2;
-  if (i >= N) return;
-  const int lane16 = threadIdx.x & 15;
-  i += (threadIdx.x >> 4) & 1;
-  const bool valid = i < N;
-  if (!valid) i = N - 1;
-  const bool on = lane16 < 12;
-  const int r = on ? lane16 : 11;
-  double* sm = reinterpret_cast<double*>(rec_smem) + (threadIdx.x >> 4) * kRecElems;
-  double* Ci_s = sm + 576;
-  double* v0 = Ci_s + kCi;          // dy_i, dy_{i+1}, then g2, G, dY3
-  const int64_t wid = node * a.Nmax + i;
-  const double* J = static_cast<const double*>(w.Jm) + (node * npts(a.Nmax) + 3 * int64_t(i)) * 144;
+  if (i0 >= N) return;
+  const int nv = N - i0 < kRecIv ? N - i0 : kRecIv;
+  const int tid = threadIdx.x, slot = tid / 12, r = tid % 12;
+  const bool valid = slot < nv;
+  const int q = valid ? slot : nv - 1;   // slots past the mesh repeat the last one and store nothing
+  double* J_s = reinterpret_cast<double*>(rec_smem);
+  double* Ci_s = J_s + (3 * kRecIv + 1) * 144;
+  double* dy_s = Ci_s + kRecIv * kCi;            // [kRecIv + 1][12]
+  double* u_s = dy_s + (kRecIv + 1) * 12;        // [kRecIv + 1][12] J dy
+  double* g2_s = u_s + (kRecIv + 1) * 12;        // [kRecIv][12] each
+  double* G_s = g2_s + kRecIv * 12;
+  double* x_s = G_s + kRecIv * 12;
+  const int64_t wid = node * a.Nmax + i0;
+  const double* J = static_cast<const double*>(w.Jm) + (node * npts(a.Nmax) + 3 * int64_t(i0)) * 144;
   const double* Ci = dir_ci(w) + wid * kCi;
-  for (int e = lane16; e < (576 + kCi) / 2; e += 16)
-    cp_async16(sm + e * 2, e < 576 / 2 ? J + e * 2 : Ci + (e - 576 / 2) * 2);
+  for (int e = tid; e < (3 * nv + 1) * 72; e += 12 * kRecIv) cp_async16(J_s + e * 2, J + e * 2);
+  for (int e = tid; e < nv * (kCi / 2); e += 12 * kRecIv) cp_async16(Ci_s + e * 2, Ci + e * 2);
   cp_async_commit();
-  double* D = w.D + (node * npts(a.Nmax) + 3 * int64_t(i)) * 12;
-  const double d0 = D[r], d3 = D[36 + r];
-  const double* res = static_cast<const double*>(w.Res) + wid * kResRows;
+  double* D = w.D + (node * npts(a.Nmax) + 3 * int64_t(i0)) * 12;
+  const double d0 = D[36 * q + r];
+  dy_s[q * 12 + r] = d0;
+  if (q == nv - 1) dy_s[nv * 12 + r] = D[36 * nv + r];
+  const double* res = static_cast<const double*>(w.Res) + (wid + q) * kResRows;
   const double r1 = res[r], r2 = res[12 + r];
   const double h = a.T[node] / N;
-  if (on) {
-    v0[r] = d0;
-    v0[12 + r] = d3;
-  }
   cp_async_wait_all();
-  __syncwarp();
-  const double u0 = h * dot12(sm + r * 12, v0), u3 = h * dot12(sm + 432 + r * 12, v0 + 12);
+  __syncthreads();
+  u_s[q * 12 + r] = h * dot12(J_s + 3 * q * 144 + r * 12, dy_s + q * 12);
+  if (q == nv - 1) u_s[nv * 12 + r] = h * dot12(J_s + 3 * nv * 144 + r * 12, dy_s + nv * 12);
+  __syncthreads();
+  const double u0 = u_s[q * 12 + r], u3 = u_s[(q + 1) * 12 + r];
   const double g1 = lob::B11 * r1 + lob::B12 * r2 - lob::S1 * d0 - lob::A1 * u0 - lob::G1 * u3;
   const double g2 = lob::B21 * r1 + lob::B22 * r2 + lob::S1 * d0 - lob::A2 * u0 - lob::G2 * u3;
-  if (on) v0[24 + r] = g2;
-  __syncwarp();
-  const double G = h * dot12(sm + 144 + r * 12, v0 + 24) - lob::B11 * g2 + lob::B21 * g1;
-  if (on) v0[36 + r] = G;
-  __syncwarp();
-  const double x = dot12(Ci_s + r * 12, v0 + 36);   // dY3
-  if (on) v0[48 + r] = x;
-  __syncwarp();
-  const double y = (h * dot12(sm + 288 + r * 12, v0 + 48) - lob::B22 * x - g2) * (1.0 / lob::B21);
-  if (valid && on) {
-    D[12 + r] = y;
-    D[24 + r] = x;
+  g2_s[q * 12 + r] = g2;
+  __syncthreads();
+  const double G = h * dot12(J_s + (3 * q + 1) * 144 + r * 12, g2_s + q * 12) - lob::B11 * g2 + lob::B21 * g1;
+  G_s[q * 12 + r] = G;
+  __syncthreads();
+  const double x = dot12(Ci_s + q * kCi + r * 12, G_s + q * 12);   // dY3
+  x_s[q * 12 + r] = x;
+  __syncthreads();
+  const double y =
+      (h * dot12(J_s + (3 * q + 2) * 144 + r * 12, x_s + q * 12) - lob::B22 * x - g2) * (1.0 / lob::B21);
+  if (valid) {
+    D[36 * q + 12 + r] = y;
+    D[36 * q + 24 + r] = x;
   }
 }
 
@@ -834,8 +841,7 @@ inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches
               tree_leaves(a.n, a.Nmax) ? a.n * ((a.Nmax + kLeafIv - 1) / kLeafIv) : 0, kLeafThreads,
               tree_smem(kLeafThreads)};
     out[2] = {"k_tree_fp64", k_tree_fp64, a.n, tt, tree_smem(tt)};
-    out[3] = {"k_recover_fp64", k_recover_fp64, ceil_div(a.n * ((a.Nmax + 1) / 2), kRecWarps), 32 * kRecWarps,
-              kRecSmem};
+    out[3] = {"k_recover_fp64", k_recover_fp64, a.n * cond_chunks(a.Nmax), 12 * kRecIv, kRecSmem};
   }
 }
 
