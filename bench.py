@@ -883,7 +883,7 @@ def roofline(kt, iters, N_h, M, prec, nq=N_QUERIES, peaks=None):
         # arithmetic (pairs of floats and split TF32 do more operations)
         # (nested over the dimensions: no products)
         "k_eval_fp64_nested": ("alu", 2.0 * 3 * M * nq, pk64, "TFLOP/s"),
-        "k_eval_fp64_nodes": ("alu", flops_eval_query(M, 3) * nq, pk64, "TFLOP/s"),
+        "k_eval_fp64_few": ("alu", 2.0 * 3 * M * nq, pk64, "TFLOP/s"),
         "k_eval_df32": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),
         "k_eval_tf32x3": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),
         "k_eval_sf_tf32x3": ("alu", flops_eval_query(M, 3) * nq, pk32, "TFLOP/s"),

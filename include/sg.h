@@ -399,7 +399,8 @@ void sg_surplus_free(sg_surplus* s);
  *          evaluated by the same polynomial)
  *   mode   SG_EVAL_FP64, or SG_EVAL_TF32X3 (contraction on tensor cores with
  *          split-TF32 operands; error bound stated with the kernel)
- *   d_out  Q x k doubles
+ *   d_out  Q x k doubles; a row depends on its query alone, to the last bit,
+ *          not on Q or on the other queries
  * Asynchronous on `stream`; the handle is read-only, so concurrent calls on
  * different streams are safe once its build is complete (a build is queued
  * on its own stream).  Errors: SG_EINVAL, SG_EUNSUPPORTED, SG_ECUDA. */

@@ -122,6 +122,39 @@ __device__ __forceinline__ void basis_row_t(double u, const double* __restrict__
   }
 }
 
+// basis_row_t in three steps for a row spread over threads, the same operations
+// in the same order: the reciprocals (zero at a hit), the factor of each level's
+// values, the values.
+__device__ __forceinline__ double basis_reciprocal(double u, double x, bool& zero) {
+  const double diff = u - x;
+  zero = diff == 0.0;
+  const double r = recip_newton(diff);
+  return zero ? 0.0 : r;
+}
+// rinv[p * stride], p = 0 .. 2^level, to wi[(l - 2) * stride], l = 2 .. level + 1
+__device__ __forceinline__ void basis_factors(const double* rinv, int stride, int level, double* wi) {
+  const int fine_n = 1 << level;
+  double P = 0.5 * (rinv[0] + rinv[fine_n * stride]);
+  for (int l = 2; l <= level + 1; ++l) {
+    const int n = 1 << (l - 1), sf = fine_n / n;
+    double nw = rinv[sf * stride];
+    for (int m = 3; m < n; m += 2) nw += rinv[m * sf * stride];
+    const double inv = recip_newton(P - nw);
+    P += nw;
+    wi[(l - 2) * stride] = l == 2 ? 0.5 * inv : -inv;
+  }
+}
+// the value of function id >= 1; hit: the point that u coincides with, or -1
+__device__ __forceinline__ double basis_value(const double* rinv, const double* wi, int stride, int level, int id,
+                                              int hit) {
+  const int fine_n = 1 << level;
+  const int l = id <= 2 ? 2 : 33 - __clz(id - 1);                       // id - 1 = 2^(l - 2) + j
+  const int sf = fine_n >> (l - 1);
+  const int p = id <= 2 ? (id - 1) * fine_n : (2 * (id - 1 - (1 << (l - 2))) + 1) * sf;
+  if (hit >= 0 && (hit & (sf - 1)) == 0) return p == hit ? 1.0 : 0.0;
+  return wi[(l - 2) * stride] * rinv[p * stride];
+}
+
 // All 1-D basis values at u to tab[id * stride]: levels 1..5 unrolled, the
 // others by the general form.
 __device__ __forceinline__ void basis_row_fast(double u, int level, const double* __restrict__ xf, double* tab,

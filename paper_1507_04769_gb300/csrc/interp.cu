@@ -117,40 +117,72 @@ __global__ void __launch_bounds__(32 * kSurpWarps)
   }
 }
 
-// Gathers rows of W into the evaluation order and into the nested order.
-__global__ void k_gather_rows(int64_t M, int k, const int32_t* __restrict__ order, const int32_t* __restrict__ nested,
-                              const double* __restrict__ W, double* __restrict__ Ws, double* __restrict__ Wt) {
+// Gathers rows of W into the evaluation order (M) and into the nested order (nrows;
+// rows that stand for no node, nested < 0, are zero).
+__global__ void k_gather_rows(int64_t M, int nrows, int k, const int32_t* __restrict__ order,
+                              const int32_t* __restrict__ nested, const double* __restrict__ W,
+                              double* __restrict__ Ws, double* __restrict__ Wt) {
   const int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (e >= M * k) return;
   const int64_t r = e / k, c = e % k;
-  Ws[e] = W[int64_t(order[r]) * k + c];
-  Wt[e] = W[int64_t(nested[r]) * k + c];
+  if (r < M) Ws[e] = W[int64_t(order[r]) * k + c];
+  if (r < nrows) Wt[e] = nested[r] < 0 ? 0.0 : W[int64_t(nested[r]) * k + c];
 }
 
 // ---------------------------------------------------------------- FP64 evaluation
 // Both kernels are bound by the FP64 pipe, which a warp's instruction holds for
 // 20 cycles whatever its active lanes.
 //
-// Nested form (many queries).  In lexicographic order of the function ids the
-// nodes are the preorder of a tree: a node's parent is the node with its last
-// active dimension set to level 1 (in the grid, which is downward closed), and
+// In lexicographic order of the function ids the nodes are the preorder of a
+// tree: a node's parent is the node with its last active dimension set to
+// level 1 (in the grid, which is downward closed), and
 //   u = value(root),  value(n) = W_n + sum over the children c of phi_c value(c)
 // with phi_c the one 1-D basis value of c's last active dimension.  That is K
 // multiply-adds per node and no products (the sum over nodes of products of
 // their active factors takes A - 1 products more per node: 7.7 FP64 operations
-// per node against 4.4 on the level-4 6-D grid).  A lane per query, 32 queries
-// per block; the block's warps take equal ranges of the preorder (a range
-// starts by entering its first node's ancestors with value 0), so that every
-// warp's control flow is uniform, and their sums are added in order.
-// Measured (K = 3, d = 6) against the per-node form at 128 threads, one query
-// each: 1e6 queries 20.2 -> 8.7 ms on the level-4 grid (the FP64 pipe's time
-// for the multiply-adds and the tables) and 114 -> 26.5 ms on the level-5 grid.
+// per node against 4.4 on the level-4 6-D grid).
+//
+// The order of the sum: the preorder is cut into ranges (four groups of one, two
+// or four, by the grid's size), each is summed by itself, and the ranges' sums
+// are added by groups (range_sum).  Both kernels perform exactly these
+// operations, so a query's result is the same to the last bit whatever the
+// number of queries in the call.
+// A range is a tree of its own: rows of the nested order, first its start (the
+// root's surplus in the range that has the root, else 0), then copies with
+// surplus 0 of its first node's ancestors, then its nodes.
+constexpr int kNestGroups = 4, kNestGroup = kNestRanges / kNestGroups;
+__device__ __forceinline__ double group_sum(const double (&g)[kNestGroups]) {
+  return __dadd_rn(__dadd_rn(g[0], g[1]), __dadd_rn(g[2], g[3]));
+}
+// v(i): the sum of range i; per: ranges of a group
+template <typename V>
+__device__ __forceinline__ double range_sum(V v, int per) {
+  double g[kNestGroups];
+#pragma unroll
+  for (int i = 0; i < kNestGroups; ++i) {
+    g[i] = v(i * per);
+#pragma unroll
+    for (int j = 1; j < kNestGroup; ++j)
+      if (j < per) g[i] = __dadd_rn(g[i], v(i * per + j));
+  }
+  return group_sum(g);
+}
+
+// Grids whose 1-D tables are too large (128 queries' in 200 KB)
+static bool fp64_eval_refused(int d, int nf) { return sizeof(double) * d * nf * kEvalThreads > 200 * 1024; }
+
+// Nested form (many queries).  A lane per query, 32 queries per block, a warp
+// per range or per group of ranges, so that every warp's control flow is
+// uniform.
+// Measured (K = 3, d = 6) against a thread per query over the products: 1e6
+// queries 20.2 -> 8.76 ms on the level-4 grid (the FP64 pipe's time for the
+// multiply-adds and the tables) and 114 -> 26.5 ms on the level-5 grid.
 constexpr int kNestQ = 32;
 
-// prog[m] of a node: table offset of its last active dimension (12 bits), its
-// depth (active dimensions, 4 bits), and for a node without children the
-// number of entries from it on that are such nodes at its depth (16 bits):
-// three quarters of the nodes are taken in runs, by a short loop.
+// prog of a row: table offset of its last active dimension (12 bits), its
+// depth (active dimensions, 4 bits; 0: a range's start or the end of the last),
+// and for a row without children the number of rows from it on that are such
+// rows at its depth (16 bits): three quarters of the nodes are taken in runs, by
+// a short loop.
 __host__ __device__ constexpr uint32_t nested_entry(uint32_t off, uint32_t depth, uint32_t run) {
   return off | depth << 12 | run << 16;
 }
@@ -160,10 +192,10 @@ struct Nested {
   const uint32_t* prog;
   const double* W;         // K columns of the surpluses in nested order, row stride k
   const double* tab;       // this query's table column
-  int k, kc, m1;           // kc: columns that exist (<= K); m1: end of the range
-  // entries base .. base + 31 of the range, staged in shared memory (an
-  // entry steers the walk, so a load from L2 would stand in its path); lp, lw:
-  // the 32 after them, one per lane, on their way
+  int k, kc, mend;         // kc: columns that exist (<= K)
+  // rows base .. base + 31 of the warp's (they end before mend), staged in
+  // shared memory (a row steers the walk, so a load from L2 would stand in
+  // its path); lp, lw: the 32 after them, one per lane, on their way
   uint32_t* sp;            // [32]
   double* sw;              // [32][K]
   int lane, base, pos;
@@ -171,9 +203,9 @@ struct Nested {
   double lw[K];
   __device__ __forceinline__ void load(int m0) {
     const int i = m0 + lane;
-    lp = i < m1 ? prog[i] : 0u;   // depth 0 ends every loop
+    lp = i < mend ? prog[i] : 0u;
 #pragma unroll
-    for (int c = 0; c < K; ++c) lw[c] = i < m1 && c < kc ? W[int64_t(i) * k + c] : 0.0;
+    for (int c = 0; c < K; ++c) lw[c] = i < mend && c < kc ? W[int64_t(i) * k + c] : 0.0;
   }
   __device__ __forceinline__ void refill() {
     __syncwarp();
@@ -188,46 +220,34 @@ struct Nested {
 };
 constexpr int nested_stage_bytes(int K) { return 32 * (8 * K + 4); }   // per warp
 
-// Adds the children (and theirs) at depth D from the current entry on to acc;
-// the first `resume` depths are ancestors of the range's first node (path:
-// their table offsets), entered with value 0.
+// Adds the children (and theirs) at depth D from the current row on to acc.
 template <int K, int D>
-__device__ __forceinline__ void nested_children(Nested<K>& t, int resume, const uint16_t* path, double (&acc)[K]) {
+__device__ __forceinline__ void nested_children(Nested<K>& t, double (&acc)[K]) {
   if constexpr (D <= kMaxDim) {
     while (true) {
-      double v[K];
-      uint32_t off;
-      const bool again = resume >= D;
-      if (again) {
-        off = path[D - 1];
-#pragma unroll
-        for (int c = 0; c < K; ++c) v[c] = 0.0;
-      } else {
-        if (t.pos == 32) t.refill();
-        const uint32_t p = t.sp[t.pos];
-        if (((p >> 12) & 15u) != uint32_t(D)) break;
-        int run = static_cast<int>(p >> 16);
-        if (run != 0) {
-          run = min(run, min(32 - t.pos, t.m1 - t.base - t.pos));
-          const uint32_t* sp = t.sp + t.pos;
-          const double* sw = t.sw + t.pos * K;
-          t.pos += run;
+      if (t.pos == 32) t.refill();
+      const uint32_t p = t.sp[t.pos];
+      if (((p >> 12) & 15u) != uint32_t(D)) break;   // (depth 0 ends every loop)
+      int run = static_cast<int>(p >> 16);
+      if (run != 0) {
+        run = min(run, 32 - t.pos);
+        const uint32_t* sp = t.sp + t.pos;
+        const double* sw = t.sw + t.pos * K;
+        t.pos += run;
 #pragma unroll 2
-          for (; run > 0; --run, ++sp, sw += K) {
-            const double phi = t.tab[(*sp & 0xFFFu) * kNestQ];
+        for (; run > 0; --run, ++sp, sw += K) {
+          const double phi = t.tab[(*sp & 0xFFFu) * kNestQ];
 #pragma unroll
-            for (int c = 0; c < K; ++c) acc[c] = fma(phi, sw[c], acc[c]);
-          }
-          continue;
+          for (int c = 0; c < K; ++c) acc[c] = fma(phi, sw[c], acc[c]);
         }
-        off = p & 0xFFFu;
-#pragma unroll
-        for (int c = 0; c < K; ++c) v[c] = t.sw[t.pos * K + c];
-        ++t.pos;
+        continue;
       }
-      const double phi = t.tab[off * kNestQ];
-      nested_children<K, D + 1>(t, again ? resume : 0, path, v);
-      resume = 0;
+      double v[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) v[c] = t.sw[t.pos * K + c];
+      ++t.pos;
+      const double phi = t.tab[(p & 0xFFFu) * kNestQ];
+      nested_children<K, D + 1>(t, v);
 #pragma unroll
       for (int c = 0; c < K; ++c) acc[c] = fma(phi, v[c], acc[c]);
     }
@@ -235,7 +255,7 @@ __device__ __forceinline__ void nested_children(Nested<K>& t, int resume, const 
 }
 
 template <int K>
-__global__ void __launch_bounds__(512, 1) k_eval_fp64_nested(EvalArgs e, int d, int c0, size_t stage0) {
+__global__ void __launch_bounds__(32 * kNestRanges, 1) k_eval_fp64_nested(EvalArgs e, int d, int c0, size_t stage0) {
   extern __shared__ double tabs_s[];   // [d * nf][kNestQ] (then the warps' sums), the warps' stages
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t q = blockIdx.x * int64_t(kNestQ) + lane;
@@ -251,129 +271,207 @@ __global__ void __launch_bounds__(512, 1) k_eval_fp64_nested(EvalArgs e, int d, 
   t.tab = tabs_s + lane;
   t.k = e.k;
   t.kc = e.k - c0 < K ? e.k - c0 : K;
-  const int m0 = static_cast<int>(e.M * warp / nw);
-  t.m1 = static_cast<int>(e.M * (warp + 1) / nw);
   t.lane = lane;
   t.sw = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(tabs_s) + stage0 + warp * nested_stage_bytes(K));
   t.sp = reinterpret_cast<uint32_t*>(t.sw + 32 * K);
-  double acc[K];
+  const int per = nw == kNestGroups ? e.per : 1;   // ranges of this warp
+  // (a warp's number is its quarter of the SM: the groups, a few per cent
+  // apart, go round the quarters from block to block)
+  const int part = (warp + blockIdx.x) & (nw - 1), r0 = part * per;
+  double total[K];
+  t.mend = e.range[r0 + per] + 1;   // (the next range's start ends the last)
+  t.base = e.range[r0] - 32;
+  t.load(t.base + 32);
+  t.refill();
+#pragma unroll 1
+  for (int j = 0; j < per; ++j) {
+    if (t.pos == 32) t.refill();
+    double acc[K];
 #pragma unroll
-  for (int c = 0; c < K; ++c) acc[c] = 0.0;
-  if (m0 < t.m1) {
-    t.base = m0 - 32;
-    t.load(m0);
-    t.refill();
-    int resume = 0;
-    if (m0 == 0) {   // the root
+    for (int c = 0; c < K; ++c) acc[c] = t.sw[t.pos * K + c];   // the range's start
+    ++t.pos;
+    nested_children<K, 1>(t, acc);
 #pragma unroll
-      for (int c = 0; c < K; ++c) acc[c] = t.sw[c];
-      t.pos = 1;
-    } else {
-      resume = static_cast<int>((t.sp[0] >> 12) & 15u) - 1;
-    }
-    nested_children<K, 1>(t, resume, e.path + int64_t(m0) * kMaxDim, acc);
+    for (int c = 0; c < K; ++c) total[c] = j == 0 ? acc[c] : __dadd_rn(total[c], acc[c]);
   }
   __syncthreads();   // the tables are read; their space takes the sums
   double* sum = tabs_s;
 #pragma unroll
-  for (int c = 0; c < K; ++c) sum[(warp * K + c) * 32 + lane] = acc[c];
+  for (int c = 0; c < K; ++c) sum[(part * K + c) * 32 + lane] = total[c];
   __syncthreads();
-  if (warp == 0 && live) {
+  for (int c = warp; c < t.kc; c += nw) {
+    double u;
+    if (nw == kNestGroups) {
+      double g[kNestGroups];
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-      double v = sum[c * 32 + lane];
-      for (int s = 1; s < nw; ++s) v += sum[(s * K + c) * 32 + lane];
-      if (c < t.kc) e.out[q * e.k + c0 + c] = v;
+      for (int s = 0; s < kNestGroups; ++s) g[s] = sum[(s * K + c) * 32 + lane];
+      u = group_sum(g);
+    } else {
+      u = range_sum([&](int r) { return sum[(r * K + c) * 32 + lane]; }, e.per);
     }
+    if (live) e.out[q * e.k + c0 + c] = u;
   }
 }
 
-// Per-node form (few queries): the lanes of a block are QB queries x node
-// streams, so that a handful of queries fills the FP64 pipe of its SM and a
-// few hundred all SMs.  A node's basis product is that of its active factors
-// (level 1 is the constant 1); nodes come in groups of equal active count.
-constexpr int kNodesThreads = 256;
+// Few queries: the same sums with the nodes over the lanes.  Only rows with
+// children (entries) need work: an entry's value is one chain of
+// multiply-adds over its children, whose values are surpluses (leaves) or
+// entries of smaller height.  Entries go by height, a block barrier between
+// heights; a thread per query, entry and output; within a height the entries
+// are sorted by their number of children, so that a warp's chains are about
+// equally long.  The chains are latency, so the node data is copied to shared
+// memory beside the tables (kStaged, where it fits), and a batch of four
+// children (lists are padded) is loaded while the one before is summed.
+constexpr int kFewBatch = 4, kFewThreads = 512;   // (or 256 threads)
 
-template <int K, int A, int QB>
-__device__ __forceinline__ void nodes_group(const EvalArgs& e, int64_t n0, int64_t n1, int stream,
-                                            const double* __restrict__ tab, int c0, int kc, double (&acc)[K]) {
-  constexpr int NS = kNodesThreads / QB;
-  for (int64_t m = n0 + stream; m < n1; m += NS) {
-    double phi = 1.0;
-    if constexpr (A > 0) {
-      const uint4 ov = *reinterpret_cast<const uint4*>(e.ops + m * kMaxDim);
-      const uint32_t o[4] = {ov.x, ov.y, ov.z, ov.w};
-      phi = tab[(o[0] & 0xFFFFu) * QB];
-#pragma unroll
-      for (int a = 1; a < A; ++a) phi *= tab[((a & 1) ? (o[a >> 1] >> 16) : (o[a >> 1] & 0xFFFFu)) * QB];
-    }
-    const double* w = e.W + m * e.k + c0;
-#pragma unroll
-    for (int c = 0; c < K; ++c)
-      if (c < kc) acc[c] = fma(phi, w[c], acc[c]);
-  }
+constexpr size_t kFewSmem = 200 * 1024;
+struct FewLayout {   // byte offsets in shared memory after the tables
+  size_t val, W, child, ent, total;
+};
+__host__ __device__ inline FewLayout few_layout(const EvalArgs& e, int d, int kc, int QB, bool staged) {
+  auto up = [](size_t x) { return (x + 15) & ~size_t(15); };
+  FewLayout L;
+  L.val = up(sizeof(double) * d * e.nf * QB);
+  // (first the rows' reciprocals, factors, coordinates and hits)
+  const size_t rows = (sizeof(double) * ((size_t(1) << e.level) + 1 + e.level + 1) + sizeof(int)) * d * QB;
+  const size_t vals = sizeof(double) * (e.fheight[kMaxDim + 1] + 1) * kc * QB;
+  L.W = L.val + up(rows > vals ? rows : vals);
+  L.child = L.W + (staged ? up(sizeof(double) * e.nrows * kc) : 0);
+  L.ent = L.child + (staged ? up(sizeof(uint32_t) * e.nchild) : 0);
+  L.total = L.ent + (staged ? sizeof(int4) * e.fheight[kMaxDim + 1] : 0);
+  return L;
 }
 
-template <int K, int QB>
-__global__ void __launch_bounds__(kNodesThreads) k_eval_fp64_nodes(EvalArgs e, int d, int c0) {
-  extern __shared__ double tabs_s[];   // [d * nf][QB], then the partial sums
-  const int tid = threadIdx.x, ql = tid % QB, stream = tid / QB;
+template <int QB, bool kStaged>
+__global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, int d, int c0, int kc) {
+  extern __shared__ __align__(16) double tabs_s[];   // [d * nf][QB], values of the entries [entry][kc][QB], node data
+  char* sm = reinterpret_cast<char*>(tabs_s);
+  const FewLayout at = few_layout(e, d, kc, QB, kStaged);
+  double* val = reinterpret_cast<double*>(sm + at.val);
+  const int tid = threadIdx.x, nt = blockDim.x;
   const int64_t q0 = blockIdx.x * int64_t(QB);
-  for (int task = tid; task < QB * d; task += kNodesThreads) {
+  const int nent = e.fheight[kMaxDim + 1];
+  const double* W = e.Wt + c0;
+  const uint4* child = reinterpret_cast<const uint4*>(e.fchild);
+  const int4* ent = e.fent;
+  int ldw = e.k;
+  if constexpr (kStaged) {
+    auto copy16 = [&](size_t dst, const void* src, int n) {   // n 16-byte words
+      for (int i = tid; i < n; i += nt) {
+        const unsigned to = static_cast<unsigned>(__cvta_generic_to_shared(sm + dst + size_t(i) * 16));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(static_cast<const char*>(src) + size_t(i) * 16));
+      }
+    };
+    copy16(at.child, e.fchild, e.nchild / 4);
+    copy16(at.ent, e.fent, nent);
+    double* Ws = reinterpret_cast<double*>(sm + at.W);
+    if (kc == e.k) {   // (the array is padded to whole words)
+      copy16(at.W, e.Wt, (e.nrows * kc + 1) / 2);
+    } else {
+      for (int i = tid; i < e.nrows * kc; i += nt) Ws[i] = W[int64_t(i / kc) * e.k + i % kc];
+    }
+    W = Ws;
+    ldw = kc;
+    child = reinterpret_cast<const uint4*>(sm + at.child);
+    ent = reinterpret_cast<const int4*>(sm + at.ent);
+  }
+  // tables: row (dim, query) = task, spread over the threads at the levels that
+  // basis_row_fast unrolls (12,000 cycles with a thread per row at level 4, 9,300 now)
+  const int rows = QB * d;
+  const bool spread = e.level >= 1 && e.level <= 5;
+  const int np = (1 << e.level) + 1;
+  double* rinv = val;                     // [np][rows]
+  double* wi = rinv + np * rows;          // [level][rows]
+  double* us = wi + e.level * rows;       // [rows]
+  int* hits = reinterpret_cast<int*>(us + rows);
+  for (int task = tid; task < rows; task += nt) {
     const int tq = task % QB, dim = task / QB;
     const int64_t q = q0 + tq;
     const double u = q < e.Q ? (e.xq[q * d + dim] - e.lo[dim]) / e.width[dim] : 0.5;
-    basis_row_fast(u, e.level, e.xf, tabs_s + (dim * e.nf) * QB + tq, QB);
-  }
-  __syncthreads();
-  const int kc = e.k - c0 < K ? e.k - c0 : K;
-  double acc[K];
-#pragma unroll
-  for (int c = 0; c < K; ++c) acc[c] = 0.0;
-  for (int a = 0; a <= kMaxDim; ++a) {
-    const int64_t n0 = e.grp[a], n1 = e.grp[a + 1];
-    if (n0 >= n1) continue;
-    switch (a) {
-      case 0: nodes_group<K, 0, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 1: nodes_group<K, 1, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 2: nodes_group<K, 2, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 3: nodes_group<K, 3, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 4: nodes_group<K, 4, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 5: nodes_group<K, 5, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 6: nodes_group<K, 6, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      case 7: nodes_group<K, 7, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
-      default: nodes_group<K, 8, QB>(e, n0, n1, stream, tabs_s + ql, c0, kc, acc); break;
+    if (spread) {
+      us[task] = u;
+      hits[task] = -1;
+    } else {
+      basis_row(u, e.level, e.xf, tabs_s + (dim * e.nf) * QB + tq, QB);
     }
   }
-  // streams of a warp by shuffles, then the warps in order
-#pragma unroll
-  for (int c = 0; c < K; ++c)
-#pragma unroll
-    for (int o = 16; o >= QB; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-  __syncthreads();
-  const int lane = tid & 31, warp = tid >> 5;
-  if (lane < QB) {
-#pragma unroll
-    for (int c = 0; c < K; ++c) tabs_s[(warp * QB + lane) * K + c] = acc[c];
+  if (spread) {
+    __syncthreads();
+    for (int i = tid; i < np * rows; i += nt) {
+      const int task = i % rows, pt = i / rows;
+      bool zero;
+      rinv[i] = basis_reciprocal(us[task], e.xf[pt], zero);
+      if (zero) hits[task] = pt;
+    }
+    __syncthreads();
+    for (int task = tid; task < rows; task += nt) basis_factors(rinv + task, rows, e.level, wi + task);
+    __syncthreads();
+    for (int i = tid; i < e.nf * rows; i += nt) {
+      const int task = i % rows, id = i / rows, tq = task % QB, dim = task / QB;
+      tabs_s[(dim * e.nf + id) * QB + tq] =
+          id == 0 ? 1.0 : basis_value(rinv + task, wi + task, rows, e.level, id, hits[task]);
+    }
   }
   __syncthreads();
-  if (tid < QB && q0 + tid < e.Q) {
+  // a list's padding: entry nent with factor 1, v + 1 * -0 = v for every v
+  for (int i = tid; i < kc * QB; i += nt) val[nent * kc * QB + i] = -0.0;
+  if constexpr (kStaged) asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  for (int h = 0; h < kMaxDim + 1; ++h) {
+    const int n = (e.fheight[h + 1] - e.fheight[h]) * kc * QB;
+    if (n == 0) continue;
+    for (int item = tid; item < n; item += nt) {
+      const int t = item / QB, q = item % QB, c = t % kc, en = e.fheight[h] + t / kc;
+      const int4 E = ent[en];
+      double v = W[E.z * ldw + c];
+      const uint4* ch = child + E.x / 4;
+      double p[kFewBatch], w[kFewBatch];
+      uint4 x4 = ch[0];
+      auto load = [&]() {
+        const uint32_t x[kFewBatch] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-      double v = tabs_s[tid * K + c];
-      for (int s = 1; s < kNodesThreads / 32; ++s) v += tabs_s[(s * QB + tid) * K + c];
-      if (c < kc) e.out[(q0 + tid) * e.k + c0 + c] = v;
+        for (int j = 0; j < kFewBatch; ++j) {
+          p[j] = tabs_s[(x[j] & 0xFFFu) * QB + q];
+          w[j] = *((x[j] & 0x1000u) ? val + ((x[j] >> 13) * kc + c) * QB + q : W + (x[j] >> 13) * ldw + c);
+        }
+      };
+      if (E.y > 0) load();
+      x4 = ch[1];   // (past the last list: padding)
+      for (int i = 0; i < E.y; i += kFewBatch) {
+        double p0[kFewBatch], w0[kFewBatch];
+#pragma unroll
+        for (int j = 0; j < kFewBatch; ++j) {
+          p0[j] = p[j];
+          w0[j] = w[j];
+        }
+        if (i + kFewBatch < E.y) {
+          load();
+          x4 = ch[i / 4 + 2];
+        }
+#pragma unroll
+        for (int j = 0; j < kFewBatch; ++j)
+          v = fma(p0[j], w0[j], v);
+      }
+      val[(en * kc + c) * QB + q] = v;
     }
+    __syncthreads();
+  }
+  for (int t = tid; t < QB * kc; t += nt) {
+    const int q = t / kc, c = t % kc;
+    if (q0 + q >= e.Q) break;
+    e.out[(q0 + q) * e.k + c0 + c] =
+        range_sum([&](int r) { return val[(e.froot[r] * kc + c) * QB + q]; }, e.per);
   }
 }
 
 template <int K>
 static int launch_eval_fp64_nested(const EvalArgs& e, int d, int c0, cudaStream_t st) {
   const int64_t blocks = ceil_div(e.Q, kNestQ);
-  // four warps per block fill the SMs (the FP64 pipe needs about four warps in
-  // flight per scheduler); with fewer blocks than that, more warps per block
-  int nw = 4;
-  while (nw < 16 && blocks * nw < int64_t(kNumSMs) * 16) nw *= 2;
+  // A warp per range leaves room for one or two blocks per SM, a warp per group
+  // for four: taken where the last wave of those would be nearly empty (level 4,
+  // 20,000 queries: 224 us against 262; 1e6: 9.2 ms against 8.8).
+  const int64_t waves = ceil_div(blocks, kNumSMs);
+  const int nw = waves <= 2 || (waves < 24 && waves % 4 == 1) ? kNestGroups * e.per : kNestGroups;
   const size_t tab = sizeof(double) * d * e.nf * kNestQ, sum = sizeof(double) * nw * K * 32;
   const size_t stage0 = tab > sum ? tab : sum, smem = stage0 + nw * nested_stage_bytes(K);
   SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64_nested<K>, smem));
@@ -383,35 +481,38 @@ static int launch_eval_fp64_nested(const EvalArgs& e, int d, int c0, cudaStream_
   return SG_OK;
 }
 
-template <int K, int QB>
-static int launch_eval_fp64_nodes(const EvalArgs& e, int d, int c0, cudaStream_t st) {
-  const size_t tab = sizeof(double) * d * e.nf * QB, sum = sizeof(double) * kNodesThreads / 32 * QB * K;
-  const size_t smem = tab > sum ? tab : sum;
-  SG_CUDA_TRY(ensure_dynamic_smem(k_eval_fp64_nodes<K, QB>, smem));
-  SG_TIMED("k_eval_fp64_nodes", st,
-           (k_eval_fp64_nodes<K, QB><<<static_cast<unsigned>(ceil_div(e.Q, QB)), kNodesThreads, smem, st>>>(e, d, c0)));
-  SG_LAUNCH_CHECK("k_eval_fp64_nodes");
+template <int QB>
+static int launch_eval_fp64_few(const EvalArgs& e, int d, int c0, int kc, int nt, cudaStream_t st) {
+  const bool staged = few_layout(e, d, kc, QB, true).total <= kFewSmem;
+  const size_t smem = few_layout(e, d, kc, QB, staged).total;
+  auto* kern = staged ? k_eval_fp64_few<QB, true> : k_eval_fp64_few<QB, false>;
+  SG_CUDA_TRY(ensure_dynamic_smem(kern, smem));
+  SG_TIMED("k_eval_fp64_few", st, (kern<<<static_cast<unsigned>(ceil_div(e.Q, QB)), nt, smem, st>>>(e, d, c0, kc)));
+  SG_LAUNCH_CHECK("k_eval_fp64_few");
   return SG_OK;
 }
 
-// K columns from c0 on.  The nested form needs 0.6 of the per-node form's
-// FP64 operations but comes in blocks of 32 queries, one SM's work at least: it
-// is taken when the queries fill two thirds of the waves of blocks they need
-// (level 4: 5,000 queries 0.124 ms per node; 8,000 queries 0.117 ms nested,
-// which the per-node form would take 0.19 ms for).  Below, the smallest number
-// of queries per block that leaves at most four blocks per SM.
+// K columns from c0 on.  The nested form comes in blocks of 32 queries, one SM's
+// work at least.  Below a wave of them, the fewest queries per block that fill one
+// wave: two blocks of 256 threads or one of 512 per SM.  Measured (K = 3, d = 6,
+// us on the level-4 and level-5 grid): 1 query 13.8 / 22.8,
+// 304: 16.3 / 44, 608: 16.8 / 44, 1,216: 23 / 70, 1,824: 34 / 111, 2,432: 34 / -;
+// nested, up to a wave: 50.7 / 134.
 template <int K>
 static int launch_eval_fp64(const EvalArgs& e, int d, int c0, cudaStream_t st) {
-  const int64_t waves = ceil_div(ceil_div(e.Q, kNestQ), kNumSMs);
-  if (3 * e.Q >= 2 * waves * kNumSMs * kNestQ) return launch_eval_fp64_nested<K>(e, d, c0, st);
-  if (e.Q <= 4 * kNumSMs) return launch_eval_fp64_nodes<K, 1>(e, d, c0, st);
-  if (e.Q <= 16 * kNumSMs) return launch_eval_fp64_nodes<K, 4>(e, d, c0, st);
-  return launch_eval_fp64_nodes<K, 16>(e, d, c0, st);
+  const int kc = e.k - c0 < K ? e.k - c0 : K;
+  if (e.Q <= 2 * kNumSMs) return launch_eval_fp64_few<1>(e, d, c0, kc, 256, st);
+  if (e.Q <= 4 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 512, st);
+  if (e.Q <= 8 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 256, st);
+  if (e.Q <= 16 * kNumSMs && few_layout(e, d, kc, 16, false).total <= kFewSmem)
+    return launch_eval_fp64_few<16>(e, d, c0, kc, 512, st);
+  if (e.Q <= 12 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 512, st);
+  return launch_eval_fp64_nested<K>(e, d, c0, st);
 }
 
 int eval_fp64(const EvalArgs& e, int d, cudaStream_t st) {
   if (d < 1 || d > kMaxDim) return fail(SG_EUNSUPPORTED, "sg_eval_feedback: d must be 1..8");
-  if (sizeof(double) * d * e.nf * kEvalThreads > 200 * 1024)
+  if (fp64_eval_refused(d, e.nf))
     return fail(SG_EUNSUPPORTED, "sg_eval_feedback: grid level too high for the FP64 kernel");
   switch (e.k) {
     case 1: return launch_eval_fp64<1>(e, d, 0, st);
@@ -453,7 +554,9 @@ struct SurplusHost {
   SfPlan sf;                    // scalar fields (its tables are in the staged bytes)
   size_t npack = 0, off = 0, ohost = 0;
   size_t oW = 0, oWs = 0, oWdf = 0, oxf = 0, oxfdf = 0, otab1 = 0, obp = 0, oerr = 0, osfb = 0;
-  size_t oWt = 0, oprog = 0, opath = 0, onested = 0;   // nested order (FP64 evaluation)
+  size_t oWt = 0, oprog = 0, onested = 0;   // nested order (FP64 evaluation)
+  size_t ofent = 0, ofchild = 0;                       // ... and its ranges' inner entries
+  int nrows = 0, per = 0, range[kNestRanges + 1] = {}, fheight[kMaxDim + 2] = {}, froot[kNestRanges] = {}, nchild = 0;
   size_t obox = 0, onact = 0, oops = 0, otcoff = 0, ofid = 0, ofpt = 0, oorder = 0, ometa = 0, obmap = 0;
   std::vector<unsigned char> staging;   // bytes [ohost, off) of the allocation, box zero
   // The same bytes in page-locked memory when it could be had (then
@@ -471,6 +574,105 @@ struct SurplusHost {
     }
   }
 };
+
+// The rows of the nested order (see k_eval_fp64_nested) from its nodes' depths and
+// table offsets.
+struct NestedRows {
+  std::vector<int32_t> node;      // place of the row's node in the nested order, or -1
+  std::vector<uint32_t> prog;     // nested_entry
+  int per;                        // ranges of a group
+  int range[kNestRanges + 1] = {};   // first rows of the ranges; the last row (an end)
+};
+NestedRows nested_rows(const std::vector<uint32_t>& depth, const std::vector<uint16_t>& path) {
+  const int64_t M = static_cast<int64_t>(depth.size());
+  // about equal ranges (within a tenth of one), cut where few ancestors have to
+  // be entered again; a range costs each query about six FP64 operations, so
+  // small grids have fewer
+  NestedRows rows;
+  rows.per = M < 150 ? 1 : (M < 2500 ? 2 : kNestGroup);
+  const int n = rows.per * kNestGroups;
+  const int64_t slack = M / (10 * n);
+  auto begin = [&](int r) {
+    const int64_t at = M * r / n;
+    int64_t best = at;
+    for (int64_t o = 1; r > 0 && r < n && o <= slack; ++o) {
+      if (depth[at - o] < depth[best]) best = at - o;
+      if (depth[at + o] < depth[best]) best = at + o;
+    }
+    return best;
+  };
+  std::vector<uint32_t> dep, off;
+  auto add = [&](int64_t node, uint32_t D, uint32_t o) {
+    rows.node.push_back(static_cast<int32_t>(node));
+    dep.push_back(D);
+    off.push_back(o);
+  };
+  for (int r = 0; r < n; ++r) {
+    const int64_t m0 = begin(r), m1 = begin(r + 1);
+    rows.range[r] = static_cast<int>(dep.size());
+    add(m0 == 0 && m1 > 0 ? 0 : -1, 0, 0);
+    if (m0 < m1)
+      for (uint32_t D = 1; D < depth[m0]; ++D) add(-1, D, path[m0 * kMaxDim + D - 1]);
+    for (int64_t m = std::max<int64_t>(m0, 1); m < m1; ++m) add(m, depth[m], path[m * kMaxDim + depth[m] - 1]);
+  }
+  rows.range[n] = static_cast<int>(dep.size());
+  add(-1, 0, 0);
+  rows.prog.resize(dep.size());
+  uint32_t run = 0;
+  for (size_t i = dep.size(); i-- > 0;) {   // a row's first child, if any, is the row after it
+    const bool leaf = dep[i] > 0 && dep[i + 1] <= dep[i];
+    run = leaf ? (run != 0 && dep[i + 1] == dep[i] && run < 0xFFFFu ? run + 1 : 1) : 0;
+    rows.prog[i] = nested_entry(off[i], dep[i], run);
+  }
+  return rows;
+}
+
+// The rows with children for k_eval_fp64_few (and the starts of empty ranges): by
+// height (fheight[h]: the first of height h + 1), within a height by falling
+// number of children; froot: the ranges' starts.
+void nested_entries(const NestedRows& rows, std::vector<int32_t>& fent, std::vector<uint32_t>& fchild,
+                    int (&fheight)[kMaxDim + 2], int (&froot)[kNestRanges]) {
+  struct Entry {
+    int32_t row;
+    int height;
+    std::vector<uint32_t> kids;   // as fchild
+  };
+  std::vector<Entry> es;
+  int open[kMaxDim + 1] = {};     // the entry at each depth on the current path
+  auto depth = [&](size_t i) { return (rows.prog[i] >> 12) & 15u; };
+  for (size_t i = 0; i + 1 < rows.prog.size(); ++i) {
+    const uint32_t D = depth(i), off = rows.prog[i] & 0xFFFu;
+    const bool entry = D == 0 || depth(i + 1) > D;
+    if (D > 0)
+      es[open[D - 1]].kids.push_back(entry ? off | 0x1000u | uint32_t(es.size()) << 13 : off | uint32_t(i) << 13);
+    if (entry) {
+      open[D] = static_cast<int>(es.size());
+      es.push_back({static_cast<int32_t>(i), 1, {}});
+    }
+  }
+  for (size_t i = es.size(); i-- > 0;)   // (an entry comes before its children)
+    for (uint32_t x : es[i].kids)
+      if (x & 0x1000u) es[i].height = std::max(es[i].height, es[x >> 13].height + 1);
+  std::vector<int32_t> by(es.size()), at(es.size());
+  std::iota(by.begin(), by.end(), 0);
+  std::stable_sort(by.begin(), by.end(), [&](int32_t a, int32_t b) {
+    return es[a].height != es[b].height ? es[a].height < es[b].height : es[a].kids.size() > es[b].kids.size();
+  });
+  for (size_t i = 0; i < by.size(); ++i) at[by[i]] = static_cast<int32_t>(i);
+  for (int h = 0; h < kMaxDim + 2; ++h)
+    fheight[h] = static_cast<int>(std::count_if(es.begin(), es.end(), [&](const Entry& x) { return x.height <= h; }));
+  int r = 0;
+  for (size_t i = 0; i < es.size(); ++i)
+    if (depth(es[i].row) == 0) froot[r++] = at[i];
+  const uint32_t pad = 0x1000u | uint32_t(es.size()) << 13;
+  for (int32_t i : by) {
+    const Entry& x = es[i];
+    fent.insert(fent.end(), {static_cast<int32_t>(fchild.size()), static_cast<int32_t>(x.kids.size()), x.row, 0});
+    for (uint32_t kid : x.kids) fchild.push_back(kid & 0x1000u ? (kid & 0x1FFFu) | uint32_t(at[kid >> 13]) << 13 : kid);
+    fchild.resize((fchild.size() + kFewBatch - 1) / kFewBatch * kFewBatch, pad);   // whole batches
+  }
+  fchild.resize(fchild.size() + 2 * kFewBatch, pad);   // read ahead, not used
+}
 
 std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   auto h = std::make_shared<SurplusHost>();
@@ -542,7 +744,7 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
     return std::lexicographical_compare(&fid[int64_t(a) * d], &fid[int64_t(a) * d] + d, &fid[int64_t(b) * d],
                                         &fid[int64_t(b) * d] + d);
   });
-  std::vector<uint32_t> prog(M, 0), depth(M, 0);
+  std::vector<uint32_t> depth(M, 0);
   std::vector<uint16_t> path(M * kMaxDim, 0);
   for (int64_t r = 0; r < M; ++r) {
     int na = 0;
@@ -552,14 +754,18 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
     }
     depth[r] = na;
   }
-  // a node's first child, if any, is the entry after it
-  uint32_t run = 0;
-  for (int64_t r = M - 1; r >= 0; --r) {
-    const bool leaf = r + 1 == M || depth[r + 1] <= depth[r];
-    const bool joins = r + 1 < M && run != 0 && depth[r + 1] == depth[r] && run < 0xFFFFu;
-    run = leaf ? (joins ? run + 1 : 1) : 0;
-    prog[r] = nested_entry(depth[r] ? path[r * kMaxDim + depth[r] - 1] : 0u, depth[r], run);
-  }
+  const NestedRows rows = nested_rows(depth, path);
+  const size_t nrows = rows.prog.size();
+  h->nrows = static_cast<int>(nrows);
+  h->per = rows.per;
+  std::copy(std::begin(rows.range), std::end(rows.range), h->range);
+  std::vector<int32_t> row_node(nrows, -1);
+  for (size_t i = 0; i < nrows; ++i)
+    if (rows.node[i] >= 0) row_node[i] = nested[rows.node[i]];
+  // the rows with children, and those (few queries)
+  std::vector<int32_t> fent;      // per entry: first child, children, row, unused
+  std::vector<uint32_t> fchild;   // per child: table offset (12 bits), whether an entry (1), entry or row
+  if (!fp64_eval_refused(d, h->nf)) nested_entries(rows, fent, fchild, h->fheight, h->froot);
 
   // one device allocation: the surplus's arrays and the build's tables; the
   // device-computed ones first, then the host-made ones (one copy)
@@ -571,7 +777,7 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   };
   h->oW = take(M * k * sizeof(double));
   h->oWs = take(M * k * sizeof(double));
-  h->oWt = take(M * k * sizeof(double));
+  h->oWt = take(nrows * k * sizeof(double));
   h->oWdf = take(M * k * sizeof(float2));
   h->oxf = take((fine_n + 1) * sizeof(double));
   h->oxfdf = take((fine_n + 1) * sizeof(float2));
@@ -594,9 +800,11 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   h->ofid = take(M * d * sizeof(uint16_t));
   h->ofpt = take(M * d * sizeof(int16_t));
   h->oorder = take(M * sizeof(int32_t));
-  h->onested = take(M * sizeof(int32_t));
-  h->oprog = take(M * sizeof(uint32_t));
-  h->opath = take(M * kMaxDim * sizeof(uint16_t));
+  h->onested = take(nrows * sizeof(int32_t));
+  h->oprog = take(nrows * sizeof(uint32_t));
+  h->ofent = take(fent.size() * sizeof(int32_t));
+  h->nchild = static_cast<int>(fchild.size());
+  h->ofchild = take(fchild.size() * sizeof(uint32_t));
   h->ometa = take(h->sf_ok ? h->sf.meta.size() : 0);
   h->obmap = take(h->sf_ok ? h->sf.bmap.size() * sizeof(int32_t) : 0);
   h->off = off;
@@ -613,9 +821,12 @@ std::shared_ptr<const SurplusHost> make_surplus_host(const sg_grid* g, int k) {
   std::memcpy(st.data() + (h->ofid - oh), fid.data(), M * d * sizeof(uint16_t));
   std::memcpy(st.data() + (h->ofpt - oh), fpt.data(), M * d * sizeof(int16_t));
   std::memcpy(st.data() + (h->oorder - oh), order.data(), M * sizeof(int32_t));
-  std::memcpy(st.data() + (h->onested - oh), nested.data(), M * sizeof(int32_t));
-  std::memcpy(st.data() + (h->oprog - oh), prog.data(), M * sizeof(uint32_t));
-  std::memcpy(st.data() + (h->opath - oh), path.data(), M * kMaxDim * sizeof(uint16_t));
+  std::memcpy(st.data() + (h->onested - oh), row_node.data(), nrows * sizeof(int32_t));
+  std::memcpy(st.data() + (h->oprog - oh), rows.prog.data(), nrows * sizeof(uint32_t));
+  if (!fent.empty()) {
+    std::memcpy(st.data() + (h->ofent - oh), fent.data(), fent.size() * sizeof(int32_t));
+    if (!fchild.empty()) std::memcpy(st.data() + (h->ofchild - oh), fchild.data(), fchild.size() * sizeof(uint32_t));
+  }
   if (h->sf_ok) {
     std::memcpy(st.data() + (h->ometa - oh), h->sf.meta.data(), h->sf.meta.size());
     std::memcpy(st.data() + (h->obmap - oh), h->sf.bmap.data(), h->sf.bmap.size() * sizeof(int32_t));
@@ -692,7 +903,14 @@ extern "C" int sg_build_surpluses(const sg_grid* g, const double* d_values, int 
   s->Ws = reinterpret_cast<double*>(base + h.oWs);
   s->Wt = reinterpret_cast<double*>(base + h.oWt);
   s->prog = reinterpret_cast<uint32_t*>(base + h.oprog);
-  s->path = reinterpret_cast<uint16_t*>(base + h.opath);
+  s->nrows = h.nrows;
+  s->per = h.per;
+  s->fent = reinterpret_cast<int4*>(base + h.ofent);
+  s->fchild = reinterpret_cast<uint32_t*>(base + h.ofchild);
+  s->nchild = h.nchild;
+  std::copy(std::begin(h.range), std::end(h.range), s->range);
+  std::copy(std::begin(h.fheight), std::end(h.fheight), s->fheight);
+  std::copy(std::begin(h.froot), std::end(h.froot), s->froot);
   s->Wdf = reinterpret_cast<float2*>(base + h.oWdf);
   s->xf = reinterpret_cast<double*>(base + h.oxf);
   s->xfdf = reinterpret_cast<float2*>(base + h.oxfdf);
@@ -758,7 +976,7 @@ extern "C" int sg_build_surpluses(const sg_grid* g, const double* d_values, int 
                  n0, n1, d, k, fine_n, d_fid, d_fpt, d_tab1, d_values, s->W)));
     SG_TRY_CLEAN(cudaGetLastError());
   }
-  SG_TIMED("k_gather_rows", st, (k_gather_rows<<<static_cast<unsigned>(ceil_div(M * k, 256)), 256, 0, st>>>(M, k, d_order, d_nested, s->W, s->Ws, s->Wt)));
+  SG_TIMED("k_gather_rows", st, (k_gather_rows<<<static_cast<unsigned>(ceil_div(std::max<int64_t>(M, h.nrows) * k, 256)), 256, 0, st>>>(M, h.nrows, k, d_order, d_nested, s->W, s->Ws, s->Wt)));
   SG_TRY_CLEAN(cudaGetLastError());
   if (split_df(fine_n + 1, s->xf, s->xfdf, st) != SG_OK || split_df(M * k, s->Ws, s->Wdf, st) != SG_OK)
     return cleanup(cudaGetLastError(), "split_df");
@@ -806,7 +1024,14 @@ extern "C" int sg_eval_feedback(const sg_surplus* s, const double* d_xq, int64_t
   e.W = s->Ws;
   e.Wt = s->Wt;
   e.prog = s->prog;
-  e.path = s->path;
+  e.nrows = s->nrows;
+  e.per = s->per;
+  e.fent = s->fent;
+  e.fchild = s->fchild;
+  e.nchild = s->nchild;
+  std::copy(std::begin(s->range), std::end(s->range), e.range);
+  std::copy(std::begin(s->fheight), std::end(s->fheight), e.fheight);
+  std::copy(std::begin(s->froot), std::end(s->froot), e.froot);
   e.lo = s->box;
   e.width = s->box + s->d;
   e.xf = s->xf;

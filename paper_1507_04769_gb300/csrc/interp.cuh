@@ -10,6 +10,7 @@ constexpr int kMaxLevel = 8;                 // finest 1-D set has 2^8 + 1 point
 constexpr int kMaxFine = 1 << kMaxLevel;
 constexpr int kMaxOut = 16;
 constexpr int kEvalThreads = 128;
+constexpr int kNestRanges = 16;              // most ranges of the FP64 evaluation's sum
 
 struct EvalArgs {
   const double* xq;
@@ -22,9 +23,16 @@ struct EvalArgs {
   const uint8_t* nact;    // M: number of active (level >= 2) dimensions
   const uint16_t* ops;    // M x kMaxDim: table offsets dim * nf + id of the active dimensions
   const double* W;        // M x k, evaluation order
-  const double* Wt;       // M x k, nested order
-  const uint32_t* prog;   // M, nested order: nested_entry of each node
-  const uint16_t* path;   // M x kMaxDim, nested order: table offsets of the active dimensions
+  const double* Wt;       // nrows x k, nested order (rows: see k_eval_fp64_nested)
+  const uint32_t* prog;   // nrows: nested_entry of each row
+  int nrows;
+  int per;                // ranges in each of its four groups
+  int range[kNestRanges + 1];   // first rows of the ranges, which are summed by themselves; the last row
+  const int4* fent;       // rows with children (entries): first child, children, row
+  const uint32_t* fchild; // their children: table offset (12 bits), whether an entry (1), entry or row
+  int nchild;                 // length of fchild (multiple of 4)
+  int fheight[kMaxDim + 2];   // entries of height h + 1 begin at fheight[h]
+  int froot[kNestRanges];     // entries that take the ranges' sums
   const double* lo;       // d
   const double* width;    // d: hi - lo (divided, so that nodes map exactly)
   const double* xf;       // 2^L + 1 points of the finest 1-D set
@@ -68,9 +76,15 @@ struct sg_surplus {
   int64_t M = 0;
   double* W = nullptr;            // M x k, grid order
   double* Ws = nullptr;           // M x k, evaluation order
-  double* Wt = nullptr;           // M x k, nested order (function ids lexicographically)
-  uint32_t* prog = nullptr;       // M, nested order: nested_entry of each node
-  uint16_t* path = nullptr;       // M x kMaxDim, nested order
+  double* Wt = nullptr;           // nested order (function ids lexicographically), as in EvalArgs
+  uint32_t* prog = nullptr;
+  int nrows = 0, per = 0;
+  int range[sg::kNestRanges + 1] = {};   // as in EvalArgs
+  int4* fent = nullptr;
+  uint32_t* fchild = nullptr;
+  int nchild = 0;
+  int fheight[sg::kMaxDim + 2] = {};
+  int froot[sg::kNestRanges] = {};
   uint8_t* nact = nullptr;        // M, evaluation order (sorted by this count)
   int64_t grp[sg::kMaxDim + 2] = {};  // first node with >= a active dimensions
   uint16_t* ops = nullptr;        // M x kMaxDim
