@@ -71,6 +71,17 @@ __device__ __forceinline__ double recip_newton(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// Whether the forms built on recip_newton hold at u: they need differences and
+// reciprocals in the normal range, and denominators away from zero (far outside
+// the box they are rounding noise, and an exact 0 would give NaN).  Elsewhere,
+// and for NaN, basis_row.  On the integer pipe: u in (-1/4, 5/4), and 0 or at
+// least 2^-1000 in size.
+__device__ __forceinline__ bool basis_in_range(double u) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(u)), a = hi & 0x7FFFFFFFu;
+  const bool inside = a < ((hi >> 31) ? 0x3FD00000u : 0x3FF40000u);
+  return inside && (a >= 0x01700000u || (a | static_cast<unsigned>(__double2loint(u))) == 0u);
+}
+
 // The FP64 basis for a level fixed at compile time (every loop unrolls, the
 // reciprocals stay in registers).  The denominators of the nested sets follow
 // from one another: the points of X^l are the even points of X^{l+1}, so with P
@@ -155,18 +166,19 @@ __device__ __forceinline__ double basis_value(const double* rinv, const double* 
   return wi[(l - 2) * stride] * rinv[p * stride];
 }
 
-// All 1-D basis values at u to tab[id * stride]: levels 1..5 unrolled, the
-// others by the general form.
+// All 1-D basis values at u to tab[id * stride]: levels 1..5 in range unrolled,
+// the others by the general form.
 __device__ __forceinline__ void basis_row_fast(double u, int level, const double* __restrict__ xf, double* tab,
                                                int stride) {
   auto out = [&](int id, double v) { tab[id * stride] = v; };
+  if (!basis_in_range(u)) level = -level;
   switch (level) {
     case 1: return basis_row_t<1>(u, xf, out);
     case 2: return basis_row_t<2>(u, xf, out);
     case 3: return basis_row_t<3>(u, xf, out);
     case 4: return basis_row_t<4>(u, xf, out);
     case 5: return basis_row_t<5>(u, xf, out);
-    default: return basis_row(u, level, xf, tab, stride);
+    default: return basis_row(u, abs(level), xf, tab, stride);
   }
 }
 

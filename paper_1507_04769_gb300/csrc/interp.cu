@@ -388,10 +388,10 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, in
     const int tq = task % QB, dim = task / QB;
     const int64_t q = q0 + tq;
     const double u = q < e.Q ? (e.xq[q * d + dim] - e.lo[dim]) / e.width[dim] : 0.5;
-    if (spread) {
-      us[task] = u;
-      hits[task] = -1;
-    } else {
+    us[task] = u;
+    hits[task] = -1;
+    if (!spread || !basis_in_range(u)) {
+      hits[task] = -2;   // done
       basis_row(u, e.level, e.xf, tabs_s + (dim * e.nf) * QB + tq, QB);
     }
   }
@@ -401,13 +401,14 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, in
       const int task = i % rows, pt = i / rows;
       bool zero;
       rinv[i] = basis_reciprocal(us[task], e.xf[pt], zero);
-      if (zero) hits[task] = pt;
+      if (zero && hits[task] != -2) hits[task] = pt;
     }
     __syncthreads();
     for (int task = tid; task < rows; task += nt) basis_factors(rinv + task, rows, e.level, wi + task);
     __syncthreads();
     for (int i = tid; i < e.nf * rows; i += nt) {
       const int task = i % rows, id = i / rows, tq = task % QB, dim = task / QB;
+      if (hits[task] == -2) continue;
       tabs_s[(dim * e.nf + id) * QB + tq] =
           id == 0 ? 1.0 : basis_value(rinv + task, wi + task, rows, e.level, id, hits[task]);
     }
