@@ -207,15 +207,15 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
   SG_CUDA_TRY(direction_setup<T>(a));
   DirLaunch dir[kDirLaunches<T>];
   direction_launches<T>(a, dir);
-  int h_cnt[2] = {0, 0};   // nodes still in the line search, nodes left to iterate
+  int h_cnt[3] = {0, 0, 0};   // nodes still in the line search, nodes left to iterate, eliminations next
   auto read_counters = [&]() -> int {
-    cudaError_t e = cudaMemcpyAsync(h_cnt, w.counters + kSearchOut, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(h_cnt, w.counters + kSearchOut, 3 * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, "counter copy");
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "solver kernels");
     return SG_OK;
   };
-  static_assert(kActiveOut == kSearchOut + 1, "read together");
+  static_assert(kActiveOut == kSearchOut + 1 && kElimOut == kSearchOut + 2, "read together");
   int rc;
   SG_CUDA_TRY(cudaMemsetAsync(w.counters, 0, kCounters * sizeof(int), st));
   SG_TIMED("k_init", st, (k_init<<<ginit, 128, 0, st>>>(a, w)));
@@ -228,10 +228,14 @@ static int run_solve(const SolveArgs& a, Workspace w, cudaStream_t st, double* l
     for (const DirLaunch& d : dir)
       if (d.grid > 0) SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
     SG_LAUNCH_CHECK("newton kernels");
-    for (int trial = 0; trial < 13; ++trial) {   // alpha = 1, 1/2, ..., 2^-10 (and one at 0 in the FP64 form)
+    for (int trial = 0; trial < 13; ++trial) {   // alpha = 1, 1/2, ..., 2^-10 (after 1 and 0 in the FP64 form)
       if constexpr (sizeof(T) == sizeof(double)) {
-        const DirLaunch d = elim_launch(a);
-        SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
+        if (trial > 0 && h_cnt[2] > 0) {
+          DirLaunch elim[kElimLaunches];
+          elim_launches(a, elim);
+          for (const DirLaunch& d : elim)
+            SG_TIMED(d.name, st, (d.fn<<<static_cast<unsigned>(d.grid), d.block, d.smem, st>>>(a, w)));
+        }
       }
       SG_TIMED("k_trial", st, (trial_kernel<T>(a)<<<gi, 128, 0, st>>>(a, w)));
       SG_TIMED("k_ls_reduce", st, (k_ls_reduce<<<gnode_warp, 128, 0, st>>>(a, w, 1)));
@@ -288,13 +292,13 @@ struct GraphBuilder {
     err = cudaGraphAddMemsetNode(&n, g, last.data(), last.size(), &p);
     last.assign(1, n);
   }
-  // Adds a WHILE node; returns its body graph (empty) through *body.
-  void loop(cudaGraphConditionalHandle h, cudaGraph_t* body) {
+  // Adds a WHILE (or IF) node; returns its body graph (empty) through *body.
+  void loop(cudaGraphConditionalHandle h, cudaGraph_t* body, cudaGraphConditionalNodeType type = cudaGraphCondTypeWhile) {
     if (err != cudaSuccess) return;
     cudaGraphNodeParams p{};
     p.type = cudaGraphNodeTypeConditional;
     p.conditional.handle = h;
-    p.conditional.type = cudaGraphCondTypeWhile;
+    p.conditional.type = type;
     p.conditional.size = 1;
     cudaGraphNode_t n;
     err = cudaGraphAddNode(&n, g, last.data(), nullptr, last.size(), &p);
@@ -304,20 +308,16 @@ struct GraphBuilder {
   }
 };
 
-// One trial of the line search: the elimination of marked nodes (FP64 form), the
-// residual at the trial point, the decision.
+// One trial of the line search: the residual at the trial point, the decision.
 template <typename T>
 static void add_trial(GraphBuilder& b, const SolveArgs& a, const Workspace& w) {
-  if constexpr (sizeof(T) == sizeof(double)) {
-    const DirLaunch d = elim_launch(a);
-    b.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
-  }
   b.kernel(trial_kernel<T>(a), static_cast<unsigned>(a.n * trial_chunks(a.Nmax)), 128, 0, a, w);
   b.kernel(k_ls_reduce, static_cast<unsigned>(ceil_div(a.n, 4)), 128, 0, a, w, 1);
 }
 
 // One Newton iteration; the first trial is in line (it is the only one for
-// nearly every node), further ones are a WHILE loop on a.h_search.
+// nearly every node), further ones are a WHILE loop on a.h_search (FP64 form:
+// after the eliminations that the last decision asked for, an IF on a.h_elim).
 template <typename T>
 static void add_iteration(GraphBuilder& b, const SolveArgs& a, const Workspace& w) {
   const int64_t np = a.n * npts(a.Nmax);
@@ -333,6 +333,17 @@ static void add_iteration(GraphBuilder& b, const SolveArgs& a, const Workspace& 
   b.loop(a.h_search, &body);
   if (b.err == cudaSuccess) {
     GraphBuilder lb{body, {}};
+    if constexpr (sizeof(T) == sizeof(double)) {
+      cudaGraph_t elim_body = nullptr;
+      lb.loop(a.h_elim, &elim_body, cudaGraphCondTypeIf);
+      if (lb.err == cudaSuccess) {
+        GraphBuilder eb{elim_body, {}};
+        DirLaunch elim[kElimLaunches];
+        elim_launches(a, elim);
+        for (const DirLaunch& d : elim) eb.kernel(d.fn, static_cast<unsigned>(d.grid), d.block, d.smem, a, w);
+        lb.err = eb.err;
+      }
+    }
     add_trial<T>(lb, a, w);
     b.err = lb.err;
   }
@@ -351,6 +362,10 @@ static cudaError_t build_solve_graph(SolveArgs a, const Workspace& w, double* la
   if ((e = cudaGraphConditionalHandleCreate(&a.h_newton, root, 0, 0)) != cudaSuccess) return e;
   if ((e = cudaGraphConditionalHandleCreate(&a.h_search, root, 0, 0)) != cudaSuccess) return e;
   a.conds = 3;
+  if (a.tree) {
+    if ((e = cudaGraphConditionalHandleCreate(&a.h_elim, root, 0, 0)) != cudaSuccess) return e;
+    a.conds |= 4;
+  }
   GraphBuilder rb{root, {}};
   rb.memset0(w.counters, kCounters * sizeof(int));
   rb.kernel(k_init, static_cast<unsigned>(ceil_div(np * kInitPer, 128)), 128, 0, a, w);
@@ -947,6 +962,10 @@ static cudaError_t build_pool_graph(SolveArgs a, const Workspace& w, uint8_t* fl
   if (e != cudaSuccess) return e;
   if ((e = cudaGraphConditionalHandleCreate(&a.h_search, root, 0, 0)) != cudaSuccess) return e;
   a.conds = 2;
+  if (a.tree) {
+    if ((e = cudaGraphConditionalHandleCreate(&a.h_elim, root, 0, 0)) != cudaSuccess) return e;
+    a.conds |= 4;
+  }
   GraphBuilder rb{root, {}};
   rb.memset0(w.counters, kEpoch * sizeof(int));
   // new slots only (searching at alpha = 0)

@@ -43,11 +43,11 @@
 // the tree is walked down for the mesh-point corrections.
 //
 // A node with a pivot too small for the arithmetic, and a node whose full step
-// is rejected by the line search, take the direction of the elimination with
-// full partial pivoting instead (k_elim_fp64, the FP32 forms' algorithm in
-// FP64).  The first has no scattering form; the second is far from its root,
-// where the path of damped Newton depends on the last bits of the direction
-// and whether it arrives is found out by following it.
+// does not pass the Armijo test (ls_node), take the direction of the elimination
+// with full partial pivoting instead (the FP32 forms' algorithm in FP64).  The first
+// has no scattering form; the second is far from its root, where the path of
+// Newton's iteration depends on the last bits of the direction and whether it
+// arrives is found out by following it.
 #pragma once
 
 #include "bvp_kernels.cuh"
@@ -87,20 +87,28 @@ static_assert(kCi + kOp <= kSegBlk, "the direction's arrays fit the region");
 
 // 1/p for the pivots of the direction: Newton's iteration (one cubic step)
 // from the approximate reciprocal instruction, which is good to about 20
-// bits.  `good` is false for a pivot too small for the arithmetic (the rows
-// are of order one) or not finite; the result is then 0.
+// bits.  `good` is false for a small pivot or one that is not finite (the result
+// is then 0).  The rows are of order one, and so are the pivots unless an
+// interval or a composition is close to having no scattering form; the
+// direction's error grows with the square of a pivot's reciprocal, to 1e-10 at
+// the line drawn here.
 __device__ __forceinline__ double dir_recip(double p, bool& good) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
   const double e = fma(-p, r, 1.0);
   r = fma(r, fma(e, e, e), r);
   const unsigned hi = static_cast<unsigned>(__double_as_longlong(p) >> 32) & 0x7FFFFFFFu;
-  good = hi >= 0x3E300000u && hi < 0x7E300000u;   // 2^-28 .. 2^996
+  good = hi >= 0x3F500000u && hi < 0x7E300000u;   // 2^-10 .. 2^996
   return good ? r : 0.0;
 }
 
 __device__ __forceinline__ void mark_elim(const Workspace& w, int64_t node) {
-  if (!(atomicOr(&w.ns[node].singular, kElimNode) & kElimNode)) atomicAdd(&w.counters[kElimCount], 1);
+  atomicOr(&w.ns[node].singular, kElimNode);
+}
+// Whether the tree forms the node's direction.  (kElimFirst, unlike kElimNode,
+// does not change while these kernels run: the answer is the block's.)
+__device__ __forceinline__ bool tree_node(const Workspace& w, int64_t node) {
+  return w.ns[node].active && !(w.ns[node].singular & kElimFirst);
 }
 
 // n contiguous entries (16-byte vectors) from or to shared or global memory
@@ -179,7 +187,7 @@ __global__ void __launch_bounds__(kCondThreads, 4) k_condense_fp64(SolveArgs a, 
   const int chunks = cond_chunks(a.Nmax);
   const int64_t node = blockIdx.x / chunks;
   int i = static_cast<int>(blockIdx.x % chunks) * kCondIv;
-  if (!w.ns[node].active) return;
+  if (!tree_node(w, node)) return;
   const int N = a.N[node];
   if (i >= N) return;
   const int slot = threadIdx.x / 12, r = threadIdx.x % 12;
@@ -579,7 +587,7 @@ __global__ void __launch_bounds__(kLeafThreads, 5) k_tree_leaf_fp64(SolveArgs a,
   const int chunks = (a.Nmax + kLeafIv - 1) / kLeafIv;
   const int64_t node = blockIdx.x / chunks;
   const int i0 = static_cast<int>(blockIdx.x % chunks) * kLeafIv;
-  if (!w.ns[node].active) return;
+  if (!tree_node(w, node)) return;
   const int N = a.N[node];
   if (i0 >= N) return;
   const int tid = threadIdx.x, lane16 = tid & 15, g = tid >> 4;
@@ -587,6 +595,17 @@ __global__ void __launch_bounds__(kLeafThreads, 5) k_tree_leaf_fp64(SolveArgs a,
   const bool bad = tree_up(dir_op(a, w) + node * a.Nmax * int64_t(kOp), i0, i0 + kLeafIv < N ? i0 + kLeafIv : N, 1,
                            kLeafIv, buf, buf + 4 * kOp, lane16 < 13 ? lane16 : 12, lane16, g, kLeafThreads / 16);
   if (__syncthreads_or(bad) && tid == 0) mark_elim(w, node);
+}
+
+// The node's line search starts: at the full step, or (marked here or before)
+// after the first trial of the others with its elimination.
+__device__ __forceinline__ void tree_ls_start(const Workspace& w, int64_t node, bool bad) {
+  NodeState s = w.ns[node];
+  if (!s.active) return;
+  if (bad) s.singular |= kElimNode;
+  s.searching = s.singular & (kElimNode | kElimFirst) ? 2 : 1;
+  s.alpha = 1.0;
+  w.ns[node] = s;
 }
 
 // Block per node.  Relations are composed in place: the result over [a, b)
@@ -597,7 +616,10 @@ __global__ void __launch_bounds__(kLeafThreads, 5) k_tree_leaf_fp64(SolveArgs a,
 __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, Workspace w) {
   extern __shared__ __align__(16) unsigned char tree_smem_raw[];
   const int64_t node = blockIdx.x;
-  if (!w.ns[node].active) return;
+  if (!tree_node(w, node)) {
+    if (threadIdx.x == 0) tree_ls_start(w, node, false);
+    return;
+  }
   const int N = a.N[node];
   const int tid = threadIdx.x, lane16 = tid & 15, g = tid >> 4, ng = blockDim.x >> 4;
   const int c = lane16 < 13 ? lane16 : 12;
@@ -650,11 +672,8 @@ __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, W
     }
   }
   bad = __syncthreads_or(bad);
-  if (tid == 0) {
-    if (bad) mark_elim(w, node);
-    ls_start(w, node);
-  }
-  if (bad) return;   // k_elim_fp64 solves it
+  if (tid == 0) tree_ls_start(w, node, bad);
+  if (bad) return;   // the elimination solves it
 
   // down the tree: the corrections at the middle of [i, e) from those at its ends
   int top = 1;
@@ -679,52 +698,87 @@ __global__ void __launch_bounds__(kTreeMaxThreads, 1) k_tree_fp64(SolveArgs a, W
   }
 }
 
-// ---------------------------------------------------------------- marked nodes
-// Block per marked node: condensation by elimination of the 24 interior
-// columns, segmented staircase, back substitution and recovery, each phase
-// over the block's warps.  A small grid, with nothing to do unless a node was
-// marked.  (The relations and inverses in the segments' region are no longer
-// read when it runs.)
-constexpr int kElimBlocks = 2 * kNumSMs, kElimWarps = 4;
-constexpr int kElimWarpSmem = 36 * kCols * 8;   // the condensation's system; the segments' tables are smaller
-static_assert(seg_smem_elems<double>() * 8 <= kElimWarpSmem && stair_smem_elems<double>() * 8 <= kElimWarpSmem &&
-                  kSegBackStages<double> * 12 * kSegLd * 8 <= kElimWarpSmem,
-              "tables fit");
-__global__ void __launch_bounds__(32 * kElimWarps) k_elim_fp64(SolveArgs a, Workspace w) {
-  if (w.counters[kElimCount] == 0) return;
+// ---------------------------------------------------------------- elimination
+// Condensation by elimination of the 24 interior columns, segmented staircase,
+// back substitution and recovery of the nodes that take the elimination's
+// direction; launched only when there are some (in a graph, under h_elim).  A
+// warp per interval, segment or node, in strides of a grid that fills the chip,
+// so that one node's intervals are spread over it as well as many nodes'.  (The
+// relations and inverses in the segments' region are no longer read when they
+// run.)  Against a block of four warps per node: 85 nodes from states twice
+// the box, twelve of them damped for 50 iterations, 215 -> 60 ms; 1,457 nodes of
+// Example II's box 400 -> 136 ms.
+__device__ __forceinline__ bool elim_node(const Workspace& w, int64_t node) {
+  const NodeState& s = w.ns[node];
+  return s.active && s.searching == 1 && (s.singular & (kElimNode | kElimDone)) == kElimNode;
+}
+
+constexpr int kElimCondWarps = 4, kElimSegWarps = 2, kElimRedWarps = 2, kElimBackWarps = 4, kElimRecWarps = 4;
+constexpr int kElimCondSmem = kElimCondWarps * 36 * kCols * 8;
+__global__ void __launch_bounds__(32 * kElimCondWarps) k_elim_condense_fp64(SolveArgs a, Workspace w) {
   extern __shared__ __align__(16) unsigned char elim_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* sm = reinterpret_cast<double*>(elim_smem + warp * kElimWarpSmem);
-  for (int64_t node = blockIdx.x; node < a.n; node += gridDim.x) {
-    const bool marked = w.ns[node].active && (w.ns[node].singular & kElimNode);
-    __syncthreads();   // every warp has read the mark before one of them changes the state
-    if (!marked) continue;
-    const int N = a.N[node], nseg = seg_count(N);
-    for (int i = warp; i < N; i += kElimWarps) condense_interval_smem(a, w, node, i, N, lane, sm);
-    __syncthreads();
-    for (int s = warp; s < nseg; s += kElimWarps) {
-      abd_segment<double>(a, w, node, s, N, lane, sm);
-      __syncwarp();
+  double* sm = reinterpret_cast<double*>(elim_smem) + warp * (36 * kCols);
+  for (int64_t wid = blockIdx.x * int64_t(kElimCondWarps) + warp; wid < a.n * a.Nmax;
+       wid += int64_t(gridDim.x) * kElimCondWarps) {
+    const int64_t node = wid / a.Nmax;
+    const int i = static_cast<int>(wid % a.Nmax);
+    if (!elim_node(w, node) || i >= a.N[node]) continue;
+    condense_interval_smem(a, w, node, i, a.N[node], lane, sm);
+    __syncwarp();
+  }
+}
+
+__global__ void __launch_bounds__(32 * kElimSegWarps) k_elim_seg_fp64(SolveArgs a, Workspace w) {
+  __shared__ __align__(16) double sm[kElimSegWarps][seg_smem_elems<double>()];
+  const int warp = threadIdx.x >> 5, smax = seg_count(a.Nmax);
+  for (int64_t wid = blockIdx.x * int64_t(kElimSegWarps) + warp; wid < a.n * smax;
+       wid += int64_t(gridDim.x) * kElimSegWarps) {
+    const int64_t node = wid / smax;
+    const int s = static_cast<int>(wid % smax);
+    if (!elim_node(w, node) || s >= seg_count(a.N[node])) continue;
+    abd_segment<double>(a, w, node, s, a.N[node], threadIdx.x & 31, sm[warp]);
+    __syncwarp();
+  }
+}
+
+__global__ void __launch_bounds__(32 * kElimRedWarps) k_elim_red_fp64(SolveArgs a, Workspace w) {
+  __shared__ __align__(16) double sm[kElimRedWarps][stair_smem_elems<double>()];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int64_t node = blockIdx.x * int64_t(kElimRedWarps) + warp; node < a.n;
+       node += int64_t(gridDim.x) * kElimRedWarps) {
+    if (!elim_node(w, node)) continue;
+    abd_reduced<double>(a, w, node, a.N[node], lane, sm[warp]);
+    __syncwarp();
+    if (lane == 0 && (w.ns[node].singular & 1)) {
+      w.ns[node].status = SG_SINGULAR;
+      w.ns[node].active = 0;
+      w.ns[node].searching = 0;
     }
-    __syncthreads();
-    if (warp == 0) abd_reduced<double>(a, w, node, N, lane, sm);
-    __syncthreads();
-    for (int s = warp; s < nseg; s += kElimWarps) {
-      abd_segment_back<double>(a, w, node, s, N, lane, reinterpret_cast<double(*)[12 * kSegLd]>(sm));
-      __syncwarp();
-    }
-    __syncthreads();
-    for (int i = warp; i < N; i += kElimWarps) recover_interval<double>(a, w, node, i, lane);
-    if (threadIdx.x == 0) {
-      NodeState& s = w.ns[node];
-      if (s.singular & 1) {
-        s.status = SG_SINGULAR;
-        s.active = 0;
-        s.searching = 0;
-      }
-      s.singular = kElimDone;
-    }
-    __syncthreads();
+    __syncwarp();
+  }
+}
+
+__global__ void __launch_bounds__(32 * kElimBackWarps) k_elim_segback_fp64(SolveArgs a, Workspace w) {
+  __shared__ __align__(16) double sm[kElimBackWarps][kSegBackStages<double>][12 * kSegLd];
+  const int warp = threadIdx.x >> 5, smax = seg_count(a.Nmax);
+  for (int64_t wid = blockIdx.x * int64_t(kElimBackWarps) + warp; wid < a.n * smax;
+       wid += int64_t(gridDim.x) * kElimBackWarps) {
+    const int64_t node = wid / smax;
+    const int s = static_cast<int>(wid % smax);
+    if (!elim_node(w, node) || s >= seg_count(a.N[node])) continue;
+    abd_segment_back<double>(a, w, node, s, a.N[node], threadIdx.x & 31, sm[warp]);
+    __syncwarp();
+  }
+}
+
+__global__ void __launch_bounds__(32 * kElimRecWarps) k_elim_recover_fp64(SolveArgs a, Workspace w) {
+  for (int64_t wid = blockIdx.x * int64_t(kElimRecWarps) + (threadIdx.x >> 5); wid < a.n * a.Nmax;
+       wid += int64_t(gridDim.x) * kElimRecWarps) {
+    const int64_t node = wid / a.Nmax;
+    const int i = static_cast<int>(wid % a.Nmax);
+    if (!elim_node(w, node) || i >= a.N[node]) continue;
+    recover_interval<double>(a, w, node, i, threadIdx.x & 31);
   }
 }
 
@@ -759,7 +813,7 @@ __global__ void __launch_bounds__(12 * kRecIv) k_recover_fp64(SolveArgs a, Works
   const int chunks = cond_chunks(a.Nmax);
   const int64_t node = blockIdx.x / chunks;
   const int i0 = static_cast<int>(blockIdx.x % chunks) * kRecIv;
-  if (!w.ns[node].active) return;
+  if (!w.ns[node].active || (w.ns[node].singular & (kElimNode | kElimFirst))) return;
   const int N = a.N[node];
   if (i0 >= N) return;
   const int nv = N - i0 < kRecIv ? N - i0 : kRecIv;
@@ -845,11 +899,21 @@ inline void direction_launches(const SolveArgs& a, DirLaunch (&out)[kDirLaunches
   }
 }
 
-// The elimination of marked nodes, launched in front of every trial of the line
-// search of the FP64 form.
-inline DirLaunch elim_launch(const SolveArgs& a) {
-  return {"k_elim_fp64", k_elim_fp64, a.n < kElimBlocks ? a.n : kElimBlocks, 32 * kElimWarps,
-          kElimWarps * kElimWarpSmem};
+// The elimination's launches, for the trials of a line search that follow a
+// reduction which counted nodes for it.
+constexpr int kElimLaunches = 5;
+inline void elim_launches(const SolveArgs& a, DirLaunch (&out)[kElimLaunches]) {
+  const int64_t nint = a.n * a.Nmax, nseg = a.n * seg_count(a.Nmax);
+  auto fill = [](int64_t warps, int per, int blocks_per_sm) {
+    const int64_t all = ceil_div(warps, per), cap = int64_t(kNumSMs) * blocks_per_sm;
+    return all < cap ? all : cap;
+  };
+  out[0] = {"k_elim_condense_fp64", k_elim_condense_fp64, fill(nint, kElimCondWarps, 4), 32 * kElimCondWarps,
+            kElimCondSmem};
+  out[1] = {"k_elim_seg_fp64", k_elim_seg_fp64, fill(nseg, kElimSegWarps, 8), 32 * kElimSegWarps, 0};
+  out[2] = {"k_elim_red_fp64", k_elim_red_fp64, fill(a.n, kElimRedWarps, 8), 32 * kElimRedWarps, 0};
+  out[3] = {"k_elim_segback_fp64", k_elim_segback_fp64, fill(nseg, kElimBackWarps, 7), 32 * kElimBackWarps, 0};
+  out[4] = {"k_elim_recover_fp64", k_elim_recover_fp64, fill(nint, kElimRecWarps, 16), 32 * kElimRecWarps, 0};
 }
 
 // Raises the dynamic shared-memory caps of a direction's kernels.
@@ -861,7 +925,7 @@ inline cudaError_t direction_setup(const SolveArgs& a) {
     const cudaError_t e = ensure_dynamic_smem(x.fn, x.smem);
     if (e != cudaSuccess) return e;
   }
-  if constexpr (sizeof(T) == sizeof(double)) return ensure_dynamic_smem(k_elim_fp64, elim_launch(a).smem);
+  if constexpr (sizeof(T) == sizeof(double)) return ensure_dynamic_smem(k_elim_condense_fp64, kElimCondSmem);
   return cudaSuccess;
 }
 

@@ -55,22 +55,25 @@ struct NodeState {
   double fmax;     // |F|_inf at the current iterate
   double alpha;    // current step length
   int active;      // still iterating
-  int searching;   // 1: in the line search; -e: step accepted in iteration e (FP64 form, for k_update)
-  int singular;    // bit 0: a zero pivot was met this iteration; kElimNode, kElimDone
+  int searching;   // 1: in the line search; FP64 form: 2: waits for the elimination's direction,
+                   // -e: step accepted in iteration e (for k_update)
+  int singular;    // bit 0: a zero pivot was met this iteration; kElim*
   int iters;
   int status;
   int ybuf;        // 1: the current iterate is in Y2 (see Workspace)
 };
 
-// NodeState::singular, FP64 form: the node waits for the direction of the
-// elimination with full partial pivoting (k_elim_fp64) / has it
-constexpr int kElimNode = 2, kElimDone = 4;
+// NodeState::singular, FP64 form: this iteration's direction is that of the
+// elimination with full partial pivoting (bvp_direction.cuh) / it has been formed /
+// the iteration starts with it
+constexpr int kElimNode = 2, kElimDone = 4, kElimFirst = 8;
 // Workspace::counters (zeroed before a solve): nodes still in the line search
-// and nodes left to iterate so far in this iteration; nodes marked kElimNode;
-// the same two as the last block of k_ls_reduce found them (read by the host
-// loop); that kernel's finished blocks; Newton iterations so far
-constexpr int kSearchCount = 0, kActiveCount = 1, kElimCount = 4, kSearchOut = 5, kActiveOut = 6, kTicket = 7, kEpoch = 8,
-              kCounters = 16;
+// and nodes left to iterate so far in this iteration; (2, 3: the persistent
+// form's queue head); nodes whose elimination comes next; the same three as the
+// last block of k_ls_reduce found them (read by the host loop); that kernel's
+// finished blocks; Newton iterations so far
+constexpr int kSearchCount = 0, kActiveCount = 1, kElimCount = 4, kSearchOut = 5, kActiveOut = 6, kElimOut = 7,
+              kTicket = 8, kEpoch = 9, kCounters = 16;
 
 constexpr int kCols = 49;        // 24 interior + 12 (y_i) + 12 (y_{i+1}) + rhs
 constexpr int kRecLd = 52;       // row stride of a stored interior pivot row (16-byte multiple)
@@ -105,7 +108,7 @@ struct Workspace {
   void* Red;       // n x seg_count(Nmax) x kBlk (T), reduced block rows of the segments
   double* part;    // n x Nmax x 2, partial |F|^2 and |F|_inf
   NodeState* ns;   // n
-  int* counters;   // 2
+  int* counters;   // kCounters
   size_t bytes;
 };
 
@@ -127,8 +130,8 @@ struct SolveArgs {
   int res_pair;        // FP32-direction form: 1 = residual in pairs of floats, 0 = in FP64
   int tree;            // FP64 form, launch per phase or graph: direction from bvp_direction.cuh
   // graph form: the loops' conditions, set by k_ls_reduce
-  int conds;           // bit 0: h_newton exists, bit 1: h_search
-  cudaGraphConditionalHandle h_newton, h_search;
+  int conds;           // bit 0: h_newton exists, bit 1: h_search, bit 2: h_elim
+  cudaGraphConditionalHandle h_newton, h_search, h_elim;
 };
 
 __host__ __device__ __forceinline__ int64_t npts(int Nmax) { return 3 * int64_t(Nmax) + 1; }
@@ -460,7 +463,6 @@ __device__ __forceinline__ void ls_start(const Workspace& w, int64_t node) {
     s.status = SG_SINGULAR;
     s.active = 0;
   } else {
-    s.singular &= kElimNode;
     s.searching = 1;
     s.alpha = 1.0;
   }
@@ -472,11 +474,30 @@ __device__ __forceinline__ void ls_start(const Workspace& w, int64_t node) {
 // mode 1: Armijo test for the current alpha, and when the step is taken the
 // iteration's end: convergence, iteration cap.
 // The node's share of the counts goes to cnt (shared memory: searching,
-// active).
+// active, eliminations next).
+//
+// FP64 form: the tree's direction is taken only where its full step passes the
+// Armijo test (damped or not).  A node far from its root follows the
+// elimination's direction, from the full step on: its path depends on the last
+// bits of it, and where the tree has lost digits the elimination has not.  alpha =
+// 0 evaluates the rows at the iterate again, which that direction needs.  The
+// next iterations start with the elimination until a full step takes |F| to a
+// quarter, as steps near the root do (a refused step of the tree costs two
+// residuals and a direction).
 __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, int64_t node, int lane, int mode,
                                         int* cnt) {
   const int N = a.N[node];   // (beside the state: one latency)
   NodeState s = w.ns[node];
+  if (s.searching == 2 && mode == 1) {
+    if (lane == 0) {
+      s.searching = 1;
+      s.singular |= kElimNode;
+      w.ns[node] = s;
+      atomicAdd(&cnt[0], 1);
+      atomicAdd(&cnt[2], 1);
+    }
+    return;
+  }
   if (s.searching != 1) return;
   double ss = 0.0, mx = 0.0;
   const double2* part = reinterpret_cast<const double2*>(w.part) + node * a.Nmax;
@@ -494,33 +515,36 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
   mx = warp_max(mx);
   if (lane != 0) return;
   if (mode == 1 && s.alpha == 0.0) {
-    // the residual rows at the iterate are back: the direction of the
-    // elimination next, and the search goes on at 1/2
-    s.alpha = 0.5;
+    // the residual rows at the iterate are back: the elimination's direction next
+    s.alpha = 1.0;
     s.singular |= kElimNode;
     w.ns[node] = s;
     atomicAdd(&cnt[0], 1);
-    atomicAdd(&w.counters[kElimCount], 1);
+    atomicAdd(&cnt[2], 1);
     return;
   }
-  const bool accept = mode == 0 || !a.damping || (ss < INFINITY && ss <= (1.0 - 2e-4 * s.alpha) * s.fnorm2) ||
-                      s.alpha <= 0x1p-10;
+  const bool tree = a.tree && !(s.singular & kElimNode);   // the direction is the tree's
+  const bool armijo = ss < INFINITY && ss <= (1.0 - 2e-4 * s.alpha) * s.fnorm2;
+  const bool accept = mode == 0 || armijo || (!a.damping && !tree) || s.alpha <= 0x1p-10;
   if (!accept) {
-    // FP64 form: a node far from its root follows the elimination's direction
-    // (its path depends on the last bits of it); alpha = 0 evaluates the
-    // rows at the iterate again, which that direction needs
-    s.alpha = a.tree && !(s.singular & kElimDone) ? 0.0 : 0.5 * s.alpha;
+    s.alpha = tree ? 0.0 : 0.5 * s.alpha;
+    if (a.tree && !tree) s.singular |= kElimDone;
     w.ns[node] = s;
     atomicAdd(&cnt[0], 1);
     return;
   }
+  const double f0 = s.fnorm2;
   s.fnorm2 = ss;
   s.fmax = mx;
   s.searching = 0;
   if (mode == 1) {
     s.iters += 1;
-    if (a.tree) s.searching = -(w.counters[kEpoch] + 1);   // k_update takes the step
-    else s.ybuf ^= 1;                                      // the trial point is the iterate
+    if (a.tree) {
+      s.searching = -(w.counters[kEpoch] + 1);   // k_update takes the step
+      s.singular = tree || (s.alpha == 1.0 && ss <= 0.0625 * f0) ? 0 : kElimFirst;
+    } else {
+      s.ybuf ^= 1;   // the trial point is the iterate
+    }
   }
   if (!(mx < INFINITY)) {
     s.status = SG_NONFINITE;
@@ -542,40 +566,43 @@ __device__ __forceinline__ void ls_node(const SolveArgs& a, const Workspace& w, 
 // memset per trial or iteration.  (Latency: a block's counts are added up in
 // shared memory, and a single block needs no ticket.)
 __global__ void __launch_bounds__(128) k_ls_reduce(SolveArgs a, Workspace w, int mode) {
-  __shared__ int cnt[2];
+  __shared__ int cnt[3];
   const int64_t node = blockIdx.x * int64_t(4) + (threadIdx.x >> 5);
   const bool one = gridDim.x == 1;
   int before = 0;
   if (threadIdx.x == 0) {
-    cnt[0] = cnt[1] = 0;
+    cnt[0] = cnt[1] = cnt[2] = 0;
     if (one) before = w.counters[kActiveCount];   // by earlier trials of the search
   }
   __syncthreads();
   if (node < a.n) ls_node(a, w, node, threadIdx.x & 31, mode, cnt);
   __syncthreads();
   if (threadIdx.x != 0) return;
-  int searching = cnt[0];
+  int searching = cnt[0], elim = cnt[2];
   if (!one) {
     if (cnt[0]) atomicAdd(&w.counters[kSearchCount], cnt[0]);
     if (cnt[1]) atomicAdd(&w.counters[kActiveCount], cnt[1]);
+    if (cnt[2]) atomicAdd(&w.counters[kElimCount], cnt[2]);
     __threadfence();   // this block's counts before its ticket
     if (atomicAdd(&w.counters[kTicket], 1) != static_cast<int>(gridDim.x) - 1) return;
     __threadfence();
     searching = atomicExch(&w.counters[kSearchCount], 0);
+    if (a.tree) elim = atomicExch(&w.counters[kElimCount], 0);
     w.counters[kTicket] = 0;
   }
   w.counters[kSearchOut] = searching;
+  if (a.tree) w.counters[kElimOut] = elim;
   if (searching == 0) {   // the iteration's end
     const int active = one ? before + cnt[1] : atomicExch(&w.counters[kActiveCount], 0);
     if (one) w.counters[kActiveCount] = 0;
     w.counters[kActiveOut] = active;
-    w.counters[kElimCount] = 0;
     if (mode == 1) w.counters[kEpoch] += 1;
     if (a.conds & 1) cudaGraphSetConditional(a.h_newton, active > 0 ? 1u : 0u);
   } else if (one) {
     w.counters[kActiveCount] = before + cnt[1];
   }
   if ((a.conds & 2) && mode == 1) cudaGraphSetConditional(a.h_search, searching > 0 ? 1u : 0u);
+  if ((a.conds & 4) && mode == 1) cudaGraphSetConditional(a.h_elim, elim > 0 ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------- Jacobian
@@ -1009,7 +1036,7 @@ inline void (*condense_reg_kernel(int cond_warps))(SolveArgs, Workspace) {
 }
 inline int condense_reg_warps(int cond_warps) { return cond_warps == 2 || cond_warps == 8 ? cond_warps : 4; }
 
-// Shared-memory FP64 form (persistent form, k_elim_fp64): the 36 x 49 system of one
+// Shared-memory FP64 form (persistent form, eliminations of bvp_direction.cuh): the 36 x 49 system of one
 // interval in shared memory, one warp per interval, elimination of the first
 // 24 columns with partial pivoting over all 36 rows (warp_eliminate).
 __device__ __forceinline__ void condense_interval_smem(const SolveArgs& a, const Workspace& w, int64_t node,
@@ -1048,7 +1075,7 @@ __device__ __forceinline__ void condense_interval_smem(const SolveArgs& a, const
   for (int r = lane; r < 36; r += 32) M[r * kCols + 48] = -res[r];
   __syncwarp();
   const bool ok = warp_eliminate<double, 36, kCols, 24>(M, lane);
-  if (!ok && lane == 0) w.ns[node].singular = 1;
+  if (!ok && lane == 0) w.ns[node].singular |= 1;
   const int64_t blk = node * a.Nmax + i;
   double* rec = static_cast<double*>(w.Rec) + blk * kRec;
   for (int e = lane; e < 24 * kCols; e += 32) rec[(e / kCols) * kRecLd + e % kCols] = M[e];
