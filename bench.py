@@ -47,6 +47,7 @@ N_QUERIES = 1_000_000
 E2E_EVAL_CHUNKS = 4        # e2e step: evaluation calls whose results go down while the next evaluates
 TOL = 1e-8
 SEG_LEN = 16   # intervals per segment of the library's segmented staircase
+LEAF_LEN = 16  # intervals per block of the FP64 tree's leaf kernel
 
 # dram__bytes_read.sum + dram__bytes_write.sum per unit of work from an ncu
 # capture of the kernel as it stands (the 600-node solve case: the first Newton
@@ -106,11 +107,27 @@ def flops_condense_fp64_interval() -> float:
     return 2.0 * (12 ** 3 + 4 * 12 * 93 + 12 * 12 * 11 + 12 * sum(24 - k for k in range(12)) + 11 * 144)
 
 
-def flops_tree_interval() -> float:
+def flops_compose() -> float:
     """One composition of two scattering relations (13 columns: the product with
-    B1, the 6 x 6 elimination, the products with A2 | C2 and with D1), and the
-    12 x 13 product on the way down."""
-    return 2.0 * (13 * (36 + 45 + 72 + 36) + 12 * 13)
+    B1, the 6 x 6 elimination, the products with A2 | C2 and with D1)."""
+    return 2.0 * 13 * (36 + 45 + 72 + 36)
+
+
+def flops_tree_down() -> float:
+    """The 12 x 13 product at a mesh point on the way down the tree."""
+    return 2.0 * 12 * 13
+
+
+def flops_point_fp64() -> float:
+    """FP64 Jacobian at a collocation point: 644 FP64 instructions (counted by
+    ncu), each with the pipe's time of a multiply-add."""
+    return 2.0 * 644
+
+
+def bytes_update() -> float:
+    """Per collocation point: read the iterate and the direction, write the
+    iterate (12 f64 each)."""
+    return 3 * 12 * 8
 
 
 def flops_recover_fp64_interval() -> float:
@@ -122,11 +139,6 @@ def flops_recover_fp64_interval() -> float:
 def flops_recover_interval() -> float:
     """Per interval: 24 x 24 product and 24 x 24 triangular solve."""
     return 2 * 576 + 576 + 24
-
-
-def bytes_point(tsize: int) -> float:
-    """Per collocation point: read y (12 f64), write F (12 f64) and J (144 x tsize)."""
-    return 12 * 8 + 12 * 8 + 144 * tsize
 
 
 def flops_eval_query(M: int, k: int) -> float:
@@ -856,28 +868,33 @@ def roofline(kt, iters, N_h, M, prec, nq=N_QUERIES, peaks=None):
     measured = bool(peaks.get("fp32_tflops")) and bool(peaks.get("fp64_tflops"))
     fp32 = prec != 0   # any form but SG_PREC_FP64 runs the direction in FP32
     suffix = "_fp32" if fp32 else "_fp64"
-    tsize = 4 if fp32 else 8
     peak_lin = pk32 if fp32 else pk64
     int_units = float(np.sum(iters * N_h))           # interval-iterations per solve
     pt_units = float(np.sum(iters * (3 * N_h + 1)))  # point-iterations per solve
     seg = -(-N_h // SEG_LEN)                            # segments per node
     seg_units = float(np.sum(iters * (N_h - seg)))      # interior segment points (panels)
     red_units = float(np.sum(iters * seg))              # reduced block rows
+    # FP64 tree: blocks of 16 intervals do their own compositions where the leaf
+    # kernel runs (few nodes), the tree the ones above (and the closing one)
+    leaf_units = float(np.sum(iters * (N_h - -(-N_h // LEAF_LEN)))) if "k_tree_leaf_fp64" in kt else 0.0
     steps_timed = None
     models = {
-        "k_condense" + suffix: ("alu", flops_condense_interval() * int_units, peak_lin, "TFLOP/s"),
         "k_condense_reg_fp32": ("alu", flops_condense_interval() * int_units, pk32, "TFLOP/s"),
-        "k_abd" + suffix: ("alu", flops_abd_interval() * int_units, peak_lin, "TFLOP/s"),
-        "k_abd_seg" + suffix: ("alu", flops_abd_seg_interval() * seg_units, peak_lin, "TFLOP/s"),
-        "k_abd_red" + suffix: ("alu", flops_abd_interval() * red_units, peak_lin, "TFLOP/s"),
-        "k_abd_segback" + suffix: ("alu", flops_abd_segback_interval() * seg_units, peak_lin, "TFLOP/s"),
+        "k_abd_seg_fp32": ("alu", flops_abd_seg_interval() * seg_units, pk32, "TFLOP/s"),
+        "k_abd_red_fp32": ("alu", flops_abd_interval() * red_units, pk32, "TFLOP/s"),
+        "k_abd_segback_fp32": ("alu", flops_abd_segback_interval() * seg_units, pk32, "TFLOP/s"),
         "k_recover" + suffix: ("alu", (flops_recover_interval() if fp32 else flops_recover_fp64_interval()) * int_units,
                                peak_lin, "TFLOP/s"),
         "k_newton_persistent" + suffix: ("alu", (flops_condense_interval() + flops_abd_interval()
                                                   + flops_recover_interval()) * int_units, peak_lin, "TFLOP/s"),
-        "k_point" + suffix: ("hbm", bytes_point(tsize) * pt_units, None, "GB/s"),
+        "k_update": ("hbm", bytes_update() * pt_units, None, "GB/s"),
+        "k_point_fp64": ("alu", flops_point_fp64() * pt_units, pk64, "TFLOP/s"),
         "k_condense_fp64": ("alu", flops_condense_fp64_interval() * int_units, pk64, "TFLOP/s"),
-        "k_tree_fp64": ("alu", flops_tree_interval() * int_units, pk64, "TFLOP/s"),
+        "k_tree_leaf_fp64": ("alu", flops_compose() * leaf_units, pk64, "TFLOP/s"),
+        "k_tree_fp64": ("alu", flops_compose() * (int_units - leaf_units) + flops_tree_down() * int_units, pk64,
+                        "TFLOP/s"),
+        # a condensation that eliminates every interval in FP64 (the k_elim kernels do so for the nodes whose
+        # step is refused, whose number is not known here)
         "k_condense_smem_fp64": ("alu", flops_condense_interval() * int_units, pk64, "TFLOP/s"),
         # the interpolant: the method's M (2k + 1) flops per query whatever the
         # arithmetic (pairs of floats and split TF32 do more operations)
