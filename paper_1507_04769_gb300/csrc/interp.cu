@@ -324,29 +324,30 @@ __global__ void __launch_bounds__(32 * kNestRanges, 1) k_eval_fp64_nested(EvalAr
 // children (lists are padded) is loaded while the one before is summed.
 constexpr int kFewBatch = 4, kFewThreads = 512;   // (or 256 threads)
 
-constexpr size_t kFewSmem = 200 * 1024;
+constexpr size_t kFewSmem = 220 * 1024;
 struct FewLayout {   // byte offsets in shared memory after the tables
   size_t val, W, child, ent, total;
 };
-__host__ __device__ inline FewLayout few_layout(const EvalArgs& e, int d, int kc, int QB, bool staged) {
+// kv columns at a time
+__host__ __device__ inline FewLayout few_layout(const EvalArgs& e, int d, int kv, int QB, bool staged) {
   auto up = [](size_t x) { return (x + 15) & ~size_t(15); };
   FewLayout L;
   L.val = up(sizeof(double) * d * e.nf * QB);
   // (first the rows' reciprocals, factors, coordinates and hits)
   const size_t rows = (sizeof(double) * ((size_t(1) << e.level) + 1 + e.level + 1) + sizeof(int)) * d * QB;
-  const size_t vals = sizeof(double) * (e.fheight[kMaxDim + 1] + 1) * kc * QB;
+  const size_t vals = sizeof(double) * (e.fheight[kMaxDim + 1] + 1) * kv * QB;
   L.W = L.val + up(rows > vals ? rows : vals);
-  L.child = L.W + (staged ? up(sizeof(double) * e.nrows * kc) : 0);
+  L.child = L.W + (staged ? up(sizeof(double) * e.nrows * kv) : 0);
   L.ent = L.child + (staged ? up(sizeof(uint32_t) * e.nchild) : 0);
   L.total = L.ent + (staged ? sizeof(int4) * e.fheight[kMaxDim + 1] : 0);
   return L;
 }
 
 template <int QB, bool kStaged>
-__global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, int d, int c0, int kc) {
-  extern __shared__ __align__(16) double tabs_s[];   // [d * nf][QB], values of the entries [entry][kc][QB], node data
+__global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, int d, int c0, int kc, int kv) {
+  extern __shared__ __align__(16) double tabs_s[];   // [d * nf][QB], values of the entries [entry][kv][QB], node data
   char* sm = reinterpret_cast<char*>(tabs_s);
-  const FewLayout at = few_layout(e, d, kc, QB, kStaged);
+  const FewLayout at = few_layout(e, d, kv, QB, kStaged);
   double* val = reinterpret_cast<double*>(sm + at.val);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int64_t q0 = blockIdx.x * int64_t(QB);
@@ -364,14 +365,9 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, in
     };
     copy16(at.child, e.fchild, e.nchild / 4);
     copy16(at.ent, e.fent, nent);
-    double* Ws = reinterpret_cast<double*>(sm + at.W);
-    if (kc == e.k) {   // (the array is padded to whole words)
-      copy16(at.W, e.Wt, (e.nrows * kc + 1) / 2);
-    } else {
-      for (int i = tid; i < e.nrows * kc; i += nt) Ws[i] = W[int64_t(i / kc) * e.k + i % kc];
-    }
-    W = Ws;
-    ldw = kc;
+    if (kv == e.k) copy16(at.W, e.Wt, (e.nrows * kv + 1) / 2);   // (the array is padded to whole words)
+    W = reinterpret_cast<const double*>(sm + at.W);
+    ldw = kv;
     child = reinterpret_cast<const uint4*>(sm + at.child);
     ent = reinterpret_cast<const int4*>(sm + at.ent);
   }
@@ -415,53 +411,65 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_eval_fp64_few(EvalArgs e, in
   }
   __syncthreads();
   // a list's padding: entry nent with factor 1, v + 1 * -0 = v for every v
-  for (int i = tid; i < kc * QB; i += nt) val[nent * kc * QB + i] = -0.0;
+  for (int i = tid; i < kv * QB; i += nt) val[nent * kv * QB + i] = -0.0;
   if constexpr (kStaged) asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  for (int h = 0; h < kMaxDim + 1; ++h) {
-    const int n = (e.fheight[h + 1] - e.fheight[h]) * kc * QB;
-    if (n == 0) continue;
-    for (int item = tid; item < n; item += nt) {
-      const int t = item / QB, q = item % QB, c = t % kc, en = e.fheight[h] + t / kc;
-      const int4 E = ent[en];
-      double v = W[E.z * ldw + c];
-      const uint4* ch = child + E.x / 4;
-      double p[kFewBatch], w[kFewBatch];
-      uint4 x4 = ch[0];
-      auto load = [&]() {
-        const uint32_t x[kFewBatch] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-        for (int j = 0; j < kFewBatch; ++j) {
-          p[j] = tabs_s[(x[j] & 0xFFFu) * QB + q];
-          w[j] = *((x[j] & 0x1000u) ? val + ((x[j] >> 13) * kc + c) * QB + q : W + (x[j] >> 13) * ldw + c);
-        }
-      };
-      if (E.y > 0) load();
-      x4 = ch[1];   // (past the last list: padding)
-      for (int i = 0; i < E.y; i += kFewBatch) {
-        double p0[kFewBatch], w0[kFewBatch];
-#pragma unroll
-        for (int j = 0; j < kFewBatch; ++j) {
-          p0[j] = p[j];
-          w0[j] = w[j];
-        }
-        if (i + kFewBatch < E.y) {
-          load();
-          x4 = ch[i / 4 + 2];
-        }
-#pragma unroll
-        for (int j = 0; j < kFewBatch; ++j)
-          v = fma(p0[j], w0[j], v);
+  for (int b = 0; b < kc; b += kv) {
+    const int kn = min(kv, kc - b);
+    if constexpr (kStaged) {
+      if (kv != e.k) {   // this pass's columns
+        double* Ws = reinterpret_cast<double*>(sm + at.W);
+        for (int i = tid; i < e.nrows * kn; i += nt) Ws[i / kn * kv + i % kn] = e.Wt[int64_t(i / kn) * e.k + c0 + b + i % kn];
+        __syncthreads();
       }
-      val[(en * kc + c) * QB + q] = v;
     }
-    __syncthreads();
-  }
-  for (int t = tid; t < QB * kc; t += nt) {
-    const int q = t / kc, c = t % kc;
-    if (q0 + q >= e.Q) break;
-    e.out[(q0 + q) * e.k + c0 + c] =
-        range_sum([&](int r) { return val[(e.froot[r] * kc + c) * QB + q]; }, e.per);
+    const double* Wb = kStaged ? W : W + b;
+    for (int h = 0; h < kMaxDim + 1; ++h) {
+      const int n = (e.fheight[h + 1] - e.fheight[h]) * kn * QB;
+      if (n == 0) continue;
+      for (int item = tid; item < n; item += nt) {
+        const int t = item / QB, q = item % QB, c = t % kn, en = e.fheight[h] + t / kn;
+        const int4 E = ent[en];
+        double v = Wb[E.z * ldw + c];
+        const uint4* ch = child + E.x / 4;
+        double p[kFewBatch], w[kFewBatch];
+        uint4 x4 = ch[0];
+        auto load = [&]() {
+          const uint32_t x[kFewBatch] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+          for (int j = 0; j < kFewBatch; ++j) {
+            p[j] = tabs_s[(x[j] & 0xFFFu) * QB + q];
+            w[j] = *((x[j] & 0x1000u) ? val + ((x[j] >> 13) * kv + c) * QB + q : Wb + (x[j] >> 13) * ldw + c);
+          }
+        };
+        if (E.y > 0) load();
+        x4 = ch[1];   // (past the last list: padding)
+        for (int i = 0; i < E.y; i += kFewBatch) {
+          double p0[kFewBatch], w0[kFewBatch];
+#pragma unroll
+          for (int j = 0; j < kFewBatch; ++j) {
+            p0[j] = p[j];
+            w0[j] = w[j];
+          }
+          if (i + kFewBatch < E.y) {
+            load();
+            x4 = ch[i / 4 + 2];
+          }
+#pragma unroll
+          for (int j = 0; j < kFewBatch; ++j)
+            v = fma(p0[j], w0[j], v);
+        }
+        val[(en * kv + c) * QB + q] = v;
+      }
+      __syncthreads();
+    }
+    for (int t = tid; t < QB * kn; t += nt) {
+      const int q = t / kn, c = t % kn;
+      if (q0 + q >= e.Q) break;
+      e.out[(q0 + q) * e.k + c0 + b + c] =
+          range_sum([&](int r) { return val[(e.froot[r] * kv + c) * QB + q]; }, e.per);
+    }
+    if (b + kv < kc) __syncthreads();   // the entries' values are read
   }
 }
 
@@ -483,31 +491,36 @@ static int launch_eval_fp64_nested(const EvalArgs& e, int d, int c0, cudaStream_
 }
 
 template <int QB>
-static int launch_eval_fp64_few(const EvalArgs& e, int d, int c0, int kc, int nt, cudaStream_t st) {
-  const bool staged = few_layout(e, d, kc, QB, true).total <= kFewSmem;
-  const size_t smem = few_layout(e, d, kc, QB, staged).total;
+static int launch_eval_fp64_few(const EvalArgs& e, int d, int c0, int kc, int nt, cudaStream_t st, int kv = 0) {
+  if (kv == 0) kv = kc;
+  const bool staged = few_layout(e, d, kv, QB, true).total <= kFewSmem;
+  const size_t smem = few_layout(e, d, kv, QB, staged).total;
   auto* kern = staged ? k_eval_fp64_few<QB, true> : k_eval_fp64_few<QB, false>;
   SG_CUDA_TRY(ensure_dynamic_smem(kern, smem));
-  SG_TIMED("k_eval_fp64_few", st, (kern<<<static_cast<unsigned>(ceil_div(e.Q, QB)), nt, smem, st>>>(e, d, c0, kc)));
+  SG_TIMED("k_eval_fp64_few", st, (kern<<<static_cast<unsigned>(ceil_div(e.Q, QB)), nt, smem, st>>>(e, d, c0, kc, kv)));
   SG_LAUNCH_CHECK("k_eval_fp64_few");
   return SG_OK;
 }
 
 // K columns from c0 on.  The nested form comes in blocks of 32 queries, one SM's
 // work at least.  Below a wave of them, the fewest queries per block that fill one
-// wave: two blocks of 256 threads or one of 512 per SM.  Measured (K = 3, d = 6,
-// us on the level-4 and level-5 grid): 1 query 13.8 / 22.8,
-// 304: 16.3 / 44, 608: 16.8 / 44, 1,216: 23 / 70, 1,824: 34 / 111, 2,432: 34 / -;
-// nested, up to a wave: 50.7 / 134.
+// wave: two blocks of 256 threads or one of 512 per SM, by what fits in shared
+// memory (16 queries: a column at a time where the entries' values of all do
+// not).  Measured (K = 3, d = 6, us on the level-4 and level-5 grid): 1 query 13.6 /
+// 22.4, 304: 16.3 / 26.2, 608: 17.1 / 43.9, 1,216: 23.2 / 68.5, 2,432: 33.7 / 108;
+// nested, up to a wave: 51.0 / 134.
 template <int K>
 static int launch_eval_fp64(const EvalArgs& e, int d, int c0, cudaStream_t st) {
   const int kc = e.k - c0 < K ? e.k - c0 : K;
-  if (e.Q <= 2 * kNumSMs) return launch_eval_fp64_few<1>(e, d, c0, kc, 256, st);
+  auto fits16 = [&](int kv) { return few_layout(e, d, kv, 16, false).total <= kFewSmem; };
+  const size_t one = few_layout(e, d, kc, 1, true).total;   // two staged blocks per SM, or one
+  const bool two = one <= kFewSmem / 2 || one > kFewSmem;
+  if (e.Q <= (two ? 2 : 1) * kNumSMs) return launch_eval_fp64_few<1>(e, d, c0, kc, 256, st);
+  if (e.Q <= 2 * kNumSMs) return launch_eval_fp64_few<2>(e, d, c0, kc, 512, st);
   if (e.Q <= 4 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 512, st);
   if (e.Q <= 8 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 256, st);
-  if (e.Q <= 16 * kNumSMs && few_layout(e, d, kc, 16, false).total <= kFewSmem)
-    return launch_eval_fp64_few<16>(e, d, c0, kc, 512, st);
-  if (e.Q <= 12 * kNumSMs) return launch_eval_fp64_few<4>(e, d, c0, kc, 512, st);
+  if (e.Q <= 16 * kNumSMs && fits16(kc)) return launch_eval_fp64_few<16>(e, d, c0, kc, 512, st);
+  if (e.Q <= 16 * kNumSMs && fits16(1)) return launch_eval_fp64_few<16>(e, d, c0, kc, 512, st, 1);
   return launch_eval_fp64_nested<K>(e, d, c0, st);
 }
 

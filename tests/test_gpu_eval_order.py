@@ -14,7 +14,7 @@ from paper_1507_04769_gb300 import serving, sg  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
-COUNTS = [1, 5, 31, 304, 305, 608, 609, 1216, 1217, 1824, 1825, 2432, 2433, 4864, 4865, 9728, 9729, 14593, 19457]
+COUNTS = [1, 5, 31, 152, 153, 304, 305, 608, 609, 1216, 1217, 1824, 1825, 2432, 2433, 4864, 4865, 9728, 9729, 14593, 19457]
 
 
 @pytest.mark.parametrize("d,L,k", [(6, 4, 3), (6, 5, 3), (6, 2, 7), (8, 3, 6), (1, 6, 2), (5, 0, 1), (2, 5, 16)])
