@@ -44,7 +44,7 @@ inline int cuda_fail(cudaError_t e, const char* where) {
 // cap below another thread's launch.
 template <typename F>
 inline cudaError_t ensure_dynamic_smem(F* func, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
+  if (bytes <= 40 * 1024) return cudaSuccess;   // (48 KB need no cap; up to 8 KB of them may be static)
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

@@ -33,3 +33,21 @@ def test_partial_controls_keep_53_bits(n, mode):
                                   keep_trajectory=True)
     u = out["ctrl"][:, 0].cpu().numpy()
     assert np.all(u == 1.0 + 2.0 ** -25 + 2.0 ** -52)
+
+
+@pytest.mark.parametrize("mode", [sg.EVAL_FP64, sg.EVAL_DF32], ids=["fp64", "df32"])
+@pytest.mark.parametrize("level", [4, 5])
+def test_block_forms_where_shared_memory_is_fullest(level, mode):
+    """Level 4 keeps its nodes in shared memory beside one, two or four trajectories'
+    tables (48 KB with the static part), level 5 reads them from global memory:
+    every form launches and gives the same bits."""
+    g = sg.Grid(6, level, LO, HI)
+    v = -(g.coords[:, :3] + 2.0 * g.coords[:, 3:])
+    S = sg.Surplus(g, v.contiguous())
+    prob = sg.problem_from(synth.attitude_params(1))
+    x0 = torch.as_tensor(synth.uniform_queries(700, LO, HI, seed=12), device="cuda")
+    full = sg.simulate_closed_loop(prob, S, x0, 3, 0.01, mode=mode)
+    for n in (2, 400):
+        part = sg.simulate_closed_loop(prob, S, x0[:n].contiguous(), 3, 0.01, mode=mode)
+        for key in ("xT", "cost"):
+            assert torch.equal(part[key], full[key][:n]), (n, key)
